@@ -698,7 +698,7 @@ static sparsepr_status_t attend_impl(const sparsepr_plan_t* p, const void* Q, co
     tm.mark(SPARSEPR_STAGE_PROBE_ROWS);
     FitArgs fa{};
     fa.BH = r.BH; fa.M = r.M; fa.d = r.d; fa.r_out = r.r_out; fa.full_rank = r.full_rank; fa.lambda = r.lambda; fa.eps_std = r.eps_std; fa.precise = r.dtype == SPARSEPR_F32;
-    fa.X = w.X; fa.Dn = w.Dn; fa.w = p->probe_w; fa.scratch = w.fit; fa.eig_ws = w.fit_eigws; fa.A = w.A; fa.c = w.c; fa.Psi = w.Psi; fa.err = p->err;
+    fa.X = w.X; fa.Dn = w.Dn; fa.w = p->probe_w; fa.scratch = w.fit; fa.eig_ws = w.fit_eigws; fa.A = w.A; fa.c = w.c; fa.At = tensor ? w.At : nullptr; fa.Psi = w.Psi; fa.err = p->err;
     launch_fit(fa, fs);
     tm.mark(SPARSEPR_STAGE_FIT);
   }
@@ -716,7 +716,7 @@ static sparsepr_status_t attend_impl(const sparsepr_plan_t* p, const void* Q, co
     cudaStreamWaitEvent(st, p->ev_join2, 0);
     tm.mark(SPARSEPR_STAGE_ATTENTION);
     if (overlap) { join_side(p, st); p->side_pending = false; }
-    if (fitted && !launch_correction_tc(w.A, w.c, w.At, w.Olo, O, r.os, r.BH, r.H, r.N, p->err, st)) return SPARSEPR_ERR_CUDA;
+    if (fitted && !launch_correction_tc(w.c, w.At, w.Olo, O, r.os, r.BH, r.H, r.N, p->err, st)) return SPARSEPR_ERR_CUDA;
     tm.mark(SPARSEPR_STAGE_CORRECTION);
   } else {
     aa.A = fitted ? w.A : nullptr; aa.c = fitted ? w.c : nullptr;      // correction fused into this kernel's epilogue

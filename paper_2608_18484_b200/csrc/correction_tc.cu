@@ -165,24 +165,6 @@ k_correction_tc(const __grid_constant__ CUtensorMap mapO, const __grid_constant_
   }
 }
 
-// A [BH][128][128] float32 (row k, column n) -> At [2][BH][n][k] bf16: first words, then what their rounding dropped
-__global__ void k_transpose_correction(const float* __restrict__ A, __nv_bfloat16* __restrict__ At) {
-  __shared__ float tile[32][33];
-  const int bh = blockIdx.z;
-  const float* a = A + (i64)bh * 128 * 128;
-  __nv_bfloat16* t = At + (i64)bh * 128 * 128;
-  const int k0 = blockIdx.y * 32, n0 = blockIdx.x * 32;
-  for (int r = threadIdx.y; r < 32; r += 8) tile[r][threadIdx.x] = a[(k0 + r) * 128 + n0 + threadIdx.x];
-  __syncthreads();
-  __nv_bfloat16* tl = At + ((i64)gridDim.z + bh) * 128 * 128;
-  for (int r = threadIdx.y; r < 32; r += 8) {
-    const float x = tile[threadIdx.x][r];
-    const __nv_bfloat16 hb = __float2bfloat16_rn(x);
-    t[(n0 + r) * 128 + k0 + threadIdx.x] = hb;
-    tl[(n0 + r) * 128 + k0 + threadIdx.x] = __float2bfloat16_rn(x - __bfloat162float(hb));
-  }
-}
-
 // Self-test of the bounded wait: one warp waits on an mbarrier that nobody arrives at (no copy in flight, no
 // tensor memory held), with a limit of 2^16 cycles; the wait gives up, the error word receives
 // SPARSEPR_ERR_TIMEOUT, the kernel returns normally and the context stays usable.
@@ -209,11 +191,10 @@ cudaError_t init_correction_tc() {
   return cudaFuncSetAttribute(tc::k_correction_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)tc::CorrSmem::total);
 }
 
-bool launch_correction_tc(const float* A, const float* c, __nv_bfloat16* At, const void* O_lo, void* O, const i64* os, int BH,
+bool launch_correction_tc(const float* c, const __nv_bfloat16* At, const void* O_lo, void* O, const i64* os, int BH,
                           int H, int N, int* err, cudaStream_t st) {
   using namespace tc;
   CUtensorMap mo, ml, ma;
-  k_transpose_correction<<<dim3(4, 4, BH), dim3(32, 8), 0, st>>>(A, At);
   if (!make_map(&mo, O, 128, N, H, BH / H, os[0], os[1], os[2], kCorrTile) ||
       !make_map(&ml, O_lo, 128, N, BH, 1, 0, (i64)N * 128, 128, kCorrTile) ||
       !make_map(&ma, At, 128, 128, 2 * BH, 1, 0, (i64)128 * 128, 128, kCorrTile))

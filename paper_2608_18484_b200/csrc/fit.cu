@@ -2,15 +2,17 @@
 // standardisation, weighted ridge normal equations solved by Cholesky, the
 // probe-residual output subspace, and the composed affine map
 //   R_hat_i = c + x_i A,  A = diag(1/s_x) B_lambda Psi_r Psi_r^T,  c = mu_R - mu_x A,
-// which is algebraically Eq. 9.  Standardisation and composition are float64; the Gram matrices and the Cholesky
-// solve are float64 for float32 tensors and float32 for 16-bit tensors; one CTA per head.
+// which is algebraically Eq. 9.  Standardisation and composition are float64; the Gram matrices and the ridge
+// solve are float64 for float32 tensors and float32 for 16-bit tensors.  The fit is a chain of short kernels, on the
+// critical path of small calls and beside the attention kernels in large ones, where every SM it holds is lost to them:
+// each stage is spread over several CTAs per head where it has the work for them.
 #include "kernels.cuh"
 
 namespace spr {
 
-// scratch per head (doubles): Xb[M*d] Rb[M*d] G[d*d] B[d*d] S[d*d] T[d*d] mu_x[d] mu_R[d] s_x[d] wt[M] flag[1]
+// scratch per head (doubles): Xb[M*d] Rb[M*d] G[d*d] B[d*d] S[d*d] mu_x[d] mu_R[d] s_x[d] wt[M] flag[1]
 struct FitLayout {
-  size_t Xb, Rb, G, B, S, T, mu_x, mu_R, s_x, wt, flag, total;
+  size_t Xb, Rb, G, B, S, mu_x, mu_R, s_x, wt, flag, total;
   __host__ __device__ FitLayout(int M, int d) {
     size_t o = 0;
     Xb = o; o += (size_t)M * d;
@@ -18,7 +20,6 @@ struct FitLayout {
     G = o; o += (size_t)d * d;
     B = o; o += (size_t)d * d;
     S = o; o += (size_t)d * d;
-    T = o; o += (size_t)d * d;
     mu_x = o; o += d; mu_R = o; o += d; s_x = o; o += d;
     wt = o; o += M;
     flag = o; o += 1;
@@ -27,244 +28,369 @@ struct FitLayout {
 };
 size_t fit_scratch_doubles(int BH, int M, int d) { return FitLayout(M, d).total * BH; }
 
-// alpha, weighted means, feature scale, standardised probes, unit-mean weights
-__global__ void __launch_bounds__(256) k_fit_prepare(FitArgs a) {
+// Probe rows a head has in flight per column slice of k_fit_prepare, columns per CTA of it.
+constexpr int kPrepCols = 32, kPrepSlices = 8;
+
+// alpha, weighted means, feature scale, standardised probes, unit-mean weights.  Bound by the latency of the loads and of
+// the float64 chains, so both are split: grid (d / 32, heads), thread (slice s, column j) takes the probes s, s + 8, ... of
+// its column, and the eight partial sums are added in a fixed order.
+// (One CTA per head with one thread per column: 26 us at M = 64, d = 128, two heads; now 6 us.)
+__global__ void __launch_bounds__(kPrepCols * kPrepSlices) k_fit_prepare(FitArgs a) {
   __shared__ double red[34];
-  const int bh = blockIdx.x, M = a.M, d = a.d;
+  __shared__ double part[2][kPrepSlices][kPrepCols];
+  constexpr int kNt = kPrepCols * kPrepSlices;
+  const int bh = blockIdx.y, M = a.M, d = a.d, tid = threadIdx.x;
+  const int jl = tid % kPrepCols, sl = tid / kPrepCols, j = blockIdx.x * kPrepCols + jl;
   const FitLayout L(M, d);
   double* sc = a.scratch + (size_t)bh * L.total;
+  pdl_wait();                                                   // the probe rows come from the kernel before
+  pdl_launch_dependents();
   const float* X = a.X + (i64)bh * M * d;
   const float* Dn = a.Dn + (i64)bh * M * d;
   const float* w = a.w + (i64)bh * M;
   double sw = 0.0, cnt = 0.0;
-  for (int p = threadIdx.x; p < M; p += 256) { sw += (double)w[p]; cnt += w[p] > 0.f ? 1.0 : 0.0; }
+  for (int p = tid; p < M; p += kNt) { sw += (double)w[p]; cnt += w[p] > 0.f ? 1.0 : 0.0; }
   sw = block_sum(sw, red);
   cnt = block_sum(cnt, red);
-  if (threadIdx.x == 0) sc[L.flag] = (sw > 0.0 && cnt > 0.0) ? 0.0 : 1.0;
+  if (tid == 0 && blockIdx.x == 0) sc[L.flag] = (sw > 0.0 && cnt > 0.0) ? 0.0 : 1.0;
   if (!(sw > 0.0)) sw = 1.0;
-  // alpha_p = w_p / sum w once per probe (float64 divisions are expensive on this part), kept in the weight slot
-  // until the unit-mean weights replace it at the end
-  for (int p = threadIdx.x; p < M; p += 256) sc[L.wt + p] = (double)w[p] / sw;
-  __syncthreads();
-  for (int j = threadIdx.x; j < d; j += 256) {
-    double mx = 0.0, mr = 0.0;
-    for (int p = 0; p < M; ++p) {
-      const double al = sc[L.wt + p], x = (double)X[p * d + j];
-      mx += al * x;
-      mr += al * ((double)Dn[p * d + j] - x);
-    }
-    double var = 0.0;
-    for (int p = 0; p < M; ++p) { const double t = (double)X[p * d + j] - mx; var += sc[L.wt + p] * t * t; }
-    const double s = sqrt(var + (double)a.eps_std), inv_s = 1.0 / s;
-    sc[L.mu_x + j] = mx; sc[L.mu_R + j] = mr; sc[L.s_x + j] = s;
-    for (int p = 0; p < M; ++p) {
-      const double x = (double)X[p * d + j];
-      sc[L.Xb + (size_t)p * d + j] = (x - mx) * inv_s;
-      sc[L.Rb + (size_t)p * d + j] = ((double)Dn[p * d + j] - x) - mr;
-    }
+  const double inv_sw = 1.0 / sw;
+  if (blockIdx.x == 0)
+    for (int p = tid; p < M; p += kNt) sc[L.wt + p] = (double)M * (double)w[p] * inv_sw;   // unit-mean weights M w_p / sum w (Appendix A.3)
+  auto total = [&](int which) {                                 // sum of the column's slices
+    double t = part[which][0][jl];
+#pragma unroll
+    for (int s = 1; s < kPrepSlices; ++s) t += part[which][s][jl];
+    return t;
+  };
+  double mx = 0.0, mr = 0.0;
+#pragma unroll 4
+  for (int p = sl; p < M; p += kPrepSlices) {
+    const double al = (double)w[p], x = (double)X[p * d + j];
+    mx = fma(al, x, mx);
+    mr = fma(al, (double)Dn[p * d + j] - x, mr);
   }
+  part[0][sl][jl] = mx; part[1][sl][jl] = mr;
   __syncthreads();
-  for (int p = threadIdx.x; p < M; p += 256) sc[L.wt + p] = (double)M * (double)w[p] / sw;   // unit-mean weights M w_p / sum w (Appendix A.3)
+  mx = total(0) * inv_sw; mr = total(1) * inv_sw;
+  __syncthreads();
+  double var = 0.0;
+#pragma unroll 4
+  for (int p = sl; p < M; p += kPrepSlices) { const double t = (double)X[p * d + j] - mx; var = fma((double)w[p] * t, t, var); }
+  part[0][sl][jl] = var;
+  __syncthreads();
+  const double s = sqrt(total(0) * inv_sw + (double)a.eps_std), inv_s = 1.0 / s;
+  if (sl == 0) { sc[L.mu_x + j] = mx; sc[L.mu_R + j] = mr; sc[L.s_x + j] = s; }
+#pragma unroll 4
+  for (int p = sl; p < M; p += kPrepSlices) {
+    const double x = (double)X[p * d + j];
+    sc[L.Xb + (size_t)p * d + j] = (x - mx) * inv_s;
+    sc[L.Rb + (size_t)p * d + j] = ((double)Dn[p * d + j] - x) - mr;
+  }
 }
 
-// blockIdx.x selects G = Xb^T W Xb + lam I, B(rhs) = Xb^T W Rb, S = Rb^T W Rb.
-// T = float for 16-bit tensors (the float64 pipe of this part is narrow: a float64 Gram is bound by it), double otherwise.
+// blockIdx.z selects G = Xb^T W Xb + lam I, B(rhs) = Xb^T W Rb, S = Rb^T W Rb; a CTA owns one kT x kT tile of it (of the
+// symmetric G and S only the tiles on and above the diagonal, mirrored), a thread a 4 x 4 or 2 x 2 block.
+// T = float for 16-bit tensors, double otherwise, with smaller tiles to spread it.
+// (One CTA per matrix with 64 entries per thread and no operand reuse in registers: 94 us at M = 64, d = 128, two heads;
+// now 18 us, of which a part is the wait for the kernel before.)
+template <typename T> constexpr int kGramTile = sizeof(T) == 4 ? 64 : 32;
 template <typename T>
 __global__ void __launch_bounds__(256) k_fit_gram(FitArgs a) {
-  extern __shared__ unsigned char sm_gram_raw[];   // [2][32][d] row chunks of the left and right factor
-  T* sm_gram = reinterpret_cast<T*>(sm_gram_raw);
-  const int bh = blockIdx.y, which = blockIdx.x, M = a.M, d = a.d;
+  constexpr int kT = kGramTile<T>, kPt = kT / 16, kRows = 32;
+  __shared__ __align__(16) T ls[kRows][kT], rs[kRows][kT];
+  const int bh = blockIdx.y, which = blockIdx.z, M = a.M, d = a.d;
+  const int nt = d / kT, i0 = (blockIdx.x / nt) * kT, j0 = (blockIdx.x % nt) * kT;
+  pdl_wait();
+  pdl_launch_dependents();
+  if (which != 1 && j0 < i0) return;
   const FitLayout L(M, d);
   double* sc = a.scratch + (size_t)bh * L.total;
-  const double* Lm = sc + (which == 2 ? L.Rb : L.Xb);
-  const double* Rm = sc + (which == 0 ? L.Xb : L.Rb);
+  const double* Lm = sc + (which == 2 ? L.Rb : L.Xb) + i0;
+  const double* Rm = sc + (which == 0 ? L.Xb : L.Rb) + j0;
   double* out = sc + (which == 0 ? L.G : which == 1 ? L.B : L.S);
-  T* ls = sm_gram;
-  T* rs = sm_gram + 32 * d;
-  const int per = d * d / 256;             // entries per thread (d = 64 or 128)
-  T acc[64];
+  const int ti = (threadIdx.x / 16) * kPt, tj = (threadIdx.x % 16) * kPt;
+  T acc[kPt][kPt];
 #pragma unroll
-  for (int e = 0; e < 64; ++e) acc[e] = T(0);
-  for (int p0 = 0; p0 < M; p0 += 32) {
-    const int nr = min(32, M - p0);
+  for (int u = 0; u < kPt; ++u)
+#pragma unroll
+    for (int v = 0; v < kPt; ++v) acc[u][v] = T(0);
+  for (int p0 = 0; p0 < M; p0 += kRows) {
+    const int nr = min(kRows, M - p0);
     __syncthreads();
-    for (int t = threadIdx.x; t < nr * d; t += 256) {
-      const int p = t / d;
-      ls[t] = (T)(Lm[(size_t)(p0 + p) * d + t % d] * sc[L.wt + p0 + p]);
-      rs[t] = (T)Rm[(size_t)(p0 + p) * d + t % d];
+#pragma unroll
+    for (int e = threadIdx.x; e < kRows * kT; e += 256) {
+      const int p = e / kT, c = e % kT;
+      if (p < nr) {
+        ls[p][c] = (T)(Lm[(size_t)(p0 + p) * d + c] * sc[L.wt + p0 + p]);
+        rs[p][c] = (T)Rm[(size_t)(p0 + p) * d + c];
+      }
     }
     __syncthreads();
+    for (int p = 0; p < nr; ++p) {
+      T x[kPt], y[kPt];
 #pragma unroll
-    for (int e = 0; e < 64; ++e) {
-      if (e < per) {
-        const int idx = threadIdx.x + e * 256, i = idx / d, j = idx % d;
-        T s = acc[e];
-        for (int p = 0; p < nr; ++p) s += ls[p * d + i] * rs[p * d + j];
-        acc[e] = s;
+      for (int u = 0; u < kPt; ++u) { x[u] = ls[p][ti + u]; y[u] = rs[p][tj + u]; }
+#pragma unroll
+      for (int u = 0; u < kPt; ++u)
+#pragma unroll
+        for (int v = 0; v < kPt; ++v) acc[u][v] = fma(x[u], y[v], acc[u][v]);
+    }
+  }
+#pragma unroll
+  for (int u = 0; u < kPt; ++u)
+#pragma unroll
+    for (int v = 0; v < kPt; ++v) {
+      const int i = i0 + ti + u, j = j0 + tj + v;
+      const double g = (double)acc[u][v] + ((which == 0 && i == j) ? (double)a.lambda : 0.0);
+      out[(size_t)i * d + j] = g;
+      if (which != 1 && i0 != j0) out[(size_t)j * d + i] = g;
+    }
+}
+
+// Ridge system (G + lam I) B = RHS by symmetric elimination G = L D L^T (no pivoting: the matrix is positive definite)
+// with the right-hand sides carried along, then back substitution; T as in k_fit_gram.
+// Everything stays in registers: warp w owns the rows w, w + 16, ..., lane l the columns l, l + 32, ... of [G | RHS].
+// Step k: the owner of row k has published it in shared memory (two buffers, so one barrier per step); every warp takes
+// its own column entries a_ik by shuffle and subtracts a_ik / a_kk times the row.  2 d barriers in all; the chain of the
+// published row (update, publish, barrier, read) sets the pace.  blockIdx.y owns kRhs right-hand sides and repeats the
+// elimination of G: the registers hold no more.
+// (Cholesky in shared memory with three barriers per column and a dot product per row of the triangular solves: 322 us
+// at d = 128 float32, 469 us float64; now 81 and 89 us, beside the eigen-solver.)
+template <typename T, int D> constexpr int kSolveRhs = sizeof(T) == 4 ? 64 : 32;
+template <typename T, int D>
+__global__ void __launch_bounds__(512, 1) k_fit_solve(FitArgs a) {
+  constexpr int kRhs = kSolveRhs<T, D>, kRpw = D / 16, kGc = D / 32, kRc = kRhs / 32, kC = kGc + kRc;
+  constexpr unsigned FULL = 0xffffffffu;
+  __shared__ T rowbuf[2][kC * 32];
+  __shared__ T dinv[D];                                          // 1 / pivot
+  const int bh = blockIdx.x, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const FitLayout L(a.M, D);
+  double* sc = a.scratch + (size_t)bh * L.total;
+  const double* G = sc + L.G;
+  double* Bm = sc + L.B + blockIdx.y * kRhs;
+  pdl_wait();
+  pdl_launch_dependents();
+  T x[kRpw][kC];
+#pragma unroll
+  for (int r = 0; r < kRpw; ++r) {
+    const int row = warp + 16 * r;
+#pragma unroll
+    for (int c = 0; c < kGc; ++c) x[r][c] = (T)G[row * D + lane + 32 * c];
+#pragma unroll
+    for (int c = 0; c < kRc; ++c) x[r][kGc + c] = (T)Bm[row * D + lane + 32 * c];
+  }
+  if (sc[L.flag] != 0.0) return;                                 // uniform: no usable probes (set by k_fit_prepare)
+  bool bad = false;
+  if (warp == 0) {
+#pragma unroll
+    for (int c = 0; c < kC; ++c) rowbuf[0][lane + 32 * c] = x[0][c];
+    if (lane == 0) dinv[0] = T(1) / x[0][0];
+  }
+#pragma unroll
+  for (int ka = 0; ka < kRpw; ++ka) {
+#pragma unroll 1
+    for (int kw = 0; kw < 16; ++kw) {
+      const int k = 16 * ka + kw;
+      __syncthreads();
+      const T* rb = rowbuf[k & 1];
+      bad |= !(rb[k] > T(0));
+      const T inv = dinv[k];
+      T rv[kC];
+#pragma unroll
+      for (int c = ka / 2; c < kC; ++c) rv[c] = rb[lane + 32 * c];
+      // the row of the next pivot first: it goes to the other buffer at once
+#pragma unroll
+      for (int r = ka; r < kRpw; ++r) {
+        if (r > ka || warp > kw) {                               // uniform: a row below k
+          const T f = __shfl_sync(FULL, x[r][ka / 2], k & 31) * inv;
+#pragma unroll
+          for (int c = ka / 2; c < kC; ++c) x[r][c] = fma(-f, rv[c], x[r][c]);
+        }
+        constexpr int kLast = kRpw - 1;
+        if (r == ka || (r == ka + 1 && r <= kLast)) {
+          const int kn = k + 1, rn = r == ka ? kw + 1 : 0;       // owner of row k + 1: (r, warp kw + 1), or (ka + 1, warp 0)
+          if ((r == ka ? kw < 15 : kw == 15) && warp == rn) {
+#pragma unroll
+            for (int c = ka / 2; c < kC; ++c) rowbuf[kn & 1][lane + 32 * c] = x[r][c];
+            const T piv = __shfl_sync(FULL, x[r][r / 2], kn & 31);
+            if (lane == 0) dinv[kn] = T(1) / piv;
+          }
+        }
       }
     }
   }
-#pragma unroll
-  for (int e = 0; e < 64; ++e) {
-    if (e < per) {
-      const int idx = threadIdx.x + e * 256, i = idx / d, j = idx % d;
-      out[idx] = (double)acc[e] + ((which == 0 && i == j) ? (double)a.lambda : 0.0);
-    }
-  }
-}
-
-// Cholesky G = L L^T in shared memory, then L Y = RHS and L^T B = Y.  T as in k_fit_gram.
-template <typename T>
-__global__ void __launch_bounds__(1024) k_fit_solve(FitArgs a) {
-  extern __shared__ unsigned char Gs_raw[];  // [d][d+1]
-  T* Gs = reinterpret_cast<T*>(Gs_raw);
-  const int bh = blockIdx.x, d = a.d, ld = d + 1;
-  const FitLayout L(a.M, d);
-  double* sc = a.scratch + (size_t)bh * L.total;
-  __shared__ int bad;
-  // (square roots and divisions are expensive in float64 on this part: one thread forms 1/sqrt(pivot), and the
-  // reciprocals of the diagonal are kept for the triangular solves)
-  __shared__ T s_inv;
-  __shared__ T dinv[128];
-  if (threadIdx.x == 0) bad = sc[L.flag] != 0.0;
-  for (int e = threadIdx.x; e < d * d; e += blockDim.x) Gs[(e / d) * ld + e % d] = (T)sc[L.G + e];
-  __syncthreads();
-  for (int k = 0; k < d; ++k) {
-    if (threadIdx.x == 0) {
-      const T piv = Gs[k * ld + k];
-      if (!(piv > T(0))) bad = 1;
-      else { s_inv = T(1) / sqrt(piv); dinv[k] = s_inv; }       // 1 / L_kk
-    }
-    __syncthreads();
-    if (bad) break;                                               // uniform
-    const T inv = s_inv;
-    for (int i = k + threadIdx.x; i < d; i += blockDim.x) Gs[i * ld + k] *= inv;   // includes the diagonal: L_kk = sqrt(piv)
-    __syncthreads();
-    // trailing update of the lower triangle: eight threads per row, columns k+1+q, k+1+q+8, ... up to the diagonal
-    for (int i = k + 1 + (int)(threadIdx.x >> 3); i < d; i += (int)(blockDim.x >> 3)) {
-      const T lik = Gs[i * ld + k];
-      for (int j = k + 1 + (int)(threadIdx.x & 7); j <= i; j += 8) Gs[i * ld + j] -= lik * Gs[j * ld + k];
-    }
-    __syncthreads();
-  }
-  __syncthreads();
-  if (bad) {
+  if (bad) {                                                     // uniform over the CTA: everyone saw every pivot
     if (threadIdx.x == 0) { sc[L.flag] = 1.0; set_error(a.err, SPARSEPR_ERR_NUMERIC); }
     return;
   }
-  // Triangular solves: eight threads per right-hand-side column.  Thread (c, q) keeps the entries i = q, q + 8, ...
-  // of its column in registers; row i of the solve is a dot product over the entries already known, split over the
-  // eight threads and added up by shuffles (fixed order).
-  double* Bm = sc + L.B;
-  constexpr int kTq = 8, kMaxPer = 128 / kTq;
-  const int c = threadIdx.x / kTq, q = threadIdx.x % kTq;
-  const int per = d / kTq;                                   // d = 64 or 128
-  if (c < d) {
-    T y[kMaxPer];
+  // back substitution: row k of the solution = y_k / pivot, once all rows below have been taken out of it
+  __syncthreads();
+  if (warp == 15) {
+    const T inv = dinv[D - 1];
 #pragma unroll
-    for (int t = 0; t < kMaxPer; ++t) y[t] = t < per ? (T)Bm[(size_t)(q + kTq * t) * d + c] : T(0);
-    for (int i = 0; i < d; ++i) {                            // forward: y_i = (b_i - sum_{j<i} L_ij y_j) / L_ii
-      T s = T(0);
-#pragma unroll
-      for (int t = 0; t < kMaxPer; ++t) {
-        const int j = q + kTq * t;
-        if (t < per && j < i) s += Gs[i * ld + j] * y[t];
-      }
-#pragma unroll
-      for (int o = 1; o < kTq; o <<= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-      const T inv = dinv[i];
-#pragma unroll
-      for (int t = 0; t < kMaxPer; ++t)
-        if (q + kTq * t == i) y[t] = (y[t] - s) * inv;
-    }
-    for (int i = d - 1; i >= 0; --i) {                       // backward: b_i = (y_i - sum_{j>i} L_ji b_j) / L_ii
-      T s = T(0);
-#pragma unroll
-      for (int t = 0; t < kMaxPer; ++t) {
-        const int j = q + kTq * t;
-        if (t < per && j > i) s += Gs[j * ld + i] * y[t];
-      }
-#pragma unroll
-      for (int o = 1; o < kTq; o <<= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-      const T inv = dinv[i];
-#pragma unroll
-      for (int t = 0; t < kMaxPer; ++t)
-        if (q + kTq * t == i) y[t] = (y[t] - s) * inv;
-    }
-#pragma unroll
-    for (int t = 0; t < kMaxPer; ++t)
-      if (t < per) Bm[(size_t)(q + kTq * t) * d + c] = (double)y[t];
+    for (int c = kGc; c < kC; ++c) { x[kRpw - 1][c] *= inv; rowbuf[(D - 1) & 1][lane + 32 * c] = x[kRpw - 1][c]; }
   }
+#pragma unroll
+  for (int kb = 0; kb < kRpw; ++kb) {
+    const int ka = kRpw - 1 - kb;
+#pragma unroll 1
+    for (int kw = 15; kw >= 0; --kw) {
+      const int k = 16 * ka + kw;
+      __syncthreads();
+      if (k == 0) break;
+      const T* rb = rowbuf[k & 1];
+      T rv[kRc];
+#pragma unroll
+      for (int c = 0; c < kRc; ++c) rv[c] = rb[lane + 32 * (kGc + c)];
+#pragma unroll
+      for (int q = 0; q <= ka; ++q) {
+        const int r = ka - q;
+        if (r < ka || warp < kw) {
+          const T f = __shfl_sync(FULL, x[r][ka / 2], k & 31);
+#pragma unroll
+          for (int c = 0; c < kRc; ++c) x[r][kGc + c] = fma(-f, rv[c], x[r][kGc + c]);
+        }
+        if (r == ka || r == ka - 1) {
+          if ((r == ka ? kw > 0 : kw == 0) && warp == (r == ka ? kw - 1 : 15)) {
+            const T inv = dinv[k - 1];
+#pragma unroll
+            for (int c = 0; c < kRc; ++c) {
+              x[r][kGc + c] *= inv;
+              rowbuf[(k - 1) & 1][lane + 32 * (kGc + c)] = x[r][kGc + c];
+            }
+          }
+        }
+      }
+    }
+  }
+#pragma unroll
+  for (int r = 0; r < kRpw; ++r)
+#pragma unroll
+    for (int c = 0; c < kRc; ++c) Bm[(warp + 16 * r) * D + lane + 32 * c] = (double)x[r][kGc + c];
 }
 
-// T = B Psi (d x r); A = diag(1/s_x) T Psi^T; c = mu_R - mu_x A
+// T = B Psi (d x r); A = diag(1/s_x) T Psi^T; c = mu_R - mu_x A.  float64 throughout.  Grid (d / 16 + 1, heads): CTA x
+// owns 16 rows of A; the last one forms c = mu_R - ((mu_x / s_x) B) Psi Psi^T.  With `At` the map is also written as the
+// two bf16 words the correction pass multiplies with: At [2][BH][n][k], first words, then what their rounding dropped.
+// (One CTA per head: 132 us at two heads of d = 128, 630 us beside the attention kernels at 24 heads; now 25 and 125 us.)
+constexpr int kCompRows = 16;
 __global__ void __launch_bounds__(256) k_fit_compose(FitArgs a, int r) {
-  const int bh = blockIdx.x, d = a.d;
+  extern __shared__ __align__(16) double sm_comp[];
+  const int bh = blockIdx.y, d = a.d, tid = threadIdx.x;
   const FitLayout L(a.M, d);
-  double* sc = a.scratch + (size_t)bh * L.total;
+  const double* sc = a.scratch + (size_t)bh * L.total;
+  pdl_wait();
+  pdl_launch_dependents();
+  const int i0 = blockIdx.x * kCompRows;
+  const bool tail = i0 >= d;
   float* A = a.A + (i64)bh * d * d;
-  float* c = a.c + (i64)bh * d;
+  float* cvec = a.c + (i64)bh * d;
+  __nv_bfloat16* Ah = a.At ? a.At + (i64)bh * d * d : nullptr;
+  __nv_bfloat16* Al = a.At ? a.At + ((i64)gridDim.y + bh) * d * d : nullptr;
+  auto put = [&](int i, int j, float x) {
+    A[(i64)i * d + j] = x;
+    if (Ah) {
+      const __nv_bfloat16 hb = __float2bfloat16_rn(x);
+      Ah[(i64)j * d + i] = hb;
+      Al[(i64)j * d + i] = __float2bfloat16_rn(x - __bfloat162float(hb));
+    }
+  };
   if (sc[L.flag] != 0.0) {                 // no usable fit: the head falls back to hard drop
-    for (int e = threadIdx.x; e < d * d; e += 256) A[e] = 0.f;
-    for (int j = threadIdx.x; j < d; j += 256) c[j] = 0.f;
+    if (tail) { for (int j = tid; j < d; j += 256) cvec[j] = 0.f; }
+    else for (int e = tid; e < kCompRows * d; e += 256) put(i0 + e % kCompRows, e / kCompRows, 0.f);
     return;
   }
-  const float* Psi = a.Psi + (i64)bh * d * r;
   const double* Bm = sc + L.B;
-  double* T = sc + L.T;
-  for (int e = threadIdx.x; e < d * r && !a.full_rank; e += 256) {
-    const int i = e / r, t = e % r;
-    double s = 0.0;
-    for (int k = 0; k < d; ++k) s += Bm[(size_t)i * d + k] * (double)Psi[k * r + t];
-    T[e] = s;
+  double* Bs = sm_comp;                    // [16][d] rows of B; tail: [2][d] halves of u, then [d] u
+  double* Ts = Bs + kCompRows * d;         // [16][r]
+  float* Ps = reinterpret_cast<float*>(Ts + kCompRows * 64);   // [d][r + 1]
+  const int ldp = r + 1;
+  if (!a.full_rank) {
+    const float* Psi = a.Psi + (i64)bh * d * r;
+    for (int e = tid; e < d * r; e += 256) Ps[(e / r) * ldp + e % r] = Psi[e];
   }
-  __shared__ double rs_x[128];             // 1 / s_x
-  for (int i = threadIdx.x; i < d; i += 256) rs_x[i] = 1.0 / sc[L.s_x + i];
-  __syncthreads();
-  double* Ad = sc + L.G;                   // G is no longer needed
-  for (int e = threadIdx.x; e < d * d; e += 256) {
-    const int i = e / d, j = e % d;
-    double s = 0.0;
-    if (a.full_rank) {
-      s = Bm[e];                           // every row of B lies in the row space of the probe residuals: B Psi Psi^T = B
-    } else {
-      for (int t = 0; t < r; ++t) s += T[i * r + t] * (double)Psi[j * r + t];
+  if (!tail) {
+    for (int e = tid; e < kCompRows * d; e += 256) Bs[e] = Bm[(size_t)i0 * d + e];
+    __syncthreads();
+    if (!a.full_rank) {
+      for (int e = tid; e < kCompRows * r; e += 256) {
+        const int i = e / r, t = e % r;
+        double s0 = 0.0, s1 = 0.0;
+        for (int k = 0; k < d; k += 2) {
+          s0 = fma(Bs[i * d + k], (double)Ps[k * ldp + t], s0);
+          s1 = fma(Bs[i * d + k + 1], (double)Ps[(k + 1) * ldp + t], s1);
+        }
+        Ts[i * r + t] = s0 + s1;
+      }
+      __syncthreads();
     }
-    s *= rs_x[i];
-    Ad[e] = s;
-    A[e] = (float)s;
+    const int i = tid % kCompRows;         // one row per thread: consecutive lanes write consecutive entries of At
+    const double rsx = 1.0 / sc[L.s_x + i0 + i];
+    for (int j = tid / kCompRows; j < d; j += 256 / kCompRows) {
+      double s = 0.0;
+      if (a.full_rank) s = Bs[i * d + j];  // every row of B lies in the row space of the probe residuals: B Psi Psi^T = B
+      else for (int t = 0; t < r; ++t) s = fma(Ts[i * r + t], (double)Ps[j * ldp + t], s);
+      put(i0 + i, j, (float)(s * rsx));
+    }
+    return;
+  }
+  // c: u = (mu_x / s_x) B by 256 / d parts of the rows, t = u Psi, c = mu_R - t Psi^T
+  const int parts = 256 / d, part = tid / d, k = tid % d, per = d / parts;
+  double u = 0.0;
+  for (int i = part * per; i < (part + 1) * per; ++i) u = fma(sc[L.mu_x + i] / sc[L.s_x + i], Bm[(size_t)i * d + k], u);
+  Bs[part * d + k] = u;
+  __syncthreads();
+  if (tid < d) {
+    double t = Bs[tid];
+    for (int q = 1; q < parts; ++q) t += Bs[q * d + tid];
+    Bs[256 + tid] = t;
   }
   __syncthreads();
-  for (int j = threadIdx.x; j < d; j += 256) {
-    double s = sc[L.mu_R + j];
-    for (int i = 0; i < d; ++i) s -= sc[L.mu_x + i] * Ad[(size_t)i * d + j];
-    c[j] = (float)s;
+  const double* us = Bs + 256;
+  if (a.full_rank) {
+    if (tid < d) cvec[tid] = (float)(sc[L.mu_R + tid] - us[tid]);
+    return;
+  }
+  if (tid < r) {
+    double t = 0.0;
+    for (int q = 0; q < d; ++q) t = fma(us[q], (double)Ps[q * ldp + tid], t);
+    Ts[tid] = t;
+  }
+  __syncthreads();
+  if (tid < d) {
+    double s = 0.0;
+    for (int t = 0; t < r; ++t) s = fma(Ts[t], (double)Ps[tid * ldp + t], s);
+    cvec[tid] = (float)(sc[L.mu_R + tid] - s);
   }
 }
 
+static size_t compose_smem(int d, int r) { return ((size_t)kCompRows * d + kCompRows * 64) * sizeof(double) + (size_t)d * (r + 1) * sizeof(float); }
+
 cudaError_t init_fit() {
-  cudaError_t e = cudaFuncSetAttribute(k_fit_solve<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, 128 * 129 * 8);
-  if (e == cudaSuccess) e = cudaFuncSetAttribute(k_fit_solve<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, 128 * 129 * 4);
-  if (e == cudaSuccess) e = cudaFuncSetAttribute(k_fit_gram<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, 2 * 32 * 128 * 8);
-  if (e == cudaSuccess) e = cudaFuncSetAttribute(k_fit_gram<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, 2 * 32 * 128 * 4);
-  return e;
+  return cudaFuncSetAttribute(k_fit_compose, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)compose_smem(128, kMaxRank));
 }
 
 void launch_fit(const FitArgs& a, cudaStream_t st) {
   const int d = a.d;
   const int r = min(a.r_out, min(a.M, d));
   const FitLayout L(a.M, d);
-  k_fit_prepare<<<a.BH, 256, 0, st>>>(a);
+  launch_pdl(k_fit_prepare, dim3(d / kPrepCols, a.BH), dim3(kPrepCols * kPrepSlices), 0, st, a);
+  const int tile = a.precise ? kGramTile<double> : kGramTile<float>, nt = d / tile;
+  const dim3 gg(nt * nt, a.BH, 3);
   if (a.precise) {
-    k_fit_gram<double><<<dim3(3, a.BH), 256, (size_t)2 * 32 * d * 8, st>>>(a);
-    k_fit_solve<double><<<a.BH, 1024, (size_t)d * (d + 1) * 8, st>>>(a);
+    launch_pdl(k_fit_gram<double>, gg, dim3(256), 0, st, a);
+    if (d == 128) launch_pdl(k_fit_solve<double, 128>, dim3(a.BH, 128 / kSolveRhs<double, 128>), dim3(512), 0, st, a);
+    else launch_pdl(k_fit_solve<double, 64>, dim3(a.BH, 64 / kSolveRhs<double, 64>), dim3(512), 0, st, a);
   } else {
-    k_fit_gram<float><<<dim3(3, a.BH), 256, (size_t)2 * 32 * d * 4, st>>>(a);
-    k_fit_solve<float><<<a.BH, 1024, (size_t)d * (d + 1) * 4, st>>>(a);
+    launch_pdl(k_fit_gram<float>, gg, dim3(256), 0, st, a);
+    if (d == 128) launch_pdl(k_fit_solve<float, 128>, dim3(a.BH, 128 / kSolveRhs<float, 128>), dim3(512), 0, st, a);
+    else launch_pdl(k_fit_solve<float, 64>, dim3(a.BH, 64 / kSolveRhs<float, 64>), dim3(512), 0, st, a);
   }
   // Psi_r: leading eigenvectors of S = Rb^T W Rb, i.e. right singular vectors of W^(1/2) Rb.
-  if (!a.full_rank) launch_eig_top(a.scratch + L.S, (i64)L.total, a.BH, d, r, 1, a.precise, a.Psi, nullptr, a.eig_ws, st);
-  k_fit_compose<<<a.BH, 256, 0, st>>>(a, r);
+  // The solve and the first kernel of the eigen-solver both only need the Gram matrices: they run side by side.
+  if (!a.full_rank) launch_eig_top(a.scratch + L.S, (i64)L.total, a.BH, d, r, 1, a.precise, a.Psi, nullptr, a.eig_ws, st, true);
+  launch_pdl(k_fit_compose, dim3(d / kCompRows + 1, a.BH), dim3(256), compose_smem(d, a.full_rank ? 0 : r), st, a, r);
 }
 
 }  // namespace spr

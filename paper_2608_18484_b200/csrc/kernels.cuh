@@ -16,10 +16,12 @@ void launch_centroid_gram(const float* kappa, const int* n, int BH, int C, int d
 // eigen.cu: leading r <= 64 eigenpairs of `batch` symmetric n x n matrices (n = 64 or 128), `stride` doubles apart.
 // scale_mode 0: columns scaled by sqrt(lambda_j / mean retained lambda); 1: orthonormal columns; precise: float64.
 // Fout [batch][n][r]; lam_out [batch][n] or null; ws: eig_scratch_doubles(batch, n) doubles of scratch.
+// beside: the matrices come from the kernel before the last one queued on `st`, and the two may run side by side (the
+// last one must have waited for its predecessor before it let dependents be scheduled).
 cudaError_t init_eigen();
 size_t eig_scratch_doubles(int batch, int n);
 void launch_eig_top(const double* Min, i64 stride, int batch, int n, int r, int scale_mode, bool precise, float* Fout,
-                    double* lam_out, double* ws, cudaStream_t st);
+                    double* lam_out, double* ws, cudaStream_t st, bool beside = false);
 void launch_project(int dtype, const void* X, const i64* xs, int BH, int H, int N, int d, int r, const float* F,
                     bool rms, float eps, float* phi, int ldphi, unsigned* maxabs, int* err, cudaStream_t st);
 // features of the semantic partition: the activations themselves as float32 rows [BH][N][d]
@@ -125,9 +127,9 @@ bool launch_attention_packed(const AttnArgs& a, const int* rem_pos, const int* r
 // one warp runs the bounded mbarrier wait into its limit (2^16 cycles) and records SPARSEPR_ERR_TIMEOUT in *err
 void launch_selftest_bounded_wait(int* err, cudaStream_t st);
 // correction_tc.cu: O <- X + X A + c in place, X = O + O_lo (two bf16 words, O_lo [BH][N][128] contiguous), d_v = 128;
-// At: bf16 scratch [2][BH][128][128] (the map as two bf16 words)
+// At [2][BH][128][128]: A transposed, as two bf16 words (from the fit)
 cudaError_t init_correction_tc();
-bool launch_correction_tc(const float* A, const float* c, __nv_bfloat16* At, const void* O_lo, void* O, const i64* os, int BH,
+bool launch_correction_tc(const float* c, const __nv_bfloat16* At, const void* O_lo, void* O, const i64* os, int BH,
                           int H, int N, int* err, cudaStream_t st);
 
 struct ProbeArgs {
@@ -160,6 +162,7 @@ struct FitArgs {
   double* scratch;                     // see fit_scratch_doubles
   double* eig_ws;                      // eig_scratch_doubles(BH, d) doubles
   float *A, *c;                        // outputs [BH][d][d], [BH][d]
+  __nv_bfloat16* At;                   // optional output [2][BH][d][d]: A transposed, as two bf16 words (correction pass)
   float* Psi;                          // [BH][d][r] scratch
   int* err;
 };
