@@ -104,8 +104,8 @@ class ClockSampler:
 # --------------------------------------------------------------------------------------
 def launches_per_call(T, fitted, tensor_path):
     """Kernels of this library launched by one plan + attend call (memsets excluded)."""
-    if tensor_path:      # per side: init, first norms, split features; per iteration: assign, recheck; T-1 updates
-        kmeans = 2 + 1 + 2 * T + (T - 1)
+    if tensor_path:      # per side: init, first norms, split features; per iteration: assign, recheck; first sums; T-1 updates
+        kmeans = 2 + 1 + 2 * T + (1 if T > 1 else 0) + (T - 1)
     else:                # init, first norms, T assignments, T-1 updates
         kmeans = 2 + T + (T - 1)
     # per side: Gram, eigen-solver (Householder, tridiagonal stage, marked-matrix fallback), projection (+ split of

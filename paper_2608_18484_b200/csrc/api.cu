@@ -257,7 +257,7 @@ struct sparsepr_plan_s {
   int *route_ptr, *route_idx, *tile_off, *tile_off128;
   RouteState* rstate;
   double* probe_dist; int* probe_idx; float* probe_w;
-  __nv_bfloat16 *xh, *xl, *mh, *ml, *Ft; float* xnorm; int* flagged; int* flagcnt; double* eigws;
+  __nv_bfloat16 *xh, *xl, *mh, *ml, *mw, *Ft; float* xnorm; int* flagged; int* flagcnt; double* eigws;
   int *rem_pos, *rem_grp, *rem_cnt;      // rows of the short group remainders (packed attention tiles)
   int* km_changed;                       // [2 sides][T + 1][BH] rows that changed group in each k-means pass
   double* Mpool;                         // [BHkv][d][d] key-response metric pooled over the query heads of a K/V head (grouped-query attention only)
@@ -296,6 +296,7 @@ void carve_plan(Carver& c, const Resolved& r, sparsepr_plan_s* p) {
   int* pidx = c.take<int>(BH * std::max(r.M, 1)); float* pw = c.take<float>(BH * std::max(r.M, 1));
   __nv_bfloat16* xh = c.take<__nv_bfloat16>(BH * N * 64); __nv_bfloat16* xl = c.take<__nv_bfloat16>(BH * N * 64);
   __nv_bfloat16* mh = c.take<__nv_bfloat16>(BH * (size_t)r.Cmax * 64); __nv_bfloat16* ml = c.take<__nv_bfloat16>(BH * (size_t)r.Cmax * 64);
+  __nv_bfloat16* mw = c.take<__nv_bfloat16>(BH * (size_t)km_padded(r.Cmax) * 8);
   float* xnorm = c.take<float>(BH * N); int* flagged = c.take<int>(BH * N);
   __nv_bfloat16* Ft = c.take<__nv_bfloat16>(BH * (size_t)3 * 64 * 128);
   int* rem_pos = c.take<int>(BH * N); int* rem_grp = c.take<int>(BH * N); int* rem_cnt = c.take<int>(BH);
@@ -309,7 +310,7 @@ void carve_plan(Carver& c, const Resolved& r, sparsepr_plan_s* p) {
     p->maxabs = maxabs; p->fx_shift = fx; p->mu = mu; p->mu2 = mu2; p->mumax = mumax; p->sums = sums; p->counts = counts;
     p->a_K = aK; p->a_Q = aQ; p->kv_perm = kvp; p->kv_inv = kvi; p->q_perm = qp; p->q_inv = qi; p->kv_off = kvo; p->q_off = qo;
     p->nk = nk; p->nq = nq; p->kappa = kappa; p->theta = theta; p->score = score; p->route_ptr = rptr; p->route_idx = ridx;
-    p->xh = xh; p->xl = xl; p->mh = mh; p->ml = ml; p->xnorm = xnorm; p->flagged = flagged;
+    p->xh = xh; p->xl = xl; p->mh = mh; p->ml = ml; p->mw = mw; p->xnorm = xnorm; p->flagged = flagged;
     p->tile_off = toff; p->tile_off128 = toff128; p->rstate = rs; p->probe_dist = pd; p->probe_idx = pidx; p->probe_w = pw;
   }
 }
@@ -370,10 +371,16 @@ void run_kmeans(const sparsepr_plan_s* p, int r, int C, int tag, int* assign, co
   launch_kmeans_init(p->phi, ld, nheads, R.N, r, C, R.seed, tag, tag == kTagQInit ? R.head_offset : R.head_offset / R.G, p->mu, p->sums, p->counts, p->maxabs, p->fx_shift, st);
   const bool tcp = kmeans_tc_supported() && r <= kMaxRank;
   float* mumax = tcp ? nullptr : p->mumax;       // the tensor-core assignment derives the norm bound from ||mu||^2 itself
-  // (with the tensor-core assignment the finalize step also writes the two bf16 words of every centroid)
+  // (with the tensor-core assignment the finalize step also writes the operands made of the centroids, and the sums
+  // live through the passes: formed once, then updated for the rows that change their group)
+  const int upd_mode = tcp ? 2 : 1;
+  auto finalize = [&](int update) {
+    launch_kmeans_finalize(p->mu, p->mu2, mumax, p->sums, p->counts, p->fx_shift, nheads, C, r, update, st,
+                           tcp ? p->mh : nullptr, tcp ? p->ml : nullptr, tcp ? p->mw : nullptr);
+  };
   // warm start: the initial centroids become the means of the current features over the previous partition's groups
-  if (warm_prev) launch_kmeans_warm_sums(p->phi, ld, nheads, R.N, r, C, warm_prev, p->sums, p->counts, p->fx_shift, st);
-  launch_kmeans_finalize(p->mu, p->mu2, mumax, p->sums, p->counts, p->fx_shift, nheads, C, r, warm_prev ? 1 : 0, st, tcp ? p->mh : nullptr, tcp ? p->ml : nullptr);
+  if (warm_prev) launch_kmeans_group_sums(p->phi, ld, nheads, R.N, r, C, warm_prev, p->sums, p->counts, p->fx_shift, st);
+  finalize(warm_prev ? upd_mode : 0);
   if (tcp) launch_split_bf16(p->phi, ld, (i64)nheads * R.N, r, p->xh, p->xl, p->xnorm, st);
   if (tcp) cudaMemsetAsync(p->flagcnt, 0, 2 * (size_t)R.BH * sizeof(int), st);
   for (int t = 1; t <= R.T; ++t) {
@@ -382,19 +389,22 @@ void run_kmeans(const sparsepr_plan_s* p, int r, int C, int tag, int* assign, co
     int* cur = changed + (size_t)t * R.BH;
     if (tcp) {
       KmeansTcArgs ka{};
-      ka.BH = nheads; ka.N = R.N; ka.C = C; ka.r = r; ka.R = ld; ka.xh = p->xh; ka.xl = p->xl; ka.mh = p->mh; ka.ml = p->ml;
+      ka.BH = nheads; ka.N = R.N; ka.C = C; ka.r = r; ka.R = ld; ka.xh = p->xh; ka.xl = p->xl; ka.mh = p->mh; ka.ml = p->ml; ka.mw = p->mw;
       ka.phi = p->phi; ka.ldphi = ld; ka.xnorm = p->xnorm; ka.mu = p->mu; ka.mu2 = p->mu2;
-      ka.assign = assign; ka.sums = upd ? p->sums : nullptr; ka.counts = upd ? p->counts : nullptr; ka.fx_shift = p->fx_shift;
+      ka.assign = assign; ka.old = t > 1 ? assign : warm_prev;
+      const bool first_sums = upd && ka.old == nullptr;        // nothing to update yet: formed from the whole assignment below
+      ka.sums = upd && !first_sums ? p->sums : nullptr; ka.counts = p->counts; ka.fx_shift = p->fx_shift;
       ka.flagged = p->flagged; ka.flag_count = p->flagcnt + (size_t)(t & 1) * R.BH; ka.flag_count_next = p->flagcnt + (size_t)((t + 1) & 1) * R.BH;
       ka.recheck_total = p->recheck; ka.err = p->err;
       ka.prev_changed = prev; ka.cur_changed = cur;
       launch_kmeans_assign_tc(ka, st);
+      if (first_sums) launch_kmeans_group_sums(p->phi, ld, nheads, R.N, r, C, assign, p->sums, p->counts, p->fx_shift, st);
     } else {
       if (!upd) cudaMemsetAsync(p->recheck, 0, sizeof(int), st);
       launch_kmeans_assign(p->phi, ld, nheads, R.N, r, p->mu, p->mu2, p->mumax, C, assign, upd ? p->sums : nullptr,
                            upd ? p->counts : nullptr, p->fx_shift, p->recheck, prev, cur, st);
     }
-    if (upd) launch_kmeans_finalize(p->mu, p->mu2, mumax, p->sums, p->counts, p->fx_shift, nheads, C, r, 1, st, tcp ? p->mh : nullptr, tcp ? p->ml : nullptr);
+    if (upd) finalize(upd_mode);
   }
 }
 
@@ -930,6 +940,7 @@ size_t sparsepr_stage_assign_workspace_bytes(int32_t n, int32_t C, int32_t r) {
   c.take<float>((size_t)n * R); c.take<float>((size_t)C * R); c.take<float>(C); c.take<float>(1); c.take<int>(4);
   c.take<__nv_bfloat16>((size_t)n * 64); c.take<__nv_bfloat16>((size_t)n * 64);
   c.take<__nv_bfloat16>((size_t)C * 64); c.take<__nv_bfloat16>((size_t)C * 64); c.take<float>(n); c.take<int>(n);
+  c.take<__nv_bfloat16>((size_t)km_padded(C) * 8);
   return c.bytes();
 }
 
@@ -948,15 +959,15 @@ sparsepr_status_t sparsepr_stage_assign(int32_t n, int32_t C, int32_t r, const f
   __nv_bfloat16* xh = c.take<__nv_bfloat16>((size_t)n * 64); __nv_bfloat16* xl = c.take<__nv_bfloat16>((size_t)n * 64);
   __nv_bfloat16* mh = c.take<__nv_bfloat16>((size_t)C * 64); __nv_bfloat16* ml = c.take<__nv_bfloat16>((size_t)C * 64);
   float* xnorm = c.take<float>(n); int* flagged = c.take<int>(n);
+  __nv_bfloat16* mw = c.take<__nv_bfloat16>((size_t)km_padded(C) * 8);
   cudaGetLastError();
   k_pad_rows<<<(unsigned)std::min<i64>(((i64)n * R + 255) / 256, 65535), 256, 0, st>>>(X, n, r, R, Xp);
   k_pad_rows<<<(unsigned)std::min<i64>(((i64)C * R + 255) / 256, 65535), 256, 0, st>>>(mu, C, r, R, mup);
-  launch_kmeans_finalize(mup, mu2, mumax, nullptr, nullptr, fx, 1, C, r, 0, st);
+  launch_kmeans_finalize(mup, mu2, mumax, nullptr, nullptr, fx, 1, C, r, 0, st, mh, ml, mw);
   if (kmeans_tc_supported() && C <= kMaxGroups) {
     launch_split_bf16(Xp, R, n, r, xh, xl, xnorm, st);
-    launch_split_bf16(mup, R, C, r, mh, ml, nullptr, st);
     KmeansTcArgs ka{};
-    ka.BH = 1; ka.N = n; ka.C = C; ka.r = r; ka.R = R; ka.xh = xh; ka.xl = xl; ka.mh = mh; ka.ml = ml;
+    ka.BH = 1; ka.N = n; ka.C = C; ka.r = r; ka.R = R; ka.xh = xh; ka.xl = xl; ka.mh = mh; ka.ml = ml; ka.mw = mw;
     ka.phi = Xp; ka.ldphi = R; ka.xnorm = xnorm; ka.mu = mup; ka.mu2 = mu2; ka.assign = a;
     ka.flagged = flagged; ka.flag_count = fx + 1; ka.recheck_total = fx + 2;
     cudaMemsetAsync(ka.flag_count, 0, sizeof(int), st);

@@ -29,10 +29,13 @@ void launch_raw_features(int dtype, const void* X, const i64* xs, int BH, int H,
                          int* err, cudaStream_t st);
 void launch_kmeans_init(const float* phi, int ldphi, int BH, int N, int r, int C, u64 seed, int tag, int head0, float* mu,
                         i64* sums, int* counts, const unsigned* maxabs_bits, int* fx_shift, cudaStream_t st);
-void launch_kmeans_warm_sums(const float* phi, int ldphi, int BH, int N, int r, int C, const int* prev, i64* sums,
+void launch_kmeans_group_sums(const float* phi, int ldphi, int BH, int N, int r, int C, const int* assign, i64* sums,
                              int* counts, const int* fx_shift, cudaStream_t st);
+// update: 1 = new centroids from the sums, which are then cleared; 2 = the same, sums and counts stay.  mh, ml, mw: operands
+// of the tensor-core assignment (all or none)
 void launch_kmeans_finalize(float* mu, float* mu2, float* mumax, i64* sums, int* counts, const int* fx_shift, int BH,
-                            int C, int r, int update, cudaStream_t st, __nv_bfloat16* mh = nullptr, __nv_bfloat16* ml = nullptr);
+                            int C, int r, int update, cudaStream_t st, __nv_bfloat16* mh = nullptr, __nv_bfloat16* ml = nullptr,
+                            __nv_bfloat16* mw = nullptr);
 // prev_changed / cur_changed [BH] (may be null): number of rows of each head whose assignment changed in the previous
 // / this pass.  A head whose previous pass changed nothing is skipped (Lloyd's iteration has reached its fixed
 // point: every later pass would reproduce the same assignment and the same centroids).
@@ -52,14 +55,20 @@ bool project_tc_supported(int dtype, int d, int r, const i64* xs);
 bool launch_project_tc(const void* X, const i64* xs, int BH, int H, int N, int r, const float* F, bool rms, float eps,
                        float* phi, int ldphi, unsigned* maxabs, __nv_bfloat16* Ft, int* err, cudaStream_t st, int f_div = 1);
 
+// centroids per product of the tensor-core assignment; ||mu_c||^2 of the places beyond C (a bf16 value, larger than any score)
+constexpr int kKmChunkCols = 128;
+constexpr float kKmFar = 2.97747e38f;
+inline int km_padded(int C) { return (C + kKmChunkCols - 1) / kKmChunkCols * kKmChunkCols; }
 // ---- kmeans_tc.cu (tcgen05 score contraction + exact recheck) --------------------------------------
 struct KmeansTcArgs {
   int BH, N, C, r, R;
-  const __nv_bfloat16 *xh, *xl, *mh, *ml;      // [BH][N][64], [BH][C][64] split operands
+  const __nv_bfloat16 *xh, *xl, *mh, *ml;      // [BH][N][64] words of x, [BH][C][64] words of -2 mu
   const float* phi; int ldphi;                 // fp32 features [BH][N][ldphi]
   const float *xnorm, *mu, *mu2;               // [BH][N], [BH][C][R], [BH][C]
   int* assign;
-  i64* sums; int* counts; const int* fx_shift; // null sums = assignment only
+  const __nv_bfloat16* mw;                     // [BH][C padded to kKmChunkCols][8]: three bf16 words of ||mu_c||^2, zeros
+  i64* sums; int* counts; const int* fx_shift; // sums over the groups `old`, brought up to date by this pass; null = assignment only
+  const int* old;                              // [BH][N] groups before this pass (may be `assign`), or null: no row was in a group
   int *flagged, *flag_count, *recheck_total, *err;   // flagged [BH][N] scratch, flag_count [BH] scratch, recheck_total: rows rechecked by this pass
   const int* prev_changed; int* cur_changed;   // [BH] or null, as for launch_kmeans_assign
   int* flag_count_next;                        // [BH] or null: the next pass's counters, zeroed by this pass (flag_count itself must arrive zeroed)

@@ -1,52 +1,112 @@
 // k-means assignment (Section 4.1) with the score contraction on the tensor cores.
 //
-// score(x, c) = ||mu_c||^2 - 2 x.mu_c.  The dot products run on tcgen05.mma with both
-// operands split into two bf16 words (x = xh + xl, mu = mh + ml; the products xh.mh,
-// xh.ml, xl.mh are accumulated in fp32 in TMEM; the dropped term is ~2^-18 relative).
-// Each row keeps its best and second-best score; a row whose gap is not larger than a
-// conservative bound on the score error is NOT decided here but handed to the exact
-// recheck (per-head row lists; float64 with the operation order of the definition for every
-// centroid that a float32 filter cannot rule out), so the final assignment always equals the
-// exact float64 decision with ties to the lowest id.
+// score(x, c) = ||mu_c||^2 - 2 x.mu_c.  The whole score comes out of tcgen05.mma: both operands are split into two bf16
+// words (x = xh + xl, -2 mu = mh + ml; the products xh.mh, xh.ml, xl.mh are accumulated in fp32 in TMEM, the dropped term is
+// ~2^-16 relative), and one more k-step multiplies a constant row (1, 1, 1, 0, ...) with the three bf16 words of ||mu_c||^2
+// (which holds all of its float32 bits).  Each row keeps its best and second-best score; a row whose gap is not larger than
+// a conservative bound on the score error is NOT decided here but handed to the exact recheck (per-head row lists; float64
+// with the operation order of the definition for every centroid that a float32 filter cannot rule out), so the final
+// assignment always equals the exact float64 decision with ties to the lowest id.
 //
-// Persistent CTAs: each owns row tiles (128 rows) of one head; centroid chunks of 256
-// stream through shared memory (resident when C <= 256).  Roles: warps 0-3 and 6-9 are two
-// epilogue groups on alternate row tiles (one row per thread: tcgen05.ld, best/second,
-// fixed-point centroid sums with warp-level pre-aggregation), warp 4 TMA producer, warp 5
-// MMA issuer.
+// Persistent CTAs: each owns row tiles (128 rows) of one head; centroid chunks of 128 stream through shared memory
+// (resident when C <= 256, and then four row tiles are in flight instead of two; the last chunk's product is as wide as
+// its centroids).  Roles: warps 0-15 are two epilogue groups of eight warps on alternate row tiles, each with two score
+// buffers of 128 columns that its chunks use in turn, warp 16 TMA producer, warps 17 and 18 MMA issuers, one per group.  In a group, warps w and
+// w + 4 share the 32 rows of a TMEM quadrant and take one half of the chunk's columns each; their results meet at a named
+// barrier.  With one buffer of 256 columns per group a product had to wait for the whole scan of the group's tile before,
+// and scan and product ran one after the other (3100 cycles per tile against 1664 of product); now the product of a
+// chunk runs while the group scans the chunk before, decides and moves rows.
+// The scan needs the best score, the gap to the second best and the index of the best.  A running best / second / index
+// costs five minimum, compare and select instructions per score on the half-rate ALU pipe.  Instead every score enters two
+// minima, each a three-input minimum over two new scores (one instruction per score together): that of its column class
+// c mod 16 (16 running minima in registers) and that of its group of 16 columns (whose running best / second / index cost
+// five instructions per 16 scores).  Class and group identify a column, so the best is in the best class and the best
+// group, and any other score lies in another class or in another group:
+//   second best = min(second best of the class minima, second best of the group minima), exactly.
+//
+// Centroid sums are exact integers (fixed point, one rounding per row and column), so they are updated instead of being
+// formed anew in every pass: a row that changes its group is subtracted from the old one and added to the new one.  After
+// the first passes few rows move, and a pass then reads the two bf16 words of the features only.
+// Measured at 24 heads of 32760 rows and 256 centroids: a pass in which no row moves 62 us (the products alone need 37, the
+// two words of the features 31), the passes of one run 62 to 168 us, 1.38 ms for 16 passes where the kernel that kept best,
+// second and index per score and formed the sums anew took 2.11 ms; 40 heads of 75600 rows, 591 centroids: 540 us per
+// pass (958).  The early passes, in which a third of the rows move, are bound by the atomics of the sums.
 #include "kernels.cuh"
 #include "tc_common.cuh"
 
 namespace spr {
 namespace tc {
 
-constexpr int kKmThreads = 320;
-constexpr int kKmChunk = 256;                         // centroids per MMA (N)
+constexpr int kKmEpiWarps = 16;
+constexpr int kKmThreads = (kKmEpiWarps + 3) * 32;   // + TMA producer, two MMA issuers
+constexpr int kKmChunk = kKmChunkCols;                // centroids per MMA (N)
 constexpr uint32_t kXBytes = 128 * 128;               // one [128 rows x 64 bf16] block
-constexpr uint32_t kMuBytes = kKmChunk * 128;         // one [256 x 64 bf16] block
+constexpr uint32_t kMuBytes = kKmChunk * 128;         // one [128 x 64 bf16] block
+constexpr uint32_t kMwBytes = kKmChunk * 16;          // [128 x 8 bf16]: the words of ||mu_c||^2
+constexpr uint32_t kMuStage = 2 * kMuBytes + kMwBytes;
 
+// Tiles: either 4 row stages and 2 centroid stages (resident) or 2 and 4; a row stage is (hi, lo) of 128 rows, a centroid
+// stage (hi, lo) and the norm words of 128 centroids.
 struct KmSmem {
-  static constexpr uint32_t x = 0;                              // 2 stages x (hi, lo)
-  static constexpr uint32_t mu = x + 2 * 2 * kXBytes;           // 2 stages x (hi, lo)
-  static constexpr uint32_t bars = mu + 2 * 2 * kMuBytes;       // 12 mbarriers
-  static constexpr uint32_t misc = bars + 12 * 8;
+  static constexpr uint32_t x = 0;
+  static constexpr uint32_t tiles = 2 * 2 * kXBytes + 4 * kMuStage;
+  static constexpr uint32_t ones = tiles;                       // [128 x 16 bf16], unswizzled: the constant rows
+  static constexpr uint32_t xchg = ones + 4096;                 // best, second, index: 3 x [2 groups][2 parities][2 halves][128]
+  static constexpr uint32_t bars = xchg + 3 * 8 * 128 * 4;
+  static constexpr uint32_t misc = bars + 32 * 8;
   static constexpr uint32_t total = misc + 32;
 };
+static_assert(4 * 2 * kXBytes + 2 * kMuStage <= KmSmem::tiles, "both stage layouts fit into the tile area");
 constexpr size_t kKmSmemBytes = KmSmem::total + 1024;
-enum KmBar { X_FULL = 0, X_EMPTY = 2, MU_FULL = 4, MU_EMPTY = 6, ACC_FULL = 8, ACC_EMPTY = 10 };
+static_assert(kKmSmemBytes + 256 <= 227 * 1024, "shared memory");
+enum KmBar { X_FULL = 0, X_EMPTY = 4, MU_FULL = 8, MU_EMPTY = 12, ACC_FULL = 16, ACC_EMPTY = 20, KM_BARS = 24 };   // 4 each
 
 struct KmParams {
   int N, C, r, R, n_chunks, ctas_per_head;
   const float* phi; int ldphi;          // fp32 features (for the centroid sums)
   const float* xnorm;                   // [BH][N]
   const float* mu2;                     // [BH][C]
+  const __nv_bfloat16* mw;              // [BH][C padded to 128][8] words of ||mu_c||^2
   int* assign;
-  i64* sums; int* counts; const int* fx_shift;
+  const int* old;                       // [BH][N] or null: the groups whose sums `sums` holds (may be `assign`; ids outside [0, C) are in no sum)
+  i64* sums; int* counts; const int* fx_shift;   // sums to be updated, or null
   int* flagged; int* flag_count;        // rows left to the exact recheck: [BH][N] row indices, [BH] their number
   int* flag_count_next;                 // [BH] or null: the counters of the next pass, zeroed here
   int* err;
   const int* prev_changed; int* cur_changed;   // [BH] or null: rows whose assignment changed in the previous / this pass
 };
+
+// one row's move between two groups, by one warp: lane = columns 2 lane and 2 lane + 1 of the row (x0, x1).  (With columns
+// lane and lane + 32, whose atomics fall into half as many sectors per instruction, a pass in which most rows move takes
+// twice as long.)
+__device__ __forceinline__ void km_move(i64* sums, int* counts, int C, int R, int r, float scl, float2 x, int from, int to, int lane) {
+  // scl = 2^shift: scaling a float32 value by a power of two is exact, so the integer is the one a float64 product gives
+  const i64 v0 = __float2ll_rn(x.x * scl), v1 = __float2ll_rn(x.y * scl);
+  const int c0 = 2 * lane;
+  if (c0 < r) {
+    atomicAdd(reinterpret_cast<u64*>(sums + (i64)to * R + c0), (u64)v0);
+    if (c0 + 1 < r) atomicAdd(reinterpret_cast<u64*>(sums + (i64)to * R + c0 + 1), (u64)v1);
+  }
+  if (lane == 0) atomicAdd(counts + to, 1);
+  if (from >= 0 && from < C) {
+    if (c0 < r) {
+      atomicAdd(reinterpret_cast<u64*>(sums + (i64)from * R + c0), (u64)(-v0));
+      if (c0 + 1 < r) atomicAdd(reinterpret_cast<u64*>(sums + (i64)from * R + c0 + 1), (u64)(-v1));
+    }
+    if (lane == 0) atomicAdd(counts + from, -1);
+  }
+}
+
+__device__ __forceinline__ float min3(float a, float b, float c) {
+  float y;
+  asm("min.f32 %0, %1, %2, %3;" : "=f"(y) : "f"(a), "f"(b), "f"(c));
+  return y;
+}
+__device__ __forceinline__ float min16(const float* s) {
+  const float a = min3(s[0], s[1], s[2]), b = min3(s[3], s[4], s[5]), c = min3(s[6], s[7], s[8]), d = min3(s[9], s[10], s[11]);
+  const float e = min3(s[12], s[13], s[14]);
+  return fminf(min3(a, b, s[15]), min3(c, d, e));
+}
 
 __global__ void __launch_bounds__(kKmThreads, 1)
 k_kmeans_assign_tc(const __grid_constant__ CUtensorMap mapXh, const __grid_constant__ CUtensorMap mapXl,
@@ -58,235 +118,269 @@ k_kmeans_assign_tc(const __grid_constant__ CUtensorMap mapXh, const __grid_const
   volatile int* misc = reinterpret_cast<volatile int*>(sm + KmSmem::misc);   // [0] tmem base, [1] abort
   const uint32_t bars = base + KmSmem::bars;
   auto bar = [&](int i) { return bars + 8u * i; };
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  constexpr unsigned FULLW = 0xffffffffu;
+  const int tid = threadIdx.x, warp = __shfl_sync(FULLW, tid >> 5, 0), lane = tid & 31;   // (uniform, and known to be)
   const int bh = blockIdx.y, cta = blockIdx.x;
 
-  __shared__ __align__(16) float mu2s[kMaxGroups];          // ||mu_c||^2, +inf beyond C
   __shared__ int s_skip;
   __shared__ float s_red[34];
+  // set-up that needs nothing from the kernels before
+  if (tid == 0) {
+    for (int i = 0; i < KM_BARS; ++i) mbar_init(bar(i), i >= ACC_EMPTY ? 8 : (i >= MU_EMPTY && i < MU_EMPTY + 4) ? 2 : 1);
+    misc[1] = 0;
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
+  if (warp == kKmEpiWarps + 1) tmem_alloc(base + KmSmem::misc, 512);
+  // the constant rows in 8 x 16-byte core matrices: row group g, k half h at g * 256 + h * 128; columns 0-2 are one
+  if (tid < 256) {
+    const uint32_t one2 = 0x3F803F80u;
+    const bool first = (tid & 8) == 0;                      // 8 rows of 16 bytes per core matrix
+    *reinterpret_cast<uint4*>(sm + KmSmem::ones + tid * 16) = first ? make_uint4(one2, 0x3F80u, 0u, 0u) : make_uint4(0u, 0u, 0u, 0u);
+  }
+  fence_async_smem();
   pdl_wait();                                               // the centroids of this pass come from the kernel before
   pdl_launch_dependents();
   if (cta == 0 && tid == 0 && prm.flag_count_next) prm.flag_count_next[bh] = 0;   // last read by the recheck two kernels back
   float mu2max = 0.f;
-  for (int c = tid; c < kMaxGroups; c += kKmThreads) {
-    const float v = c < prm.C ? prm.mu2[(i64)bh * prm.C + c] : INFINITY;
-    mu2s[c] = v;
-    if (c < prm.C) mu2max = fmaxf(mu2max, v);
-  }
+  for (int c = tid; c < prm.C; c += kKmThreads) mu2max = fmaxf(mu2max, prm.mu2[(i64)bh * prm.C + c]);
   // a head whose previous pass changed no assignment has reached the fixed point of the iteration: skipped
   if (tid == 0) s_skip = (prm.err != nullptr && *reinterpret_cast<volatile int*>(prm.err) == SPARSEPR_ERR_TIMEOUT) ||
                          (prm.prev_changed != nullptr && prm.prev_changed[bh] == 0);
+  tc_fence_before();
   // largest centroid norm of the head, rounded up: it enters the bound on the score error only
-  const float mm_head = sqrtf(block_max(mu2max, s_red)) * 1.000001f;
+  const float mm = sqrtf(block_max(mu2max, s_red)) * 1.000001f;
   __syncthreads();
-  if (s_skip) return;
+  tc_fence_after();
+  const uint32_t tmem = (uint32_t)misc[0];
+  volatile int* abort_flag = &misc[1];
 
   const int row_tiles = (prm.N + 127) / 128;
   // contiguous chunk of row tiles per CTA: CTAs that run at the same time then work on distant
   // tokens, i.e. on different clusters, and do not contend for the same centroid sums
   const int per_cta = (row_tiles + prm.ctas_per_head - 1) / prm.ctas_per_head;
   const int tile0 = cta * per_cta;
-  const int my_tiles = max(0, min(per_cta, row_tiles - tile0));
+  const int my_tiles = __any_sync(0xffffffffu, s_skip) ? 0 : max(0, min(per_cta, row_tiles - tile0));
   const int n_chunks = prm.n_chunks;
-  const int steps = my_tiles * n_chunks;
   const int n_pairs = (my_tiles + 1) / 2;
-  if (tid == 0) {
-    for (int i = 0; i < 12; ++i) mbar_init(bar(i), (i == ACC_EMPTY || i == ACC_EMPTY + 1) ? 128 : 1);
-    misc[1] = 0;
-    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-  }
-  if (warp == 5) tmem_alloc(base + KmSmem::misc, 512);
-  tc_fence_before();
-  __syncthreads();
-  tc_fence_after();
-  const uint32_t tmem = (uint32_t)misc[0];
-  volatile int* abort_flag = &misc[1];
+  const bool resident = n_chunks <= 2;
+  const int xst = resident ? 4 : 2;                         // row stages
+  const int xlog = resident ? 2 : 1;
+  const uint32_t mu_base = base + (uint32_t)xst * 2 * kXBytes;
 
-  if (warp == 4) {
+  if (warp == kKmEpiWarps) {
     // =========================== TMA producer ============================================
     if (lane == 0) {
-      // Step order: the row tiles are taken in pairs, and inside a pair the centroid chunks are interleaved
-      // (tile 0 chunk 0, tile 1 chunk 0, tile 0 chunk 1, ...): score buffer b then only ever holds tiles of parity b,
-      // i.e. belongs to one epilogue group, whose waits follow the buffer's phases in order.  (With the chunks of a
-      // tile back to back both groups would share both buffers, and a group waiting for a phase that lies two ahead
-      // of the barrier's current one takes the parity test for passed.)  v counts the steps that exist.
+      // Step order: the row tiles are taken in pairs, and inside a pair the centroid chunks are interleaved (tile 0
+      // chunk 0, tile 1 chunk 0, tile 0 chunk 1, ...), so that both tiles use the chunk that a centroid stage holds.
+      // Tile t of a pair belongs to epilogue group t, and the group's k-th chunk to its buffer k mod 2: the waits on a
+      // buffer's barriers follow its phases in order.  v counts the chunks loaded.
+      const __nv_bfloat16* mw = prm.mw + (i64)bh * n_chunks * kKmChunk * 8;
       int v = 0;
-      int pair = 0, r2 = 0;                                    // sidx = pair * 2 n_chunks + r2
-      for (int sidx = 0; sidx < n_pairs * 2 * n_chunks; ++sidx) {
-        const int tl = 2 * pair + (r2 & 1), ch = r2 >> 1;
-        if (++r2 == 2 * n_chunks) { r2 = 0; ++pair; }
-        if (tl >= my_tiles) continue;
-        if (n_chunks > 1 || v == 0) {
-          const int ms = n_chunks > 1 ? (v & 1) : 0;
-          if (n_chunks > 1 && !mbar_wait(bar(MU_EMPTY + ms), ((v >> 1) & 1) ^ 1, abort_flag)) break;
-          mbar_expect_tx(bar(MU_FULL + ms), 2 * kMuBytes);
-          tma_load_4d(base + KmSmem::mu + ms * 2 * kMuBytes, &mapMh, bar(MU_FULL + ms), 0, ch * kKmChunk, bh, 0);
-          tma_load_4d(base + KmSmem::mu + ms * 2 * kMuBytes + kMuBytes, &mapMl, bar(MU_FULL + ms), 0, ch * kKmChunk, bh, 0);
+      bool go = true;
+      for (int pair = 0; pair < n_pairs && go; ++pair) {
+        const int nt = min(2, my_tiles - 2 * pair);
+        for (int ch = 0; ch < n_chunks && go; ++ch) {
+          if (!resident || pair == 0) {
+            const int ms = v & 3;
+            if (!mbar_wait(bar(MU_EMPTY + ms), ((v >> 2) & 1) ^ 1, abort_flag)) { go = false; break; }
+            const uint32_t dst = mu_base + ms * kMuStage;
+            mbar_expect_tx(bar(MU_FULL + ms), kMuStage);
+            tma_load_4d(dst, &mapMh, bar(MU_FULL + ms), 0, ch * kKmChunk, bh, 0);
+            tma_load_4d(dst + kMuBytes, &mapMl, bar(MU_FULL + ms), 0, ch * kKmChunk, bh, 0);
+            bulk_load(dst + 2 * kMuBytes, mw + (i64)ch * kKmChunk * 8, kMwBytes, bar(MU_FULL + ms));
+            ++v;
+          }
+          for (int t = 0; ch == 0 && t < nt; ++t) {
+            const int tl = 2 * pair + t, xs = tl & (xst - 1);
+            if (!mbar_wait(bar(X_EMPTY + xs), ((tl >> xlog) & 1) ^ 1, abort_flag)) { go = false; break; }
+            const int row0 = (tile0 + tl) * 128;
+            mbar_expect_tx(bar(X_FULL + xs), 2 * kXBytes);
+            tma_load_4d(base + KmSmem::x + xs * 2 * kXBytes, &mapXh, bar(X_FULL + xs), 0, row0, bh, 0);
+            tma_load_4d(base + KmSmem::x + xs * 2 * kXBytes + kXBytes, &mapXl, bar(X_FULL + xs), 0, row0, bh, 0);
+          }
         }
-        if (ch == 0) {
-          const int xs = tl & 1;
-          if (!mbar_wait(bar(X_EMPTY + xs), ((tl >> 1) & 1) ^ 1, abort_flag)) break;
-          const int row0 = (tile0 + tl) * 128;
-          mbar_expect_tx(bar(X_FULL + xs), 2 * kXBytes);
-          tma_load_4d(base + KmSmem::x + xs * 2 * kXBytes, &mapXh, bar(X_FULL + xs), 0, row0, bh, 0);
-          tma_load_4d(base + KmSmem::x + xs * 2 * kXBytes + kXBytes, &mapXl, bar(X_FULL + xs), 0, row0, bh, 0);
-        }
-        ++v;
       }
     }
-  } else if (warp == 5) {
-    // =========================== MMA issuer ================================================
-    if (lane == 0) {
-      // The issuing thread shares its warp scheduler with epilogue warps that leave it few issue slots, and the next
-      // product of a score buffer can only be issued once the epilogue has released it: every instruction of this
-      // loop is on the critical path.  Descriptors are therefore built once (only their 16-byte address field moves),
-      // the step order is tracked with counters instead of divisions, and the k-steps are unrolled.
-      const uint32_t idesc = idesc_bf16(0, kKmChunk);
+  } else if (warp > kKmEpiWarps) {
+    // =========================== MMA issuers (one per group) ================================
+    {
+      // The whole warp walks the steps and one elected lane issues; loop control goes through votes so that it is known to
+      // be uniform and descriptors stay in uniform registers.  A step costs its issuer about 500 cycles of barriers and
+      // commits besides 31 per product: with one issuer for both groups the tensor pipe idled a third of the time.
+      // Descriptors are built once (only their 16-byte address field moves) and the k-steps are unrolled.
+      const int t = warp - (kKmEpiWarps + 1);
       const int ksteps = prm.R / 16;
-      const uint64_t x_desc0 = smem_desc(base + KmSmem::x, 16), m_desc0 = smem_desc(base + KmSmem::mu, 16);
-      int v = 0;                                               // same step order as the producer
-      int pair = 0, r2 = 0;                                    // sidx = pair * 2 n_chunks + r2
-      for (int sidx = 0; sidx < n_pairs * 2 * n_chunks; ++sidx) {
-        const int tl = 2 * pair + (r2 & 1), ch = r2 >> 1;
-        if (++r2 == 2 * n_chunks) { r2 = 0; ++pair; }
-        if (tl >= my_tiles) continue;
-        const int xs = tl & 1, ms = n_chunks > 1 ? (v & 1) : 0;
-        const int ab = tl & 1, au = (tl >> 1) * n_chunks + ch;   // score buffer and how often it has been used before
-        if (ch == 0 && !mbar_wait(bar(X_FULL + xs), (tl >> 1) & 1, abort_flag)) break;
-        if ((n_chunks > 1 || v == 0) && !mbar_wait(bar(MU_FULL + ms), n_chunks > 1 ? ((v >> 1) & 1) : 0, abort_flag)) break;
-        if (!mbar_wait(bar(ACC_EMPTY + ab), (au & 1) ^ 1, abort_flag)) break;
-        tc_fence_after();
-        const uint32_t d = tmem + (uint32_t)ab * 256u;
-        const uint64_t xh = x_desc0 + (uint64_t)((xs * 2 * kXBytes) >> 4), xl = xh + (uint64_t)(kXBytes >> 4);
-        const uint64_t mh = m_desc0 + (uint64_t)((ms * 2 * kMuBytes) >> 4), ml = mh + (uint64_t)(kMuBytes >> 4);
-        // x_h mu_h + x_h mu_l + x_l mu_h; one k-step = 16 columns = 32 bytes = 2 address units
+      // the last chunk's product covers its centroids only (a multiple of 16 columns)
+      const int n_last = min(kKmChunk, (prm.C - (n_chunks - 1) * kKmChunk + 15) & ~15);
+      const uint32_t idesc_full = idesc_bf16(0, kKmChunk), idesc_last = idesc_bf16(0, n_last);
+      const uint64_t x_desc0 = smem_desc(base + KmSmem::x, 16), m_desc0 = smem_desc(mu_base, 16);
+      // unswizzled operands of the norm step.  A: k halves 128 bytes apart, row groups 256; B: one core matrix per 8
+      // centroids, 128 bytes apart; its second k half is multiplied by zeros and reads the first one again (stride 0)
+      const uint64_t one_desc = smem_desc_plain(base + KmSmem::ones, 128, 256);
+      const uint64_t w_desc0 = smem_desc_plain(mu_base + 2 * kMuBytes, 0, 128);
+      const uint32_t tm = __shfl_sync(0xffffffffu, tmem, 0);
+      int k = 0;                                               // chunks so far
+      bool go = true;
+      for (int pair = 0; pair < n_pairs && go; ++pair) {
+        const int tl = 2 * pair + t, xs = tl & (xst - 1);
+        const bool have = tl < my_tiles;
+        for (int ch = 0; ch < n_chunks; ++ch, ++k) {
+          const int ms = resident ? ch : (k & 3), ab = 2 * t + (k & 1);
+          if (!resident || pair == 0) go = __all_sync(FULLW, mbar_wait(bar(MU_FULL + ms), resident ? 0 : ((k >> 2) & 1), abort_flag));
+          if (have && ch == 0) go = __all_sync(FULLW, go && mbar_wait(bar(X_FULL + xs), (tl >> xlog) & 1, abort_flag));
+          if (have) go = __all_sync(FULLW, go && mbar_wait(bar(ACC_EMPTY + ab), ((k >> 1) & 1) ^ 1, abort_flag));
+          if (!go) break;
+          tc_fence_after();
+          const uint32_t d = tm + (uint32_t)ab * kKmChunk;
+          const uint32_t idesc = ch == n_chunks - 1 ? idesc_last : idesc_full;
+          const uint64_t moff = (uint64_t)((ms * kMuStage) >> 4);
+          const uint64_t mh = m_desc0 + moff, ml = mh + (uint64_t)(kMuBytes >> 4), wd = w_desc0 + moff;
+          const uint64_t xh = x_desc0 + (uint64_t)((xs * 2 * kXBytes) >> 4), xl = xh + (uint64_t)(kXBytes >> 4);
+          if (elect_one()) {
+            if (have) {
+              // ||mu||^2 + x_h mu_h + x_h mu_l + x_l mu_h; one k-step = 16 columns = 32 bytes = 2 address units
+              umma_bf16(d, one_desc, wd, idesc, 0);
 #pragma unroll
-        for (int kk = 0; kk < 4; ++kk) if (kk < ksteps) umma_bf16(d, xh + 2 * kk, mh + 2 * kk, idesc, kk > 0);
-#pragma unroll
-        for (int kk = 0; kk < 4; ++kk) if (kk < ksteps) umma_bf16(d, xh + 2 * kk, ml + 2 * kk, idesc, 1);
-#pragma unroll
-        for (int kk = 0; kk < 4; ++kk) if (kk < ksteps) umma_bf16(d, xl + 2 * kk, mh + 2 * kk, idesc, 1);
-        if (ch == n_chunks - 1) umma_commit(bar(X_EMPTY + xs));
-        if (n_chunks > 1) umma_commit(bar(MU_EMPTY + ms));
-        umma_commit(bar(ACC_FULL + ab));
-        ++v;
+              for (int kk = 0; kk < 4; ++kk)
+                if (kk < ksteps) {
+                  umma_bf16(d, xh + 2 * kk, mh + 2 * kk, idesc, 1);
+                  umma_bf16(d, xh + 2 * kk, ml + 2 * kk, idesc, 1);
+                  umma_bf16(d, xl + 2 * kk, mh + 2 * kk, idesc, 1);
+                }
+              umma_commit(bar(ACC_FULL + ab));
+              if (ch == n_chunks - 1) umma_commit(bar(X_EMPTY + xs));
+              if (!resident) umma_commit(bar(MU_EMPTY + ms));
+            } else if (!resident) {
+              mbar_arrive(bar(MU_EMPTY + ms));                 // the last pair has one tile
+            }
+          }
+          __syncwarp();
+        }
       }
     }
   } else {
     // =========================== epilogue: argmin, sums =====================================
-    // two groups of four warps (warps 0-3 and 6-9) take alternate row tiles
     const uint32_t FULL = 0xffffffffu;
-    const int grp = warp < 4 ? 0 : 1, wq = warp & 3;
-    const uint32_t lane_addr = (uint32_t)(wq * 32) << 16;
-    const float mm = mm_head;
+    const int grp = warp >> 3, hh = (warp >> 2) & 1, wq = warp & 3;
+    const uint32_t acc_addr0 = tmem + ((uint32_t)(wq * 32) << 16) + (uint32_t)grp * (2 * kKmChunk);
+    float* xb = reinterpret_cast<float*>(sm + KmSmem::xchg);    // best; second 1024 on; index 2048 on
+    const float scl = prm.sums ? __int_as_float((127 + prm.fx_shift[bh]) << 23) : 0.f;
     bool ok = true;
-    for (int tl = grp; tl < my_tiles; tl += 2) {
-      const int row = (tile0 + tl) * 128 + wq * 32 + lane;
-      float best = 3.0e38f, second = 3.0e38f;
-      int bi = 0;
-      // features of the warp's 32 rows for this lane's two columns (used by the centroid sums);
-      // issued before the score wait so that the loads overlap it
-      float pv0[32], pv1[32];
-      const float xn = row < prm.N ? prm.xnorm[(i64)bh * prm.N + row] : 0.f;   // needed after the scores: fetched now
-      // the row's group of the previous pass, for the count of rows that move (same reason: its latency is hidden here)
-      const int old_a = (prm.prev_changed != nullptr && row < prm.N) ? prm.assign[(i64)bh * prm.N + row] : -1;
-      if (prm.sums) {
-        const int rowbase = (tile0 + tl) * 128 + wq * 32;
-        // this lane's columns are (2 lane, 2 lane + 1): one 8-byte load per row (ldphi is a multiple of 16, and
-        // columns r..ldphi-1 hold zeros, so a pair that straddles r reads a zero)
-        const bool cok = 2 * lane < prm.r;
-        if (rowbase + 31 < prm.N) {                            // every tile but the last of a head (uniform)
-          const float* xb = prm.phi + ((i64)bh * prm.N + rowbase) * prm.ldphi + 2 * lane;
+    for (int tl = grp, k = 0; tl < my_tiles; tl += 2) {
+      const int rowbase = (tile0 + tl) * 128 + wq * 32, row = rowbase + lane;
+      const i64 gr = (i64)bh * prm.N + row;
+      const bool mine = row < prm.N && (lane >> 4) == hh;      // the two warps of a quadrant finish 16 of its rows each
+      const float xn = mine ? prm.xnorm[gr] : 0.f;             // needed after the scores: fetched now
+      const int old_a = (prm.old != nullptr && mine) ? prm.old[gr] : -1;
+      float cls[16];                                           // minima over the column classes c mod 16
 #pragma unroll
-          for (int rr = 0; rr < 32; ++rr) {
-            const float2 x2 = cok ? *reinterpret_cast<const float2*>(xb + rr * prm.ldphi) : make_float2(0.f, 0.f);
-            pv0[rr] = x2.x; pv1[rr] = x2.y;
-          }
-        } else {
-#pragma unroll
-          for (int rr = 0; rr < 32; ++rr) {
-            const int rw = min(rowbase + rr, prm.N - 1);
-            const float* xr = prm.phi + ((i64)bh * prm.N + rw) * prm.ldphi + 2 * lane;
-            const float2 x2 = cok ? *reinterpret_cast<const float2*>(xr) : make_float2(0.f, 0.f);
-            pv0[rr] = x2.x; pv1[rr] = x2.y;
-          }
-        }
-      }
-      for (int ch = 0; ch < n_chunks; ++ch) {
-        const int ab = tl & 1, au = (tl >> 1) * n_chunks + ch;   // this group's score buffer and its phase
-        ok = __all_sync(FULL, ok && mbar_wait(bar(ACC_FULL + ab), au & 1, abort_flag));
-        if (!ok) continue;
-        tc_fence_after();
-        const int c0 = ch * kKmChunk;
-        const int nvalid = min(kKmChunk, prm.C - c0);
+      for (int j = 0; j < 16; ++j) cls[j] = kKmFar;
+      float gb = kKmFar, gs = kKmFar;                          // best and second best of the minima of 16 columns
+      int gi = 0;                                              // index of the best (c / 16)
+      for (int ch = 0; ch < n_chunks; ++ch, ++k) {             // k: chunks of this group so far
+        const int ab = 2 * grp + (k & 1);
+        ok = __all_sync(FULL, ok && mbar_wait(bar(ACC_FULL + ab), (k >> 1) & 1, abort_flag));
+        if (ok) {
+          tc_fence_after();
+          const uint32_t acc_addr = acc_addr0 + (uint32_t)(k & 1) * kKmChunk;
+          const int c0 = ch * kKmChunk;
+          const int ng = (min(kKmChunk, prm.C - c0) + 15) >> 4;    // groups of 16 columns that hold centroids
+          const int ns = (ng + 1) >> 1, s_mid = (ns + 1) >> 1;     // 32-column steps; this warp's half of them
+          const int s1 = hh ? ns : s_mid;
 #pragma unroll 1
-        for (int g = 0; g < kKmChunk / 32; ++g) {
-          if (g * 32 >= nvalid) break;                       // uniform: whole column groups beyond C
-          float t[32];
-          tmem_ld32(tmem + lane_addr + (uint32_t)ab * 256u + g * 32, t);
+          for (int st = hh ? s_mid : 0; st < s1; ++st) {
+            float t[32];
+            tmem_ld32(acc_addr + st * 32, t);
+            auto group = [&](float cm, int g) {
+              gs = fminf(gs, fmaxf(cm, gb));
+              gi = cm < gb ? g : gi;
+              gb = fminf(gb, cm);
+            };
+            group(min16(t), (c0 >> 4) + 2 * st);
+            if (2 * st + 1 < ng) {                             // uniform (the product wrote no columns beyond ng groups)
+              group(min16(t + 16), (c0 >> 4) + 2 * st + 1);
 #pragma unroll
-          for (int j = 0; j < 32; j += 4) {
-            const int c = c0 + g * 32 + j;
-            const float4 m4 = *reinterpret_cast<const float4*>(mu2s + c);
-            const float mv[4] = {m4.x, m4.y, m4.z, m4.w};
+              for (int j = 0; j < 16; ++j) cls[j] = min3(cls[j], t[j], t[16 + j]);
+            } else {
 #pragma unroll
-            for (int u = 0; u < 4; ++u) {
-              const float s = fmaf(-2.f, t[j + u], mv[u]);
-              second = fminf(second, fmaxf(s, best));
-              bi = s < best ? c + u : bi;
-              best = fminf(best, s);
+              for (int j = 0; j < 16; ++j) cls[j] = fminf(cls[j], t[j]);
             }
           }
+          tc_fence_before();
         }
-        tc_fence_before();
-        mbar_arrive(bar(ACC_EMPTY + ab));
+        __syncwarp();
+        if (lane == 0) mbar_arrive(bar(ACC_EMPTY + ab));
       }
+      // second best of the class minima (tournament) and the class of the best
+      float tb[8], ts[8];
+#pragma unroll
+      for (int j = 0; j < 8; ++j) { tb[j] = fminf(cls[2 * j], cls[2 * j + 1]); ts[j] = fmaxf(cls[2 * j], cls[2 * j + 1]); }
+#pragma unroll
+      for (int w = 4; w > 0; w >>= 1)
+#pragma unroll
+        for (int j = 0; j < w; ++j) {
+          const float hi = fmaxf(tb[j], tb[j + w]);
+          ts[j] = min3(hi, ts[j], ts[j + w]);
+          tb[j] = fminf(tb[j], tb[j + w]);
+        }
+      int cj = 0;
+#pragma unroll
+      for (int j = 1; j < 16; ++j) cj = cls[j] == tb[0] ? j : cj;
+      float best = tb[0], second = fminf(ts[0], gs);
+      int bi = gi * 16 + cj;
+      {
+        // the two halves of the columns
+        float* xc = xb + ((grp * 2 + ((tl >> 1) & 1)) * 2) * 128 + wq * 32 + lane;
+        xc[hh * 128] = best; xc[1024 + hh * 128] = second; reinterpret_cast<int*>(xc)[2048 + hh * 128] = bi;
+        asm volatile("bar.sync %0, 64;" ::"r"(1 + grp * 4 + wq) : "memory");
+        const float ob = xc[(hh ^ 1) * 128], os = xc[1024 + (hh ^ 1) * 128];
+        const int oi = reinterpret_cast<const int*>(xc)[2048 + (hh ^ 1) * 128];
+        second = min3(fmaxf(best, ob), second, os);
+        bi = ob < best ? oi : bi;
+        best = fminf(best, ob);
+      }
+      bi = min(bi, prm.C - 1);                               // (only rows of non-finite scores could point past C)
       // decide, or hand the row to the exact recheck
-      const bool valid = ok && row < prm.N;
       bool decided = false, moved = false;
-      if (valid) {
-        // bound on |computed score - true score|: split-operand products (2^-13 relative with
-        // margin), fp32 accumulation and the final combination
-        const float E = 2.5e-4f * xn * mm + 1.0e-6f * (mm * mm + xn * mm);
+      if (ok && mine) {
+        // Bound on |computed score - true score|.  A bf16 rounding is off by at most 2^-8 relative, so the words of x and
+        // of 2 mu leave 2^-16 each and the dropped product xl.ml another 2^-16 of 2 |x| |mu|: 9.2e-5 in all.  Accumulation
+        // in fp32: 13 steps that add 17 terms, each aligned to the largest and cut at 2^-24 of it, which is at most
+        // 2 |x| |mu| + |mu|^2: 1.4e-5 of that.
+        const float E = 1.25e-4f * xn * mm + 1.5e-5f * mm * mm;
         decided = second - best > 2.f * E;
         if (decided) {
           moved = old_a != bi;
-          prm.assign[(i64)bh * prm.N + row] = bi;
+          if (moved || prm.old != prm.assign) prm.assign[gr] = bi;
         } else {                                             // the recheck writes (and compares) this row's assignment
           const int pos = atomicAdd(prm.flag_count + bh, 1);
           prm.flagged[(i64)bh * prm.N + pos] = row;
         }
       }
       if (prm.cur_changed != nullptr) {
-        const int nmoved = __popc(__ballot_sync(FULL, moved));
+        const int nmoved = __popc(__ballot_sync(FULL, decided && (moved || prm.prev_changed == nullptr)));
         if (lane == 0 && nmoved) atomicAdd(prm.cur_changed + bh, nmoved);
       }
       if (prm.sums) {
-        // warp-level pre-aggregation: lanes = feature columns (2 lane, 2 lane + 1); the 32 rows of the
-        // warp were prefetched above; one fixed-point atomic per (cluster, column)
-        unsigned todo = __ballot_sync(FULL, decided);
-        // 2^shift as a float: scaling a float32 partial sum by a power of two is exact, so the conversion below
-        // gives the same integer as a float64 product would
-        const float scl = __int_as_float((127 + prm.fx_shift[bh]) << 23);
+        // rows that changed their group, four at a time (the latency of their features is the cost)
+        unsigned todo = __ballot_sync(FULL, decided && moved);
+        i64* sums = prm.sums + (i64)bh * prm.C * prm.R;
+        int* counts = prm.counts + (i64)bh * prm.C;
         while (todo) {
-          const int leader = __ffs(todo) - 1;
-          const int cl = __shfl_sync(FULL, bi, leader);
-          const unsigned members = __ballot_sync(FULL, decided && bi == cl) & todo;
-          todo &= ~members;
-          // float32 partial sums in a fixed order (hence reproducible), one
-          // conversion to fixed point per (cluster, column)
-          // (four interleaved partial sums: one chain of 32 dependent additions would set the pace of this loop)
-          float2 a2[4] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f), make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
+          int rr[4];
+          float2 x2[4];
 #pragma unroll
-          for (int rr = 0; rr < 32; ++rr)
-            if ((members >> rr) & 1u) a2[rr & 3] = __fadd2_rn(a2[rr & 3], make_float2(pv0[rr], pv1[rr]));   // one packed add per member row
-          const float2 a01 = __fadd2_rn(__fadd2_rn(a2[0], a2[1]), __fadd2_rn(a2[2], a2[3]));
-          const float a0 = a01.x, a1 = a01.y;
-          const i64 acc0 = __float2ll_rn(a0 * scl), acc1 = __float2ll_rn(a1 * scl);
-          i64* s = prm.sums + ((i64)bh * prm.C + cl) * prm.R;
-          if (2 * lane < prm.r) atomicAdd(reinterpret_cast<u64*>(s + 2 * lane), (u64)acc0);
-          if (2 * lane + 1 < prm.r) atomicAdd(reinterpret_cast<u64*>(s + 2 * lane + 1), (u64)acc1);
-          if (lane == 0) atomicAdd(prm.counts + (i64)bh * prm.C + cl, __popc(members));
+          for (int u = 0; u < 4; ++u) {
+            rr[u] = todo ? __ffs(todo) - 1 : -1;
+            todo &= todo - 1;
+            x2[u] = make_float2(0.f, 0.f);
+            if (rr[u] >= 0 && 2 * lane < prm.r)              // (ldphi is a multiple of 16 and columns r..ldphi-1 hold zeros)
+              x2[u] = *reinterpret_cast<const float2*>(prm.phi + ((i64)bh * prm.N + rowbase + rr[u]) * prm.ldphi + 2 * lane);
+          }
+#pragma unroll
+          for (int u = 0; u < 4; ++u)
+            if (rr[u] >= 0)
+              km_move(sums, counts, prm.C, prm.R, prm.r, scl, x2[u], __shfl_sync(FULL, old_a, rr[u]), __shfl_sync(FULL, bi, rr[u]), lane);
         }
       }
     }
@@ -298,7 +392,7 @@ k_kmeans_assign_tc(const __grid_constant__ CUtensorMap mapXh, const __grid_const
     if (tid == 0) set_error(prm.err, SPARSEPR_ERR_TIMEOUT);
     __syncthreads();
   }
-  if (warp == 5) {
+  if (warp == kKmEpiWarps + 1) {
     tc_fence_after();
     tmem_dealloc(tmem, 512);
   }
@@ -319,7 +413,7 @@ __global__ void __launch_bounds__(256) k_assign_recheck_staged(const int* __rest
                                                                const float* __restrict__ mu, int C, int* __restrict__ assign,
                                                                i64* __restrict__ sums, int* __restrict__ counts,
                                                                const int* __restrict__ fx_shift, int* __restrict__ recheck_total,
-                                                               int first_pass, int* __restrict__ cur_changed) {
+                                                               const int* __restrict__ old, int count_all, int* __restrict__ cur_changed) {
   extern __shared__ __align__(16) float rs_smem[];
   const unsigned FULL = 0xffffffffu;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -421,17 +515,15 @@ __global__ void __launch_bounds__(256) k_assign_recheck_staged(const int* __rest
       }
     }
     bi = min(max(bi, 0), C - 1);
+    const int old_a = old != nullptr ? old[gr] : -1;
+    __syncwarp();                                              // everyone has read it (`old` may be `assign`)
     if (lane == 0) {
-      if (cur_changed != nullptr && (first_pass || assign[gr] != bi)) atomicAdd(cur_changed + bh, 1);
+      if (cur_changed != nullptr && (count_all || old_a != bi)) atomicAdd(cur_changed + bh, 1);
       assign[gr] = bi;
     }
-    if (sums) {
-      // 2^shift as a float: scaling a float32 value by a power of two is exact, so the conversion gives the same
-      // integer as the float64 product
+    if (sums && old_a != bi) {
       const float scl = __int_as_float((127 + fx_shift[bh]) << 23);
-      i64* sp = sums + ((i64)bh * C + bi) * R;
-      for (int t = lane; t < r; t += 32) atomicAdd(reinterpret_cast<u64*>(sp + t), (u64)__float2ll_rn(xs[t] * scl));
-      if (lane == 0) atomicAdd(counts + (i64)bh * C + bi, 1);
+      km_move(sums + (i64)bh * C * R, counts + (i64)bh * C, C, R, r, scl, 2 * lane < R ? *reinterpret_cast<const float2*>(xs + 2 * lane) : make_float2(0.f, 0.f), old_a, bi, lane);
     }
   }
 }
@@ -445,7 +537,7 @@ __global__ void __launch_bounds__(256) k_assign_recheck(const int* __restrict__ 
                                                         const float* __restrict__ mu, int C, int* __restrict__ assign,
                                                         i64* __restrict__ sums, int* __restrict__ counts,
                                                         const int* __restrict__ fx_shift, int* __restrict__ recheck_total,
-                                                        int first_pass, int* __restrict__ cur_changed) {
+                                                        const int* __restrict__ old, int count_all, int* __restrict__ cur_changed) {
   __shared__ double s_best[8];
   __shared__ int s_bi[8];
   const unsigned FULL = 0xffffffffu;
@@ -497,16 +589,16 @@ __global__ void __launch_bounds__(256) k_assign_recheck(const int* __restrict__ 
       const int oi = s_bi[w];
       if (oi >= 0 && (bi < 0 || ob < best || (ob == best && oi < bi))) { best = ob; bi = oi; }
     }
+    const int old_a = old != nullptr ? old[gr] : -1;
+    __syncthreads();                                           // everyone has read it (`old` may be `assign`)
     if (tid == 0) {
-      if (cur_changed != nullptr && (first_pass || assign[gr] != bi)) atomicAdd(cur_changed + bh, 1);
+      if (cur_changed != nullptr && (count_all || old_a != bi)) atomicAdd(cur_changed + bh, 1);
       assign[gr] = bi;
     }
-    if (sums) {
+    if (sums && old_a != bi && warp == 0) {
       const float* x = phi + gr * ldphi;
-      const double scl = ldexp(1.0, fx_shift[bh]);
-      i64* sp = sums + ((i64)bh * C + bi) * R;
-      if (tid < r) atomicAdd(reinterpret_cast<u64*>(sp + tid), (u64)__double2ll_rn((double)x[tid] * scl));
-      if (tid == 0) atomicAdd(counts + (i64)bh * C + bi, 1);
+      const float scl = __int_as_float((127 + fx_shift[bh]) << 23);
+      km_move(sums + (i64)bh * C * R, counts + (i64)bh * C, C, R, r, scl, 2 * lane < R ? *reinterpret_cast<const float2*>(x + 2 * lane) : make_float2(0.f, 0.f), old_a, bi, lane);
     }
     __syncthreads();
   }
@@ -557,7 +649,8 @@ void launch_split_bf16(const float* x, int ld, i64 rows, int r, __nv_bfloat16* h
   launch_pdl(tc::k_split_bf16, dim3((unsigned)((rows * 8 + 255) / 256)), dim3(256), 0, st, x, ld, rows, r, hi, lo, norm);
 }
 
-// One assignment pass.  xh/xl: bf16 [BH][N][64]; mh/ml: bf16 [BH][C][64]; sums may be null (no update wanted).
+// One assignment pass.  xh/xl: bf16 [BH][N][64]; mh/ml: bf16 [BH][C][64]; sums may be null (no update wanted), else they
+// hold the sums over the groups `old`, which may be `assign` itself.
 bool launch_kmeans_assign_tc(const KmeansTcArgs& a, cudaStream_t st) {
   using namespace tc;
   CUtensorMap mxh, mxl, mmh, mml;
@@ -586,7 +679,7 @@ bool launch_kmeans_assign_tc(const KmeansTcArgs& a, cudaStream_t st) {
   }
   p.phi = a.phi; p.ldphi = a.ldphi; p.xnorm = a.xnorm; p.mu2 = a.mu2; p.assign = a.assign;
   p.sums = a.sums; p.counts = a.counts; p.fx_shift = a.fx_shift; p.flagged = a.flagged; p.flag_count = a.flag_count; p.err = a.err;
-  p.prev_changed = a.prev_changed; p.cur_changed = a.cur_changed; p.flag_count_next = a.flag_count_next;
+  p.old = a.old; p.mw = a.mw; p.prev_changed = a.prev_changed; p.cur_changed = a.cur_changed; p.flag_count_next = a.flag_count_next;
   // the three kernels of a pass (assignment, exact recheck, new centroids) follow each other with programmatic
   // dependent launches: 48 short dependent launches per k-means run otherwise pay their launch latency one by one
   launch_pdl(k_kmeans_assign_tc, dim3(p.ctas_per_head, a.BH), dim3(kKmThreads), kKmSmemBytes, st, mxh, mxl, mmh, mml, p);
@@ -594,11 +687,11 @@ bool launch_kmeans_assign_tc(const KmeansTcArgs& a, cudaStream_t st) {
   const int per_head = std::max(1, 2 * sm_count() / a.BH);
   if (rs <= kRecheckSmemMax)
     launch_pdl(k_assign_recheck_staged, dim3(per_head, a.BH), dim3(256), rs, st, a.flagged, a.flag_count, a.phi, a.ldphi, a.N, a.r, a.R, a.mu, a.C,
-               a.assign, a.sums, a.counts, a.fx_shift, a.recheck_total, (int)(a.prev_changed == nullptr), a.cur_changed);
+               a.assign, a.sums, a.counts, a.fx_shift, a.recheck_total, a.old, (int)(a.prev_changed == nullptr), a.cur_changed);
   else
     k_assign_recheck<<<dim3(std::max(1, 4 * sm_count() / a.BH), a.BH), 256, 0, st>>>(a.flagged, a.flag_count, a.phi, a.ldphi, a.N, a.r, a.R, a.mu, a.C,
                                                                                      a.assign, a.sums, a.counts, a.fx_shift, a.recheck_total,
-                                                                                     a.prev_changed == nullptr, a.cur_changed);
+                                                                                     a.old, (int)(a.prev_changed == nullptr), a.cur_changed);
   return true;
 }
 

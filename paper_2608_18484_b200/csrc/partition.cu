@@ -387,7 +387,7 @@ __global__ void k_kmeans_init(const float* __restrict__ phi, int ldphi, int N, i
     frexpf(m, &e2);                                  // m < 2^e2
     int nb = 0;
     while ((1ll << nb) < (i64)N) ++nb;
-    int sh = 61 - nb - e2;
+    int sh = min(61 - nb, 50) - e2;                  // (50: what k_kmeans_group_sums adds up in int32)
     fx_shift[bh] = max(-60, min(sh, 60));
   }
 }
@@ -401,7 +401,8 @@ __global__ void __launch_bounds__(1024) k_kmeans_finalize(float* __restrict__ mu
                                                           float* __restrict__ mumax, i64* __restrict__ sums,
                                                           int* __restrict__ counts, const int* __restrict__ fx_shift,
                                                           int C, int r, int R, int update,
-                                                          __nv_bfloat16* __restrict__ mh, __nv_bfloat16* __restrict__ ml) {
+                                                          __nv_bfloat16* __restrict__ mh, __nv_bfloat16* __restrict__ ml,
+                                                          __nv_bfloat16* __restrict__ mw, int Cpad) {
   __shared__ float red[34];
   const int bh = blockIdx.x;
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = blockDim.x >> 5;
@@ -409,6 +410,15 @@ __global__ void __launch_bounds__(1024) k_kmeans_finalize(float* __restrict__ mu
   pdl_launch_dependents();
   const double inv_sc = update ? ldexp(1.0, -fx_shift[bh]) : 0.0;
   float mx = 0.f;
+  auto store_words = [&](float v, int c) {                       // the three bf16 words of ||mu_c||^2, then zeros
+    const __nv_bfloat16 w0 = __float2bfloat16_rn(v);
+    const float v1 = v - __bfloat162float(w0);
+    const __nv_bfloat16 w1 = __float2bfloat16_rn(v1), w2 = __float2bfloat16_rn(v1 - __bfloat162float(w1));
+    const uint32_t lo = (uint32_t)__bfloat16_as_ushort(w0) | ((uint32_t)__bfloat16_as_ushort(w1) << 16);
+    *reinterpret_cast<uint4*>(mw + ((i64)bh * Cpad + c) * 8) = make_uint4(lo, __bfloat16_as_ushort(w2), 0u, 0u);
+  };
+  if (mw != nullptr && blockIdx.y == 0)
+    for (int c = C + threadIdx.x; c < Cpad; c += blockDim.x) store_words(kKmFar, c);
   for (int c = blockIdx.y * nw + w; c < C; c += nw * gridDim.y) {
     float* m = mu + ((i64)bh * C + c) * R;
     i64* s = sums + ((i64)bh * C + c) * R;
@@ -420,13 +430,13 @@ __global__ void __launch_bounds__(1024) k_kmeans_finalize(float* __restrict__ mu
         v = m[k];
         if (update) {
           if (cnt > 0 && k < r) { v = (float)((double)s[k] * inv_sc / (double)cnt); m[k] = v; }
-          s[k] = 0;
+          if (update == 1) s[k] = 0;
         }
         n2 += (double)v * (double)v;
       }
       if (mh != nullptr && k < 64) {
-        // the two bf16 words of the centroid for the tensor-core assignment, [C][64] with zeros beyond r
-        const float x = k < r ? v : 0.f;
+        // the two bf16 words of -2 mu for the tensor-core assignment, [C][64] with zeros beyond r
+        const float x = k < r ? -2.f * v : 0.f;
         const __nv_bfloat16 hb = __float2bfloat16_rn(x);
         mh[((i64)bh * C + c) * 64 + k] = hb;
         ml[((i64)bh * C + c) * 64 + k] = __float2bfloat16_rn(x - __bfloat162float(hb));
@@ -436,7 +446,8 @@ __global__ void __launch_bounds__(1024) k_kmeans_finalize(float* __restrict__ mu
     __syncwarp();
     if (lane == 0) {
       mu2[(i64)bh * C + c] = (float)n2;
-      if (update) counts[(i64)bh * C + c] = 0;
+      if (update == 1) counts[(i64)bh * C + c] = 0;
+      if (mw != nullptr) store_words((float)n2, c);
       mx = fmaxf(mx, (float)sqrt(n2) * 1.0000002f);
     }
   }
@@ -446,53 +457,66 @@ __global__ void __launch_bounds__(1024) k_kmeans_finalize(float* __restrict__ mu
   }
 }
 
-// Warm start (Appendix C.1): fixed-point sums and counts of the CURRENT features over the groups of a previous
-// partition `prev` [BH][N]; the update step that follows turns them into the initial centroids (a group that the
-// previous partition left empty keeps the strided row k_kmeans_init gave it).  One warp per 32 consecutive rows,
-// lanes = feature columns (2 lane, 2 lane + 1), one atomic per (cluster present in the warp, column).  Entries of
-// `prev` outside [0, C) are ignored.
-__global__ void __launch_bounds__(256) k_kmeans_warm_sums(const float* __restrict__ phi, int ldphi, int N, int r, int R, int C,
-                                                          const int* __restrict__ prev, i64* __restrict__ sums,
-                                                          int* __restrict__ counts, const int* __restrict__ fx_shift) {
+// Fixed-point sums and counts of the features over the groups of a partition [BH][N] (ids outside [0, C) are ignored): the
+// first centroids of a warm start (Appendix C.1; a group that the previous partition left empty keeps the strided row
+// k_kmeans_init gave it), and the sums after the first tensor-core assignment, which later passes only update.
+// Every row is rounded once, as in a later move of that row, so the sums stay exact: x 2^shift = h 2^26 + l with
+// h = rint(x 2^(shift - 26)) and l = rint of what is left, both below 2^26 and added over up to 32 rows in int32.
+// One warp per 32 consecutive rows, lane = columns lane and lane + 32, two rows in flight, one atomic per (group present in
+// the warp, column).  Bound by those atomics (a warp's 32 rows fall into about 20 groups after a cold start): 67 us at
+// 24 heads of 32760 rows and 64 columns, 48 us on the partition of a call before (few groups per warp).
+__global__ void __launch_bounds__(256) k_kmeans_group_sums(const float* __restrict__ phi, int ldphi, int N, int r, int R, int C,
+                                                           const int* __restrict__ assign, i64* __restrict__ sums,
+                                                           int* __restrict__ counts, const int* __restrict__ fx_shift) {
   const unsigned FULL = 0xffffffffu;
+  pdl_wait();                                                   // the assignment comes from the kernels before
+  pdl_launch_dependents();
   const int bh = blockIdx.y, lane = threadIdx.x & 31;
   const int rowbase = (blockIdx.x * 8 + (threadIdx.x >> 5)) * 32;
   if (rowbase >= N) return;
   const int row = rowbase + lane;
   int cl_mine = -1;
-  if (row < N) { const int c = prev[(i64)bh * N + row]; if (c >= 0 && c < C) cl_mine = c; }
-  const float scl = __int_as_float((127 + fx_shift[bh]) << 23);
+  if (row < N) { const int c = assign[(i64)bh * N + row]; if (c >= 0 && c < C) cl_mine = c; }
+  const float s_hi = __int_as_float((127 + fx_shift[bh] - 26) << 23);
   for (int cb = 0; cb < R; cb += 64) {                         // 64 columns at a time (two passes for raw activations)
-    const int col = cb + 2 * lane;
-    const bool cok = col < r;
-    float pv0[32], pv1[32];
-#pragma unroll
-    for (int rr = 0; rr < 32; ++rr) {
-      const int rw = min(rowbase + rr, N - 1);
-      const float2 x2 = cok ? *reinterpret_cast<const float2*>(phi + ((i64)bh * N + rw) * ldphi + col) : make_float2(0.f, 0.f);
-      pv0[rr] = x2.x; pv1[rr] = x2.y;
-    }
+    const int col = cb + lane;
+    const bool ok0 = col < r, ok1 = col + 32 < r;
+    const float* p = phi + ((i64)bh * N + rowbase) * ldphi + col;
     unsigned todo = __ballot_sync(FULL, cl_mine >= 0);
     while (todo) {
       const int leader = __ffs(todo) - 1;
       const int cl = __shfl_sync(FULL, cl_mine, leader);
-      const unsigned members = __ballot_sync(FULL, cl_mine == cl) & todo;
-      todo &= ~members;
-      float a0 = 0.f, a1 = 0.f;
-#pragma unroll
-      for (int rr = 0; rr < 32; ++rr)
-        if ((members >> rr) & 1u) { a0 += pv0[rr]; a1 += pv1[rr]; }
-      i64* sp = sums + ((i64)bh * C + cl) * R;
-      if (col < r) atomicAdd(reinterpret_cast<u64*>(sp + col), (u64)__float2ll_rn(a0 * scl));
-      if (col + 1 < r) atomicAdd(reinterpret_cast<u64*>(sp + col + 1), (u64)__float2ll_rn(a1 * scl));
-      if (lane == 0 && cb == 0) atomicAdd(counts + (i64)bh * C + cl, __popc(members));
+      unsigned m = __ballot_sync(FULL, cl_mine == cl);
+      todo &= ~m;
+      const int n = __popc(m);
+      int h0 = 0, h1 = 0, l0 = 0, l1 = 0;
+      auto add = [&](float xa, float xc) {
+        const float y0 = xa * s_hi, y1 = xc * s_hi;
+        const int a0 = __float2int_rn(y0), a1 = __float2int_rn(y1);
+        h0 += a0; h1 += a1;
+        l0 += __float2int_rn((y0 - (float)a0) * 67108864.f); l1 += __float2int_rn((y1 - (float)a1) * 67108864.f);
+      };
+      while (m) {
+        const float* pa = p + (i64)(__ffs(m) - 1) * ldphi;
+        m &= m - 1;
+        const float* pb = m ? p + (i64)(__ffs(m) - 1) * ldphi : nullptr;
+        m &= m - 1;
+        const float a0 = ok0 ? pa[0] : 0.f, a1 = ok1 ? pa[32] : 0.f;
+        const float b0 = ok0 && pb ? pb[0] : 0.f, b1 = ok1 && pb ? pb[32] : 0.f;
+        add(a0, a1);
+        add(b0, b1);
+      }
+      i64* sp = sums + ((i64)bh * C + cl) * R + col;
+      if (ok0) atomicAdd(reinterpret_cast<u64*>(sp), (u64)((i64)h0 * 67108864ll + l0));
+      if (ok1) atomicAdd(reinterpret_cast<u64*>(sp + 32), (u64)((i64)h1 * 67108864ll + l1));
+      if (lane == 0 && cb == 0) atomicAdd(counts + (i64)bh * C + cl, n);
     }
   }
 }
-void launch_kmeans_warm_sums(const float* phi, int ldphi, int BH, int N, int r, int C, const int* prev, i64* sums,
-                             int* counts, const int* fx_shift, cudaStream_t st) {
+void launch_kmeans_group_sums(const float* phi, int ldphi, int BH, int N, int r, int C, const int* assign, i64* sums,
+                              int* counts, const int* fx_shift, cudaStream_t st) {
   const int R = feature_ld(r);
-  k_kmeans_warm_sums<<<dim3((N + 255) / 256, BH), 256, 0, st>>>(phi, ldphi, N, r, R, C, prev, sums, counts, fx_shift);
+  launch_pdl(k_kmeans_group_sums, dim3((N + 255) / 256, BH), dim3(256), 0, st, phi, ldphi, N, r, R, C, assign, sums, counts, fx_shift);
 }
 
 void launch_kmeans_init(const float* phi, int ldphi, int BH, int N, int r, int C, u64 seed, int tag, int head0, float* mu,
@@ -502,14 +526,14 @@ void launch_kmeans_init(const float* phi, int ldphi, int BH, int N, int r, int C
   launch_pdl(k_kmeans_init, grid, dim3(256), 0, st, phi, ldphi, N, r, R, C, seed, tag, head0, mu, sums, counts, maxabs_bits, fx_shift);
 }
 void launch_kmeans_finalize(float* mu, float* mu2, float* mumax, i64* sums, int* counts, const int* fx_shift, int BH,
-                            int C, int r, int update, cudaStream_t st, __nv_bfloat16* mh, __nv_bfloat16* ml) {
-  const int R = feature_ld(r);
+                            int C, int r, int update, cudaStream_t st, __nv_bfloat16* mh, __nv_bfloat16* ml, __nv_bfloat16* mw) {
+  const int R = feature_ld(r), Cpad = km_padded(C);
   if (mumax != nullptr) {
-    k_kmeans_finalize<<<BH, 1024, 0, st>>>(mu, mu2, mumax, sums, counts, fx_shift, C, r, R, update, mh, ml);
+    k_kmeans_finalize<<<BH, 1024, 0, st>>>(mu, mu2, mumax, sums, counts, fx_shift, C, r, R, update, mh, ml, mw, Cpad);
   } else {
     // one warp per centroid, spread over enough CTAs to fill the GPU
     const int parts = std::max(1, std::min(32, (C + 7) / 8));
-    launch_pdl(k_kmeans_finalize, dim3(BH, parts), dim3(256), 0, st, mu, mu2, (float*)nullptr, sums, counts, fx_shift, C, r, R, update, mh, ml);
+    launch_pdl(k_kmeans_finalize, dim3(BH, parts), dim3(256), 0, st, mu, mu2, (float*)nullptr, sums, counts, fx_shift, C, r, R, update, mh, ml, mw, Cpad);
   }
 }
 
