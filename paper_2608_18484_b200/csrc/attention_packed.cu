@@ -90,7 +90,8 @@ k_attention_packed(const __grid_constant__ Maps mapsK, const __grid_constant__ M
   volatile int* misc = reinterpret_cast<volatile int*>(sm + Smem::misc);   // [0] tmem, [1] abort, [2] boxes, [3] skip, [8..41] scan scratch
   const uint32_t bars = base + Smem::bars;
   auto bar = [&](int i) { return bars + 8u * i; };
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  constexpr uint32_t FULLW = 0xffffffffu;
+  const int tid = threadIdx.x, warp = __shfl_sync(FULLW, tid >> 5, 0), lane = tid & 31;   // (uniform, and known to be)
   const int bh = blockIdx.y, m0 = blockIdx.x * kTile;
   const int cnt = prm.rem_cnt[bh];
   if (m0 >= cnt) return;
@@ -150,8 +151,8 @@ k_attention_packed(const __grid_constant__ Maps mapsK, const __grid_constant__ M
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
-  const uint32_t tmem = (uint32_t)misc[0];
-  const int total_boxes = misc[2];
+  const uint32_t tmem = __shfl_sync(FULLW, (uint32_t)misc[0], 0);
+  const int total_boxes = __shfl_sync(FULLW, misc[2], 0);
   const int n_tiles = (total_boxes + kSubPerTile - 1) / kSubPerTile;
   volatile int* abort_flag = &misc[1];
 
@@ -210,50 +211,58 @@ k_attention_packed(const __grid_constant__ Maps mapsK, const __grid_constant__ M
       }
     }
   } else if (warp == 9) {
-    // =========================== Q K^T issuer (the two products are issued by two threads) ====
-    if (lane == 0) {
+    // =========================== Q K^T issuer (the two products are issued by two warps, as in the 128-row kernel) ====
+    {
       const uint32_t idesc_qk = idesc_bf16(0, 128);
       const uint64_t k_desc0 = smem_desc(base + Smem::k, 16);
-      bool ok = mbar_wait(bar(Q_FULL), 0, abort_flag);
+      bool ok = __all_sync(FULLW, mbar_wait(bar(Q_FULL), 0, abort_flag));
       for (int i = 0; i < n_tiles && ok; ++i) {
         const int s = i % kStages;
         // score buffer i mod 2 is free once every softmax thread holds tile i - 2 in registers
-        if (i >= 2 && !mbar_wait(bar(S_FREE + (i & 1)), ((i - 2) >> 1) & 1, abort_flag)) { ok = false; break; }
-        if (!mbar_wait(bar(K_FULL + s), (i / kStages) & 1, abort_flag)) { ok = false; break; }
+        if (i >= 2) ok = mbar_wait(bar(S_FREE + (i & 1)), ((i - 2) >> 1) & 1, abort_flag);
+        ok = __all_sync(FULLW, ok && mbar_wait(bar(K_FULL + s), (i / kStages) & 1, abort_flag));
+        if (!ok) break;
         tc_fence_after();
         const uint32_t d = tmem + (uint32_t)(i & 1) * 128u;
         const uint64_t kd = k_desc0 + (uint64_t)(s * (kTileBytes >> 4));
+        if (elect_one()) {
 #pragma unroll
-        for (int kk = 0; kk < kD / 16; ++kk) {
-          const uint64_t koff = (uint64_t)((kk >> 2) * (kHalfBytes >> 4) + (kk & 3) * 2);
-          umma_bf16_ts(d, tmem + 448u + kk * 8, kd + koff, idesc_qk, kk > 0);
+          for (int kk = 0; kk < kD / 16; ++kk) {
+            const uint64_t koff = (uint64_t)((kk >> 2) * (kHalfBytes >> 4) + (kk & 3) * 2);
+            umma_bf16_ts(d, tmem + 448u + kk * 8, kd + koff, idesc_qk, kk > 0);
+          }
+          umma_commit(bar(K_EMPTY + s));
+          umma_commit(bar(S_FULL + (i & 1)));
         }
-        umma_commit(bar(K_EMPTY + s));
-        umma_commit(bar(S_FULL + (i & 1)));
+        __syncwarp();
       }
     }
   } else if (warp == 11) {
     // =========================== P V issuer ==================================================
-    if (lane == 0) {
+    {
       const uint32_t idesc_pv = idesc_bf16(1, 128);
       const uint64_t v_desc0 = smem_desc(base + Smem::v, kHalfBytes);
       bool ok = true;
       for (int i = 0; i < n_tiles && ok; ++i) {
         const int s = i % kStages;
-        if (!mbar_wait(bar(META_FULL + (i & 7)), (i >> 3) & 1, abort_flag)) { ok = false; break; }
-        const int nsub = (int)meta[i & 7].nsub;
-        if (!mbar_wait(bar(V_FULL + s), (i / kStages) & 1, abort_flag)) { ok = false; break; }
-        if (!mbar_wait(bar(P_FULL), i & 1, abort_flag)) { ok = false; break; }
+        ok = mbar_wait(bar(META_FULL + (i & 7)), (i >> 3) & 1, abort_flag);
+        const int nsub = __shfl_sync(FULLW, (int)meta[i & 7].nsub, 0);
+        ok = ok && mbar_wait(bar(V_FULL + s), (i / kStages) & 1, abort_flag);
+        ok = __all_sync(FULLW, ok && mbar_wait(bar(P_FULL), i & 1, abort_flag));
+        if (!ok) break;
         tc_fence_after();
         const uint64_t vd = v_desc0 + (uint64_t)(s * (kTileBytes >> 4));
+        if (elect_one()) {
 #pragma unroll
-        for (int kk = 0; kk < kSubPerTile; ++kk)
-          if (kk < nsub)
-            umma_bf16_ts(tmem + 320u, tmem + 256u + kk * 8, vd + (uint64_t)(kk * (kSubBytes >> 4)), idesc_pv, (i > 0 || kk > 0) ? 1u : 0u);
-        umma_commit(bar(V_EMPTY + s));
-        umma_commit(bar(P_EMPTY));
+          for (int kk = 0; kk < kSubPerTile; ++kk)
+            if (kk < nsub)
+              umma_bf16_ts(tmem + 320u, tmem + 256u + kk * 8, vd + (uint64_t)(kk * (kSubBytes >> 4)), idesc_pv, (i > 0 || kk > 0) ? 1u : 0u);
+          umma_commit(bar(V_EMPTY + s));
+          umma_commit(bar(P_EMPTY));
+        }
+        __syncwarp();
       }
-      if (ok) umma_commit(bar(O_DONE));                        // completes at once when there was no tile
+      if (ok && elect_one()) umma_commit(bar(O_DONE));         // completes at once when there was no tile
     }
   } else if (warp < 8) {
     // =========================== softmax (warps 0-7) =======================================

@@ -5,9 +5,9 @@
 //   warps 0-7  softmax: warps w and w+4 share the 32 rows of TMEM quadrant w and split the
 //              128 scores of a row in two halves (keys 0-63 / 64-127 of the tile)
 //   warp  8    TMA producer of Q and the key tiles (+ tile meta ring)
-//   warp  9    issues Q K^T (one thread); owns the TMEM allocation
+//   warp  9    issues Q K^T (one elected lane); owns the TMEM allocation
 //   warp  10   TMA producer of the value tiles
-//   warp  11   issues P V (one thread)
+//   warp  11   issues P V (one elected lane)
 // The routed keys/values arrive as one concatenated sequence of 16-row boxes (tiles of 128 keys, only
 // range ends are ragged); consecutive boxes of one key range are fetched by one copy per set bit of their
 // number (tensor maps with 16-, 32-, 64- and 128-row boxes).  Data path per key tile i:
@@ -102,7 +102,8 @@ k_attention_tc(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__
   const uint32_t bars = base + Smem::bars;
   auto bar = [&](int i) { return bars + 8u * i; };
 
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  constexpr uint32_t FULLW = 0xffffffffu;
+  const int tid = threadIdx.x, warp = __shfl_sync(FULLW, tid >> 5, 0), lane = tid & 31;   // (uniform, and known to be)
   const int bh = blockIdx.y, b = bh / prm.H, h = bh % prm.H;
   // ---- which query tile ---------------------------------------------------------------
   // Few dependent global reads: one round finds the query group of this tile (every thread tests one group),
@@ -171,8 +172,8 @@ k_attention_tc(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
-  const uint32_t tmem = (uint32_t)misc[0];
-  const int total_boxes = misc[2];
+  const uint32_t tmem = __shfl_sync(FULLW, (uint32_t)misc[0], 0);
+  const int total_boxes = __shfl_sync(FULLW, misc[2], 0);
   const int n_tiles = (total_boxes + kSubPerTile - 1) / kSubPerTile;
   volatile int* abort_flag = &misc[1];
 
@@ -255,53 +256,65 @@ k_attention_tc(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__
     // The two products are issued by two threads on different warp schedulers: an issuing thread shares its
     // scheduler with two softmax warps that rarely leave it a slot, and the score tile two steps ahead must not
     // queue behind the P V of the current one.
-    if (lane == 0 && n_tiles > 0) {
+    // The whole warp walks the tiles and one elected lane issues; loop control goes through votes, so that it is known
+    // to be uniform and the descriptors stay in uniform registers.  With a loop in one thread (divergent exits) an
+    // instruction cost its issuer about 70 cycles instead of 31: dense launch 12.7 -> 11.9 ms, block-sparse stage of the
+    // 480p-like call 4.95 -> 4.43 ms.
+    if (n_tiles > 0) {
       const uint32_t idesc_qk = idesc_bf16(0, 128);
       // descriptors are built once; inside the loops only their address field moves (in 16-byte units)
       const uint64_t q_desc = smem_desc(base + Smem::q, 16);
       const uint64_t k_desc0 = smem_desc(base + Smem::k, 16);
-      bool ok = mbar_wait(bar(Q_FULL), 0, abort_flag);
+      bool ok = __all_sync(FULLW, mbar_wait(bar(Q_FULL), 0, abort_flag));
       for (int i = 0; i < n_tiles && ok; ++i) {
         const int s = i % kKStages;
         // score buffer i mod 2 is free once every softmax thread holds tile i - 2 in registers
-        if (i >= 2 && !mbar_wait(bar(S_FREE + (i & 1)), ((i - 2) >> 1) & 1, abort_flag)) { ok = false; break; }
-        if (!mbar_wait(bar(K_FULL + s), (i / kKStages) & 1, abort_flag)) { ok = false; break; }
+        if (i >= 2) ok = mbar_wait(bar(S_FREE + (i & 1)), ((i - 2) >> 1) & 1, abort_flag);
+        ok = __all_sync(FULLW, ok && mbar_wait(bar(K_FULL + s), (i / kKStages) & 1, abort_flag));
+        if (!ok) break;
         tc_fence_after();
         const uint32_t d = tmem + (uint32_t)(i & 1) * 128u;
         const uint64_t kd = k_desc0 + (uint64_t)(s * (kTileBytes >> 4));
+        if (elect_one()) {
 #pragma unroll
-        for (int kk = 0; kk < kD / 16; ++kk) {
-          const uint64_t koff = (uint64_t)((kk >> 2) * (kHalfBytes >> 4) + (kk & 3) * 2);     // compile-time constant
-          umma_bf16(d, q_desc + koff, kd + koff, idesc_qk, kk > 0);
+          for (int kk = 0; kk < kD / 16; ++kk) {
+            const uint64_t koff = (uint64_t)((kk >> 2) * (kHalfBytes >> 4) + (kk & 3) * 2);     // compile-time constant
+            umma_bf16(d, q_desc + koff, kd + koff, idesc_qk, kk > 0);
+          }
+          umma_commit(bar(K_EMPTY + s));
+          umma_commit(bar(S_FULL + (i & 1)));
         }
-        umma_commit(bar(K_EMPTY + s));
-        umma_commit(bar(S_FULL + (i & 1)));
+        __syncwarp();
       }
     }
   } else if (warp == 11) {
     // =========================== P V issuer ==============================================
-    if (lane == 0 && n_tiles > 0) {
+    if (n_tiles > 0) {
       const uint32_t idesc_pv = idesc_bf16(1, 128);
       const uint64_t v_desc0 = smem_desc(base + Smem::v, kHalfBytes);
       bool ok = true;
       for (int i = 0; i < n_tiles && ok; ++i) {
         const int s = i % kVStages;
-        if (!mbar_wait(bar(META_FULL + (i & 7)), (i >> 3) & 1, abort_flag)) { ok = false; break; }
-        const int nsub = (int)meta[i & 7].y;
-        if (!mbar_wait(bar(V_FULL + s), (i / kVStages) & 1, abort_flag)) { ok = false; break; }
-        if (!mbar_wait(bar(P_FULL + (i & 1)), (i >> 1) & 1, abort_flag)) { ok = false; break; }   // P(i) in TMEM, O rescaled if needed
+        ok = mbar_wait(bar(META_FULL + (i & 7)), (i >> 3) & 1, abort_flag);
+        const int nsub = __shfl_sync(FULLW, (int)meta[i & 7].y, 0);
+        ok = ok && mbar_wait(bar(V_FULL + s), (i / kVStages) & 1, abort_flag);
+        ok = __all_sync(FULLW, ok && mbar_wait(bar(P_FULL + (i & 1)), (i >> 1) & 1, abort_flag));   // P(i) in TMEM, O rescaled if needed
+        if (!ok) break;
         tc_fence_after();
         const uint32_t d = tmem + 320u;
         const uint32_t pa = tmem + ((i & 1) ? 448u : 256u);
         const uint64_t vd = v_desc0 + (uint64_t)(s * (kTileBytes >> 4));
+        if (elect_one()) {
 #pragma unroll
-        for (int kk = 0; kk < kSubPerTile; ++kk)
-          if (kk < nsub)
-            umma_bf16_ts(d, pa + kk * 8, vd + (uint64_t)(kk * (kSubBytes >> 4)), idesc_pv, (i > 0 || kk > 0) ? 1u : 0u);
-        umma_commit(bar(V_EMPTY + s));
-        umma_commit(bar(P_EMPTY + (i & 1)));
+          for (int kk = 0; kk < kSubPerTile; ++kk)
+            if (kk < nsub)
+              umma_bf16_ts(d, pa + kk * 8, vd + (uint64_t)(kk * (kSubBytes >> 4)), idesc_pv, (i > 0 || kk > 0) ? 1u : 0u);
+          umma_commit(bar(V_EMPTY + s));
+          umma_commit(bar(P_EMPTY + (i & 1)));
+        }
+        __syncwarp();
       }
-      if (ok) umma_commit(bar(O_DONE));
+      if (ok && elect_one()) umma_commit(bar(O_DONE));
     }
   } else if (warp < 8) {
     // =========================== softmax (warps 0-7) =======================================
