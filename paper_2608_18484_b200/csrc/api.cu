@@ -340,7 +340,7 @@ void carve_attend(Carver& c, const Resolved& r, AttendWs* w) {
   void* Qg = c.take<char>(BH * N * d * r.es);
   void* Kg = c.take<char>(BH * N * d * r.es);
   void* Vg = c.take<char>(BH * N * d * r.es);
-  const bool staged = r.dtype == SPARSEPR_BF16 && r.d == 128 && r.mode == 0 && r.M > 0;
+  const bool staged = r.dtype == SPARSEPR_BF16 && r.mode == 0 && r.M > 0;
   __nv_bfloat16* Olo = c.take<__nv_bfloat16>(staged ? BH * N * d : 0);
   const size_t M1 = std::max(r.M, 1);
   // tensor-core probe kernel: one CTA per (128 probe rows, key slice), about one wave
@@ -534,7 +534,7 @@ static sparsepr_status_t plan_impl(const sparsepr_shape_t* shape, const sparsepr
     launch_eig_top(metric, (i64)r.d * r.d, r.BHkv, r.d, r.rK, 0, r.dtype == SPARSEPR_F32, p->FK, p->lam, p->eigws, st);
     tm.mark(SPARSEPR_STAGE_KEY_METRIC);
     if (project_tc_supported(r.dtype, r.d, r.rK, r.ks)) {
-      if (!launch_project_tc(K, r.ks, r.BHkv, r.Hkv, r.N, r.rK, p->FK, false, 0.f, p->phi, r.RK, p->maxabs, p->Ft, p->err, st)) { delete p; return SPARSEPR_ERR_CUDA; }
+      if (!launch_project_tc(K, r.ks, r.BHkv, r.Hkv, r.N, r.d, r.rK, p->FK, false, 0.f, p->phi, r.RK, p->maxabs, p->Ft, p->err, st)) { delete p; return SPARSEPR_ERR_CUDA; }
     } else {
       launch_project(r.dtype, K, r.ks, r.BHkv, r.Hkv, r.N, r.d, r.rK, p->FK, false, 0.f, p->phi, r.RK, p->maxabs, p->err, st);
     }
@@ -555,7 +555,7 @@ static sparsepr_status_t plan_impl(const sparsepr_shape_t* shape, const sparsepr
     launch_eig_top(p->Mmat, (i64)r.d * r.d, r.BHkv, r.d, r.rQ, 0, r.dtype == SPARSEPR_F32, p->FQ, p->lam, p->eigws, st);
     tm.mark(SPARSEPR_STAGE_QUERY_METRIC);
     if (project_tc_supported(r.dtype, r.d, r.rQ, r.qs)) {
-      if (!launch_project_tc(Q, r.qs, r.BH, r.H, r.N, r.rQ, p->FQ, true, r.eps_rms, p->phi, r.RQ, p->maxabs, p->Ft, p->err, st, r.G)) { delete p; return SPARSEPR_ERR_CUDA; }
+      if (!launch_project_tc(Q, r.qs, r.BH, r.H, r.N, r.d, r.rQ, p->FQ, true, r.eps_rms, p->phi, r.RQ, p->maxabs, p->Ft, p->err, st, r.G)) { delete p; return SPARSEPR_ERR_CUDA; }
     } else {
       launch_project(r.dtype, Q, r.qs, r.BH, r.H, r.N, r.d, r.rQ, p->FQ, true, r.eps_rms, p->phi, r.RQ, p->maxabs, p->err, st);
     }
@@ -726,7 +726,7 @@ static sparsepr_status_t attend_impl(const sparsepr_plan_t* p, const void* Q, co
     cudaStreamWaitEvent(st, p->ev_join2, 0);
     tm.mark(SPARSEPR_STAGE_ATTENTION);
     if (overlap) { join_side(p, st); p->side_pending = false; }
-    if (fitted && !launch_correction_tc(w.c, w.At, w.Olo, O, r.os, r.BH, r.H, r.N, p->err, st)) return SPARSEPR_ERR_CUDA;
+    if (fitted && !launch_correction_tc(w.c, w.At, w.Olo, O, r.os, r.BH, r.H, r.N, r.d, p->err, st)) return SPARSEPR_ERR_CUDA;
     tm.mark(SPARSEPR_STAGE_CORRECTION);
   } else {
     aa.A = fitted ? w.A : nullptr; aa.c = fitted ? w.c : nullptr;      // correction fused into this kernel's epilogue
@@ -827,7 +827,7 @@ sparsepr_status_t sparsepr_plan_stats(const sparsepr_plan_t* p, sparsepr_stats_t
     out->nonempty_q_groups_min = std::min(out->nonempty_q_groups_min, neQ);
     // pairs issued by the tiled kernel over the concatenated routed keys: the tensor-core kernel uses
     // 128-row query tiles and 128-key tiles built from 16-row boxes, the float32 kernel 64 x 64 tiles
-    const bool tcpath = r.dtype == SPARSEPR_BF16 && r.d == 128;
+    const bool tcpath = r.dtype == SPARSEPR_BF16;
     const int qtile = tcpath ? 128 : 64, ktile = tcpath ? 128 : 64, box = tcpath ? 16 : 1;
     const int* rpp = &rp[(size_t)bh * (r.Cq + 1)];
     const int* rii = &ri[(size_t)bh * r.Cq * r.Ck];

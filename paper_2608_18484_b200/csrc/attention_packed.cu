@@ -1,4 +1,4 @@
-// Block-sparse attention (Eq. 3) for the short remainders of the query groups (bf16, d = d_v = 128).
+// Block-sparse attention (Eq. 3) for the short remainders of the query groups (bf16, D = d = d_v = 64 or 128).
 //
 // A query group of n rows gives floor(n / 128) full tiles to the 128-row kernel; when the n mod 128 rows
 // that are left are at most kRemRows they come here.  An M = 128 tensor-core tile for a handful of rows
@@ -15,7 +15,7 @@
 //              boxes (tiles of 128 keys, every box inside one group), and publishes the group of every box;
 //   warp  10   V producer
 //   warp  9    issues Q K^T (one thread); owns the TMEM allocation;  warp 11 issues P V (one thread)
-// TMEM: S_0 [0,128), S_1 [128,256), P [256,320), O [320,448), Q [448,512); both products take their A
+// TMEM: S_0 [0,128), S_1 [128,256), P [256,320), O [320,320+D), Q [448,448+D/2); both products take their A
 // operand from tensor memory.  Reference maxima move lazily (growth beyond 2^8), as in the 128-row kernel.
 // Every mbarrier wait is bounded; on expiry the CTA records SPARSEPR_ERR_TIMEOUT and leaves.
 #include <cuda.h>
@@ -29,21 +29,20 @@ namespace packed {
 constexpr int kThreads = 384;
 constexpr int kPolyOf8 = 3;                           // pairs of every 8 whose exponential is a polynomial on the FMA pipe
 constexpr int kTile = 128;
-constexpr int kD = 128;
 constexpr int kSub = 16;                               // rows per TMA box of the K/V stream
 constexpr int kSubPerTile = kTile / kSub;
 constexpr uint32_t kHalfBytes = kTile * 128;          // [128 rows x 64 bf16]
-constexpr uint32_t kTileBytes = 2 * kHalfBytes;       // 32 KB
+template <int D> constexpr uint32_t kTileBytes = (D / 64) * kHalfBytes;   // 32 KB at D = 128, 16 KB at D = 64
 constexpr uint32_t kSubBytes = kSub * 128;
 constexpr int kStages = 2;
 
 // per key tile: number of boxes, valid rows of every box (4 bits each, minus one), K/V group of every box
 struct Meta { uint32_t cnt_bits, nsub; unsigned short grp[kSubPerTile]; uint32_t pad[2]; };   // 32 bytes
 
-struct Smem {
+template <int D> struct Smem {
   static constexpr uint32_t k = 0;
-  static constexpr uint32_t v = k + kStages * kTileBytes;
-  static constexpr uint32_t bitmap = v + kStages * kTileBytes;           // [kMaxGroups/32 words][128 rows]
+  static constexpr uint32_t v = k + kStages * kTileBytes<D>;
+  static constexpr uint32_t bitmap = v + kStages * kTileBytes<D>;           // [kMaxGroups/32 words][128 rows]
   static constexpr uint32_t uni = bitmap + (kMaxGroups / 32) * 128 * 4;  // [kMaxGroups/32] union of the rows' route bitmaps
   static constexpr uint32_t ranges = uni + (kMaxGroups / 32) * 4;        // int2[kMaxGroups] (start, length) of the wanted K/V groups
   static constexpr uint32_t gid = ranges + kMaxGroups * 8;               // unsigned short[kMaxGroups] their group ids
@@ -54,7 +53,7 @@ struct Smem {
   static constexpr uint32_t misc = bars + 32 * 8;
   static constexpr uint32_t total = misc + 256;
 };
-static_assert(Smem::total <= 227 * 1024, "shared memory");
+static_assert(Smem<128>::total <= 227 * 1024, "shared memory");
 enum Bar { Q_FULL = 0, K_FULL = 1, K_EMPTY = K_FULL + kStages, V_FULL = K_EMPTY + kStages, V_EMPTY = V_FULL + kStages,
            S_FULL = V_EMPTY + kStages, S_FREE = S_FULL + 2, P_FULL = S_FREE + 2, P_EMPTY, O_DONE, META_FULL, kNumBars = META_FULL + 8 };
 static_assert(kNumBars <= 32, "barrier area");
@@ -67,28 +66,32 @@ struct Params {
   float scale_log2;
   const int *rem_pos, *rem_grp, *rem_cnt;      // [BH][N] group-major position and query group of every packed row; [BH] their number
   const int *kv_off, *route_ptr, *route_idx, *q_perm;
-  const __nv_bfloat16* Qg;                     // [BH][N][128] group-major
+  const __nv_bfloat16* Qg;                     // [BH][N][D] group-major
   __nv_bfloat16* O; i64 os[3];
   float* O_sparse;
-  __nv_bfloat16* O_lo;             // optional [BH][N][128]: o - bf16(o), original order (second word for the correction pass)
+  __nv_bfloat16* O_lo;             // optional [BH][N][D]: o - bf16(o), original order (second word for the correction pass)
   int* err;
 };
 
+template <int D>
 __global__ void __launch_bounds__(kThreads, 1)
 k_attention_packed(const __grid_constant__ Maps mapsK, const __grid_constant__ Maps mapsV, Params prm) {
+  using SM = Smem<D>;
+  constexpr int kHalves = D / 64;                                          // 64-column blocks of a row
+  constexpr int kOc = D / 2;                                               // query / output columns of a thread
   extern __shared__ __align__(1024) unsigned char smem_raw[];
   const uint32_t base = smem_u32(smem_raw);
   unsigned char* sm = smem_raw;
-  unsigned* bitmap = reinterpret_cast<unsigned*>(sm + Smem::bitmap);
-  unsigned* uni = reinterpret_cast<unsigned*>(sm + Smem::uni);
-  int2* ranges = reinterpret_cast<int2*>(sm + Smem::ranges);
-  unsigned short* gid = reinterpret_cast<unsigned short*>(sm + Smem::gid);
-  int* idx = reinterpret_cast<int*>(sm + Smem::idx);
-  float* xmax = reinterpret_cast<float*>(sm + Smem::xchg);
+  unsigned* bitmap = reinterpret_cast<unsigned*>(sm + SM::bitmap);
+  unsigned* uni = reinterpret_cast<unsigned*>(sm + SM::uni);
+  int2* ranges = reinterpret_cast<int2*>(sm + SM::ranges);
+  unsigned short* gid = reinterpret_cast<unsigned short*>(sm + SM::gid);
+  int* idx = reinterpret_cast<int*>(sm + SM::idx);
+  float* xmax = reinterpret_cast<float*>(sm + SM::xchg);
   float* xsum = xmax + 4 * 128;
-  Meta* meta = reinterpret_cast<Meta*>(sm + Smem::meta);
-  volatile int* misc = reinterpret_cast<volatile int*>(sm + Smem::misc);   // [0] tmem, [1] abort, [2] boxes, [3] skip, [8..41] scan scratch
-  const uint32_t bars = base + Smem::bars;
+  Meta* meta = reinterpret_cast<Meta*>(sm + SM::meta);
+  volatile int* misc = reinterpret_cast<volatile int*>(sm + SM::misc);   // [0] tmem, [1] abort, [2] boxes, [3] skip, [8..41] scan scratch
+  const uint32_t bars = base + SM::bars;
   auto bar = [&](int i) { return bars + 8u * i; };
   constexpr uint32_t FULLW = 0xffffffffu;
   const int tid = threadIdx.x, warp = __shfl_sync(FULLW, tid >> 5, 0), lane = tid & 31;   // (uniform, and known to be)
@@ -113,7 +116,7 @@ k_attention_packed(const __grid_constant__ Maps mapsK, const __grid_constant__ M
     misc[1] = 0; misc[2] = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
-  if (warp == 9) tmem_alloc(base + Smem::misc, 512);
+  if (warp == 9) tmem_alloc(base + SM::misc, 512);
   // route bitmap of every row of the tile, transposed: bitmap[word][row]
   for (int e = tid; e < words * 128; e += kThreads) bitmap[e] = 0u;
   __syncthreads();
@@ -162,7 +165,7 @@ k_attention_packed(const __grid_constant__ Maps mapsK, const __grid_constant__ M
     if (n_tiles > 0) {
       const bool is_k = warp == 8;
       const int full0 = is_k ? K_FULL : V_FULL, empty0 = is_k ? K_EMPTY : V_EMPTY;
-      const uint32_t buf0 = base + (is_k ? Smem::k : Smem::v);
+      const uint32_t buf0 = base + (is_k ? SM::k : SM::v);
       const Maps* maps = is_k ? &mapsK : &mapsV;
       int ri = 0, off = 0;
       bool ok = true;
@@ -201,12 +204,12 @@ k_attention_packed(const __grid_constant__ Maps mapsK, const __grid_constant__ M
           __syncwarp();
           if (lane == 0) mbar_arrive(bar(META_FULL + (i & 7)));
         }
-        if (lane == 0) mbar_expect_tx(bar(full0 + s), nsub * 2 * kSubBytes);
+        if (lane == 0) mbar_expect_tx(bar(full0 + s), nsub * kHalves * kSubBytes);
         __syncwarp();
         if (my_k >= 0) {
-          const uint32_t dst = buf0 + s * kTileBytes + lane * kSubBytes;
-          tma_load_4d(dst, &maps->m[my_k], bar(full0 + s), 0, my_start, kvh, 0);
-          tma_load_4d(dst + kHalfBytes, &maps->m[my_k], bar(full0 + s), 64, my_start, kvh, 0);
+          const uint32_t dst = buf0 + s * kTileBytes<D> + lane * kSubBytes;
+#pragma unroll
+          for (int c = 0; c < kHalves; ++c) tma_load_4d(dst + c * kHalfBytes, &maps->m[my_k], bar(full0 + s), 64 * c, my_start, kvh, 0);
         }
       }
     }
@@ -214,7 +217,7 @@ k_attention_packed(const __grid_constant__ Maps mapsK, const __grid_constant__ M
     // =========================== Q K^T issuer (the two products are issued by two warps, as in the 128-row kernel) ====
     {
       const uint32_t idesc_qk = idesc_bf16(0, 128);
-      const uint64_t k_desc0 = smem_desc(base + Smem::k, 16);
+      const uint64_t k_desc0 = smem_desc(base + SM::k, 16);
       bool ok = __all_sync(FULLW, mbar_wait(bar(Q_FULL), 0, abort_flag));
       for (int i = 0; i < n_tiles && ok; ++i) {
         const int s = i % kStages;
@@ -224,10 +227,10 @@ k_attention_packed(const __grid_constant__ Maps mapsK, const __grid_constant__ M
         if (!ok) break;
         tc_fence_after();
         const uint32_t d = tmem + (uint32_t)(i & 1) * 128u;
-        const uint64_t kd = k_desc0 + (uint64_t)(s * (kTileBytes >> 4));
+        const uint64_t kd = k_desc0 + (uint64_t)(s * (kTileBytes<D> >> 4));
         if (elect_one()) {
 #pragma unroll
-          for (int kk = 0; kk < kD / 16; ++kk) {
+          for (int kk = 0; kk < D / 16; ++kk) {
             const uint64_t koff = (uint64_t)((kk >> 2) * (kHalfBytes >> 4) + (kk & 3) * 2);
             umma_bf16_ts(d, tmem + 448u + kk * 8, kd + koff, idesc_qk, kk > 0);
           }
@@ -240,8 +243,8 @@ k_attention_packed(const __grid_constant__ Maps mapsK, const __grid_constant__ M
   } else if (warp == 11) {
     // =========================== P V issuer ==================================================
     {
-      const uint32_t idesc_pv = idesc_bf16(1, 128);
-      const uint64_t v_desc0 = smem_desc(base + Smem::v, kHalfBytes);
+      const uint32_t idesc_pv = idesc_bf16(1, D);
+      const uint64_t v_desc0 = smem_desc(base + SM::v, kHalfBytes);
       bool ok = true;
       for (int i = 0; i < n_tiles && ok; ++i) {
         const int s = i % kStages;
@@ -251,7 +254,7 @@ k_attention_packed(const __grid_constant__ Maps mapsK, const __grid_constant__ M
         ok = __all_sync(FULLW, ok && mbar_wait(bar(P_FULL), i & 1, abort_flag));
         if (!ok) break;
         tc_fence_after();
-        const uint64_t vd = v_desc0 + (uint64_t)(s * (kTileBytes >> 4));
+        const uint64_t vd = v_desc0 + (uint64_t)(s * (kTileBytes<D> >> 4));
         if (elect_one()) {
 #pragma unroll
           for (int kk = 0; kk < kSubPerTile; ++kk)
@@ -271,24 +274,25 @@ k_attention_packed(const __grid_constant__ Maps mapsK, const __grid_constant__ M
     const uint32_t lane_addr = (uint32_t)(wq * 32) << 16;
     const uint32_t FULL = 0xffffffffu;
     const uint32_t p_addr = tmem + lane_addr + 256u + (uint32_t)hh * 32u;
-    const uint32_t o_addr = tmem + lane_addr + 320u + (uint32_t)hh * 64u;
+    const uint32_t o_addr = tmem + lane_addr + 320u + (uint32_t)(hh * kOc);
     const float sc = prm.scale_log2;
     const int my_pos = row < nrows ? rpos[row] : -1;
-    // this thread's half (64 of 128 dimensions) of its query row goes to tensor memory, two bf16 per column
+    // this thread's half (kOc of D dimensions) of its query row goes to tensor memory, two bf16 per column
     {
-      uint32_t qw[32];
+      uint32_t qw[kOc / 2];
       if (my_pos >= 0) {
-        const uint4* qp = reinterpret_cast<const uint4*>(prm.Qg + ((i64)bh * prm.N + my_pos) * kD + hh * 64);
+        const uint4* qp = reinterpret_cast<const uint4*>(prm.Qg + ((i64)bh * prm.N + my_pos) * D + hh * kOc);
 #pragma unroll
-        for (int c = 0; c < 8; ++c) {
+        for (int c = 0; c < kOc / 8; ++c) {
           const uint4 u = qp[c];
           qw[4 * c] = u.x; qw[4 * c + 1] = u.y; qw[4 * c + 2] = u.z; qw[4 * c + 3] = u.w;
         }
       } else {
 #pragma unroll
-        for (int c = 0; c < 32; ++c) qw[c] = 0u;
+        for (int c = 0; c < kOc / 2; ++c) qw[c] = 0u;
       }
-      tmem_st32u(tmem + lane_addr + 448u + (uint32_t)hh * 32u, qw);
+      if constexpr (D == 128) tmem_st32u(tmem + lane_addr + 448u + (uint32_t)hh * 32u, qw);
+      else tmem_st16u(tmem + lane_addr + 448u + (uint32_t)hh * 16u, qw);
       tc_fence_before();
       mbar_arrive(bar(Q_FULL));
     }
@@ -367,7 +371,7 @@ k_attention_packed(const __grid_constant__ Maps mapsK, const __grid_constant__ M
         p_free = true;
         tc_fence_after();
 #pragma unroll
-        for (int q = 0; q < 2; ++q) {
+        for (int q = 0; q < kOc / 32; ++q) {
           float t[32];
           tmem_ld32(o_addr + q * 32, t);
 #pragma unroll
@@ -420,12 +424,12 @@ k_attention_packed(const __grid_constant__ Maps mapsK, const __grid_constant__ M
     const float inv = ltot > 0.f ? 1.f / ltot : 0.f;
     if (ok) {
       tc_fence_after();
-      float o[64];
+      float o[kOc];
 #pragma unroll
-      for (int c = 0; c < 64; ++c) o[c] = 0.f;
+      for (int c = 0; c < kOc; ++c) o[c] = 0.f;
       if (n_tiles > 0) {
 #pragma unroll
-        for (int q = 0; q < 2; ++q) {
+        for (int q = 0; q < kOc / 32; ++q) {
           float t[32];
           tmem_ld32(o_addr + q * 32, t);
 #pragma unroll
@@ -435,18 +439,18 @@ k_attention_packed(const __grid_constant__ Maps mapsK, const __grid_constant__ M
       if (my_pos >= 0) {
         const int dst = prm.q_perm[(i64)bh * prm.N + my_pos];
         const int b = bh / prm.H, h = bh % prm.H;
-        __nv_bfloat16* op = prm.O + b * prm.os[0] + h * prm.os[1] + (i64)dst * prm.os[2] + hh * 64;
+        __nv_bfloat16* op = prm.O + b * prm.os[0] + h * prm.os[1] + (i64)dst * prm.os[2] + hh * kOc;
 #pragma unroll
-        for (int ch = 0; ch < 8; ++ch) {
+        for (int ch = 0; ch < kOc / 8; ++ch) {
           float v8[8];
 #pragma unroll
           for (int k = 0; k < 8; ++k) v8[k] = o[ch * 8 + k];
           store8(op + ch * 8, v8);
         }
         if (prm.O_lo) {                                        // what the bf16 rounding above dropped
-          __nv_bfloat16* lp = prm.O_lo + ((i64)bh * prm.N + dst) * kD + hh * 64;
+          __nv_bfloat16* lp = prm.O_lo + ((i64)bh * prm.N + dst) * D + hh * kOc;
 #pragma unroll
-          for (int ch = 0; ch < 8; ++ch) {
+          for (int ch = 0; ch < kOc / 8; ++ch) {
             float v8[8];
 #pragma unroll
             for (int k = 0; k < 8; ++k) v8[k] = o[ch * 8 + k] - __bfloat162float(__float2bfloat16_rn(o[ch * 8 + k]));
@@ -454,9 +458,9 @@ k_attention_packed(const __grid_constant__ Maps mapsK, const __grid_constant__ M
           }
         }
         if (prm.O_sparse) {
-          float* sp = prm.O_sparse + ((i64)bh * prm.N + dst) * kD + hh * 64;
+          float* sp = prm.O_sparse + ((i64)bh * prm.N + dst) * D + hh * kOc;
 #pragma unroll
-          for (int ch = 0; ch < 8; ++ch) {
+          for (int ch = 0; ch < kOc / 8; ++ch) {
             float v8[8];
 #pragma unroll
             for (int k = 0; k < 8; ++k) v8[k] = o[ch * 8 + k];
@@ -547,7 +551,10 @@ __global__ void __launch_bounds__(1024) k_remainder_rows(const int* __restrict__
 }  // namespace tc
 
 cudaError_t init_attention_packed() {
-  return cudaFuncSetAttribute(tc::packed::k_attention_packed, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)tc::packed::Smem::total);
+  using namespace tc::packed;
+  const cudaError_t e = cudaFuncSetAttribute(k_attention_packed<128>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Smem<128>::total);
+  if (e != cudaSuccess) return e;
+  return cudaFuncSetAttribute(k_attention_packed<64>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Smem<64>::total);
 }
 
 void launch_remainder_rows(const int* q_off, const int* route_ptr, const int* route_idx, int BH, int Cq, int Ck, int N, int* rem_pos,
@@ -556,15 +563,16 @@ void launch_remainder_rows(const int* q_off, const int* route_ptr, const int* ro
 }
 
 // Short remainders of every query group, packed (the 128-row kernel must have been given tile offsets that leave
-// them out).  Q, K, V group-major [BH][N][128] bf16; rem_* from launch_remainder_rows.
+// them out).  Q, K, V group-major [BH][N][d] bf16; rem_* from launch_remainder_rows.
 bool launch_attention_packed(const AttnArgs& a, const int* rem_pos, const int* rem_grp, const int* rem_cnt, cudaStream_t st) {
   using namespace tc;
   using namespace tc::packed;
+  const int d = a.d;
   Maps mk, mv;
   const int kvd = a.kv_div < 1 ? 1 : a.kv_div;
   for (int k = 0; k < 4; ++k)
-    if (!make_map(&mk.m[k], a.K, kD, a.N, a.BH / kvd, 1, 0, (i64)a.N * kD, kD, kSub << k) ||
-        !make_map(&mv.m[k], a.V, kD, a.N, a.BH / kvd, 1, 0, (i64)a.N * kD, kD, kSub << k))
+    if (!make_map(&mk.m[k], a.K, d, a.N, a.BH / kvd, 1, 0, (i64)a.N * d, d, kSub << k) ||
+        !make_map(&mv.m[k], a.V, d, a.N, a.BH / kvd, 1, 0, (i64)a.N * d, d, kSub << k))
       return false;
   Params p{};
   p.kv_div = kvd;
@@ -577,7 +585,8 @@ bool launch_attention_packed(const AttnArgs& a, const int* rem_pos, const int* r
   // a group contributes at most kRemRows of every 128 rows it has beyond a multiple of 128, so the packed rows of a
   // head never exceed N; CTAs past the head's count return at once
   const int tiles = (a.N + kTile - 1) / kTile;
-  k_attention_packed<<<dim3(tiles, a.BH), kThreads, Smem::total, st>>>(mk, mv, p);
+  if (d == 128) k_attention_packed<128><<<dim3(tiles, a.BH), kThreads, Smem<128>::total, st>>>(mk, mv, p);
+  else k_attention_packed<64><<<dim3(tiles, a.BH), kThreads, Smem<64>::total, st>>>(mk, mv, p);
   return true;
 }
 

@@ -1,4 +1,5 @@
-// Block-sparse / dense attention on the sm_100a tensor cores (bf16, d = d_v = 128).
+// Block-sparse / dense attention on the sm_100a tensor cores (bf16, D = d = d_v = 64 or 128; at 64 the products are half
+// as long and the softmax threads, which set the pace, do the same work per score).
 //
 // One CTA processes one 128-row query tile (of one query group, Eq. 3; or of the whole
 // head for dense attention, Eq. 1).  Roles:
@@ -44,21 +45,20 @@ namespace tc {
 
 constexpr int kThreads = 384;
 constexpr int kTile = 128;            // query rows per CTA, keys per tile
-constexpr int kD = 128;
 constexpr int kSub = 16;              // rows per TMA box of the K/V stream
 constexpr int kSubPerTile = kTile / kSub;
 constexpr uint32_t kHalfBytes = kTile * 128;          // one [128 rows x 64 bf16] swizzled block
-constexpr uint32_t kTileBytes = 2 * kHalfBytes;       // 32 KB
+template <int D> constexpr uint32_t kTileBytes = (D / 64) * kHalfBytes;      // 32 KB at D = 128, 16 KB at D = 64
 constexpr uint32_t kSubBytes = kSub * 128;            // 2 KB per box
 constexpr int kPolyOf8 = 3;            // pairs of every 8 whose exponential is a polynomial on the FMA pipe
 constexpr int kKStages = 2;            // K tiles in flight (consumed by Q K^T)
 constexpr int kVStages = 2;            // V tiles in flight (consumed by P V)
 
-struct Smem {                          // offsets from a 1024-byte aligned base
+template <int D> struct Smem {         // offsets from a 1024-byte aligned base
   static constexpr uint32_t q = 0;
-  static constexpr uint32_t k = q + kTileBytes;
-  static constexpr uint32_t v = k + kKStages * kTileBytes;
-  static constexpr uint32_t ranges = v + kVStages * kTileBytes;
+  static constexpr uint32_t k = q + kTileBytes<D>;
+  static constexpr uint32_t v = k + kKStages * kTileBytes<D>;
+  static constexpr uint32_t ranges = v + kVStages * kTileBytes<D>;
   static constexpr uint32_t xchg = ranges + kMaxGroups * 8;     // float [2 tile parities][2 halves][128] row maxima; float [2][128] row sums
   static constexpr uint32_t meta = xchg + 6 * 128 * 4;            // uint2[8]: ring of per-tile box counts
   static constexpr uint32_t bars = meta + 8 * 8;                  // kNumBars mbarriers
@@ -66,7 +66,7 @@ struct Smem {                          // offsets from a 1024-byte aligned base
   static constexpr uint32_t dst = misc + 64;                      // int [128]: where the rows of this tile go (original token index)
   static constexpr uint32_t total = dst + kTile * 4;
 };
-constexpr size_t kSmemBytes = Smem::total;                        // the dynamic segment is 1024-byte aligned and the only shared memory
+template <int D> constexpr size_t kSmemBytes = Smem<D>::total;                        // the dynamic segment is 1024-byte aligned and the only shared memory
 
 enum Bar { Q_FULL = 0, K_FULL = 1, K_EMPTY = K_FULL + kKStages, V_FULL = K_EMPTY + kKStages, V_EMPTY = V_FULL + kVStages,
            S_FULL = V_EMPTY + kVStages, S_FREE = S_FULL + 2, P_FULL = S_FREE + 2, P_EMPTY = P_FULL + 2, O_DONE = P_EMPTY + 2, META_FULL,
@@ -80,7 +80,7 @@ struct Params {
   const int *q_off, *kv_off, *route_ptr, *route_idx, *q_perm, *tile_off;
   __nv_bfloat16* O; i64 os[3];
   float* O_sparse;
-  __nv_bfloat16* O_lo;             // optional [BH][N][128]: o - bf16(o), original order (second word for the correction pass)
+  __nv_bfloat16* O_lo;             // optional [BH][N][D]: o - bf16(o), original order (second word for the correction pass)
   int* err;
 };
 
@@ -88,18 +88,22 @@ struct Maps { CUtensorMap m[4]; };      // the same tensor with boxes of 16, 32,
 
 __device__ __forceinline__ uint32_t pack_bf16(float a, float b) { return pack_bf16x2(a, b); }
 
+template <int D>
 __global__ void __launch_bounds__(kThreads, 1)
 k_attention_tc(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__ CUtensorMap mapQ64,
                const __grid_constant__ Maps mapsK, const __grid_constant__ Maps mapsV, Params prm) {
+  using SM = Smem<D>;
+  constexpr int kHalves = D / 64;                                          // 64-column blocks of a row
+  constexpr int kOc = D / 2;                                               // output columns of a thread
   extern __shared__ __align__(1024) unsigned char smem_raw[];
   const uint32_t base = smem_u32(smem_raw);
   unsigned char* sm = smem_raw;
-  int2* ranges = reinterpret_cast<int2*>(sm + Smem::ranges);
-  float* xmax = reinterpret_cast<float*>(sm + Smem::xchg);                 // [2][2][128] half-row maxima of the current / next tile
+  int2* ranges = reinterpret_cast<int2*>(sm + SM::ranges);
+  float* xmax = reinterpret_cast<float*>(sm + SM::xchg);                 // [2][2][128] half-row maxima of the current / next tile
   float* xsum = xmax + 4 * 128;                                            // [2][128] half-row sums (end)
-  uint2* meta = reinterpret_cast<uint2*>(sm + Smem::meta);
-  volatile int* misc = reinterpret_cast<volatile int*>(sm + Smem::misc);   // [0] tmem base, [1] abort, [2] total boxes, [3] leave, [4] query group, [5] its first tile
-  const uint32_t bars = base + Smem::bars;
+  uint2* meta = reinterpret_cast<uint2*>(sm + SM::meta);
+  volatile int* misc = reinterpret_cast<volatile int*>(sm + SM::misc);   // [0] tmem base, [1] abort, [2] total boxes, [3] leave, [4] query group, [5] its first tile
+  const uint32_t bars = base + SM::bars;
   auto bar = [&](int i) { return bars + 8u * i; };
 
   constexpr uint32_t FULLW = 0xffffffffu;
@@ -111,7 +115,7 @@ k_attention_tc(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__
   // second round reads the group's rows and routes.
   // Once any CTA has recorded a timeout the remaining CTAs of the launch leave at once (also if the
   // shared-memory base is not aligned as the swizzled tiles require).
-  int* kv_stage = reinterpret_cast<int*>(sm + Smem::k);
+  int* kv_stage = reinterpret_cast<int*>(sm + SM::k);
   if (tid == 0) {
     misc[3] = (prm.err != nullptr && *reinterpret_cast<volatile int*>(prm.err) == SPARSEPR_ERR_TIMEOUT) || (base & 1023u) != 0;
     if ((base & 1023u) != 0) set_error(prm.err, SPARSEPR_ERR_CUDA);
@@ -145,7 +149,7 @@ k_attention_tc(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__
   }
   const bool dup = prm.sparse && nrows <= kTile / 2;           // every row twice: lanes r and r + 64 (see the header)
   // destination rows of the tile, fetched now so that the epilogue does not wait for them
-  int* dsts = reinterpret_cast<int*>(sm + Smem::dst);
+  int* dsts = reinterpret_cast<int*>(sm + SM::dst);
   if (tid < kTile) dsts[tid] = tid < nrows ? (prm.sparse ? prm.q_perm[(i64)bh * prm.N + row0 + tid] : row0 + tid) : -1;
 
   // ---- set-up: barriers, TMEM, key ranges ---------------------------------------------------
@@ -155,7 +159,7 @@ k_attention_tc(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__
     misc[1] = 0; misc[2] = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
-  if (warp == 9) tmem_alloc(base + Smem::misc, 512);
+  if (warp == 9) tmem_alloc(base + SM::misc, 512);
   __syncthreads();
   {
     int boxes = 0;
@@ -187,21 +191,21 @@ k_attention_tc(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__
       const int c2 = (prm.sparse ? bh : h) / prm.kv_div;       // K/V head (group-major copies: [BH / kv_div]; originals: [B][H / kv_div])
       if (is_k && lane == 0) {
         const int q2 = prm.sparse ? bh : h;
-        mbar_expect_tx(bar(Q_FULL), kTileBytes);
+        mbar_expect_tx(bar(Q_FULL), kTileBytes<D>);
         if (dup) {
           // the same 64 rows into both halves of the tile (rows 64-127 of a [128 x 64] block start 8 KB in)
           for (int part = 0; part < 2; ++part) {
-            tma_load_4d(base + Smem::q + part * (kHalfBytes / 2), &mapQ64, bar(Q_FULL), 0, row0, q2, c3);
-            tma_load_4d(base + Smem::q + kHalfBytes + part * (kHalfBytes / 2), &mapQ64, bar(Q_FULL), 64, row0, q2, c3);
+            for (int c = 0; c < kHalves; ++c)
+              tma_load_4d(base + SM::q + c * kHalfBytes + part * (kHalfBytes / 2), &mapQ64, bar(Q_FULL), 64 * c, row0, q2, c3);
           }
         } else {
-          tma_load_4d(base + Smem::q, &mapQ, bar(Q_FULL), 0, row0, q2, c3);
-          tma_load_4d(base + Smem::q + kHalfBytes, &mapQ, bar(Q_FULL), 64, row0, q2, c3);
+          for (int c = 0; c < kHalves; ++c)
+            tma_load_4d(base + SM::q + c * kHalfBytes, &mapQ, bar(Q_FULL), 64 * c, row0, q2, c3);
         }
       }
       const int nst = is_k ? kKStages : kVStages;
       const int full0 = is_k ? K_FULL : V_FULL, empty0 = is_k ? K_EMPTY : V_EMPTY;
-      const uint32_t buf0 = base + (is_k ? Smem::k : Smem::v);
+      const uint32_t buf0 = base + (is_k ? SM::k : SM::v);
       const Maps* maps = is_k ? &mapsK : &mapsV;
       int ri = 0, off = 0;
       bool ok = true;
@@ -240,19 +244,19 @@ k_attention_tc(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__
             meta[i & 7] = make_uint2(cnt_bits, (uint32_t)nsub);
             mbar_arrive(bar(META_FULL + (i & 7)));
           }
-          mbar_expect_tx(bar(full0 + s), nsub * 2 * kSubBytes);
+          mbar_expect_tx(bar(full0 + s), nsub * kHalves * kSubBytes);
         }
         __syncwarp();
         if (my_k >= 0) {
-          const uint32_t dst = buf0 + s * kTileBytes + lane * kSubBytes;
-          tma_load_4d(dst, &maps->m[my_k], bar(full0 + s), 0, my_start, c2, c3);
-          tma_load_4d(dst + kHalfBytes, &maps->m[my_k], bar(full0 + s), 64, my_start, c2, c3);
+          const uint32_t dst = buf0 + s * kTileBytes<D> + lane * kSubBytes;
+#pragma unroll
+          for (int c = 0; c < kHalves; ++c) tma_load_4d(dst + c * kHalfBytes, &maps->m[my_k], bar(full0 + s), 64 * c, my_start, c2, c3);
         }
       }
     }
   } else if (warp == 9) {
     // =========================== Q K^T issuer ============================================
-    // TMEM columns: S_0 [0,128), S_1 [128,256), P_0 [256,320) and P_1 [448,512) (two bf16 per column), O [320,448).
+    // TMEM columns: S_0 [0,128), S_1 [128,256), P_0 [256,320) and P_1 [448,512) (two bf16 per column), O [320,320+D).
     // The two products are issued by two threads on different warp schedulers: an issuing thread shares its
     // scheduler with two softmax warps that rarely leave it a slot, and the score tile two steps ahead must not
     // queue behind the P V of the current one.
@@ -263,8 +267,8 @@ k_attention_tc(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__
     if (n_tiles > 0) {
       const uint32_t idesc_qk = idesc_bf16(0, 128);
       // descriptors are built once; inside the loops only their address field moves (in 16-byte units)
-      const uint64_t q_desc = smem_desc(base + Smem::q, 16);
-      const uint64_t k_desc0 = smem_desc(base + Smem::k, 16);
+      const uint64_t q_desc = smem_desc(base + SM::q, 16);
+      const uint64_t k_desc0 = smem_desc(base + SM::k, 16);
       bool ok = __all_sync(FULLW, mbar_wait(bar(Q_FULL), 0, abort_flag));
       for (int i = 0; i < n_tiles && ok; ++i) {
         const int s = i % kKStages;
@@ -274,10 +278,10 @@ k_attention_tc(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__
         if (!ok) break;
         tc_fence_after();
         const uint32_t d = tmem + (uint32_t)(i & 1) * 128u;
-        const uint64_t kd = k_desc0 + (uint64_t)(s * (kTileBytes >> 4));
+        const uint64_t kd = k_desc0 + (uint64_t)(s * (kTileBytes<D> >> 4));
         if (elect_one()) {
 #pragma unroll
-          for (int kk = 0; kk < kD / 16; ++kk) {
+          for (int kk = 0; kk < D / 16; ++kk) {
             const uint64_t koff = (uint64_t)((kk >> 2) * (kHalfBytes >> 4) + (kk & 3) * 2);     // compile-time constant
             umma_bf16(d, q_desc + koff, kd + koff, idesc_qk, kk > 0);
           }
@@ -290,8 +294,8 @@ k_attention_tc(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__
   } else if (warp == 11) {
     // =========================== P V issuer ==============================================
     if (n_tiles > 0) {
-      const uint32_t idesc_pv = idesc_bf16(1, 128);
-      const uint64_t v_desc0 = smem_desc(base + Smem::v, kHalfBytes);
+      const uint32_t idesc_pv = idesc_bf16(1, D);
+      const uint64_t v_desc0 = smem_desc(base + SM::v, kHalfBytes);
       bool ok = true;
       for (int i = 0; i < n_tiles && ok; ++i) {
         const int s = i % kVStages;
@@ -303,7 +307,7 @@ k_attention_tc(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__
         tc_fence_after();
         const uint32_t d = tmem + 320u;
         const uint32_t pa = tmem + ((i & 1) ? 448u : 256u);
-        const uint64_t vd = v_desc0 + (uint64_t)(s * (kTileBytes >> 4));
+        const uint64_t vd = v_desc0 + (uint64_t)(s * (kTileBytes<D> >> 4));
         if (elect_one()) {
 #pragma unroll
           for (int kk = 0; kk < kSubPerTile; ++kk)
@@ -325,26 +329,26 @@ k_attention_tc(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__
     const uint32_t lane_addr = (uint32_t)(wq * 32) << 16;
     const uint32_t FULL = 0xffffffffu;
     const uint32_t p_addr0 = tmem + lane_addr + 256u + (uint32_t)hh * 32u;      // P of even tiles; odd tiles 192 columns on
-    const uint32_t o_addr = tmem + lane_addr + 320u + (uint32_t)hh * 64u;
+    const uint32_t o_addr = tmem + lane_addr + 320u + (uint32_t)(hh * kOc);
     float m_ref = -INFINITY, l = 0.f;
     bool ok = true;
     const float sc = prm.scale_log2;
-    // the 64 finished output columns [64 hh, 64 hh + 64) of tile row r: bf16 at the original token index, the part that
+    // the finished output columns [kOc hh, kOc hh + kOc) of tile row r: bf16 at the original token index, the part that
     // the rounding dropped as a second word, float32 on request
-    auto store_row = [&](int r, const float (&o)[64]) {
+    auto store_row = [&](int r, const float (&o)[kOc]) {
       const int dst = prm.sparse ? prm.q_perm[(i64)bh * prm.N + row0 + r] : row0 + r;
-      __nv_bfloat16* op = prm.O + b * prm.os[0] + h * prm.os[1] + (i64)dst * prm.os[2] + hh * 64;
+      __nv_bfloat16* op = prm.O + b * prm.os[0] + h * prm.os[1] + (i64)dst * prm.os[2] + hh * kOc;
 #pragma unroll
-      for (int ch = 0; ch < 8; ++ch) {
+      for (int ch = 0; ch < kOc / 8; ++ch) {
         float v8[8];
 #pragma unroll
         for (int k = 0; k < 8; ++k) v8[k] = o[ch * 8 + k];
         store8(op + ch * 8, v8);
       }
       if (prm.O_lo) {                                          // what the bf16 rounding above dropped
-        __nv_bfloat16* lp = prm.O_lo + ((i64)bh * prm.N + dst) * kD + hh * 64;
+        __nv_bfloat16* lp = prm.O_lo + ((i64)bh * prm.N + dst) * D + hh * kOc;
 #pragma unroll
-        for (int ch = 0; ch < 8; ++ch) {
+        for (int ch = 0; ch < kOc / 8; ++ch) {
           float v8[8];
 #pragma unroll
           for (int k = 0; k < 8; ++k) v8[k] = o[ch * 8 + k] - __bfloat162float(__float2bfloat16_rn(o[ch * 8 + k]));
@@ -352,9 +356,9 @@ k_attention_tc(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__
         }
       }
       if (prm.O_sparse) {
-        float* sp = prm.O_sparse + ((i64)bh * prm.N + dst) * kD + hh * 64;
+        float* sp = prm.O_sparse + ((i64)bh * prm.N + dst) * D + hh * kOc;
 #pragma unroll
-        for (int ch = 0; ch < 8; ++ch) {
+        for (int ch = 0; ch < kOc / 8; ++ch) {
           float v8[8];
 #pragma unroll
           for (int k = 0; k < 8; ++k) v8[k] = o[ch * 8 + k];
@@ -426,7 +430,7 @@ k_attention_tc(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__
           if (!ok) continue;
           tc_fence_after();
 #pragma unroll
-          for (int q = 0; q < 2; ++q) {
+          for (int q = 0; q < kOc / 32; ++q) {
             float t[32];
             tmem_ld32(o_addr + q * 32, t);
 #pragma unroll
@@ -462,13 +466,13 @@ k_attention_tc(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__
       // ---- row sums of the four threads, sum of the two accumulators, normalise, store -----------------
       if (n_tiles > 0) ok = __all_sync(FULL, ok && mbar_wait(bar(O_DONE), 0, abort_flag));
       xsum[slot * 64 + vr] = l;
-      float o[64];
+      float o[kOc];
 #pragma unroll
-      for (int c = 0; c < 64; ++c) o[c] = 0.f;
+      for (int c = 0; c < kOc; ++c) o[c] = 0.f;
       if (ok && n_tiles > 0) {
         tc_fence_after();
 #pragma unroll
-        for (int q = 0; q < 2; ++q) {
+        for (int q = 0; q < kOc / 32; ++q) {
           float t[32];
           tmem_ld32(o_addr + q * 32, t);
 #pragma unroll
@@ -477,17 +481,17 @@ k_attention_tc(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__
       }
       // the copy at lane r + 64 hands its accumulator over through the Q tile's shared memory (every product that
       // reads it has completed): [half][column][row], conflict-free for consecutive rows
-      float* ex = reinterpret_cast<float*>(sm + Smem::q);
+      float* ex = reinterpret_cast<float*>(sm + SM::q);
       if (u == 1) {
 #pragma unroll
-        for (int c = 0; c < 64; ++c) ex[(hh * 64 + c) * 64 + vr] = o[c];
+        for (int c = 0; c < kOc; ++c) ex[(hh * kOc + c) * 64 + vr] = o[c];
       }
       asm volatile("bar.sync %0, 128;" ::"r"(1 + q0) : "memory");
       if (u == 0) {
         const float ltot = (xsum[vr] + xsum[64 + vr]) + (xsum[128 + vr] + xsum[192 + vr]);
         const float inv = ltot > 0.f ? 1.f / ltot : 0.f;
 #pragma unroll
-        for (int c = 0; c < 64; ++c) o[c] = inv != 0.f ? (o[c] + ex[(hh * 64 + c) * 64 + vr]) * inv : 0.f;
+        for (int c = 0; c < kOc; ++c) o[c] = inv != 0.f ? (o[c] + ex[(hh * kOc + c) * 64 + vr]) * inv : 0.f;
         if (ok && vr < nrows) store_row(vr, o);
       }
     } else {
@@ -556,7 +560,7 @@ k_attention_tc(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__
         if (!ok) continue;
         tc_fence_after();
 #pragma unroll
-        for (int q = 0; q < 2; ++q) {
+        for (int q = 0; q < kOc / 32; ++q) {
           float t[32];
           tmem_ld32(o_addr + q * 32, t);
 #pragma unroll
@@ -592,14 +596,14 @@ k_attention_tc(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__
     asm volatile("bar.sync %0, 64;" ::"r"(1 + wq) : "memory");
     const float ltot = l + xsum[(hh ^ 1) * 128 + row];
     const float inv = ltot > 0.f ? 1.f / ltot : 0.f;
-    // this thread finishes output columns [64 hh, 64 hh + 64) of its row
-    float o[64];
+    // this thread finishes output columns [kOc hh, kOc hh + kOc) of its row
+    float o[kOc];
 #pragma unroll
-    for (int c = 0; c < 64; ++c) o[c] = 0.f;
+    for (int c = 0; c < kOc; ++c) o[c] = 0.f;
     if (ok && n_tiles > 0) {
       tc_fence_after();
 #pragma unroll
-      for (int q = 0; q < 2; ++q) {
+      for (int q = 0; q < kOc / 32; ++q) {
         float t[32];
         tmem_ld32(o_addr + q * 32, t);
 #pragma unroll
@@ -609,18 +613,19 @@ k_attention_tc(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__
     if (prm.O_sparse) {
       if (ok && row < nrows) store_row(row, o);
     } else {
-      // Coalesced stores: a thread holds 64 columns of one row, and storing them directly makes every 16-byte store
+      // Coalesced stores: a thread holds half the columns of one row, and storing them directly makes every 16-byte store
       // of a warp touch 32 different lines.  The tile is staged in shared memory instead (the K and V rings are idle:
-      // every product has completed), rows 272 bytes apart so that the 16-byte accesses of a quarter warp fall into
-      // different banks, and written out with 16 lanes per row.
-      constexpr uint32_t kPitch = 2 * kD + 16;
-      unsigned char* st_hi = sm + Smem::k;
-      unsigned char* st_lo = sm + Smem::v;
+      // every product has completed), rows 16 bytes more than their length apart so that the 16-byte accesses of a
+      // quarter warp fall into different banks, and written out with 16 (D = 64: 8) lanes per row.
+      constexpr uint32_t kPitch = 2 * D + 16;
+      static_assert(kTile * kPitch <= 2 * kTileBytes<D>, "the rings hold the staged tile");
+      unsigned char* st_hi = sm + SM::k;
+      unsigned char* st_lo = sm + SM::v;
       {
-        uint4* ph = reinterpret_cast<uint4*>(st_hi + row * kPitch + hh * 128);
-        uint4* pl = reinterpret_cast<uint4*>(st_lo + row * kPitch + hh * 128);
+        uint4* ph = reinterpret_cast<uint4*>(st_hi + row * kPitch + hh * D);
+        uint4* pl = reinterpret_cast<uint4*>(st_lo + row * kPitch + hh * D);
 #pragma unroll
-        for (int ch = 0; ch < 8; ++ch) {
+        for (int ch = 0; ch < kOc / 8; ++ch) {
           uint32_t wh[4], wl[4];
 #pragma unroll
           for (int k = 0; k < 4; ++k) {
@@ -633,17 +638,18 @@ k_attention_tc(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__
         }
       }
       asm volatile("bar.sync 6, 256;" ::: "memory");
-      const int c16 = lane & 15;
+      constexpr int kLpr = D / 8, kRpi = 32 / kLpr;               // lanes per row, rows per step of a warp
+      const int c16 = lane % kLpr;
 #pragma unroll
-      for (int it = 0; it < 8; ++it) {
-        const int r = warp * 16 + 2 * it + (lane >> 4);
+      for (int it = 0; it < 16 / kRpi; ++it) {
+        const int r = warp * 16 + kRpi * it + lane / kLpr;
         const int dst = dsts[r];
         if (ok && r < nrows) {
           const uint4 vh = *reinterpret_cast<const uint4*>(st_hi + r * kPitch + c16 * 16);
           *reinterpret_cast<uint4*>(prm.O + b * prm.os[0] + h * prm.os[1] + (i64)dst * prm.os[2] + c16 * 8) = vh;
           if (prm.O_lo) {
             const uint4 vl = *reinterpret_cast<const uint4*>(st_lo + r * kPitch + c16 * 16);
-            *reinterpret_cast<uint4*>(prm.O_lo + ((i64)bh * prm.N + dst) * kD + c16 * 8) = vl;
+            *reinterpret_cast<uint4*>(prm.O_lo + ((i64)bh * prm.N + dst) * D + c16 * 8) = vl;
           }
         }
       }
@@ -702,15 +708,18 @@ bool make_map(CUtensorMap* m, const void* ptr, int cols, int rows, int H, int B,
 }  // namespace tc
 
 cudaError_t init_attention_tc() {
-  return cudaFuncSetAttribute(tc::k_attention_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)tc::kSmemBytes);
+  const cudaError_t e = cudaFuncSetAttribute(tc::k_attention_tc<128>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)tc::kSmemBytes<128>);
+  if (e != cudaSuccess) return e;
+  return cudaFuncSetAttribute(tc::k_attention_tc<64>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)tc::kSmemBytes<64>);
 }
 
 bool attention_tc_supported(const AttnArgs& a) {
-  return a.dtype == SPARSEPR_BF16 && a.d == 128 && tc::tma_available();
+  return a.dtype == SPARSEPR_BF16 && (a.d == 64 || a.d == 128) && tc::tma_available();
 }
 
 bool launch_attention_tc(const AttnArgs& a, cudaStream_t st) {
   using namespace tc;
+  const int d = a.d;
   CUtensorMap mq, mq64;
   Maps mk, mv;
   const bool sparse = a.route_ptr != nullptr;
@@ -718,17 +727,17 @@ bool launch_attention_tc(const AttnArgs& a, cudaStream_t st) {
   const int kvd = a.kv_div < 1 ? 1 : a.kv_div;
   bool ok;
   if (sparse) {
-    ok = make_map(&mq, a.Q, kD, a.N, a.BH, 1, 0, (i64)a.N * kD, kD, kTile) &&
-         make_map(&mq64, a.Q, kD, a.N, a.BH, 1, 0, (i64)a.N * kD, kD, kTile / 2);
+    ok = make_map(&mq, a.Q, d, a.N, a.BH, 1, 0, (i64)a.N * d, d, kTile) &&
+         make_map(&mq64, a.Q, d, a.N, a.BH, 1, 0, (i64)a.N * d, d, kTile / 2);
     for (int k = 0; k < 4 && ok; ++k)
-      ok = make_map(&mk.m[k], a.K, kD, a.N, a.BH / kvd, 1, 0, (i64)a.N * kD, kD, kSub << k) &&
-           make_map(&mv.m[k], a.V, kD, a.N, a.BH / kvd, 1, 0, (i64)a.N * kD, kD, kSub << k);
+      ok = make_map(&mk.m[k], a.K, d, a.N, a.BH / kvd, 1, 0, (i64)a.N * d, d, kSub << k) &&
+           make_map(&mv.m[k], a.V, d, a.N, a.BH / kvd, 1, 0, (i64)a.N * d, d, kSub << k);
   } else {
-    ok = make_map(&mq, a.Q, kD, a.N, a.H, B, a.qs[0], a.qs[1], a.qs[2], kTile) &&
-         make_map(&mq64, a.Q, kD, a.N, a.H, B, a.qs[0], a.qs[1], a.qs[2], kTile / 2);
+    ok = make_map(&mq, a.Q, d, a.N, a.H, B, a.qs[0], a.qs[1], a.qs[2], kTile) &&
+         make_map(&mq64, a.Q, d, a.N, a.H, B, a.qs[0], a.qs[1], a.qs[2], kTile / 2);
     for (int k = 0; k < 4 && ok; ++k)
-      ok = make_map(&mk.m[k], a.K, kD, a.N, a.H / kvd, B, a.ks[0], a.ks[1], a.ks[2], kSub << k) &&
-           make_map(&mv.m[k], a.V, kD, a.N, a.H / kvd, B, a.vs[0], a.vs[1], a.vs[2], kSub << k);
+      ok = make_map(&mk.m[k], a.K, d, a.N, a.H / kvd, B, a.ks[0], a.ks[1], a.ks[2], kSub << k) &&
+           make_map(&mv.m[k], a.V, d, a.N, a.H / kvd, B, a.vs[0], a.vs[1], a.vs[2], kSub << k);
   }
   if (!ok) return false;
   Params p{};
@@ -739,7 +748,8 @@ bool launch_attention_tc(const AttnArgs& a, cudaStream_t st) {
   p.O = (__nv_bfloat16*)a.O; for (int i = 0; i < 3; ++i) p.os[i] = a.os[i];
   p.O_sparse = a.O_sparse; p.O_lo = (__nv_bfloat16*)a.O_lo; p.err = a.err;
   const int tiles = (a.N + kTile - 1) / kTile + (sparse ? a.Cq : 0);
-  k_attention_tc<<<dim3(tiles, a.BH), kThreads, kSmemBytes, st>>>(mq, mq64, mk, mv, p);
+  if (d == 128) k_attention_tc<128><<<dim3(tiles, a.BH), kThreads, kSmemBytes<128>, st>>>(mq, mq64, mk, mv, p);
+  else k_attention_tc<64><<<dim3(tiles, a.BH), kThreads, kSmemBytes<64>, st>>>(mq, mq64, mk, mv, p);
   return true;
 }
 

@@ -48,11 +48,11 @@ void launch_group_means(int dtype, const void* X, const i64* xs, int BH, int H, 
 void launch_gather_rows(int dtype, const void* X, const i64* xs, int BH, int H, const int* perm, int N, int d, void* out,
                         cudaStream_t st);
 
-// project_tc.cu: the same projection on the tensor cores (bf16, d = 128, r <= 64); Ft: bf16 scratch [BH][3][64][128]
+// project_tc.cu: the same projection on the tensor cores (bf16, d = 64 or 128, r <= 64); Ft: bf16 scratch [BH][3][64][d]
 cudaError_t init_project_tc();
 bool project_tc_supported(int dtype, int d, int r, const i64* xs);
 // f_div: heads that share one feature map (F is indexed by bh / f_div)
-bool launch_project_tc(const void* X, const i64* xs, int BH, int H, int N, int r, const float* F, bool rms, float eps,
+bool launch_project_tc(const void* X, const i64* xs, int BH, int H, int N, int d, int r, const float* F, bool rms, float eps,
                        float* phi, int ldphi, unsigned* maxabs, __nv_bfloat16* Ft, int* err, cudaStream_t st, int f_div = 1);
 
 // centroids per product of the tensor-core assignment; ||mu_c||^2 of the places beyond C (a bf16 value, larger than any score)
@@ -118,7 +118,7 @@ cudaError_t init_attention_simt();
 // tile_off [BH][Cq+1]: prefix of the tiles per query group; small_rem > 0 leaves out a last tile of at most small_rem rows
 void launch_tile_offsets(const int* q_off, int BH, int Cq, int tile_rows, int small_rem, int* tile_off, cudaStream_t st);
 void launch_attention_simt(const AttnArgs& a, cudaStream_t st);
-// ---- attention_tc.cu (tcgen05 / TMEM / TMA; bf16, d = 128) -------------------------------------
+// ---- attention_tc.cu (tcgen05 / TMEM / TMA; bf16, d = 64 or 128) -------------------------------------
 cudaError_t init_attention_tc();
 bool attention_tc_supported(const AttnArgs& a);
 // tile_off in `a` must have been built for 128-row tiles; a.A and a.c are ignored (no correction epilogue)
@@ -135,11 +135,11 @@ void launch_remainder_rows(const int* q_off, const int* route_ptr, const int* ro
 bool launch_attention_packed(const AttnArgs& a, const int* rem_pos, const int* rem_grp, const int* rem_cnt, cudaStream_t st);
 // one warp runs the bounded mbarrier wait into its limit (2^16 cycles) and records SPARSEPR_ERR_TIMEOUT in *err
 void launch_selftest_bounded_wait(int* err, cudaStream_t st);
-// correction_tc.cu: O <- X + X A + c in place, X = O + O_lo (two bf16 words, O_lo [BH][N][128] contiguous), d_v = 128;
-// At [2][BH][128][128]: A transposed, as two bf16 words (from the fit)
+// correction_tc.cu: O <- X + X A + c in place, X = O + O_lo (two bf16 words, O_lo [BH][N][d] contiguous), d_v = d = 64 or 128;
+// At [2][BH][d][d]: A transposed, as two bf16 words (from the fit)
 cudaError_t init_correction_tc();
 bool launch_correction_tc(const float* c, const __nv_bfloat16* At, const void* O_lo, void* O, const i64* os, int BH,
-                          int H, int N, int* err, cudaStream_t st);
+                          int H, int N, int d, int* err, cudaStream_t st);
 
 struct ProbeArgs {
   int dtype, BH, H, N, d, M, Ck, Cq, n_split;
@@ -154,7 +154,7 @@ struct ProbeArgs {
 size_t probe_partial_floats(int BH, int n_split, int M, int d);
 void launch_probe_rows(const ProbeArgs& a, cudaStream_t st);
 void launch_probe_merge(const ProbeArgs& a, cudaStream_t st);
-// probe_tc.cu: the same partial states from the tensor-core kernel (bf16, d = 128); Qp: scratch [BH][M][128] bf16
+// probe_tc.cu: the same partial states from the tensor-core kernel (bf16, d = 64 or 128); Qp: scratch [BH][M][d] bf16
 cudaError_t init_probe_tc();
 bool probe_tc_supported(const ProbeArgs& a);
 bool launch_probe_rows_tc(const ProbeArgs& a, __nv_bfloat16* Qp, int* err, cudaStream_t st);

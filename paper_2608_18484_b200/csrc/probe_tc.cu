@@ -1,4 +1,4 @@
-// Exact probe rows on the tensor cores (Appendix A.1-A.2; bf16, d = d_v = 128).
+// Exact probe rows on the tensor cores (Appendix A.1-A.2; bf16, D = d = d_v = 64 or 128).
 //
 // For every probe row one pass over ALL keys (group-major order) maintains two
 // online-softmax states: the keys retained by the probe's query group (Z_S, N_S) and the
@@ -10,7 +10,7 @@
 //              with one warp per scheduler the loop ran at the latency of its instructions)
 //   warp  8    K producer (also builds the per-tile list of K/V-group runs), warp 9 V producer
 //   warp  10   tcgen05.mma issuer, owns TMEM
-// TMEM: S0 [0,128), S1 [128,256), O_S [256,384), O_U [384,512).  The exponentials of a tile
+// TMEM: S0 [0,128), S1 [128,256), O_S [256,256+D), O_U [384,384+D).  The exponentials of a tile
 // are written back over its score buffer as bf16: retained weights in columns [0,64),
 // omitted weights in [64,128); the two P V products read them from TMEM.
 #include "kernels.cuh"
@@ -23,17 +23,17 @@ constexpr int kPbThreads = 352;
 constexpr int kPbWarpK = 8, kPbWarpV = 9, kPbWarpMma = 10;
 constexpr int kPbTile = 128;
 constexpr uint32_t kPbHalf = 128 * 128;              // [128 rows x 64 bf16] swizzled block
-constexpr uint32_t kPbTileBytes = 2 * kPbHalf;
+template <int D> constexpr uint32_t kPbTileBytes = (D / 64) * kPbHalf;
 constexpr int kPbKStages = 2, kPbVStages = 2;
 constexpr int kPbMaxRuns = 8;                        // K/V-group runs per key tile
 
 struct PbMeta { int ncols, nruns; unsigned short grp[kPbMaxRuns]; unsigned char end[kPbMaxRuns]; };   // 32 bytes
 
-struct PbSmem {
+template <int D> struct PbSmem {
   static constexpr uint32_t q = 0;
-  static constexpr uint32_t k = q + kPbTileBytes;
-  static constexpr uint32_t v = k + kPbKStages * kPbTileBytes;
-  static constexpr uint32_t bitmap = v + kPbVStages * kPbTileBytes;        // [kMaxGroups/32 words][128 rows]
+  static constexpr uint32_t k = q + kPbTileBytes<D>;
+  static constexpr uint32_t v = k + kPbKStages * kPbTileBytes<D>;
+  static constexpr uint32_t bitmap = v + kPbVStages * kPbTileBytes<D>;        // [kMaxGroups/32 words][128 rows]
   static constexpr uint32_t meta = bitmap + (kMaxGroups / 32) * 128 * 4;   // PbMeta[8]
   static constexpr uint32_t xchg = meta + 8 * 32;                          // float [2][2][2][128] half-row maxima of both states, [2][2][128] sums
   static constexpr uint32_t bars = xchg + 12 * 128 * 4;
@@ -50,20 +50,23 @@ struct PbParams {
   int kv_div;                     // query heads per K/V head: the K/V maps and kv_off are indexed by bh / kv_div
   float scale_log2;
   const int *probe_idx, *q_assign, *kv_off, *route_ptr, *route_idx;
-  float* partial;                 // [BH][n_split][M][2][130]
+  float* partial;                 // [BH][n_split][M][2][D + 2]
   int* err;
 };
 
+template <int D>
 __global__ void __launch_bounds__(kPbThreads, 1)
 k_probe_rows_tc(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__ CUtensorMap mapK,
                 const __grid_constant__ CUtensorMap mapV, PbParams prm) {
+  using SM = PbSmem<D>;
+  constexpr int kHalves = D / 64, kOc = D / 2;                             // 64-column blocks of a row; output columns of a thread
   extern __shared__ __align__(1024) unsigned char smem_raw[];
   const uint32_t base = smem_u32(smem_raw);
   unsigned char* sm = smem_raw;
-  unsigned* bitmap = reinterpret_cast<unsigned*>(sm + PbSmem::bitmap);
-  PbMeta* meta = reinterpret_cast<PbMeta*>(sm + PbSmem::meta);
-  volatile int* misc = reinterpret_cast<volatile int*>(sm + PbSmem::misc);   // [0] tmem, [1] abort, [3] skip
-  const uint32_t bars = base + PbSmem::bars;
+  unsigned* bitmap = reinterpret_cast<unsigned*>(sm + SM::bitmap);
+  PbMeta* meta = reinterpret_cast<PbMeta*>(sm + SM::meta);
+  volatile int* misc = reinterpret_cast<volatile int*>(sm + SM::misc);   // [0] tmem, [1] abort, [3] skip
+  const uint32_t bars = base + SM::bars;
   auto bar = [&](int i) { return bars + 8u * i; };
   constexpr uint32_t FULLW = 0xffffffffu;
   const int tid = threadIdx.x, warp = __shfl_sync(FULLW, tid >> 5, 0), lane = tid & 31;   // (uniform, and known to be)
@@ -87,7 +90,7 @@ k_probe_rows_tc(const __grid_constant__ CUtensorMap mapQ, const __grid_constant_
     misc[1] = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
-  if (warp == kPbWarpMma) tmem_alloc(base + PbSmem::misc, 512);
+  if (warp == kPbWarpMma) tmem_alloc(base + SM::misc, 512);
   // route bitmap of every probe row, transposed: bitmap[word][row]
   for (int e = tid; e < words * 128; e += kPbThreads) bitmap[e] = 0u;
   __syncthreads();
@@ -127,13 +130,12 @@ k_probe_rows_tc(const __grid_constant__ CUtensorMap mapQ, const __grid_constant_
     if (lane == 0 && p_begin < p_end) {
       const bool is_k = warp == kPbWarpK;
       if (is_k) {
-        mbar_expect_tx(bar(PQ_FULL), kPbTileBytes);
-        tma_load_4d(base + PbSmem::q, &mapQ, bar(PQ_FULL), 0, m0, bh, 0);
-        tma_load_4d(base + PbSmem::q + kPbHalf, &mapQ, bar(PQ_FULL), 64, m0, bh, 0);
+        mbar_expect_tx(bar(PQ_FULL), kPbTileBytes<D>);
+        for (int c = 0; c < kHalves; ++c) tma_load_4d(base + SM::q + c * kPbHalf, &mapQ, bar(PQ_FULL), 64 * c, m0, bh, 0);
       }
       const int nst = is_k ? kPbKStages : kPbVStages;
       const int full0 = is_k ? PK_FULL : PV_FULL, empty0 = is_k ? PK_EMPTY : PV_EMPTY;
-      const uint32_t buf0 = base + (is_k ? PbSmem::k : PbSmem::v);
+      const uint32_t buf0 = base + (is_k ? SM::k : SM::v);
       const CUtensorMap* map = is_k ? &mapK : &mapV;
       int g = 0;
       { int lo = 0, hi = prm.Ck - 1; while (lo < hi) { const int mid = (lo + hi + 1) >> 1; if (kvoff[mid] <= p_begin) lo = mid; else hi = mid - 1; } g = lo; }
@@ -147,9 +149,8 @@ k_probe_rows_tc(const __grid_constant__ CUtensorMap mapQ, const __grid_constant_
           meta[i & 7] = mt;
           mbar_arrive(bar(PMETA_FULL + (i & 7)));
         }
-        mbar_expect_tx(bar(full0 + s), kPbTileBytes);
-        tma_load_4d(buf0 + s * kPbTileBytes, map, bar(full0 + s), 0, pos, kvh, 0);
-        tma_load_4d(buf0 + s * kPbTileBytes + kPbHalf, map, bar(full0 + s), 64, pos, kvh, 0);
+        mbar_expect_tx(bar(full0 + s), kPbTileBytes<D>);
+        for (int c = 0; c < kHalves; ++c) tma_load_4d(buf0 + s * kPbTileBytes<D> + c * kPbHalf, map, bar(full0 + s), 64 * c, pos, kvh, 0);
         pos += nc;
       }
     }
@@ -158,19 +159,19 @@ k_probe_rows_tc(const __grid_constant__ CUtensorMap mapQ, const __grid_constant_
     // The whole warp walks the tiles and one elected lane issues; loop control goes through votes (known to be uniform):
     // 522 -> 433 us at 24 heads of 32760 keys beside the attention kernels.
     if (p_begin < p_end) {
-      const uint32_t idesc_qk = idesc_bf16(0, 128), idesc_pv = idesc_bf16(1, 128);
-      const uint64_t q_desc = smem_desc(base + PbSmem::q, 16), k_desc0 = smem_desc(base + PbSmem::k, 16);
-      const uint64_t v_desc0 = smem_desc(base + PbSmem::v, kPbHalf);
+      const uint32_t idesc_qk = idesc_bf16(0, 128), idesc_pv = idesc_bf16(1, D);
+      const uint64_t q_desc = smem_desc(base + SM::q, 16), k_desc0 = smem_desc(base + SM::k, 16);
+      const uint64_t v_desc0 = smem_desc(base + SM::v, kPbHalf);
       bool ok = __all_sync(FULLW, mbar_wait(bar(PQ_FULL), 0, abort_flag));
       auto issue_qk = [&](int i) -> bool {
         const int s = i % kPbKStages;
         if (!__all_sync(FULLW, mbar_wait(bar(PK_FULL + s), (i / kPbKStages) & 1, abort_flag))) return false;
         tc_fence_after();
         const uint32_t d = tmem + (uint32_t)(i & 1) * 128u;
-        const uint64_t kd = k_desc0 + (uint64_t)(s * (kPbTileBytes >> 4));
+        const uint64_t kd = k_desc0 + (uint64_t)(s * (kPbTileBytes<D> >> 4));
         if (elect_one()) {
 #pragma unroll
-          for (int kk = 0; kk < 8; ++kk) {
+          for (int kk = 0; kk < D / 16; ++kk) {
             const uint64_t koff = (uint64_t)((kk >> 2) * (kPbHalf >> 4) + (kk & 3) * 2);
             umma_bf16(d, q_desc + koff, kd + koff, idesc_qk, kk > 0);
           }
@@ -197,7 +198,7 @@ k_probe_rows_tc(const __grid_constant__ CUtensorMap mapQ, const __grid_constant_
         if (!ok) break;
         tc_fence_after();
         const uint32_t pbuf = tmem + (uint32_t)(i & 1) * 128u;
-        const uint64_t vd = v_desc0 + (uint64_t)(s * (kPbTileBytes >> 4));
+        const uint64_t vd = v_desc0 + (uint64_t)(s * (kPbTileBytes<D> >> 4));
         if (elect_one()) {
 #pragma unroll
           for (int which = 0; which < 2; ++which)               // retained weights -> O_S, omitted -> O_U
@@ -219,7 +220,7 @@ k_probe_rows_tc(const __grid_constant__ CUtensorMap mapQ, const __grid_constant_
     const uint32_t lane_addr = (uint32_t)(wq * 32) << 16;
     const uint32_t FULL = 0xffffffffu;
     const float sc = prm.scale_log2;
-    float* xmax = reinterpret_cast<float*>(sm + PbSmem::xchg);             // [parity][half][state][row]
+    float* xmax = reinterpret_cast<float*>(sm + SM::xchg);             // [parity][half][state][row]
     float* xsum = xmax + 8 * 128;                                          // [half][state][row]
     float mS = -INFINITY, mU = -INFINITY, lS = 0.f, lU = 0.f;
     bool ok = true;
@@ -289,10 +290,11 @@ k_probe_rows_tc(const __grid_constant__ CUtensorMap mapQ, const __grid_constant_
       if (i > 0 && __any_sync(FULL, moveS || moveU)) {           // rescale this half of the O_S / O_U rows (rare)
         tc_fence_after();
 #pragma unroll
-        for (int q = 0; q < 4; ++q) {
+        for (int q = 0; q < 2 * (kOc / 32); ++q) {
           float t[32];
-          const float f = q < 2 ? cS : cU;
-          const uint32_t a = tmem + lane_addr + 256u + (uint32_t)(q >> 1) * 128u + (uint32_t)hh * 64u + (uint32_t)(q & 1) * 32u;
+          constexpr int kQ = kOc / 32;
+          const float f = q < kQ ? cS : cU;
+          const uint32_t a = tmem + lane_addr + 256u + (uint32_t)(q / kQ) * 128u + (uint32_t)(hh * kOc + (q % kQ) * 32);
           tmem_ld32(a, t);
 #pragma unroll
           for (int c = 0; c < 32; ++c) t[c] *= f;
@@ -342,19 +344,20 @@ k_probe_rows_tc(const __grid_constant__ CUtensorMap mapQ, const __grid_constant_
     lS += xsum[((hh ^ 1) * 2 + 0) * 128 + row];
     lU += xsum[((hh ^ 1) * 2 + 1) * 128 + row];
     if (row < nrows && hh == 0) {
-      float* out = prm.partial + ((((i64)bh * prm.n_split + split) * prm.M + m0 + row) * 2) * 130;
+      float* out = prm.partial + ((((i64)bh * prm.n_split + split) * prm.M + m0 + row) * 2) * (D + 2);
       const bool good = ok && any;
       out[0] = (good && lS > 0.f) ? mS * sc : -INFINITY; out[1] = good ? lS : 0.f;
-      out[130] = (good && lU > 0.f) ? mU * sc : -INFINITY; out[131] = good ? lU : 0.f;
+      out[D + 2] = (good && lU > 0.f) ? mU * sc : -INFINITY; out[D + 3] = good ? lU : 0.f;
     }
     if (ok && any) {
       tc_fence_after();
 #pragma unroll
-      for (int q = 0; q < 4; ++q) {                             // this half's 64 columns of O_S, then of O_U
+      for (int q = 0; q < 2 * (kOc / 32); ++q) {                // this half's columns of O_S, then of O_U
+        constexpr int kQ = kOc / 32;
         float t[32];
-        tmem_ld32(tmem + lane_addr + 256u + (uint32_t)(q >> 1) * 128u + (uint32_t)hh * 64u + (uint32_t)(q & 1) * 32u, t);
+        tmem_ld32(tmem + lane_addr + 256u + (uint32_t)(q / kQ) * 128u + (uint32_t)(hh * kOc + (q % kQ) * 32), t);
         if (row < nrows) {
-          float* out = prm.partial + ((((i64)bh * prm.n_split + split) * prm.M + m0 + row) * 2 + (q >> 1)) * 130 + 2 + hh * 64 + (q & 1) * 32;
+          float* out = prm.partial + ((((i64)bh * prm.n_split + split) * prm.M + m0 + row) * 2 + q / kQ) * (D + 2) + 2 + hh * kOc + (q % kQ) * 32;
 #pragma unroll
           for (int c = 0; c < 32; ++c) out[c] = t[c];
         }
@@ -374,36 +377,39 @@ k_probe_rows_tc(const __grid_constant__ CUtensorMap mapQ, const __grid_constant_
   }
 }
 
-// probe rows of Q gathered into a dense [BH][M][128] bf16 buffer (rows of missing probes are zero)
+// probe rows of Q gathered into a dense [BH][M][d] bf16 buffer (rows of missing probes are zero)
 __global__ void k_gather_probe_q(const __nv_bfloat16* __restrict__ Q, i64 sb, i64 sh, i64 sn, int H,
-                                 const int* __restrict__ probe_idx, int M, __nv_bfloat16* __restrict__ out) {
+                                 const int* __restrict__ probe_idx, int M, int d, __nv_bfloat16* __restrict__ out) {
   const int bh = blockIdx.y, b = bh / H, h = bh % H;
-  const int t = blockIdx.x * blockDim.x + threadIdx.x;          // 16 threads per row
-  const int m = t >> 4, c = (t & 15) * 8;
+  const int t = blockIdx.x * blockDim.x + threadIdx.x;          // d / 8 threads per row
+  const int m = t / (d / 8), c = t % (d / 8) * 8;
   if (m >= M) return;
   const int pi = probe_idx[(i64)bh * M + m];
   uint4 v = make_uint4(0, 0, 0, 0);
   if (pi >= 0) v = *reinterpret_cast<const uint4*>(Q + b * sb + h * sh + (i64)pi * sn + c);
-  *reinterpret_cast<uint4*>(out + ((i64)bh * M + m) * 128 + c) = v;
+  *reinterpret_cast<uint4*>(out + ((i64)bh * M + m) * d + c) = v;
 }
 
 }  // namespace tc
 
 cudaError_t init_probe_tc() {
-  return cudaFuncSetAttribute(tc::k_probe_rows_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)tc::PbSmem::total);
+  const cudaError_t e = cudaFuncSetAttribute(tc::k_probe_rows_tc<128>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)tc::PbSmem<128>::total);
+  if (e != cudaSuccess) return e;
+  return cudaFuncSetAttribute(tc::k_probe_rows_tc<64>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)tc::PbSmem<64>::total);
 }
-bool probe_tc_supported(const ProbeArgs& a) { return a.dtype == SPARSEPR_BF16 && a.d == 128 && tc::tma_available(); }
+bool probe_tc_supported(const ProbeArgs& a) { return a.dtype == SPARSEPR_BF16 && (a.d == 64 || a.d == 128) && tc::tma_available(); }
 
-// Qp: scratch [BH][M][128] bf16.  Writes a.partial in the layout k_probe_merge reads.
+// Qp: scratch [BH][M][d] bf16.  Writes a.partial in the layout k_probe_merge reads.
 bool launch_probe_rows_tc(const ProbeArgs& a, __nv_bfloat16* Qp, int* err, cudaStream_t st) {
   const int kvd = a.kv_div < 1 ? 1 : a.kv_div;
   using namespace tc;
-  k_gather_probe_q<<<dim3((a.M * 16 + 255) / 256, a.BH), 256, 0, st>>>((const __nv_bfloat16*)a.Q, a.qs[0], a.qs[1], a.qs[2], a.H,
-                                                                     a.probe_idx, a.M, Qp);
+  const int d = a.d;
+  k_gather_probe_q<<<dim3((a.M * (d / 8) + 255) / 256, a.BH), 256, 0, st>>>((const __nv_bfloat16*)a.Q, a.qs[0], a.qs[1], a.qs[2], a.H,
+                                                                     a.probe_idx, a.M, d, Qp);
   CUtensorMap mq, mk, mv;
-  if (!make_map(&mq, Qp, 128, a.M, a.BH, 1, 0, (i64)a.M * 128, 128, 128) ||
-      !make_map(&mk, a.Kg, 128, a.N, a.BH / kvd, 1, 0, (i64)a.N * 128, 128, 128) ||
-      !make_map(&mv, a.Vg, 128, a.N, a.BH / kvd, 1, 0, (i64)a.N * 128, 128, 128))
+  if (!make_map(&mq, Qp, d, a.M, a.BH, 1, 0, (i64)a.M * d, d, 128) ||
+      !make_map(&mk, a.Kg, d, a.N, a.BH / kvd, 1, 0, (i64)a.N * d, d, 128) ||
+      !make_map(&mv, a.Vg, d, a.N, a.BH / kvd, 1, 0, (i64)a.N * d, d, 128))
     return false;
   PbParams p{};
   p.BH = a.BH; p.N = a.N; p.M = a.M; p.Ck = a.Ck; p.Cq = a.Cq; p.n_split = a.n_split;
@@ -411,7 +417,9 @@ bool launch_probe_rows_tc(const ProbeArgs& a, __nv_bfloat16* Qp, int* err, cudaS
   p.kv_div = kvd;
   p.probe_idx = a.probe_idx; p.q_assign = a.q_assign; p.kv_off = a.kv_off; p.route_ptr = a.route_ptr; p.route_idx = a.route_idx;
   p.partial = a.partial; p.err = err;
-  k_probe_rows_tc<<<dim3(a.n_split, (a.M + 127) / 128, a.BH), kPbThreads, PbSmem::total, st>>>(mq, mk, mv, p);
+  const dim3 grid(a.n_split, (a.M + 127) / 128, a.BH);
+  if (d == 128) k_probe_rows_tc<128><<<grid, kPbThreads, PbSmem<128>::total, st>>>(mq, mk, mv, p);
+  else k_probe_rows_tc<64><<<grid, kPbThreads, PbSmem<64>::total, st>>>(mq, mk, mv, p);
   return true;
 }
 

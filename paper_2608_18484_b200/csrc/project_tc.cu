@@ -1,9 +1,9 @@
-// Response projections on the sm_100a tensor cores (bf16 tensors, d = 128):
+// Response projections on the sm_100a tensor cores (bf16 tensors, D = d = 64 or 128):
 //   phi_K = K F_K (Eq. 6),  phi_Q = RMS-normalised Q F_Q (Eq. 7).
 // X is bf16 and enters the MMA unchanged; the float32 feature map F is split into three bf16
 // terms (F = F1 + F2 + F3 up to 2^-24), so the three accumulated products reproduce the float32
 // projection.  The pass is bandwidth bound: X is read once by TMA, phi written once.
-// Persistent CTAs own contiguous row tiles of one head; F^T (3 x [64 x 128] bf16) stays in
+// Persistent CTAs own contiguous row tiles of one head; F^T (3 x [64 x D] bf16) stays in
 // shared memory.  Roles: warps 0-3 epilogue (one row per thread: normalisation, store, max |phi|),
 // warp 4 (one lane) TMA loads and tcgen05.mma, TMEM owner.  Two X stages and two accumulators
 // let the loads, the MMAs and the epilogue of consecutive tiles overlap.
@@ -18,13 +18,13 @@ namespace tc {
 
 constexpr int kPjThreads = 160;
 constexpr uint32_t kPjXHalf = 128 * 128;            // [128 rows x 64 bf16]
-constexpr uint32_t kPjXBytes = 2 * kPjXHalf;
+template <int D> constexpr uint32_t kPjXBytes = (D / 64) * kPjXHalf;
 constexpr uint32_t kPjFHalf = 64 * 128;             // [64 rows x 64 bf16]
-constexpr uint32_t kPjFBytes = 2 * kPjFHalf;
-struct PjSmem {
+template <int D> constexpr uint32_t kPjFBytes = (D / 64) * kPjFHalf;
+template <int D> struct PjSmem {
   static constexpr uint32_t x = 0;                              // 2 stages
-  static constexpr uint32_t f = x + 2 * kPjXBytes;              // 3 terms
-  static constexpr uint32_t bars = f + 3 * kPjFBytes;           // F_FULL, X_FULL[2], X_EMPTY[2], ACC_FULL[2], ACC_EMPTY[2]
+  static constexpr uint32_t f = x + 2 * kPjXBytes<D>;              // 3 terms
+  static constexpr uint32_t bars = f + 3 * kPjFBytes<D>;           // F_FULL, X_FULL[2], X_EMPTY[2], ACC_FULL[2], ACC_EMPTY[2]
   static constexpr uint32_t misc = bars + 16 * 8;
   static constexpr uint32_t total = misc + 16;
 };
@@ -38,14 +38,17 @@ struct PjParams {
   int* err;
 };
 
+template <int D>
 __global__ void __launch_bounds__(kPjThreads)
 k_project_tc(const __grid_constant__ CUtensorMap mapX, const __grid_constant__ CUtensorMap mapF, PjParams prm) {
   pdl_wait();                                                   // the split feature map comes from the kernel before
   pdl_launch_dependents();
+  using SM = PjSmem<D>;
+  constexpr int kHalves = D / 64;
   extern __shared__ __align__(1024) unsigned char smem_raw[];
   const uint32_t base = smem_u32(smem_raw);
-  volatile int* misc = reinterpret_cast<volatile int*>(smem_raw + PjSmem::misc);   // [0] tmem base, [1] abort, [2] skip
-  const uint32_t bars = base + PjSmem::bars;
+  volatile int* misc = reinterpret_cast<volatile int*>(smem_raw + SM::misc);   // [0] tmem base, [1] abort, [2] skip
+  const uint32_t bars = base + SM::bars;
   auto bar = [&](int i) { return bars + 8u * i; };
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int bh = blockIdx.y, b = bh / prm.H, h = bh % prm.H;
@@ -62,7 +65,7 @@ k_project_tc(const __grid_constant__ CUtensorMap mapX, const __grid_constant__ C
   }
   __syncthreads();
   if (misc[2] || my_tiles == 0) return;
-  if (warp == 4) tmem_alloc(base + PjSmem::misc, 128);
+  if (warp == 4) tmem_alloc(base + SM::misc, 128);
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
@@ -74,15 +77,13 @@ k_project_tc(const __grid_constant__ CUtensorMap mapX, const __grid_constant__ C
       auto load_x = [&](int t) {
         const int s = t & 1;
         const int row0 = (tile0 + t) * 128;
-        mbar_expect_tx(bar(PX_FULL + s), kPjXBytes);
-        tma_load_4d(base + PjSmem::x + s * kPjXBytes, &mapX, bar(PX_FULL + s), 0, row0, h, b);
-        tma_load_4d(base + PjSmem::x + s * kPjXBytes + kPjXHalf, &mapX, bar(PX_FULL + s), 64, row0, h, b);
+        mbar_expect_tx(bar(PX_FULL + s), kPjXBytes<D>);
+        for (int c = 0; c < kHalves; ++c) tma_load_4d(base + SM::x + s * kPjXBytes<D> + c * kPjXHalf, &mapX, bar(PX_FULL + s), 64 * c, row0, h, b);
       };
-      mbar_expect_tx(bar(PF_FULL), 3 * kPjFBytes);
+      mbar_expect_tx(bar(PF_FULL), 3 * kPjFBytes<D>);
 #pragma unroll
       for (int t = 0; t < 3; ++t) {
-        tma_load_4d(base + PjSmem::f + t * kPjFBytes, &mapF, bar(PF_FULL), 0, 0, t, bh);
-        tma_load_4d(base + PjSmem::f + t * kPjFBytes + kPjFHalf, &mapF, bar(PF_FULL), 64, 0, t, bh);
+        for (int c = 0; c < kHalves; ++c) tma_load_4d(base + SM::f + t * kPjFBytes<D> + c * kPjFHalf, &mapF, bar(PF_FULL), 64 * c, 0, t, bh);
       }
       load_x(0);
       bool ok = mbar_wait(bar(PF_FULL), 0, abort_flag);
@@ -97,13 +98,13 @@ k_project_tc(const __grid_constant__ CUtensorMap mapX, const __grid_constant__ C
         if (!mbar_wait(bar(PX_FULL + s), (t >> 1) & 1, abort_flag)) { ok = false; break; }
         if (t >= 2 && !mbar_wait(bar(PACC_EMPTY + s), ((t - 2) >> 1) & 1, abort_flag)) { ok = false; break; }
         tc_fence_after();
-        const uint64_t xd = smem_desc(base + PjSmem::x + s * kPjXBytes, 16);
+        const uint64_t xd = smem_desc(base + SM::x + s * kPjXBytes<D>, 16);
         const uint32_t d = tmem + (uint32_t)s * 64u;
 #pragma unroll
         for (int term = 0; term < 3; ++term) {
-          const uint64_t fd = smem_desc(base + PjSmem::f + term * kPjFBytes, 16);
+          const uint64_t fd = smem_desc(base + SM::f + term * kPjFBytes<D>, 16);
 #pragma unroll
-          for (int kk = 0; kk < 8; ++kk) {
+          for (int kk = 0; kk < D / 16; ++kk) {
             const uint64_t xoff = (uint64_t)((kk >> 2) * (kPjXHalf >> 4) + (kk & 3) * 2);
             const uint64_t foff = (uint64_t)((kk >> 2) * (kPjFHalf >> 4) + (kk & 3) * 2);
             umma_bf16(d, xd + xoff, fd + foff, idesc, (term > 0 || kk > 0) ? 1u : 0u);
@@ -166,20 +167,20 @@ k_project_tc(const __grid_constant__ CUtensorMap mapX, const __grid_constant__ C
   }
 }
 
-// F [BH][128][r] float32 -> Ft [BH][3][64][128] bf16: term t, row j (output column, zero beyond r), column k
+// F [BH][d][r] float32 -> Ft [BH][3][64][d] bf16: term t, row j (output column, zero beyond r), column k
 // (f_div heads share one feature map: the query heads of a K/V head under grouped-query attention)
-__global__ void k_split_feature_map(const float* __restrict__ F, int r, __nv_bfloat16* __restrict__ Ft, int f_div) {
+__global__ void k_split_feature_map(const float* __restrict__ F, int r, int d, __nv_bfloat16* __restrict__ Ft, int f_div) {
   pdl_wait();                                                   // the feature map comes from the kernels before
   pdl_launch_dependents();
   const int bh = blockIdx.y;
-  for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < 64 * 128; e += gridDim.x * blockDim.x) {
-    const int j = e / 128, k = e % 128;
-    float x = j < r ? F[((i64)(bh / f_div) * 128 + k) * r + j] : 0.f;
-    __nv_bfloat16* out = Ft + (i64)bh * 3 * 64 * 128 + e;
+  for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < 64 * d; e += gridDim.x * blockDim.x) {
+    const int j = e / d, k = e % d;
+    float x = j < r ? F[((i64)(bh / f_div) * d + k) * r + j] : 0.f;
+    __nv_bfloat16* out = Ft + (i64)bh * 3 * 64 * d + e;
 #pragma unroll
     for (int t = 0; t < 3; ++t) {
       const __nv_bfloat16 hb = __float2bfloat16_rn(x);
-      out[(i64)t * 64 * 128] = hb;
+      out[(i64)t * 64 * d] = hb;
       x -= __bfloat162float(hb);
     }
   }
@@ -188,26 +189,29 @@ __global__ void k_split_feature_map(const float* __restrict__ F, int r, __nv_bfl
 }  // namespace tc
 
 cudaError_t init_project_tc() {
-  return cudaFuncSetAttribute(tc::k_project_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)tc::PjSmem::total);
+  const cudaError_t e = cudaFuncSetAttribute(tc::k_project_tc<128>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)tc::PjSmem<128>::total);
+  if (e != cudaSuccess) return e;
+  return cudaFuncSetAttribute(tc::k_project_tc<64>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)tc::PjSmem<64>::total);
 }
 bool project_tc_supported(int dtype, int d, int r, const i64* xs) {
-  return dtype == SPARSEPR_BF16 && d == 128 && r <= 64 && xs[2] % 8 == 0 && xs[1] % 8 == 0 && xs[0] % 8 == 0 && tc::tma_available();
+  return dtype == SPARSEPR_BF16 && (d == 64 || d == 128) && r <= 64 && xs[2] % 8 == 0 && xs[1] % 8 == 0 && xs[0] % 8 == 0 && tc::tma_available();
 }
 
-// Ft: bf16 scratch [BH][3][64][128]
-bool launch_project_tc(const void* X, const i64* xs, int BH, int H, int N, int r, const float* F, bool rms, float eps,
+// Ft: bf16 scratch [BH][3][64][d]
+bool launch_project_tc(const void* X, const i64* xs, int BH, int H, int N, int d, int r, const float* F, bool rms, float eps,
                        float* phi, int ldphi, unsigned* maxabs, __nv_bfloat16* Ft, int* err, cudaStream_t st, int f_div) {
   using namespace tc;
   CUtensorMap mx, mf;
-  launch_pdl(tc::k_split_feature_map, dim3(8, BH), dim3(256), 0, st, F, r, Ft, f_div < 1 ? 1 : f_div);
-  if (!make_map(&mx, X, 128, N, H, BH / H, xs[0], xs[1], xs[2], 128) ||
-      !make_map(&mf, Ft, 128, 64, 3, BH, (i64)3 * 64 * 128, (i64)64 * 128, 128, 64))
+  launch_pdl(tc::k_split_feature_map, dim3(8, BH), dim3(256), 0, st, F, r, d, Ft, f_div < 1 ? 1 : f_div);
+  if (!make_map(&mx, X, d, N, H, BH / H, xs[0], xs[1], xs[2], 128) ||
+      !make_map(&mf, Ft, d, 64, 3, BH, (i64)3 * 64 * d, (i64)64 * d, d, 64))
     return false;
   PjParams p{};
   p.H = H; p.N = N; p.r = r; p.ldphi = ldphi; p.rms = rms; p.eps = eps; p.phi = phi; p.maxabs_bits = maxabs; p.err = err;
   const int row_tiles = (N + 127) / 128;
   p.ctas_per_head = std::max(1, std::min(row_tiles, (2 * sm_count()) / BH));
-  launch_pdl(k_project_tc, dim3(p.ctas_per_head, BH), dim3(kPjThreads), PjSmem::total, st, mx, mf, p);
+  if (d == 128) launch_pdl(k_project_tc<128>, dim3(p.ctas_per_head, BH), dim3(kPjThreads), PjSmem<128>::total, st, mx, mf, p);
+  else launch_pdl(k_project_tc<64>, dim3(p.ctas_per_head, BH), dim3(kPjThreads), PjSmem<64>::total, st, mx, mf, p);
   return true;
 }
 
