@@ -108,14 +108,14 @@ def launches_per_call(T, fitted, tensor_path):
         kmeans = 2 + 1 + 2 * T + (1 if T > 1 else 0) + (T - 1)
     else:                # init, first norms, T assignments, T-1 updates
         kmeans = 2 + T + (T - 1)
-    # per side: Gram, eigen-solver (Householder, tridiagonal stage, marked-matrix fallback), projection (+ split of
+    # per side: Gram, eigen-solver (Householder, vectors, orthogonalisation, back-transformation, marked-matrix fallback), projection (+ split of
     # the feature map), k-means, sort + means; then probes; route; tile offsets + remainder rows
-    plan = 2 * (4 + (2 if tensor_path else 1) + kmeans + 2) + 2 + 2 + 3
+    plan = 2 * (6 + (2 if tensor_path else 1) + kmeans + 2) + 2 + 2 + 3
     if not fitted:
         plan -= 2
     attend = 3 + 1 + (1 if tensor_path else 0)       # gathers, attention (+ the packed-remainder kernel)
     if fitted:
-        attend += (3 if tensor_path else 2) + 7 + 1  # probe rows (+gather) + merge, fit (eigen-solver: three launches), probe write
+        attend += (3 if tensor_path else 2) + 9 + 1  # probe rows (+gather) + merge, fit (eigen-solver: five launches), probe write
         attend += 1 if tensor_path else 0            # correction pass
     return plan + attend
 
