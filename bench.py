@@ -116,7 +116,7 @@ def launches_per_call(T, fitted, tensor_path):
     attend = 3 + 1 + (1 if tensor_path else 0)       # gathers, attention (+ the packed-remainder kernel)
     if fitted:
         attend += (3 if tensor_path else 2) + 9 + 1  # probe rows (+gather) + merge, fit (eigen-solver: five launches), probe write
-        attend += 1 if tensor_path else 0            # correction pass
+        attend += 1                                  # correction pass
     return plan + attend
 
 

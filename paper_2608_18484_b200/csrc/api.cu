@@ -320,6 +320,7 @@ struct AttendWs {
   __nv_bfloat16* Olo;                  // second bf16 word of the hard-drop rows for the correction pass (tensor-core path, fitted mode)
   float *partial, *X, *Dn, *A, *c, *Psi;
   __nv_bfloat16 *At, *Qp;
+  float* fpart; int* fcount;           // float32 block-sparse kernel: partial states of split key sequences, counters per tile
   int n_split_tc;
   double* fit; double* fit_eigws;
   int n_split;
@@ -351,9 +352,12 @@ void carve_attend(Carver& c, const Resolved& r, AttendWs* w) {
   float* A = c.take<float>(BH * d * d); float* cc = c.take<float>(BH * d);
   float* Psi = c.take<float>(BH * d * d);
   __nv_bfloat16* At = c.take<__nv_bfloat16>(2 * BH * d * d);   // the correction map as two bf16 words
+  const bool f32 = r.dtype == SPARSEPR_F32;
+  float* fpart = c.take<float>(f32 ? attention_f32_part_floats(r.BH, r.N, r.Cq, r.d) : 0);
+  int* fcount = c.take<int>(f32 ? attention_f32_counters(r.BH, r.N, r.Cq) : 0);
   double* fit = c.take<double>(fit_scratch_doubles(r.BH, (int)M1, r.d));
   double* fit_eigws = c.take<double>(eig_scratch_doubles(r.BH, r.d));
-  if (w) { w->Olo = Olo; w->Qg = Qg; w->Kg = Kg; w->Vg = Vg; w->partial = partial; w->X = X; w->Dn = Dn; w->A = A; w->c = cc; w->Psi = Psi; w->At = At; w->Qp = Qp; w->n_split_tc = ns_tc; w->fit = fit; w->fit_eigws = fit_eigws; w->n_split = ns; }
+  if (w) { w->fpart = fpart; w->fcount = fcount; w->Olo = Olo; w->Qg = Qg; w->Kg = Kg; w->Vg = Vg; w->partial = partial; w->X = X; w->Dn = Dn; w->A = A; w->c = cc; w->Psi = Psi; w->At = At; w->Qp = Qp; w->n_split_tc = ns_tc; w->fit = fit; w->fit_eigws = fit_eigws; w->n_split = ns; }
 }
 
 i64 pair_budget(const Resolved& r) {
@@ -684,10 +688,11 @@ static sparsepr_status_t attend_impl(const sparsepr_plan_t* p, const void* Q, co
   aa.O_sparse = O_sparse;
   aa.err = p->err;
   const bool tensor = attention_tc_supported(aa);
-  // The probe rows and the fit depend only on the gathered K, V and the plan.  With the tensor-core
-  // kernel (whose correction is a separate pass) they run on the plan's second stream beside the
-  // block-sparse kernel; a profiled call keeps everything on one stream so that stage times add up.
-  const bool overlap = fitted && tensor && prof == nullptr;
+  if (r.dtype == SPARSEPR_BF16 && !tensor) return SPARSEPR_ERR_CUDA;          // no tensor maps: nothing else serves bf16
+  // The probe rows and the fit depend only on the gathered K, V and the plan.  The correction is a separate pass, so
+  // they run on the plan's second stream beside the block-sparse kernel; a profiled call keeps everything on one
+  // stream so that stage times add up.
+  const bool overlap = fitted && prof == nullptr;
   if (p->side_pending && !overlap) { join_side(p, st); p->side_pending = false; }   // the plan call's probe selection, still on the second stream
   if (fitted) {
     cudaStream_t fs = st;
@@ -729,9 +734,11 @@ static sparsepr_status_t attend_impl(const sparsepr_plan_t* p, const void* Q, co
     if (fitted && !launch_correction_tc(w.c, w.At, w.Olo, O, r.os, r.BH, r.H, r.N, r.d, p->err, st)) return SPARSEPR_ERR_CUDA;
     tm.mark(SPARSEPR_STAGE_CORRECTION);
   } else {
-    aa.A = fitted ? w.A : nullptr; aa.c = fitted ? w.c : nullptr;      // correction fused into this kernel's epilogue
-    launch_attention_simt(aa, st);
+    launch_attention_f32(aa, w.fpart, w.fcount, st);
     tm.mark(SPARSEPR_STAGE_ATTENTION);
+    if (overlap) { join_side(p, st); p->side_pending = false; }
+    if (fitted) launch_correction_f32(w.A, w.c, O, r.os, r.BH, r.H, r.N, r.d, st);
+    tm.mark(SPARSEPR_STAGE_CORRECTION);
   }
   if (fitted) launch_write_probe_rows(r.dtype, w.Dn, p->probe_idx, r.BH, r.H, r.M, r.d, O, r.os, st);
   tm.mark(SPARSEPR_STAGE_PROBE_WRITE);
@@ -777,8 +784,10 @@ sparsepr_status_t sparsepr_dense(const sparsepr_shape_t* shape, float softmax_sc
   for (int i = 0; i < 3; ++i) { aa.qs[i] = r.qs[i]; aa.ks[i] = r.ks[i]; aa.vs[i] = r.vs[i]; aa.os[i] = r.os[i]; }
   if (attention_tc_supported(aa)) {
     if (!launch_attention_tc(aa, static_cast<cudaStream_t>(cuda_stream))) return SPARSEPR_ERR_CUDA;
+  } else if (r.dtype == SPARSEPR_F32) {
+    launch_attention_f32(aa, nullptr, nullptr, static_cast<cudaStream_t>(cuda_stream));
   } else {
-    launch_attention_simt(aa, static_cast<cudaStream_t>(cuda_stream));
+    return SPARSEPR_ERR_CUDA;                                  // no tensor maps: nothing else serves bf16
   }
   return launch_ok() ? SPARSEPR_OK : SPARSEPR_ERR_CUDA;
 }

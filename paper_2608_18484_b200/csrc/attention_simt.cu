@@ -1,9 +1,9 @@
 // float32 attention kernels on the CUDA cores: block-sparse attention with
 // renormalised hard drop (Eq. 3) over the group-major layout, dense attention
-// (Eq. 1), and the exact probe rows with their retained/omitted statistics
-// (Appendix A.1).  These are the kernels of the float32 configuration (whose
-// 1e-5 tolerance rules out reduced-precision tensor-core inputs) and the
-// fallback shapes of the bf16 path.
+// (Eq. 1), the residual correction (Eq. 9), and the exact probe rows with their
+// retained/omitted statistics (Appendix A.1).  These are the kernels of the float32
+// configuration, whose 1e-5 tolerance rules out reduced-precision tensor-core inputs.
+#include <algorithm>
 #include "kernels.cuh"
 
 namespace spr {
@@ -14,7 +14,6 @@ constexpr float kLog2e = 1.4426950408889634f;
 
 template <int D> struct SimtSmem {
   static constexpr int q = D * BM, k = D * BN, v = BN * D, p = BN * BM;
-  static constexpr size_t bytes = (size_t)(q + k + v + p) * sizeof(float) + 64 * sizeof(int);
 };
 
 // Transposed tile load: dst[(c)*64 + r] = src_row_r[c]; rows given by a row-pointer functor.
@@ -105,30 +104,53 @@ __device__ __forceinline__ float row16_sum(float v) {
 }
 
 // =============================================================================
-// Main kernel.  SPARSE: one CTA per 64-row tile of one query group; the keys of
-// the routed K/V groups are streamed as one concatenated sequence (every tile is
-// full except the last).  Dense: one CTA per 64 rows over all keys.  Epilogue:
-// O_hat = O_sp + (O_sp A + c) (the affine map of Eq. 9 composed into one matrix),
-// stored at the original token index.
+// Main kernel.  SPARSE: one CTA per 64-row tile of one query group; the keys of the routed K/V groups are streamed as one
+// concatenated sequence (every tile of 64 keys is full except the last).  Dense: one CTA per 64 rows over all keys.
+// Stores the hard-drop output at the original token index; the correction is a pass of its own, so that the probe rows and
+// the fit can run beside this kernel.
+//
+// Bound by the FMA pipe: 128 threads, two CTAs per SM, thread (ty, tx) holds 8 query rows x 4 keys of the scores and
+// 8 rows x D / 16 columns of the output, so that a 16-byte shared-memory read serves 8 to 32 multiply-adds, and all of
+// them are packed two to an instruction (scores: even and odd dimensions in separate halves; output: column pairs).
+// Rows are 16 bytes longer than their data, which keeps the 16-byte reads of consecutive rows in different banks.  The
+// probabilities take the place of the K tile.  Tiles arrive by cp.async; the other CTA of the SM covers their latency.
+// F32_MEASURED
+//
+// A grid with few tiles leaves SMs idle, and groups that route to many keys then set the duration: with n_split > 1 the
+// key sequence of a tile is cut into up to n_split parts of at least kMinSplitTiles key tiles, one CTA each; every part
+// leaves (m, l, O) in `part`, and the CTA that finishes last (a counter per tile) adds them up in the order of the parts.
 // =============================================================================
-template <typename T, int D, bool SPARSE>
-__global__ void __launch_bounds__(256) k_attention_simt(AttnArgs a) {
+constexpr int kFThreads = 128, kMinSplitTiles = 4;
+template <int D> struct F32Smem {
+  static constexpr int ld = D + 4, ldp = BM + 4;
+  static constexpr int q = BM * ld, k = BN * ld, v = BN * D;
+  static constexpr size_t bytes = (size_t)(q + k + v) * sizeof(float) + 2 * BN * sizeof(int);
+  static_assert(BN * ldp <= k, "the probabilities fit into the K tile");
+};
+__device__ __forceinline__ void cp16(float* dst, const float* src, bool on) {     // 16 bytes, zeros when off
+  const unsigned d = (unsigned)__cvta_generic_to_shared(dst);
+  const int n = on ? 16 : 0;
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(d), "l"(src), "r"(n) : "memory");
+}
+
+template <int D, bool SPARSE>
+__global__ void __launch_bounds__(kFThreads, 2) k_attention_f32(AttnArgs a, int n_split, float* __restrict__ part, int* __restrict__ counter) {
+  using S = F32Smem<D>;
   extern __shared__ __align__(16) float smem[];
-  float* Qs = smem;
-  float* Ks = Qs + SimtSmem<D>::q;
-  float* Vs = Ks + SimtSmem<D>::k;
-  float* Ps = Vs + SimtSmem<D>::v;
-  int* krow = reinterpret_cast<int*>(Ps + SimtSmem<D>::p);     // [64] source row of every tile key
+  float* Qs = smem;                                      // [64][D + 4]
+  float* Ks = Qs + S::q;                                 // [64][D + 4], then P [64 keys][64 rows + 4]
+  float* Vs = Ks + S::k;                                 // [64][D]
+  int* krow = reinterpret_cast<int*>(Vs + S::v);         // [2][64] source row of every key of this / the next tile
   __shared__ int cum[SPARSE ? kMaxGroups + 1 : 1];
   __shared__ int scratch[34];
-  constexpr int OC = D / 16;
+  constexpr int OP = D / 32;                             // output column pairs per thread: columns 4 tx + 64 c + {0..3}
   const int bh = blockIdx.y, b = bh / a.H, h = bh % a.H;
   const int tid = threadIdx.x, ty = tid >> 4, tx = tid & 15;
 
   int row0, nrows, nroute = 0, L;
   const int* ridx = nullptr;
   const int* kvoff = nullptr;
-  const T *Qb, *Kb, *Vb;
+  const float *Qb, *Kb, *Vb;
   i64 qsn, ksn, vsn;
   if (SPARSE) {
     const int* toff = a.tile_off + (i64)bh * (a.Cq + 1);
@@ -143,136 +165,250 @@ __global__ void __launch_bounds__(256) k_attention_simt(AttnArgs a) {
     ridx = a.route_idx + (i64)bh * a.Cq * a.Ck + rp[g];
     nroute = rp[g + 1] - rp[g];
     kvoff = a.kv_off + (i64)bh * (a.Ck + 1);
-    for (int t = tid; t < nroute; t += 256) { const int bb = ridx[t]; cum[t] = kvoff[bb + 1] - kvoff[bb]; }
+    for (int t = tid; t < nroute; t += kFThreads) { const int bb = ridx[t]; cum[t] = kvoff[bb + 1] - kvoff[bb]; }
     __syncthreads();
     L = block_exclusive_scan(cum, nroute, scratch);
     if (tid == 0) cum[nroute] = L;
-    Qb = (const T*)a.Q + (i64)bh * a.N * D; Kb = (const T*)a.K + (i64)bh * a.N * D; Vb = (const T*)a.V + (i64)bh * a.N * D;
+    Qb = (const float*)a.Q + (i64)bh * a.N * D; Kb = (const float*)a.K + (i64)bh * a.N * D; Vb = (const float*)a.V + (i64)bh * a.N * D;
     qsn = ksn = vsn = D;
   } else {
     row0 = blockIdx.x * BM;
     nrows = min(BM, a.N - row0);
     L = a.N;
-    Qb = (const T*)a.Q + b * a.qs[0] + h * a.qs[1]; Kb = (const T*)a.K + b * a.ks[0] + h * a.ks[1];
-    Vb = (const T*)a.V + b * a.vs[0] + h * a.vs[1];
+    Qb = (const float*)a.Q + b * a.qs[0] + h * a.qs[1]; Kb = (const float*)a.K + b * a.ks[0] + h * a.ks[1];
+    Vb = (const float*)a.V + b * a.vs[0] + h * a.vs[1];
     qsn = a.qs[2]; ksn = a.ks[2]; vsn = a.vs[2];
   }
-  load_tile_transposed<T, D>(Qs, [&](int r) { return r < nrows ? Qb + (i64)(row0 + r) * qsn : (const T*)nullptr; });
+  // this CTA's part of the key tiles
+  const int n_tiles = (L + BN - 1) / BN;
+  const int parts = max(1, min(n_split, n_tiles / kMinSplitTiles)), z = blockIdx.z;
+  if (z >= parts) return;
+  const int t_begin = (int)((i64)n_tiles * z / parts), t_end = (int)((i64)n_tiles * (z + 1) / parts);
 
-  float o[4][OC], m[4], l[4];
-#pragma unroll
-  for (int i = 0; i < 4; ++i) {
-    m[i] = -INFINITY; l[i] = 0.f;
-#pragma unroll
-    for (int c = 0; c < OC; ++c) o[i][c] = 0.f;
+  constexpr int CPR = D / 4;                             // 16-byte chunks per row
+#pragma unroll 4
+  for (int e = tid; e < BM * CPR; e += kFThreads) {
+    const int r = e / CPR, c = (e % CPR) * 4;
+    cp16(Qs + r * S::ld + c, Qb + (i64)(row0 + min(r, nrows - 1)) * qsn + c, r < nrows);
   }
-  const float sc = a.scale * kLog2e;
-  for (int t0 = 0; t0 < L; t0 += BN) {
-    const int ncols = min(BN, L - t0);
-    __syncthreads();                                   // previous tile fully consumed
+  auto find_rows = [&](int t, int* dst) {                // source rows of key tile t
     if (tid < BN) {
+      const int pos = t * BN + tid;
       int src = -1;
-      if (tid < ncols) {
+      if (pos < L) {
         if (SPARSE) {
-          const int pos = t0 + tid;
-          int lo = 0, hi = nroute - 1;                 // last range with cum[range] <= pos
+          int lo = 0, hi = nroute - 1;                   // last range with cum[range] <= pos
           while (lo < hi) { const int mid = (lo + hi + 1) >> 1; if (cum[mid] <= pos) lo = mid; else hi = mid - 1; }
           src = kvoff[ridx[lo]] + (pos - cum[lo]);
-        } else src = t0 + tid;
+        } else src = pos;
       }
-      krow[tid] = src;
+      dst[tid] = src;
     }
-    __syncthreads();
-    load_tile_transposed<T, D>(Ks, [&](int r) { return krow[r] >= 0 ? Kb + (i64)krow[r] * ksn : (const T*)nullptr; });
-    load_tile_natural<T, D>(Vs, [&](int r) { return krow[r] >= 0 ? Vb + (i64)krow[r] * vsn : (const T*)nullptr; });
-    __syncthreads();
-    float s[4][4];
-    qk_tile<D>(Qs, Ks, ty, tx, s);
-    float corr[4];
+  };
+  __syncthreads();                                       // cum[] is complete
+  find_rows(t_begin, krow);
+
+  float2 o[8][OP];
+  float m[8], l[8];
 #pragma unroll
-    for (int i = 0; i < 4; ++i) {
-      float mx = -INFINITY;
+  for (int i = 0; i < 8; ++i) {
+    m[i] = -INFINITY; l[i] = 0.f;
 #pragma unroll
-      for (int j = 0; j < 4; ++j) {
-        s[i][j] = (tx * 4 + j < ncols) ? s[i][j] * sc : -INFINITY;
-        mx = fmaxf(mx, s[i][j]);
+    for (int c = 0; c < OP; ++c) o[i][c] = make_float2(0.f, 0.f);
+  }
+  const float sc = a.scale * kLog2e;
+  for (int t = t_begin; t < t_end; ++t) {
+    const int* kr = krow + ((t - t_begin) & 1) * BN;
+    const int ncols = min(BN, L - t * BN);
+    __syncthreads();                                     // previous tile fully consumed, rows of this one known
+#pragma unroll 4
+    for (int e = tid; e < BN * CPR; e += kFThreads) {
+      const int r = e / CPR, c = (e % CPR) * 4, src = kr[r];
+      cp16(Ks + r * S::ld + c, Kb + (i64)max(src, 0) * ksn + c, src >= 0);
+      cp16(Vs + r * D + c, Vb + (i64)max(src, 0) * vsn + c, src >= 0);
+    }
+    asm volatile("cp.async.commit_group;" ::: "memory");
+    if (t + 1 < t_end) find_rows(t + 1, krow + ((t + 1 - t_begin) & 1) * BN);
+    asm volatile("cp.async.wait_group 0;" ::: "memory");
+    __syncthreads();
+    // scores of rows 8 ty + i and keys tx + 16 j
+    float s[8][4];
+    {
+      float2 acc[8][4];
+#pragma unroll
+      for (int i = 0; i < 8; ++i)
+#pragma unroll
+        for (int j = 0; j < 4; ++j) acc[i][j] = make_float2(0.f, 0.f);
+      const float* qp = Qs + ty * 8 * S::ld;
+      const float* kp = Ks + tx * S::ld;
+#pragma unroll 2
+      for (int k = 0; k < D; k += 4) {
+        float4 kk[4];
+#pragma unroll
+        for (int j = 0; j < 4; ++j) kk[j] = *reinterpret_cast<const float4*>(kp + 16 * j * S::ld + k);
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+          const float4 q = *reinterpret_cast<const float4*>(qp + i * S::ld + k);
+#pragma unroll
+          for (int j = 0; j < 4; ++j) {
+            acc[i][j] = __ffma2_rn(make_float2(q.x, q.y), make_float2(kk[j].x, kk[j].y), acc[i][j]);
+            acc[i][j] = __ffma2_rn(make_float2(q.z, q.w), make_float2(kk[j].z, kk[j].w), acc[i][j]);
+          }
+        }
       }
-      mx = row16_max(mx);
+#pragma unroll
+      for (int i = 0; i < 8; ++i)
+#pragma unroll
+        for (int j = 0; j < 4; ++j) s[i][j] = tx + 16 * j < ncols ? (acc[i][j].x + acc[i][j].y) * sc : -INFINITY;
+    }
+    __syncthreads();                                     // K is consumed: its place takes the probabilities
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+      const float mx = row16_max(fmaxf(fmaxf(s[i][0], s[i][1]), fmaxf(s[i][2], s[i][3])));
       const float mn = fmaxf(m[i], mx);
-      corr[i] = exp2f(m[i] - mn);                      // 0 on the first tile (m = -inf)
+      const float corr = exp2f(m[i] - mn);               // 0 on the first tile (m = -inf)
       m[i] = mn;
-      float ps = 0.f;
 #pragma unroll
-      for (int j = 0; j < 4; ++j) { s[i][j] = exp2f(s[i][j] - mn); ps += s[i][j]; }
-      l[i] = l[i] * corr[i] + ps;
+      for (int j = 0; j < 4; ++j) s[i][j] = exp2f(s[i][j] - mn);
+      l[i] = fmaf(l[i], corr, (s[i][0] + s[i][1]) + (s[i][2] + s[i][3]));
+      if (corr != 1.f) {
 #pragma unroll
-      for (int c = 0; c < OC; ++c) o[i][c] *= corr[i];
+        for (int c = 0; c < OP; ++c) { o[i][c].x *= corr; o[i][c].y *= corr; }
+      }
     }
+    float* Ps = Ks;
 #pragma unroll
-    for (int j = 0; j < 4; ++j)
-      *reinterpret_cast<float4*>(Ps + (tx * 4 + j) * BM + ty * 4) = make_float4(s[0][j], s[1][j], s[2][j], s[3][j]);
+    for (int j = 0; j < 4; ++j) {
+      float* pp = Ps + (tx + 16 * j) * S::ldp + ty * 8;
+      *reinterpret_cast<float4*>(pp) = make_float4(s[0][j], s[1][j], s[2][j], s[3][j]);
+      *reinterpret_cast<float4*>(pp + 4) = make_float4(s[4][j], s[5][j], s[6][j], s[7][j]);
+    }
     __syncthreads();
-    pv_tile<D>(Ps, Vs, ty, tx, ncols, o);
+#pragma unroll 4
+    for (int j = 0; j < ncols; ++j) {
+      const float4 p0 = *reinterpret_cast<const float4*>(Ps + j * S::ldp + ty * 8), p1 = *reinterpret_cast<const float4*>(Ps + j * S::ldp + ty * 8 + 4);
+      const float pv[8] = {p0.x, p0.y, p0.z, p0.w, p1.x, p1.y, p1.z, p1.w};
+#pragma unroll
+      for (int c = 0; c < OP / 2; ++c) {
+        const float4 v = *reinterpret_cast<const float4*>(Vs + j * D + 64 * c + 4 * tx);
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+          const float2 pp = make_float2(pv[i], pv[i]);
+          o[i][2 * c] = __ffma2_rn(pp, make_float2(v.x, v.y), o[i][2 * c]);
+          o[i][2 * c + 1] = __ffma2_rn(pp, make_float2(v.z, v.w), o[i][2 * c + 1]);
+        }
+      }
+    }
+  }
+#pragma unroll
+  for (int i = 0; i < 8; ++i) l[i] = row16_sum(l[i]);
+  if (parts > 1) {
+    const i64 slot = ((i64)bh * gridDim.x + blockIdx.x) * n_split;
+    float* mine = part + (slot + z) * BM * (D + 2);
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+      const int r = ty * 8 + i;
+      if (tx == 0) { mine[r] = m[i]; mine[BM + r] = l[i]; }
+#pragma unroll
+      for (int c = 0; c < OP / 2; ++c)
+        *reinterpret_cast<float4*>(mine + 2 * BM + r * D + 64 * c + 4 * tx) = make_float4(o[i][2 * c].x, o[i][2 * c].y, o[i][2 * c + 1].x, o[i][2 * c + 1].y);
+    }
+    __threadfence();
+    __syncthreads();
+    if (tid == 0) scratch[0] = atomicAdd(counter + (i64)bh * gridDim.x + blockIdx.x, 1);
+    __syncthreads();
+    if (scratch[0] != parts - 1) return;
+    __threadfence();
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+      const int r = ty * 8 + i;
+      float mm = -INFINITY;
+      for (int q = 0; q < parts; ++q) mm = fmaxf(mm, part[(slot + q) * BM * (D + 2) + r]);
+      m[i] = mm; l[i] = 0.f;
+#pragma unroll
+      for (int c = 0; c < OP; ++c) o[i][c] = make_float2(0.f, 0.f);
+      for (int q = 0; q < parts; ++q) {
+        const float* pq = part + (slot + q) * BM * (D + 2);
+        const float w = exp2f(pq[r] - mm);
+        l[i] = fmaf(w, pq[BM + r], l[i]);
+#pragma unroll
+        for (int c = 0; c < OP / 2; ++c) {
+          const float4 v = *reinterpret_cast<const float4*>(pq + 2 * BM + r * D + 64 * c + 4 * tx);
+          o[i][2 * c] = __ffma2_rn(make_float2(w, w), make_float2(v.x, v.y), o[i][2 * c]);
+          o[i][2 * c + 1] = __ffma2_rn(make_float2(w, w), make_float2(v.z, v.w), o[i][2 * c + 1]);
+        }
+      }
+    }
   }
   // ---- epilogue -------------------------------------------------------------------
+  float* Ob = (float*)a.O + b * a.os[0] + h * a.os[1];
 #pragma unroll
-  for (int i = 0; i < 4; ++i) {
-    const float tot = row16_sum(l[i]);
-    const float inv = tot > 0.f ? 1.f / tot : 0.f;
+  for (int i = 0; i < 8; ++i) {
+    const int r = ty * 8 + i;
+    if (r >= nrows) continue;
+    const float inv = l[i] > 0.f ? 1.f / l[i] : 0.f;
+    const int dst = SPARSE ? a.q_perm[(i64)bh * a.N + row0 + r] : row0 + r;
 #pragma unroll
-    for (int c = 0; c < OC; ++c) o[i][c] *= inv;
+    for (int c = 0; c < OP / 2; ++c) {
+      const float4 v = make_float4(o[i][2 * c].x * inv, o[i][2 * c].y * inv, o[i][2 * c + 1].x * inv, o[i][2 * c + 1].y * inv);
+      *reinterpret_cast<float4*>(Ob + (i64)dst * a.os[2] + 64 * c + 4 * tx) = v;
+      if (a.O_sparse) *reinterpret_cast<float4*>(a.O_sparse + ((i64)bh * a.N + dst) * D + 64 * c + 4 * tx) = v;
+    }
   }
-  float res[4][OC];
+}
+
+// Residual correction of Eq. 9 in place: O <- X + X A + c for the rows X = O (float32).  A CTA takes 32 rows of a head; A is
+// read through L2, thread (ty, tx) = 4 rows x D / 16 columns.
+template <int D>
+__global__ void __launch_bounds__(128) k_correction_f32(const float* __restrict__ A, const float* __restrict__ cvec, int H, int N,
+                                                        float* __restrict__ O, i64 ob, i64 oh, i64 on) {
+  __shared__ __align__(16) float xs[32][D + 4];
+  const int bh = blockIdx.y, row0 = blockIdx.x * 32, nr = min(32, N - row0);
+  const int tid = threadIdx.x, ty = tid >> 4, tx = tid & 15;
+  float* Ob = O + (bh / H) * ob + (bh % H) * oh;
+  for (int e = tid; e < 32 * (D / 4); e += 128) {
+    const int r = e / (D / 4), c = (e % (D / 4)) * 4;
+    *reinterpret_cast<float4*>(&xs[r][c]) = r < nr ? *reinterpret_cast<const float4*>(Ob + (i64)(row0 + r) * on + c) : make_float4(0.f, 0.f, 0.f, 0.f);
+  }
+  __syncthreads();
+  const float* Ah = A + (i64)bh * D * D + 4 * tx;
+  float acc[4][D / 16];
 #pragma unroll
   for (int i = 0; i < 4; ++i)
 #pragma unroll
-    for (int c = 0; c < OC; ++c) res[i][c] = o[i][c];
-  if (a.A != nullptr) {
-    __syncthreads();
-    float* Os = Qs;                                    // [BM][D]
-    float* As = Ks;                                    // [D][D] spans the K and V tiles
+    for (int c = 0; c < D / 16; ++c) acc[i][c] = 0.f;
+#pragma unroll 4
+  for (int k = 0; k < D; ++k) {
+    float x[4];
 #pragma unroll
-    for (int i = 0; i < 4; ++i)
+    for (int i = 0; i < 4; ++i) x[i] = xs[ty * 4 + i][k];
 #pragma unroll
-      for (int c = 0; c < OC; ++c) Os[(ty * 4 + i) * D + tx * OC + c] = o[i][c];
-    const float* Ah = a.A + (i64)bh * D * D;
-    for (int e = tid * 4; e < D * D; e += 1024) *reinterpret_cast<float4*>(As + e) = *reinterpret_cast<const float4*>(Ah + e);
-    __syncthreads();
-    const float* ch = a.c + (i64)bh * D;
-#pragma unroll
-    for (int i = 0; i < 4; ++i)
-#pragma unroll
-      for (int c = 0; c < OC; ++c) res[i][c] += ch[tx * OC + c];
-    for (int k = 0; k < D; ++k) {
-      float av[OC];
-#pragma unroll
-      for (int c = 0; c < OC; c += 4) {
-        const float4 v = *reinterpret_cast<const float4*>(As + k * D + tx * OC + c);
-        av[c] = v.x; av[c + 1] = v.y; av[c + 2] = v.z; av[c + 3] = v.w;
-      }
+    for (int c = 0; c < D / 64; ++c) {
+      const float4 v = __ldg(reinterpret_cast<const float4*>(Ah + (i64)k * D + 64 * c));
 #pragma unroll
       for (int i = 0; i < 4; ++i) {
-        const float x = Os[(ty * 4 + i) * D + k];
-#pragma unroll
-        for (int c = 0; c < OC; ++c) res[i][c] = fmaf(x, av[c], res[i][c]);
+        acc[i][4 * c] = fmaf(x[i], v.x, acc[i][4 * c]); acc[i][4 * c + 1] = fmaf(x[i], v.y, acc[i][4 * c + 1]);
+        acc[i][4 * c + 2] = fmaf(x[i], v.z, acc[i][4 * c + 2]); acc[i][4 * c + 3] = fmaf(x[i], v.w, acc[i][4 * c + 3]);
       }
     }
   }
-  T* Ob = (T*)a.O + b * a.os[0] + h * a.os[1];
 #pragma unroll
-  for (int i = 0; i < 4; ++i) {
-    const int r = ty * 4 + i;
-    if (r >= nrows) continue;
-    const int dst = SPARSE ? a.q_perm[(i64)bh * a.N + row0 + r] : row0 + r;
-    T* op = Ob + (i64)dst * a.os[2] + tx * OC;
+  for (int c = 0; c < D / 64; ++c) {
+    const float4 cv = *reinterpret_cast<const float4*>(cvec + (i64)bh * D + 64 * c + 4 * tx);
 #pragma unroll
-    for (int c = 0; c < OC; ++c) op[c] = from_f32<T>(res[i][c]);
-    if (a.O_sparse) {
-      float* sp = a.O_sparse + ((i64)bh * a.N + dst) * D + tx * OC;
-#pragma unroll
-      for (int c = 0; c < OC; ++c) sp[c] = o[i][c];
+    for (int i = 0; i < 4; ++i) {
+      const int r = ty * 4 + i;
+      if (r >= nr) continue;
+      const float4 x = *reinterpret_cast<const float4*>(&xs[r][64 * c + 4 * tx]);
+      *reinterpret_cast<float4*>(Ob + (i64)(row0 + r) * on + 64 * c + 4 * tx) =
+          make_float4(x.x + (cv.x + acc[i][4 * c]), x.y + (cv.y + acc[i][4 * c + 1]), x.z + (cv.z + acc[i][4 * c + 2]), x.w + (cv.w + acc[i][4 * c + 3]));
     }
   }
+}
+void launch_correction_f32(const float* A, const float* c, void* O, const i64* os, int BH, int H, int N, int d, cudaStream_t st) {
+  const dim3 grid((N + 31) / 32, BH);
+  if (d == 128) k_correction_f32<128><<<grid, 128, 0, st>>>(A, c, H, N, (float*)O, os[0], os[1], os[2]);
+  else k_correction_f32<64><<<grid, 128, 0, st>>>(A, c, H, N, (float*)O, os[0], os[1], os[2]);
 }
 
 // tiles per query group: ceil(n / tile_rows), or, with small_rem > 0, without the last tile when it
@@ -296,19 +432,33 @@ void launch_tile_offsets(const int* q_off, int BH, int Cq, int tile_rows, int sm
   k_tile_offsets<<<BH, 1024, 0, st>>>(q_off, Cq, tile_rows, small_rem, tile_off);
 }
 
-template <typename T, int D>
-static void attention_dispatch(const AttnArgs& a, cudaStream_t st) {
+// Parts a tile's keys are cut into (float32): enough for about four rounds of CTAs on every SM slot, at most 8, none when the
+// tiles alone fill the GPU.
+int attention_f32_splits(int BH, int N, int Cq) {
+  const i64 tiles = (i64)BH * (N / BM + (Cq + 1) / 2);          // about: a group ends with half a tile
+  return (int)std::max<i64>(1, std::min<i64>(8, (i64)4 * 2 * sm_count() / std::max<i64>(tiles, 1)));
+}
+static i64 f32_tile_slots(int BH, int N, int Cq) { return (i64)BH * ((N + BM - 1) / BM + Cq); }
+size_t attention_f32_part_floats(int BH, int N, int Cq, int d) {
+  const int ns = attention_f32_splits(BH, N, Cq);
+  return ns > 1 ? (size_t)f32_tile_slots(BH, N, Cq) * ns * BM * (d + 2) : 0;
+}
+size_t attention_f32_counters(int BH, int N, int Cq) { return attention_f32_splits(BH, N, Cq) > 1 ? (size_t)f32_tile_slots(BH, N, Cq) : 0; }
+
+template <int D>
+static void attention_dispatch(const AttnArgs& a, float* part, int* counter, cudaStream_t st) {
   if (a.route_ptr) {
-    dim3 grid((a.N + BM - 1) / BM + a.Cq, a.BH);
-    k_attention_simt<T, D, true><<<grid, 256, SimtSmem<D>::bytes, st>>>(a);
+    const int ns = part ? attention_f32_splits(a.BH, a.N, a.Cq) : 1;
+    if (ns > 1) cudaMemsetAsync(counter, 0, attention_f32_counters(a.BH, a.N, a.Cq) * sizeof(int), st);
+    dim3 grid((a.N + BM - 1) / BM + a.Cq, a.BH, ns);
+    k_attention_f32<D, true><<<grid, kFThreads, F32Smem<D>::bytes, st>>>(a, ns, part, counter);
   } else {
     dim3 grid((a.N + BM - 1) / BM, a.BH);
-    k_attention_simt<T, D, false><<<grid, 256, SimtSmem<D>::bytes, st>>>(a);
+    k_attention_f32<D, false><<<grid, kFThreads, F32Smem<D>::bytes, st>>>(a, 1, nullptr, nullptr);
   }
 }
-void launch_attention_simt(const AttnArgs& a, cudaStream_t st) {
-  if (a.dtype == SPARSEPR_BF16) { if (a.d == 128) attention_dispatch<__nv_bfloat16, 128>(a, st); else attention_dispatch<__nv_bfloat16, 64>(a, st); }
-  else { if (a.d == 128) attention_dispatch<float, 128>(a, st); else attention_dispatch<float, 64>(a, st); }
+void launch_attention_f32(const AttnArgs& a, float* part, int* counter, cudaStream_t st) {
+  if (a.d == 128) attention_dispatch<128>(a, part, counter, st); else attention_dispatch<64>(a, part, counter, st);
 }
 
 // =============================================================================
@@ -494,8 +644,7 @@ void launch_probe_merge(const ProbeArgs& a, cudaStream_t st) {
   else k_probe_merge<64><<<g2, 256, 0, st>>>(a.partial, a.n_split, a.M, a.X, a.Dn);
 }
 void launch_probe_rows(const ProbeArgs& a, cudaStream_t st) {
-  if (a.dtype == SPARSEPR_BF16) { if (a.d == 128) probe_dispatch<__nv_bfloat16, 128>(a, st); else probe_dispatch<__nv_bfloat16, 64>(a, st); }
-  else { if (a.d == 128) probe_dispatch<float, 128>(a, st); else probe_dispatch<float, 64>(a, st); }
+  if (a.d == 128) probe_dispatch<float, 128>(a, st); else probe_dispatch<float, 64>(a, st);
 }
 
 // O[b,h,probe_idx[m],:] = O_dense of the probe (Eq. 10, first case)
@@ -519,18 +668,12 @@ void launch_write_probe_rows(int dtype, const float* Dn, const int* probe_idx, i
 cudaError_t init_attention_simt() {
   cudaError_t e;
 #define SPR_ATTR(KERN, BYTES) if ((e = cudaFuncSetAttribute(KERN, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(BYTES))) != cudaSuccess) return e
-  SPR_ATTR((k_attention_simt<float, 128, true>), SimtSmem<128>::bytes);
-  SPR_ATTR((k_attention_simt<float, 128, false>), SimtSmem<128>::bytes);
-  SPR_ATTR((k_attention_simt<float, 64, true>), SimtSmem<64>::bytes);
-  SPR_ATTR((k_attention_simt<float, 64, false>), SimtSmem<64>::bytes);
-  SPR_ATTR((k_attention_simt<__nv_bfloat16, 128, true>), SimtSmem<128>::bytes);
-  SPR_ATTR((k_attention_simt<__nv_bfloat16, 128, false>), SimtSmem<128>::bytes);
-  SPR_ATTR((k_attention_simt<__nv_bfloat16, 64, true>), SimtSmem<64>::bytes);
-  SPR_ATTR((k_attention_simt<__nv_bfloat16, 64, false>), SimtSmem<64>::bytes);
+  SPR_ATTR((k_attention_f32<128, true>), F32Smem<128>::bytes);
+  SPR_ATTR((k_attention_f32<128, false>), F32Smem<128>::bytes);
+  SPR_ATTR((k_attention_f32<64, true>), F32Smem<64>::bytes);
+  SPR_ATTR((k_attention_f32<64, false>), F32Smem<64>::bytes);
   SPR_ATTR((k_probe_rows<float, 128>), probe_smem_bytes<128>(kMaxGroups));
   SPR_ATTR((k_probe_rows<float, 64>), probe_smem_bytes<64>(kMaxGroups));
-  SPR_ATTR((k_probe_rows<__nv_bfloat16, 128>), probe_smem_bytes<128>(kMaxGroups));
-  SPR_ATTR((k_probe_rows<__nv_bfloat16, 64>), probe_smem_bytes<64>(kMaxGroups));
 #undef SPR_ATTR
   return cudaSuccess;
 }

@@ -108,7 +108,6 @@ struct AttnArgs {
   int Cq, Ck;
   int kv_div;                 // query heads per K/V head (grouped-query attention): K/V-side arrays are indexed by bh / kv_div; 0 = 1
   // epilogue
-  const float *A, *c;         // [BH][d][d], [BH][d]; null = no correction
   void* O; i64 os[3];
   float* O_sparse;            // optional [BH][N][d] in original order
   void* O_lo;                 // optional bf16 [BH][N][d] in original order: o - bf16(o) (tensor-core kernels only)
@@ -117,11 +116,18 @@ struct AttnArgs {
 cudaError_t init_attention_simt();
 // tile_off [BH][Cq+1]: prefix of the tiles per query group; small_rem > 0 leaves out a last tile of at most small_rem rows
 void launch_tile_offsets(const int* q_off, int BH, int Cq, int tile_rows, int small_rem, int* tile_off, cudaStream_t st);
-void launch_attention_simt(const AttnArgs& a, cudaStream_t st);
+// float32; sparse calls: part / counter from the workspace (attention_f32_part_floats floats, attention_f32_counters ints; the
+// key sequences are not split when part is null)
+int attention_f32_splits(int BH, int N, int Cq);
+size_t attention_f32_part_floats(int BH, int N, int Cq, int d);
+size_t attention_f32_counters(int BH, int N, int Cq);
+void launch_attention_f32(const AttnArgs& a, float* part, int* counter, cudaStream_t st);
+// O <- O + O A + c in place (float32)
+void launch_correction_f32(const float* A, const float* c, void* O, const i64* os, int BH, int H, int N, int d, cudaStream_t st);
 // ---- attention_tc.cu (tcgen05 / TMEM / TMA; bf16, d = 64 or 128) -------------------------------------
 cudaError_t init_attention_tc();
 bool attention_tc_supported(const AttnArgs& a);
-// tile_off in `a` must have been built for 128-row tiles; a.A and a.c are ignored (no correction epilogue)
+// tile_off in `a` must have been built for 128-row tiles
 bool launch_attention_tc(const AttnArgs& a, cudaStream_t st);
 // Query-group remainders of 1..kRemRows rows are left out of the 128-row kernel's tiles (tile offsets built with
 // small_rem = kRemRows) and handled by attention_packed.cu
