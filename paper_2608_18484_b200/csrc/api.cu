@@ -254,7 +254,8 @@ struct sparsepr_plan_s {
   float *mu, *mu2, *mumax; i64* sums; int* counts;
   int *a_K, *a_Q, *kv_perm, *kv_inv, *q_perm, *q_inv, *kv_off, *q_off, *nk, *nq;
   float *kappa, *theta, *score;
-  int *route_ptr, *route_idx, *tile_off, *tile_off128;
+  int *route_ptr, *route_idx, *tile_off128;
+  int4* f32_items; int *f32_keys, *f32_count;   // float32: the attention kernel's list of CTAs
   RouteState* rstate;
   double* probe_dist; int* probe_idx; float* probe_w;
   __nv_bfloat16 *xh, *xl, *mh, *ml, *mw, *Ft; float* xnorm; int* flagged; int* flagcnt; double* eigws;
@@ -289,8 +290,10 @@ void carve_plan(Carver& c, const Resolved& r, sparsepr_plan_s* p) {
   float* kappa = c.take<float>(BH * r.Ck * d); float* theta = c.take<float>(BH * r.Cq * d);
   float* score = c.take<float>(BH * (size_t)r.Cq * r.Ck);
   int* rptr = c.take<int>(BH * (r.Cq + 1)); int* ridx = c.take<int>(BH * (size_t)r.Cq * r.Ck);
-  int* toff = c.take<int>(BH * (r.Cq + 1));
-  int* toff128 = c.take<int>(BH * (r.Cq + 1));
+  const bool f32 = r.dtype == SPARSEPR_F32;
+  int* toff128 = c.take<int>(f32 ? 0 : BH * (r.Cq + 1));
+  int4* items = c.take<int4>(f32 ? attention_f32_items((int)BH, (int)N, r.Cq) : 0);
+  int* ikeys = c.take<int>(f32 ? BH * r.Cq : 0); int* icount = c.take<int>(f32 ? 1 : 0);
   RouteState* rs = c.take<RouteState>(BH);
   double* pd = c.take<double>(BH * N);
   int* pidx = c.take<int>(BH * std::max(r.M, 1)); float* pw = c.take<float>(BH * std::max(r.M, 1));
@@ -299,7 +302,7 @@ void carve_plan(Carver& c, const Resolved& r, sparsepr_plan_s* p) {
   __nv_bfloat16* mw = c.take<__nv_bfloat16>(BH * (size_t)km_padded(r.Cmax) * 8);
   float* xnorm = c.take<float>(BH * N); int* flagged = c.take<int>(BH * N);
   __nv_bfloat16* Ft = c.take<__nv_bfloat16>(BH * (size_t)3 * 64 * 128);
-  int* rem_pos = c.take<int>(BH * N); int* rem_grp = c.take<int>(BH * N); int* rem_cnt = c.take<int>(BH);
+  int* rem_pos = c.take<int>(f32 ? 0 : BH * N); int* rem_grp = c.take<int>(f32 ? 0 : BH * N); int* rem_cnt = c.take<int>(f32 ? 0 : BH);
   int* km_changed = c.take<int>(2 * (size_t)(r.T + 1) * BH);
   int* flagcnt = c.take<int>(2 * BH);                       // two sets of per-head counters, used by alternate passes
   double* eigws = c.take<double>(eig_scratch_doubles((int)BH, r.d));
@@ -311,7 +314,18 @@ void carve_plan(Carver& c, const Resolved& r, sparsepr_plan_s* p) {
     p->a_K = aK; p->a_Q = aQ; p->kv_perm = kvp; p->kv_inv = kvi; p->q_perm = qp; p->q_inv = qi; p->kv_off = kvo; p->q_off = qo;
     p->nk = nk; p->nq = nq; p->kappa = kappa; p->theta = theta; p->score = score; p->route_ptr = rptr; p->route_idx = ridx;
     p->xh = xh; p->xl = xl; p->mh = mh; p->ml = ml; p->mw = mw; p->xnorm = xnorm; p->flagged = flagged;
-    p->tile_off = toff; p->tile_off128 = toff128; p->rstate = rs; p->probe_dist = pd; p->probe_idx = pidx; p->probe_w = pw;
+    p->tile_off128 = toff128; p->f32_items = items; p->f32_keys = ikeys; p->f32_count = icount; p->rstate = rs; p->probe_dist = pd; p->probe_idx = pidx; p->probe_w = pw;
+  }
+}
+
+// the attention kernels' tiles of a plan with routes
+void launch_tiles(const sparsepr_plan_s* p, cudaStream_t st) {
+  const Resolved& r = p->r;
+  if (r.dtype == SPARSEPR_F32) {
+    launch_f32_items(p->q_off, p->kv_off, p->route_ptr, p->route_idx, r.BH, r.N, r.Cq, r.Ck, p->f32_keys, p->f32_items, p->f32_count, st);
+  } else {
+    launch_tile_offsets(p->q_off, r.BH, r.Cq, 128, kRemRows, p->tile_off128, st);
+    launch_remainder_rows(p->q_off, p->route_ptr, p->route_idx, r.BH, r.Cq, r.Ck, r.N, p->rem_pos, p->rem_grp, p->rem_cnt, st);
   }
 }
 
@@ -354,7 +368,7 @@ void carve_attend(Carver& c, const Resolved& r, AttendWs* w) {
   __nv_bfloat16* At = c.take<__nv_bfloat16>(2 * BH * d * d);   // the correction map as two bf16 words
   const bool f32 = r.dtype == SPARSEPR_F32;
   float* fpart = c.take<float>(f32 ? attention_f32_part_floats(r.BH, r.N, r.Cq, r.d) : 0);
-  int* fcount = c.take<int>(f32 ? attention_f32_counters(r.BH, r.N, r.Cq) : 0);
+  int* fcount = c.take<int>(f32 ? attention_f32_items(r.BH, r.N, r.Cq) : 0);
   double* fit = c.take<double>(fit_scratch_doubles(r.BH, (int)M1, r.d));
   double* fit_eigws = c.take<double>(eig_scratch_doubles(r.BH, r.d));
   if (w) { w->fpart = fpart; w->fcount = fcount; w->Olo = Olo; w->Qg = Qg; w->Kg = Kg; w->Vg = Vg; w->partial = partial; w->X = X; w->Dn = Dn; w->A = A; w->c = cc; w->Psi = Psi; w->At = At; w->Qp = Qp; w->n_split_tc = ns_tc; w->fit = fit; w->fit_eigws = fit_eigws; w->n_split = ns; }
@@ -580,9 +594,7 @@ static sparsepr_status_t plan_impl(const sparsepr_shape_t* shape, const sparsepr
   launch_cell_scores(p->theta, p->kappa, p->nq, p->nk, r.BH, r.Cq, r.Ck, r.d, r.scale, p->score, r.G, st);
   launch_route_select(p->score, p->nq, p->nk, r.BH, r.Cq, r.Ck, pair_budget(r), r.density >= 1.0f, p->route_ptr,
                       p->route_idx, p->rstate, nullptr, r.G, st);
-  launch_tile_offsets(p->q_off, r.BH, r.Cq, 64, 0, p->tile_off, st);
-  launch_tile_offsets(p->q_off, r.BH, r.Cq, 128, kRemRows, p->tile_off128, st);
-  launch_remainder_rows(p->q_off, p->route_ptr, p->route_idx, r.BH, r.Cq, r.Ck, r.N, p->rem_pos, p->rem_grp, p->rem_cnt, st);
+  launch_tiles(p, st);
   if (overlap) p->side_pending = true;          // not joined here: the probes are not needed before the attend call
   tm.mark(SPARSEPR_STAGE_ROUTE);
   tm.finish();
@@ -649,9 +661,7 @@ sparsepr_status_t sparsepr_plan_import(const sparsepr_shape_t* shape, const spar
   k_sizes_from_off<<<dim3((r.Ck + 255) / 256, r.BHkv), 256, 0, st>>>(p->kv_off, r.Ck, p->nk);
   k_sizes_from_off<<<dim3((r.Cq + 255) / 256, r.BH), 256, 0, st>>>(p->q_off, r.Cq, p->nq);
   launch_count_pairs(p->q_off, p->kv_off, p->route_ptr, p->route_idx, r.BH, r.Cq, r.Ck, p->rstate, r.G, st);
-  launch_tile_offsets(p->q_off, r.BH, r.Cq, 64, 0, p->tile_off, st);
-  launch_tile_offsets(p->q_off, r.BH, r.Cq, 128, kRemRows, p->tile_off128, st);
-  launch_remainder_rows(p->q_off, p->route_ptr, p->route_idx, r.BH, r.Cq, r.Ck, r.N, p->rem_pos, p->rem_grp, p->rem_cnt, st);
+  launch_tiles(p, st);
   if (!launch_ok() || cudaStreamSynchronize(st) != cudaSuccess) { delete p; return SPARSEPR_ERR_CUDA; }
   *out = p;
   return SPARSEPR_OK;
@@ -683,7 +693,7 @@ static sparsepr_status_t attend_impl(const sparsepr_plan_t* p, const void* Q, co
   aa.dtype = r.dtype; aa.BH = r.BH; aa.H = r.H; aa.N = r.N; aa.d = r.d; aa.scale = r.scale;
   aa.Q = w.Qg; aa.K = w.Kg; aa.V = w.Vg;
   aa.q_off = p->q_off; aa.kv_off = p->kv_off; aa.route_ptr = p->route_ptr; aa.route_idx = p->route_idx;
-  aa.q_perm = p->q_perm; aa.tile_off = p->tile_off; aa.Cq = r.Cq; aa.Ck = r.Ck; aa.kv_div = r.G;
+  aa.q_perm = p->q_perm; aa.tile_off = p->tile_off128; aa.Cq = r.Cq; aa.Ck = r.Ck; aa.kv_div = r.G;
   aa.O = O; for (int i = 0; i < 3; ++i) aa.os[i] = r.os[i];
   aa.O_sparse = O_sparse;
   aa.err = p->err;
@@ -718,7 +728,6 @@ static sparsepr_status_t attend_impl(const sparsepr_plan_t* p, const void* Q, co
     tm.mark(SPARSEPR_STAGE_FIT);
   }
   if (tensor) {
-    aa.tile_off = p->tile_off128;
     // with a correction to follow, the block-sparse kernels also store what the bf16 rounding of O dropped
     if (fitted) aa.O_lo = w.Olo;
     // the packed remainder tiles are few and long, the 128-row tiles many and short: they share the GPU instead of
@@ -734,6 +743,7 @@ static sparsepr_status_t attend_impl(const sparsepr_plan_t* p, const void* Q, co
     if (fitted && !launch_correction_tc(w.c, w.At, w.Olo, O, r.os, r.BH, r.H, r.N, r.d, p->err, st)) return SPARSEPR_ERR_CUDA;
     tm.mark(SPARSEPR_STAGE_CORRECTION);
   } else {
+    aa.items = p->f32_items; aa.n_items = p->f32_count;
     launch_attention_f32(aa, w.fpart, w.fcount, st);
     tm.mark(SPARSEPR_STAGE_ATTENTION);
     if (overlap) { join_side(p, st); p->side_pending = false; }
@@ -835,7 +845,8 @@ sparsepr_status_t sparsepr_plan_stats(const sparsepr_plan_t* p, sparsepr_stats_t
     out->nonempty_kv_groups_min = std::min(out->nonempty_kv_groups_min, neK);
     out->nonempty_q_groups_min = std::min(out->nonempty_q_groups_min, neQ);
     // pairs issued by the tiled kernel over the concatenated routed keys: the tensor-core kernel uses
-    // 128-row query tiles and 128-key tiles built from 16-row boxes, the float32 kernel 64 x 64 tiles
+    // 128-row query tiles and 128-key tiles built from 16-row boxes, the float32 kernel equal tiles of up to 64 rows, done in
+    // eighths, and 64 keys
     const bool tcpath = r.dtype == SPARSEPR_BF16;
     const int qtile = tcpath ? 128 : 64, ktile = tcpath ? 128 : 64, box = tcpath ? 16 : 1;
     const int* rpp = &rp[(size_t)bh * (r.Cq + 1)];
@@ -862,7 +873,8 @@ sparsepr_status_t sparsepr_plan_stats(const sparsepr_plan_t* p, sparsepr_stats_t
         const int n = rpp[a + 1] - rpp[a];
         packed_order.push_back(((unsigned long long)(r.Ck - n) << 24) | ((unsigned long long)(n > 0 ? rii[rpp[a]] : 0) << 12) | (unsigned long long)a);
       } else {
-        out->padded_tile_pairs += (i64)((nrow + qtile - 1) / qtile) * qtile * kt * ktile;
+        const int nt = (nrow + qtile - 1) / qtile, rows = nt ? (nrow + nt - 1) / nt : 0;
+        out->padded_tile_pairs += (i64)nt * (tcpath ? qtile : std::max(16, (rows + 7) / 8 * 8)) * kt * ktile;
       }
     }
     std::sort(packed_order.begin(), packed_order.end());

@@ -104,23 +104,21 @@ __device__ __forceinline__ float row16_sum(float v) {
 }
 
 // =============================================================================
-// Main kernel.  SPARSE: one CTA per 64-row tile of one query group; the keys of the routed K/V groups are streamed as one
-// concatenated sequence (every tile of 64 keys is full except the last).  Dense: one CTA per 64 rows over all keys.
-// Stores the hard-drop output at the original token index; the correction is a pass of its own, so that the probe rows and
-// the fit can run beside this kernel.
+// Main kernel.  SPARSE: one CTA per item of a list (below): up to 64 rows of one query group against the keys of its routed
+// K/V groups, streamed as one concatenated sequence (every tile of 64 keys is full except the last), or against a part of
+// them.  Dense: one CTA per 64 rows over all keys.  Stores the hard-drop output at the original token index; the correction
+// is a pass of its own, so that the probe rows and the fit can run beside this kernel.
 //
-// Bound by the FMA pipe: 128 threads, two CTAs per SM, thread (ty, tx) holds 8 query rows x 4 keys of the scores and
-// 8 rows x D / 16 columns of the output, so that a 16-byte shared-memory read serves 8 to 32 multiply-adds, and all of
+// Bound by the FMA pipe: 128 threads, two CTAs per SM, thread (ty, tx) holds R query rows x 4 keys of the scores and
+// R rows x D / 16 columns of the output, so that a 16-byte shared-memory read serves 8 to 32 multiply-adds, and all of
 // them are packed two to an instruction (scores: even and odd dimensions in separate halves; output: column pairs).
 // Rows are 16 bytes longer than their data, which keeps the 16-byte reads of consecutive rows in different banks.  The
-// probabilities take the place of the K tile.  Tiles arrive by cp.async; the other CTA of the SM covers their latency.
-// F32_MEASURED
-//
-// A grid with few tiles leaves SMs idle, and groups that route to many keys then set the duration: with n_split > 1 the
-// key sequence of a tile is cut into up to n_split parts of at least kMinSplitTiles key tiles, one CTA each; every part
-// leaves (m, l, O) in `part`, and the CTA that finishes last (a counter per tile) adds them up in the order of the parts.
+// probabilities take the place of the K tile.  Tiles arrive by cp.async, V under the scores; the other CTA of the SM covers
+// the latency of K.
+// 8 heads, 7161 tokens, d = 128, routed density 0.24: 4040 us with 256 threads and blocks of 4 x 4 single multiply-adds, 2640 us
+// with packed 8 x 4 blocks, 1610 us with equal row tiles, parts and descending order; dense 47 of the 74 TFLOP/s of the pipe.
 // =============================================================================
-constexpr int kFThreads = 128, kMinSplitTiles = 4;
+constexpr int kFThreads = 128;
 template <int D> struct F32Smem {
   static constexpr int ld = D + 4, ldp = BM + 4;
   static constexpr int q = BM * ld, k = BN * ld, v = BN * D;
@@ -133,63 +131,33 @@ __device__ __forceinline__ void cp16(float* dst, const float* src, bool on) {   
   asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(d), "l"(src), "r"(n) : "memory");
 }
 
-template <int D, bool SPARSE>
-__global__ void __launch_bounds__(kFThreads, 2) k_attention_f32(AttnArgs a, int n_split, float* __restrict__ part, int* __restrict__ counter) {
+// what a CTA works on: rows row0 .. row0 + nrows of head bh against key tiles [t_begin, t_end) of L keys
+struct F32Work {
+  int bh, row0, nrows, L, t_begin, t_end, z, parts, slot, nroute;
+  const int *ridx, *kvoff;                               // routed groups and group offsets of the head (SPARSE)
+  const float *Qb, *Kb, *Vb;
+  i64 qsn, ksn, vsn;
+};
+
+// R: rows per thread, ceil(nrows / 8).  Row ty R + i of the tile sits in row ty 8 + i of the shared-memory tiles, so that all R share
+// one layout with aligned 16-byte rows.
+template <int D, bool SPARSE, int R>
+__device__ __forceinline__ void attend_f32(const AttnArgs& a, const F32Work& w, float* smem, const int* cum, int* scratch, float* __restrict__ part,
+                                           int* __restrict__ counter) {
   using S = F32Smem<D>;
-  extern __shared__ __align__(16) float smem[];
   float* Qs = smem;                                      // [64][D + 4]
   float* Ks = Qs + S::q;                                 // [64][D + 4], then P [64 keys][64 rows + 4]
   float* Vs = Ks + S::k;                                 // [64][D]
   int* krow = reinterpret_cast<int*>(Vs + S::v);         // [2][64] source row of every key of this / the next tile
-  __shared__ int cum[SPARSE ? kMaxGroups + 1 : 1];
-  __shared__ int scratch[34];
   constexpr int OP = D / 32;                             // output column pairs per thread: columns 4 tx + 64 c + {0..3}
-  const int bh = blockIdx.y, b = bh / a.H, h = bh % a.H;
-  const int tid = threadIdx.x, ty = tid >> 4, tx = tid & 15;
-
-  int row0, nrows, nroute = 0, L;
-  const int* ridx = nullptr;
-  const int* kvoff = nullptr;
-  const float *Qb, *Kb, *Vb;
-  i64 qsn, ksn, vsn;
-  if (SPARSE) {
-    const int* toff = a.tile_off + (i64)bh * (a.Cq + 1);
-    if ((int)blockIdx.x >= toff[a.Cq]) return;
-    int lo = 0, hi = a.Cq - 1;                      // last group g with toff[g] <= blockIdx.x
-    while (lo < hi) { const int mid = (lo + hi + 1) >> 1; if (toff[mid] <= (int)blockIdx.x) lo = mid; else hi = mid - 1; }
-    const int g = lo;
-    const int* qoff = a.q_off + (i64)bh * (a.Cq + 1);
-    row0 = qoff[g] + ((int)blockIdx.x - toff[g]) * BM;
-    nrows = min(BM, qoff[g + 1] - row0);
-    const int* rp = a.route_ptr + (i64)bh * (a.Cq + 1);
-    ridx = a.route_idx + (i64)bh * a.Cq * a.Ck + rp[g];
-    nroute = rp[g + 1] - rp[g];
-    kvoff = a.kv_off + (i64)bh * (a.Ck + 1);
-    for (int t = tid; t < nroute; t += kFThreads) { const int bb = ridx[t]; cum[t] = kvoff[bb + 1] - kvoff[bb]; }
-    __syncthreads();
-    L = block_exclusive_scan(cum, nroute, scratch);
-    if (tid == 0) cum[nroute] = L;
-    Qb = (const float*)a.Q + (i64)bh * a.N * D; Kb = (const float*)a.K + (i64)bh * a.N * D; Vb = (const float*)a.V + (i64)bh * a.N * D;
-    qsn = ksn = vsn = D;
-  } else {
-    row0 = blockIdx.x * BM;
-    nrows = min(BM, a.N - row0);
-    L = a.N;
-    Qb = (const float*)a.Q + b * a.qs[0] + h * a.qs[1]; Kb = (const float*)a.K + b * a.ks[0] + h * a.ks[1];
-    Vb = (const float*)a.V + b * a.vs[0] + h * a.vs[1];
-    qsn = a.qs[2]; ksn = a.ks[2]; vsn = a.vs[2];
-  }
-  // this CTA's part of the key tiles
-  const int n_tiles = (L + BN - 1) / BN;
-  const int parts = max(1, min(n_split, n_tiles / kMinSplitTiles)), z = blockIdx.z;
-  if (z >= parts) return;
-  const int t_begin = (int)((i64)n_tiles * z / parts), t_end = (int)((i64)n_tiles * (z + 1) / parts);
-
   constexpr int CPR = D / 4;                             // 16-byte chunks per row
+  constexpr int RV = (R + 3) / 4;                        // 16-byte pieces of a thread's probabilities of one key
+  const int tid = threadIdx.x, ty = tid >> 4, tx = tid & 15;
+  const int L = w.L;
 #pragma unroll 4
-  for (int e = tid; e < BM * CPR; e += kFThreads) {
+  for (int e = tid; e < 8 * R * CPR; e += kFThreads) {
     const int r = e / CPR, c = (e % CPR) * 4;
-    cp16(Qs + r * S::ld + c, Qb + (i64)(row0 + min(r, nrows - 1)) * qsn + c, r < nrows);
+    cp16(Qs + (r / R * 8 + r % R) * S::ld + c, w.Qb + (i64)(w.row0 + min(r, w.nrows - 1)) * w.qsn + c, r < w.nrows);
   }
   auto find_rows = [&](int t, int* dst) {                // source rows of key tile t
     if (tid < BN) {
@@ -197,46 +165,50 @@ __global__ void __launch_bounds__(kFThreads, 2) k_attention_f32(AttnArgs a, int 
       int src = -1;
       if (pos < L) {
         if (SPARSE) {
-          int lo = 0, hi = nroute - 1;                   // last range with cum[range] <= pos
+          int lo = 0, hi = w.nroute - 1;                 // last range with cum[range] <= pos
           while (lo < hi) { const int mid = (lo + hi + 1) >> 1; if (cum[mid] <= pos) lo = mid; else hi = mid - 1; }
-          src = kvoff[ridx[lo]] + (pos - cum[lo]);
+          src = w.kvoff[w.ridx[lo]] + (pos - cum[lo]);
         } else src = pos;
       }
       dst[tid] = src;
     }
   };
-  __syncthreads();                                       // cum[] is complete
-  find_rows(t_begin, krow);
+  find_rows(w.t_begin, krow);
 
-  float2 o[8][OP];
-  float m[8], l[8];
+  float2 o[R][OP];
+  float m[R], l[R];
 #pragma unroll
-  for (int i = 0; i < 8; ++i) {
+  for (int i = 0; i < R; ++i) {
     m[i] = -INFINITY; l[i] = 0.f;
 #pragma unroll
     for (int c = 0; c < OP; ++c) o[i][c] = make_float2(0.f, 0.f);
   }
   const float sc = a.scale * kLog2e;
-  for (int t = t_begin; t < t_end; ++t) {
-    const int* kr = krow + ((t - t_begin) & 1) * BN;
+  for (int t = w.t_begin; t < w.t_end; ++t) {
+    const int* kr = krow + ((t - w.t_begin) & 1) * BN;
     const int ncols = min(BN, L - t * BN);
     __syncthreads();                                     // previous tile fully consumed, rows of this one known
-#pragma unroll 4
+#pragma unroll 8
     for (int e = tid; e < BN * CPR; e += kFThreads) {
       const int r = e / CPR, c = (e % CPR) * 4, src = kr[r];
-      cp16(Ks + r * S::ld + c, Kb + (i64)max(src, 0) * ksn + c, src >= 0);
-      cp16(Vs + r * D + c, Vb + (i64)max(src, 0) * vsn + c, src >= 0);
+      cp16(Ks + r * S::ld + c, w.Kb + (i64)max(src, 0) * w.ksn + c, src >= 0);
     }
     asm volatile("cp.async.commit_group;" ::: "memory");
-    if (t + 1 < t_end) find_rows(t + 1, krow + ((t + 1 - t_begin) & 1) * BN);
-    asm volatile("cp.async.wait_group 0;" ::: "memory");
+#pragma unroll 8
+    for (int e = tid; e < BN * CPR; e += kFThreads) {
+      const int r = e / CPR, c = (e % CPR) * 4, src = kr[r];
+      cp16(Vs + r * D + c, w.Vb + (i64)max(src, 0) * w.vsn + c, src >= 0);
+    }
+    asm volatile("cp.async.commit_group;" ::: "memory");
+    if (t + 1 < w.t_end) find_rows(t + 1, krow + ((t + 1 - w.t_begin) & 1) * BN);
+    asm volatile("cp.async.wait_group 1;" ::: "memory"); // Q and K
     __syncthreads();
-    // scores of rows 8 ty + i and keys tx + 16 j
-    float s[8][4];
+    // scores of rows ty R + i and keys tx + 16 j
+    float s[R][4];
     {
-      float2 acc[8][4];
+      float2 acc[R][4];
 #pragma unroll
-      for (int i = 0; i < 8; ++i)
+      for (int i = 0; i < R; ++i)
 #pragma unroll
         for (int j = 0; j < 4; ++j) acc[i][j] = make_float2(0.f, 0.f);
       const float* qp = Qs + ty * 8 * S::ld;
@@ -246,24 +218,27 @@ __global__ void __launch_bounds__(kFThreads, 2) k_attention_f32(AttnArgs a, int 
         float4 kk[4];
 #pragma unroll
         for (int j = 0; j < 4; ++j) kk[j] = *reinterpret_cast<const float4*>(kp + 16 * j * S::ld + k);
+        float4 q[R];
 #pragma unroll
-        for (int i = 0; i < 8; ++i) {
-          const float4 q = *reinterpret_cast<const float4*>(qp + i * S::ld + k);
+        for (int i = 0; i < R; ++i) q[i] = *reinterpret_cast<const float4*>(qp + i * S::ld + k);
 #pragma unroll
-          for (int j = 0; j < 4; ++j) {
-            acc[i][j] = __ffma2_rn(make_float2(q.x, q.y), make_float2(kk[j].x, kk[j].y), acc[i][j]);
-            acc[i][j] = __ffma2_rn(make_float2(q.z, q.w), make_float2(kk[j].z, kk[j].w), acc[i][j]);
-          }
-        }
+        for (int i = 0; i < R; ++i)
+#pragma unroll
+          for (int j = 0; j < 4; ++j) acc[i][j] = __ffma2_rn(make_float2(q[i].x, q[i].y), make_float2(kk[j].x, kk[j].y), acc[i][j]);
+#pragma unroll
+        for (int i = 0; i < R; ++i)
+#pragma unroll
+          for (int j = 0; j < 4; ++j) acc[i][j] = __ffma2_rn(make_float2(q[i].z, q[i].w), make_float2(kk[j].z, kk[j].w), acc[i][j]);
       }
 #pragma unroll
-      for (int i = 0; i < 8; ++i)
+      for (int i = 0; i < R; ++i)
 #pragma unroll
         for (int j = 0; j < 4; ++j) s[i][j] = tx + 16 * j < ncols ? (acc[i][j].x + acc[i][j].y) * sc : -INFINITY;
     }
+    asm volatile("cp.async.wait_group 0;" ::: "memory"); // V
     __syncthreads();                                     // K is consumed: its place takes the probabilities
 #pragma unroll
-    for (int i = 0; i < 8; ++i) {
+    for (int i = 0; i < R; ++i) {
       const float mx = row16_max(fmaxf(fmaxf(s[i][0], s[i][1]), fmaxf(s[i][2], s[i][3])));
       const float mn = fmaxf(m[i], mx);
       const float corr = exp2f(m[i] - mn);               // 0 on the first tile (m = -inf)
@@ -280,19 +255,25 @@ __global__ void __launch_bounds__(kFThreads, 2) k_attention_f32(AttnArgs a, int 
 #pragma unroll
     for (int j = 0; j < 4; ++j) {
       float* pp = Ps + (tx + 16 * j) * S::ldp + ty * 8;
-      *reinterpret_cast<float4*>(pp) = make_float4(s[0][j], s[1][j], s[2][j], s[3][j]);
-      *reinterpret_cast<float4*>(pp + 4) = make_float4(s[4][j], s[5][j], s[6][j], s[7][j]);
+#pragma unroll
+      for (int u = 0; u < RV; ++u)
+        *reinterpret_cast<float4*>(pp + 4 * u) = make_float4(s[4 * u][j], 4 * u + 1 < R ? s[min(4 * u + 1, R - 1)][j] : 0.f,
+                                                             4 * u + 2 < R ? s[min(4 * u + 2, R - 1)][j] : 0.f, 4 * u + 3 < R ? s[min(4 * u + 3, R - 1)][j] : 0.f);
     }
     __syncthreads();
 #pragma unroll 4
     for (int j = 0; j < ncols; ++j) {
-      const float4 p0 = *reinterpret_cast<const float4*>(Ps + j * S::ldp + ty * 8), p1 = *reinterpret_cast<const float4*>(Ps + j * S::ldp + ty * 8 + 4);
-      const float pv[8] = {p0.x, p0.y, p0.z, p0.w, p1.x, p1.y, p1.z, p1.w};
+      float pv[4 * RV];
+#pragma unroll
+      for (int u = 0; u < RV; ++u) {
+        const float4 p = *reinterpret_cast<const float4*>(Ps + j * S::ldp + ty * 8 + 4 * u);
+        pv[4 * u] = p.x; pv[4 * u + 1] = p.y; pv[4 * u + 2] = p.z; pv[4 * u + 3] = p.w;
+      }
 #pragma unroll
       for (int c = 0; c < OP / 2; ++c) {
         const float4 v = *reinterpret_cast<const float4*>(Vs + j * D + 64 * c + 4 * tx);
 #pragma unroll
-        for (int i = 0; i < 8; ++i) {
+        for (int i = 0; i < R; ++i) {
           const float2 pp = make_float2(pv[i], pv[i]);
           o[i][2 * c] = __ffma2_rn(pp, make_float2(v.x, v.y), o[i][2 * c]);
           o[i][2 * c + 1] = __ffma2_rn(pp, make_float2(v.z, v.w), o[i][2 * c + 1]);
@@ -301,13 +282,12 @@ __global__ void __launch_bounds__(kFThreads, 2) k_attention_f32(AttnArgs a, int 
     }
   }
 #pragma unroll
-  for (int i = 0; i < 8; ++i) l[i] = row16_sum(l[i]);
-  if (parts > 1) {
-    const i64 slot = ((i64)bh * gridDim.x + blockIdx.x) * n_split;
-    float* mine = part + (slot + z) * BM * (D + 2);
+  for (int i = 0; i < R; ++i) l[i] = row16_sum(l[i]);
+  if (SPARSE && w.parts > 1) {
+    float* mine = part + (i64)(w.slot + w.z) * BM * (D + 2);
 #pragma unroll
-    for (int i = 0; i < 8; ++i) {
-      const int r = ty * 8 + i;
+    for (int i = 0; i < R; ++i) {
+      const int r = ty * R + i;
       if (tx == 0) { mine[r] = m[i]; mine[BM + r] = l[i]; }
 #pragma unroll
       for (int c = 0; c < OP / 2; ++c)
@@ -315,46 +295,166 @@ __global__ void __launch_bounds__(kFThreads, 2) k_attention_f32(AttnArgs a, int 
     }
     __threadfence();
     __syncthreads();
-    if (tid == 0) scratch[0] = atomicAdd(counter + (i64)bh * gridDim.x + blockIdx.x, 1);
+    if (tid == 0) scratch[0] = atomicAdd(counter + w.slot, 1);
     __syncthreads();
-    if (scratch[0] != parts - 1) return;
+    if (scratch[0] != w.parts - 1) return;
     __threadfence();
 #pragma unroll
-    for (int i = 0; i < 8; ++i) {
-      const int r = ty * 8 + i;
+    for (int i = 0; i < R; ++i) {
+      const int r = ty * R + i;
       float mm = -INFINITY;
-      for (int q = 0; q < parts; ++q) mm = fmaxf(mm, part[(slot + q) * BM * (D + 2) + r]);
+      for (int q = 0; q < w.parts; ++q) mm = fmaxf(mm, part[(i64)(w.slot + q) * BM * (D + 2) + r]);
       m[i] = mm; l[i] = 0.f;
 #pragma unroll
       for (int c = 0; c < OP; ++c) o[i][c] = make_float2(0.f, 0.f);
-      for (int q = 0; q < parts; ++q) {
-        const float* pq = part + (slot + q) * BM * (D + 2);
-        const float w = exp2f(pq[r] - mm);
-        l[i] = fmaf(w, pq[BM + r], l[i]);
+      for (int q = 0; q < w.parts; ++q) {
+        const float* pq = part + (i64)(w.slot + q) * BM * (D + 2);
+        const float f = exp2f(pq[r] - mm);
+        l[i] = fmaf(f, pq[BM + r], l[i]);
 #pragma unroll
         for (int c = 0; c < OP / 2; ++c) {
           const float4 v = *reinterpret_cast<const float4*>(pq + 2 * BM + r * D + 64 * c + 4 * tx);
-          o[i][2 * c] = __ffma2_rn(make_float2(w, w), make_float2(v.x, v.y), o[i][2 * c]);
-          o[i][2 * c + 1] = __ffma2_rn(make_float2(w, w), make_float2(v.z, v.w), o[i][2 * c + 1]);
+          o[i][2 * c] = __ffma2_rn(make_float2(f, f), make_float2(v.x, v.y), o[i][2 * c]);
+          o[i][2 * c + 1] = __ffma2_rn(make_float2(f, f), make_float2(v.z, v.w), o[i][2 * c + 1]);
         }
       }
     }
   }
   // ---- epilogue -------------------------------------------------------------------
-  float* Ob = (float*)a.O + b * a.os[0] + h * a.os[1];
+  float* Ob = (float*)a.O + w.bh / a.H * a.os[0] + w.bh % a.H * a.os[1];
 #pragma unroll
-  for (int i = 0; i < 8; ++i) {
-    const int r = ty * 8 + i;
-    if (r >= nrows) continue;
+  for (int i = 0; i < R; ++i) {
+    const int r = ty * R + i;
+    if (r >= w.nrows) continue;
     const float inv = l[i] > 0.f ? 1.f / l[i] : 0.f;
-    const int dst = SPARSE ? a.q_perm[(i64)bh * a.N + row0 + r] : row0 + r;
+    const int dst = SPARSE ? a.q_perm[(i64)w.bh * a.N + w.row0 + r] : w.row0 + r;
 #pragma unroll
     for (int c = 0; c < OP / 2; ++c) {
       const float4 v = make_float4(o[i][2 * c].x * inv, o[i][2 * c].y * inv, o[i][2 * c + 1].x * inv, o[i][2 * c + 1].y * inv);
       *reinterpret_cast<float4*>(Ob + (i64)dst * a.os[2] + 64 * c + 4 * tx) = v;
-      if (a.O_sparse) *reinterpret_cast<float4*>(a.O_sparse + ((i64)bh * a.N + dst) * D + 64 * c + 4 * tx) = v;
+      if (a.O_sparse) *reinterpret_cast<float4*>(a.O_sparse + ((i64)w.bh * a.N + dst) * D + 64 * c + 4 * tx) = v;
     }
   }
+}
+
+template <int D>
+__global__ void __launch_bounds__(kFThreads, 2) k_attention_f32_sparse(AttnArgs a, float* __restrict__ part, int* __restrict__ counter) {
+  extern __shared__ __align__(16) float smem[];
+  __shared__ int cum[kMaxGroups + 1];
+  __shared__ int scratch[34];
+  if ((int)blockIdx.x >= *a.n_items) return;
+  const int4 it = a.items[blockIdx.x];
+  F32Work w;
+  w.bh = it.x / a.Cq; w.row0 = it.y; w.nrows = it.z & 0xFF; w.z = (it.z >> 8) & 0xFF; w.parts = it.z >> 16; w.slot = it.w;
+  const int g = it.x % a.Cq;
+  const int* rp = a.route_ptr + (i64)w.bh * (a.Cq + 1);
+  w.ridx = a.route_idx + (i64)w.bh * a.Cq * a.Ck + rp[g];
+  w.nroute = rp[g + 1] - rp[g];
+  w.kvoff = a.kv_off + (i64)w.bh * (a.Ck + 1);
+  for (int t = threadIdx.x; t < w.nroute; t += kFThreads) { const int bb = w.ridx[t]; cum[t] = w.kvoff[bb + 1] - w.kvoff[bb]; }
+  __syncthreads();
+  w.L = block_exclusive_scan(cum, w.nroute, scratch);    // ends with a barrier
+  const i64 base = (i64)w.bh * a.N * D;
+  w.Qb = (const float*)a.Q + base; w.Kb = (const float*)a.K + base; w.Vb = (const float*)a.V + base;
+  w.qsn = w.ksn = w.vsn = D;
+  const int n_tiles = (w.L + BN - 1) / BN;
+  w.t_begin = (int)((i64)n_tiles * w.z / w.parts); w.t_end = (int)((i64)n_tiles * (w.z + 1) / w.parts);
+  switch ((w.nrows + 7) >> 3) {
+    case 1: case 2: attend_f32<D, true, 2>(a, w, smem, cum, scratch, part, counter); break;
+    case 3: attend_f32<D, true, 3>(a, w, smem, cum, scratch, part, counter); break;
+    case 4: attend_f32<D, true, 4>(a, w, smem, cum, scratch, part, counter); break;
+    case 5: attend_f32<D, true, 5>(a, w, smem, cum, scratch, part, counter); break;
+    case 6: attend_f32<D, true, 6>(a, w, smem, cum, scratch, part, counter); break;
+    case 7: attend_f32<D, true, 7>(a, w, smem, cum, scratch, part, counter); break;
+    default: attend_f32<D, true, 8>(a, w, smem, cum, scratch, part, counter);
+  }
+}
+template <int D>
+__global__ void __launch_bounds__(kFThreads, 2) k_attention_f32_dense(AttnArgs a) {
+  extern __shared__ __align__(16) float smem[];
+  F32Work w;
+  w.bh = blockIdx.y; w.row0 = blockIdx.x * BM; w.nrows = min(BM, a.N - w.row0); w.L = a.N;
+  w.t_begin = 0; w.t_end = (w.L + BN - 1) / BN; w.parts = 1;
+  const int b = w.bh / a.H, h = w.bh % a.H;
+  w.Qb = (const float*)a.Q + b * a.qs[0] + h * a.qs[1]; w.Kb = (const float*)a.K + b * a.ks[0] + h * a.ks[1];
+  w.Vb = (const float*)a.V + b * a.vs[0] + h * a.vs[1];
+  w.qsn = a.qs[2]; w.ksn = a.ks[2]; w.vsn = a.vs[2];
+  attend_f32<D, false, 8>(a, w, smem, nullptr, nullptr, nullptr, nullptr);
+}
+
+// ---- the list of items: which rows and keys, longest first ---------------------------
+// The groups of a plan differ by more than ten times in rows and in routed keys.  A group's rows are cut into tiles of equal
+// size, at most 64 rows, whose CTA does the work of 8 ceil(rows / 8) rows; the keys of a tile are cut into parts of about
+// `chunk` key tiles; the items are issued in descending order of their work, so that no long one is left for the end.
+// Every part of a cut tile leaves (m, l, O) in `part`, and the CTA that finishes last (a counter per tile) adds them up in
+// the order of the parts.  The chunk is the smallest of the series 4, 6, 8, 12, 16, 24 ... that gives at most max_items items
+// (attention_f32_items): fine enough for a small list to fill the GPU, and for the kernels of the probes and the fit to find
+// free slots beside a large one (they would wait for the longest items of the first wave), coarse enough that the parts
+// cost little.
+__global__ void __launch_bounds__(1024) k_route_keys(const int* __restrict__ kv_off, const int* __restrict__ route_ptr, const int* __restrict__ route_idx, int Cq,
+                                                     int Ck, int* __restrict__ keys) {
+  const int bh = blockIdx.y, g = blockIdx.x * 32 + (threadIdx.x >> 5);
+  if (g >= Cq) return;
+  const int* rp = route_ptr + (i64)bh * (Cq + 1);
+  const int* ri = route_idx + (i64)bh * Cq * Ck;
+  const int* ko = kv_off + (i64)bh * (Ck + 1);
+  int L = 0;
+  for (int t = rp[g] + (threadIdx.x & 31); t < rp[g + 1]; t += 32) { const int b = ri[t]; L += ko[b + 1] - ko[b]; }
+  L = warp_sum(L);
+  if ((threadIdx.x & 31) == 0) keys[(i64)bh * Cq + g] = L;
+}
+constexpr int kItemBuckets = 1024, kChunks = 15;
+__device__ __forceinline__ int item_chunk(int j) { return (j & 1 ? 6 : 4) << (j >> 1); }       // 4, 6, 8 .. 512
+__device__ __forceinline__ int item_parts(int nt, int j) {                                     // j = kChunks: whole
+  const int c = item_chunk(j);
+  return j < kChunks ? min(max((nt + c / 2) / c, 1), 255) : 1;
+}
+__global__ void __launch_bounds__(kItemBuckets) k_f32_items(const int* __restrict__ q_off, const int* __restrict__ keys, int BH, int Cq, int max_items, int shift,
+                                                            int4* __restrict__ items, int* __restrict__ n_items) {
+  __shared__ int hist[kItemBuckets];
+  __shared__ int scratch[34];
+  __shared__ int slots, sum[kChunks];
+  hist[threadIdx.x] = 0;
+  if (threadIdx.x == 0) slots = 0;
+  if (threadIdx.x < kChunks) sum[threadIdx.x] = 0;
+  __syncthreads();
+  int n_of[kChunks] = {}, first, n, tiles, rows, nt;
+  auto group = [&](int e) {
+    const int* qo = q_off + (i64)(e / Cq) * (Cq + 1) + e % Cq;
+    first = qo[0]; n = qo[1] - first;
+    tiles = (n + BM - 1) / BM; rows = n > 0 ? (n + tiles - 1) / tiles : 0; nt = (keys[e] + BN - 1) / BN;
+    return n > 0;
+  };
+  for (int e = threadIdx.x; e < BH * Cq; e += kItemBuckets)
+    if (group(e)) {
+#pragma unroll
+      for (int j = 0; j < kChunks; ++j) n_of[j] += tiles * item_parts(nt, j);
+    }
+#pragma unroll
+  for (int j = 0; j < kChunks; ++j) {
+    const int v = __reduce_add_sync(0xffffffffu, n_of[j]);
+    if ((threadIdx.x & 31) == 0) atomicAdd(&sum[j], v);
+  }
+  __syncthreads();
+  int j = 0;
+  while (j < kChunks && sum[j] > max_items) ++j;
+  int total = 0;
+  for (int pass = 0; pass < 2; ++pass) {
+    for (int e = threadIdx.x; e < BH * Cq; e += kItemBuckets) {
+      if (!group(e)) continue;
+      const int parts = item_parts(nt, j);
+      const int bucket = kItemBuckets - 1 - min(kItemBuckets - 1, (((nt + parts - 1) / parts + 1) * ((rows + 7) / 8 + 1)) >> shift);
+      int at = atomicAdd(&hist[bucket], tiles * parts);
+      if (pass == 0) continue;
+      const int slot = parts > 1 ? atomicAdd(&slots, tiles * parts) : 0;
+      for (int t = 0; t < tiles; ++t)
+        for (int z = 0; z < parts; ++z, ++at)
+          items[at] = make_int4(e, first + t * rows, min(rows, n - t * rows) | z << 8 | parts << 16, slot + t * parts);
+    }
+    __syncthreads();
+    if (pass == 0) total = block_exclusive_scan(hist, kItemBuckets, scratch);
+  }
+  if (threadIdx.x == 0) *n_items = total;
 }
 
 // Residual correction of Eq. 9 in place: O <- X + X A + c for the rows X = O (float32).  A CTA takes 32 rows of a head; A is
@@ -432,29 +532,25 @@ void launch_tile_offsets(const int* q_off, int BH, int Cq, int tile_rows, int sm
   k_tile_offsets<<<BH, 1024, 0, st>>>(q_off, Cq, tile_rows, small_rem, tile_off);
 }
 
-// Parts a tile's keys are cut into (float32): enough for about four rounds of CTAs on every SM slot, at most 8, none when the
-// tiles alone fill the GPU.
-int attention_f32_splits(int BH, int N, int Cq) {
-  const i64 tiles = (i64)BH * (N / BM + (Cq + 1) / 2);          // about: a group ends with half a tile
-  return (int)std::max<i64>(1, std::min<i64>(8, (i64)4 * 2 * sm_count() / std::max<i64>(tiles, 1)));
+// Items of a list at most: four rounds of CTAs on every SM slot, and twice as many as tiles.
+size_t attention_f32_items(int BH, int N, int Cq) { return std::max((size_t)4 * 2 * sm_count(), (size_t)2 * BH * ((N + BM - 1) / BM + Cq)); }
+size_t attention_f32_part_floats(int BH, int N, int Cq, int d) { return attention_f32_items(BH, N, Cq) * BM * (d + 2); }
+void launch_f32_items(const int* q_off, const int* kv_off, const int* route_ptr, const int* route_idx, int BH, int N, int Cq, int Ck, int* keys, int4* items,
+                      int* n_items, cudaStream_t st) {
+  k_route_keys<<<dim3((Cq + 31) / 32, BH), 1024, 0, st>>>(kv_off, route_ptr, route_idx, Cq, Ck, keys);
+  int shift = 0;
+  while ((((N + BN - 1) / BN + 1) * 9) >> shift >= kItemBuckets) ++shift;
+  k_f32_items<<<1, kItemBuckets, 0, st>>>(q_off, keys, BH, Cq, (int)attention_f32_items(BH, N, Cq), shift, items, n_items);
 }
-static i64 f32_tile_slots(int BH, int N, int Cq) { return (i64)BH * ((N + BM - 1) / BM + Cq); }
-size_t attention_f32_part_floats(int BH, int N, int Cq, int d) {
-  const int ns = attention_f32_splits(BH, N, Cq);
-  return ns > 1 ? (size_t)f32_tile_slots(BH, N, Cq) * ns * BM * (d + 2) : 0;
-}
-size_t attention_f32_counters(int BH, int N, int Cq) { return attention_f32_splits(BH, N, Cq) > 1 ? (size_t)f32_tile_slots(BH, N, Cq) : 0; }
 
 template <int D>
 static void attention_dispatch(const AttnArgs& a, float* part, int* counter, cudaStream_t st) {
-  if (a.route_ptr) {
-    const int ns = part ? attention_f32_splits(a.BH, a.N, a.Cq) : 1;
-    if (ns > 1) cudaMemsetAsync(counter, 0, attention_f32_counters(a.BH, a.N, a.Cq) * sizeof(int), st);
-    dim3 grid((a.N + BM - 1) / BM + a.Cq, a.BH, ns);
-    k_attention_f32<D, true><<<grid, kFThreads, F32Smem<D>::bytes, st>>>(a, ns, part, counter);
+  if (a.items) {
+    const unsigned items = (unsigned)attention_f32_items(a.BH, a.N, a.Cq);
+    cudaMemsetAsync(counter, 0, items * sizeof(int), st);
+    k_attention_f32_sparse<D><<<items, kFThreads, F32Smem<D>::bytes, st>>>(a, part, counter);
   } else {
-    dim3 grid((a.N + BM - 1) / BM, a.BH);
-    k_attention_f32<D, false><<<grid, kFThreads, F32Smem<D>::bytes, st>>>(a, 1, nullptr, nullptr);
+    k_attention_f32_dense<D><<<dim3((a.N + BM - 1) / BM, a.BH), kFThreads, F32Smem<D>::bytes, st>>>(a);
   }
 }
 void launch_attention_f32(const AttnArgs& a, float* part, int* counter, cudaStream_t st) {
@@ -668,10 +764,10 @@ void launch_write_probe_rows(int dtype, const float* Dn, const int* probe_idx, i
 cudaError_t init_attention_simt() {
   cudaError_t e;
 #define SPR_ATTR(KERN, BYTES) if ((e = cudaFuncSetAttribute(KERN, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(BYTES))) != cudaSuccess) return e
-  SPR_ATTR((k_attention_f32<128, true>), F32Smem<128>::bytes);
-  SPR_ATTR((k_attention_f32<128, false>), F32Smem<128>::bytes);
-  SPR_ATTR((k_attention_f32<64, true>), F32Smem<64>::bytes);
-  SPR_ATTR((k_attention_f32<64, false>), F32Smem<64>::bytes);
+  SPR_ATTR(k_attention_f32_sparse<128>, F32Smem<128>::bytes);
+  SPR_ATTR(k_attention_f32_dense<128>, F32Smem<128>::bytes);
+  SPR_ATTR(k_attention_f32_sparse<64>, F32Smem<64>::bytes);
+  SPR_ATTR(k_attention_f32_dense<64>, F32Smem<64>::bytes);
   SPR_ATTR((k_probe_rows<float, 128>), probe_smem_bytes<128>(kMaxGroups));
   SPR_ATTR((k_probe_rows<float, 64>), probe_smem_bytes<64>(kMaxGroups));
 #undef SPR_ATTR

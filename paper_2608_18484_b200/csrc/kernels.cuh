@@ -106,6 +106,7 @@ struct AttnArgs {
   // sparse metadata (null for dense)
   const int *q_off, *kv_off, *route_ptr, *route_idx, *q_perm, *tile_off;
   int Cq, Ck;
+  const int4* items; const int* n_items;       // float32: the list of launch_f32_items
   int kv_div;                 // query heads per K/V head (grouped-query attention): K/V-side arrays are indexed by bh / kv_div; 0 = 1
   // epilogue
   void* O; i64 os[3];
@@ -116,11 +117,12 @@ struct AttnArgs {
 cudaError_t init_attention_simt();
 // tile_off [BH][Cq+1]: prefix of the tiles per query group; small_rem > 0 leaves out a last tile of at most small_rem rows
 void launch_tile_offsets(const int* q_off, int BH, int Cq, int tile_rows, int small_rem, int* tile_off, cudaStream_t st);
-// float32; sparse calls: part / counter from the workspace (attention_f32_part_floats floats, attention_f32_counters ints; the
-// key sequences are not split when part is null)
-int attention_f32_splits(int BH, int N, int Cq);
+// float32, sparse calls.  The list of CTAs (attention_f32_items entries, `keys` [BH][Cq]), made once the routes are known; part /
+// counter: workspace of attention_f32_part_floats floats and attention_f32_items ints.
+size_t attention_f32_items(int BH, int N, int Cq);
 size_t attention_f32_part_floats(int BH, int N, int Cq, int d);
-size_t attention_f32_counters(int BH, int N, int Cq);
+void launch_f32_items(const int* q_off, const int* kv_off, const int* route_ptr, const int* route_idx, int BH, int N, int Cq, int Ck, int* keys, int4* items,
+                      int* n_items, cudaStream_t st);
 void launch_attention_f32(const AttnArgs& a, float* part, int* counter, cudaStream_t st);
 // O <- O + O A + c in place (float32)
 void launch_correction_f32(const float* A, const float* c, void* O, const i64* os, int BH, int H, int N, int d, cudaStream_t st);
