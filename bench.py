@@ -109,7 +109,7 @@ def launches_per_call(T, fitted, tensor_path):
     else:                # init, first norms, T assignments, T-1 updates
         kmeans = 2 + T + (T - 1)
     # per side: Gram, eigen-solver (Householder, vectors, orthogonalisation, back-transformation, marked-matrix fallback), projection (+ split of
-    # the feature map), k-means, sort + means; then probes; route; tile offsets + remainder rows
+    # the feature map), k-means, sort + means; then probes; route; list of tiles (2) + remainder rows
     plan = 2 * (6 + (2 if tensor_path else 1) + kmeans + 2) + 2 + 2 + 3
     if not fitted:
         plan -= 2

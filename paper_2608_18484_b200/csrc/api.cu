@@ -254,8 +254,8 @@ struct sparsepr_plan_s {
   float *mu, *mu2, *mumax; i64* sums; int* counts;
   int *a_K, *a_Q, *kv_perm, *kv_inv, *q_perm, *q_inv, *kv_off, *q_off, *nk, *nq;
   float *kappa, *theta, *score;
-  int *route_ptr, *route_idx, *tile_off128;
-  int4* f32_items; int *f32_keys, *f32_count;   // float32: the attention kernel's list of CTAs
+  int *route_ptr, *route_idx;
+  int4* items; int *item_keys, *n_items;   // the attention kernel's list of CTAs
   RouteState* rstate;
   double* probe_dist; int* probe_idx; float* probe_w;
   __nv_bfloat16 *xh, *xl, *mh, *ml, *mw, *Ft; float* xnorm; int* flagged; int* flagcnt; double* eigws;
@@ -291,9 +291,8 @@ void carve_plan(Carver& c, const Resolved& r, sparsepr_plan_s* p) {
   float* score = c.take<float>(BH * (size_t)r.Cq * r.Ck);
   int* rptr = c.take<int>(BH * (r.Cq + 1)); int* ridx = c.take<int>(BH * (size_t)r.Cq * r.Ck);
   const bool f32 = r.dtype == SPARSEPR_F32;
-  int* toff128 = c.take<int>(f32 ? 0 : BH * (r.Cq + 1));
-  int4* items = c.take<int4>(f32 ? attention_f32_items((int)BH, (int)N, r.Cq) : 0);
-  int* ikeys = c.take<int>(f32 ? BH * r.Cq : 0); int* icount = c.take<int>(f32 ? 1 : 0);
+  int4* items = c.take<int4>(f32 ? attention_f32_items((int)BH, (int)N, r.Cq) : BH * attention_tc_items((int)N, r.Cq));
+  int* ikeys = c.take<int>(BH * r.Cq); int* icount = c.take<int>(f32 ? 1 : BH);
   RouteState* rs = c.take<RouteState>(BH);
   double* pd = c.take<double>(BH * N);
   int* pidx = c.take<int>(BH * std::max(r.M, 1)); float* pw = c.take<float>(BH * std::max(r.M, 1));
@@ -314,7 +313,7 @@ void carve_plan(Carver& c, const Resolved& r, sparsepr_plan_s* p) {
     p->a_K = aK; p->a_Q = aQ; p->kv_perm = kvp; p->kv_inv = kvi; p->q_perm = qp; p->q_inv = qi; p->kv_off = kvo; p->q_off = qo;
     p->nk = nk; p->nq = nq; p->kappa = kappa; p->theta = theta; p->score = score; p->route_ptr = rptr; p->route_idx = ridx;
     p->xh = xh; p->xl = xl; p->mh = mh; p->ml = ml; p->mw = mw; p->xnorm = xnorm; p->flagged = flagged;
-    p->tile_off128 = toff128; p->f32_items = items; p->f32_keys = ikeys; p->f32_count = icount; p->rstate = rs; p->probe_dist = pd; p->probe_idx = pidx; p->probe_w = pw;
+    p->items = items; p->item_keys = ikeys; p->n_items = icount; p->rstate = rs; p->probe_dist = pd; p->probe_idx = pidx; p->probe_w = pw;
   }
 }
 
@@ -322,9 +321,9 @@ void carve_plan(Carver& c, const Resolved& r, sparsepr_plan_s* p) {
 void launch_tiles(const sparsepr_plan_s* p, cudaStream_t st) {
   const Resolved& r = p->r;
   if (r.dtype == SPARSEPR_F32) {
-    launch_f32_items(p->q_off, p->kv_off, p->route_ptr, p->route_idx, r.BH, r.N, r.Cq, r.Ck, p->f32_keys, p->f32_items, p->f32_count, st);
+    launch_f32_items(p->q_off, p->kv_off, p->route_ptr, p->route_idx, r.BH, r.N, r.Cq, r.Ck, p->item_keys, p->items, p->n_items, st);
   } else {
-    launch_tile_offsets(p->q_off, r.BH, r.Cq, 128, kRemRows, p->tile_off128, st);
+    launch_tc_items(p->q_off, p->kv_off, p->route_ptr, p->route_idx, r.BH, r.N, r.Cq, r.Ck, r.G, p->item_keys, p->items, p->n_items, st);
     launch_remainder_rows(p->q_off, p->route_ptr, p->route_idx, r.BH, r.Cq, r.Ck, r.N, p->rem_pos, p->rem_grp, p->rem_cnt, st);
   }
 }
@@ -693,7 +692,7 @@ static sparsepr_status_t attend_impl(const sparsepr_plan_t* p, const void* Q, co
   aa.dtype = r.dtype; aa.BH = r.BH; aa.H = r.H; aa.N = r.N; aa.d = r.d; aa.scale = r.scale;
   aa.Q = w.Qg; aa.K = w.Kg; aa.V = w.Vg;
   aa.q_off = p->q_off; aa.kv_off = p->kv_off; aa.route_ptr = p->route_ptr; aa.route_idx = p->route_idx;
-  aa.q_perm = p->q_perm; aa.tile_off = p->tile_off128; aa.Cq = r.Cq; aa.Ck = r.Ck; aa.kv_div = r.G;
+  aa.q_perm = p->q_perm; aa.items = p->items; aa.n_items = p->n_items; aa.Cq = r.Cq; aa.Ck = r.Ck; aa.kv_div = r.G;
   aa.O = O; for (int i = 0; i < 3; ++i) aa.os[i] = r.os[i];
   aa.O_sparse = O_sparse;
   aa.err = p->err;
@@ -743,7 +742,6 @@ static sparsepr_status_t attend_impl(const sparsepr_plan_t* p, const void* Q, co
     if (fitted && !launch_correction_tc(w.c, w.At, w.Olo, O, r.os, r.BH, r.H, r.N, r.d, p->err, st)) return SPARSEPR_ERR_CUDA;
     tm.mark(SPARSEPR_STAGE_CORRECTION);
   } else {
-    aa.items = p->f32_items; aa.n_items = p->f32_count;
     launch_attention_f32(aa, w.fpart, w.fcount, st);
     tm.mark(SPARSEPR_STAGE_ATTENTION);
     if (overlap) { join_side(p, st); p->side_pending = false; }

@@ -391,15 +391,16 @@ __global__ void __launch_bounds__(kFThreads, 2) k_attention_f32_dense(AttnArgs a
 // (attention_f32_items): fine enough for a small list to fill the GPU, and for the kernels of the probes and the fit to find
 // free slots beside a large one (they would wait for the longest items of the first wave), coarse enough that the parts
 // cost little.
+// keys of every group's routes, in boxes of `box` rows of which only the last of a range may be short
 __global__ void __launch_bounds__(1024) k_route_keys(const int* __restrict__ kv_off, const int* __restrict__ route_ptr, const int* __restrict__ route_idx, int Cq,
-                                                     int Ck, int* __restrict__ keys) {
+                                                     int Ck, int kv_div, int box, int* __restrict__ keys) {
   const int bh = blockIdx.y, g = blockIdx.x * 32 + (threadIdx.x >> 5);
   if (g >= Cq) return;
   const int* rp = route_ptr + (i64)bh * (Cq + 1);
   const int* ri = route_idx + (i64)bh * Cq * Ck;
-  const int* ko = kv_off + (i64)bh * (Ck + 1);
+  const int* ko = kv_off + (i64)(bh / kv_div) * (Ck + 1);
   int L = 0;
-  for (int t = rp[g] + (threadIdx.x & 31); t < rp[g + 1]; t += 32) { const int b = ri[t]; L += ko[b + 1] - ko[b]; }
+  for (int t = rp[g] + (threadIdx.x & 31); t < rp[g + 1]; t += 32) { const int b = ri[t]; L += (ko[b + 1] - ko[b] + box - 1) / box; }
   L = warp_sum(L);
   if ((threadIdx.x & 31) == 0) keys[(i64)bh * Cq + g] = L;
 }
@@ -511,36 +512,51 @@ void launch_correction_f32(const float* A, const float* c, void* O, const i64* o
   else k_correction_f32<64><<<grid, 128, 0, st>>>(A, c, H, N, (float*)O, os[0], os[1], os[2]);
 }
 
-// tiles per query group: ceil(n / tile_rows), or, with small_rem > 0, without the last tile when it
-// would hold at most small_rem rows (those rows belong to the remainder kernel)
-__global__ void __launch_bounds__(1024) k_tile_offsets(const int* __restrict__ q_off, int Cq, int tile_rows, int small_rem,
-                                                       int* __restrict__ tile_off) {
-  __shared__ int cnt[kMaxGroups];
-  __shared__ int scratch[34];
-  const int bh = blockIdx.x;
-  const int* qo = q_off + (i64)bh * (Cq + 1);
-  for (int a = threadIdx.x; a < Cq; a += blockDim.x) {
-    const int n = qo[a + 1] - qo[a], rem = n % tile_rows;
-    cnt[a] = n / tile_rows + (rem > small_rem ? 1 : 0);
-  }
-  __syncthreads();
-  const int total = block_exclusive_scan(cnt, Cq, scratch);
-  for (int a = threadIdx.x; a < Cq; a += blockDim.x) tile_off[(i64)bh * (Cq + 1) + a] = cnt[a];
-  if (threadIdx.x == 0) tile_off[(i64)bh * (Cq + 1) + Cq] = total;
-}
-void launch_tile_offsets(const int* q_off, int BH, int Cq, int tile_rows, int small_rem, int* tile_off, cudaStream_t st) {
-  k_tile_offsets<<<BH, 1024, 0, st>>>(q_off, Cq, tile_rows, small_rem, tile_off);
-}
-
 // Items of a list at most: four rounds of CTAs on every SM slot, and twice as many as tiles.
 size_t attention_f32_items(int BH, int N, int Cq) { return std::max((size_t)4 * 2 * sm_count(), (size_t)2 * BH * ((N + BM - 1) / BM + Cq)); }
 size_t attention_f32_part_floats(int BH, int N, int Cq, int d) { return attention_f32_items(BH, N, Cq) * BM * (d + 2); }
 void launch_f32_items(const int* q_off, const int* kv_off, const int* route_ptr, const int* route_idx, int BH, int N, int Cq, int Ck, int* keys, int4* items,
                       int* n_items, cudaStream_t st) {
-  k_route_keys<<<dim3((Cq + 31) / 32, BH), 1024, 0, st>>>(kv_off, route_ptr, route_idx, Cq, Ck, keys);
+  k_route_keys<<<dim3((Cq + 31) / 32, BH), 1024, 0, st>>>(kv_off, route_ptr, route_idx, Cq, Ck, 1, 1, keys);
   int shift = 0;
   while ((((N + BN - 1) / BN + 1) * 9) >> shift >= kItemBuckets) ++shift;
   k_f32_items<<<1, kItemBuckets, 0, st>>>(q_off, keys, BH, Cq, (int)attention_f32_items(BH, N, Cq), shift, items, n_items);
+}
+
+// The 128-row tensor-core kernel: the tiles of a head, longest first (per head, not over all of them: tiles of one head run together
+// and share its keys in L2).  Every 128 rows of a group are a tile; a last tile of at most small_rem rows is left to the
+// remainder kernel.  Item: first row, boxes of 16 keys, place of the group's routes in the head's list, rows << 16 | routes.
+__global__ void __launch_bounds__(kItemBuckets) k_tc_items(const int* __restrict__ q_off, const int* __restrict__ route_ptr, const int* __restrict__ boxes, int Cq, int small_rem,
+                                                           int shift, int cap, int4* __restrict__ items, int* __restrict__ n_items) {
+  __shared__ int hist[kItemBuckets];
+  __shared__ int scratch[34];
+  const int bh = blockIdx.x;
+  const int* qo = q_off + (i64)bh * (Cq + 1);
+  const int* rp = route_ptr + (i64)bh * (Cq + 1);
+  hist[threadIdx.x] = 0;
+  __syncthreads();
+  int total = 0;
+  for (int pass = 0; pass < 2; ++pass) {
+    for (int a = threadIdx.x; a < Cq; a += kItemBuckets) {
+      const int first = qo[a], n = qo[a + 1] - first, rem = n % 128, tiles = n / 128 + (rem > small_rem ? 1 : 0), bx = boxes[(i64)bh * Cq + a];
+      if (tiles == 0) continue;
+      int at = atomicAdd(&hist[kItemBuckets - 1 - min(kItemBuckets - 1, bx >> shift)], tiles);
+      if (pass == 0) continue;
+      const int r0 = rp[a], nr = rp[a + 1] - r0;
+      for (int t = 0; t < tiles; ++t, ++at) items[(i64)bh * cap + at] = make_int4(first + 128 * t, bx, r0, min(128, n - 128 * t) << 16 | nr);
+    }
+    __syncthreads();
+    if (pass == 0) total = block_exclusive_scan(hist, kItemBuckets, scratch);
+  }
+  if (threadIdx.x == 0) n_items[bh] = total;
+}
+int attention_tc_items(int N, int Cq) { return (N + 127) / 128 + Cq; }
+void launch_tc_items(const int* q_off, const int* kv_off, const int* route_ptr, const int* route_idx, int BH, int N, int Cq, int Ck, int kv_div, int* boxes, int4* items,
+                     int* n_items, cudaStream_t st) {
+  k_route_keys<<<dim3((Cq + 31) / 32, BH), 1024, 0, st>>>(kv_off, route_ptr, route_idx, Cq, Ck, kv_div, 16, boxes);
+  int shift = 0;
+  while (((N + 15) / 16 + Ck) >> shift >= kItemBuckets) ++shift;
+  k_tc_items<<<BH, kItemBuckets, 0, st>>>(q_off, route_ptr, boxes, Cq, kRemRows, shift, attention_tc_items(N, Cq), items, n_items);
 }
 
 template <int D>

@@ -77,7 +77,8 @@ struct Params {
   int BH, H, N, Cq, Ck, sparse;
   int kv_div;                      // query heads per K/V head: K/V tensors, their maps and kv_off are indexed by head / kv_div
   float scale_log2;
-  const int *q_off, *kv_off, *route_ptr, *route_idx, *q_perm, *tile_off;
+  const int *kv_off, *route_idx, *q_perm;
+  const int4* items; const int* n_items;       // block-sparse: the tiles of a head (launch_tc_items)
   __nv_bfloat16* O; i64 os[3];
   float* O_sparse;
   __nv_bfloat16* O_lo;             // optional [BH][N][D]: o - bf16(o), original order (second word for the correction pass)
@@ -102,7 +103,7 @@ k_attention_tc(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__
   float* xmax = reinterpret_cast<float*>(sm + SM::xchg);                 // [2][2][128] half-row maxima of the current / next tile
   float* xsum = xmax + 4 * 128;                                            // [2][128] half-row sums (end)
   uint2* meta = reinterpret_cast<uint2*>(sm + SM::meta);
-  volatile int* misc = reinterpret_cast<volatile int*>(sm + SM::misc);   // [0] tmem base, [1] abort, [2] total boxes, [3] leave, [4] query group, [5] its first tile
+  volatile int* misc = reinterpret_cast<volatile int*>(sm + SM::misc);   // [0] tmem base, [1] abort, [3] leave
   const uint32_t bars = base + SM::bars;
   auto bar = [&](int i) { return bars + 8u * i; };
 
@@ -110,74 +111,57 @@ k_attention_tc(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__
   const int tid = threadIdx.x, warp = __shfl_sync(FULLW, tid >> 5, 0), lane = tid & 31;   // (uniform, and known to be)
   const int bh = blockIdx.y, b = bh / prm.H, h = bh % prm.H;
   // ---- which query tile ---------------------------------------------------------------
-  // Few dependent global reads: one round finds the query group of this tile (every thread tests one group),
-  // reads the error word and stages the key-group offsets in shared memory (the K ring is still idle); the
-  // second round reads the group's rows and routes.
+  // Few dependent global reads before the first copy can start: the item (rows, place of the routes), the routed groups,
+  // their ranges.  (Looking the tile up in prefix sums over the query groups took two reads more and two barriers, 5400 cycles
+  // of a CTA's 130000 at 480p-like size; with that and tiles in group order: attend on a kept plan, 12 heads of 25200 tokens,
+  // 1446 us, now 1417; call with 16 heads of d = 64 and 17550 tokens 2540 us, now 2494.)
   // Once any CTA has recorded a timeout the remaining CTAs of the launch leave at once (also if the
   // shared-memory base is not aligned as the swizzled tiles require).
-  int* kv_stage = reinterpret_cast<int*>(sm + SM::k);
+  int4 item = make_int4((int)blockIdx.x * kTile, 0, 0, (min(kTile, prm.N - (int)blockIdx.x * kTile) << 16) | 1);
+  bool none = false;
+  if (prm.sparse) {
+    none = (int)blockIdx.x >= prm.n_items[bh];                 // beyond this head's tiles
+    item = prm.items[(i64)bh * gridDim.x + blockIdx.x];
+  }
   if (tid == 0) {
     misc[3] = (prm.err != nullptr && *reinterpret_cast<volatile int*>(prm.err) == SPARSEPR_ERR_TIMEOUT) || (base & 1023u) != 0;
     if ((base & 1023u) != 0) set_error(prm.err, SPARSEPR_ERR_CUDA);
-    misc[4] = -1;
+    misc[1] = 0;
   }
   __syncthreads();
-  if (prm.sparse) {
-    const int* toff = prm.tile_off + (i64)bh * (prm.Cq + 1);
-    const int* kvo = prm.kv_off + (i64)(bh / prm.kv_div) * (prm.Ck + 1);
-    for (int g = tid; g < prm.Cq; g += kThreads)
-      if (toff[g] <= (int)blockIdx.x && (int)blockIdx.x < toff[g + 1]) { misc[4] = g; misc[5] = toff[g]; }
-    for (int g = tid; g <= prm.Ck; g += kThreads) kv_stage[g] = kvo[g];
-    __syncthreads();
-  }
-  if (misc[3] || (prm.sparse && misc[4] < 0)) return;        // error, or a tile index beyond this head's tiles
-  int row0, nrows, nroute;
-  const int* ridx = nullptr;
-  if (prm.sparse) {
-    const int g = misc[4];
-    const int* qoff = prm.q_off + (i64)bh * (prm.Cq + 1);
-    const int* rp = prm.route_ptr + (i64)bh * (prm.Cq + 1);
-    const int q0 = qoff[g], q1 = qoff[g + 1], r0 = rp[g], r1 = rp[g + 1];
-    row0 = q0 + ((int)blockIdx.x - misc[5]) * kTile;
-    nrows = min(kTile, q1 - row0);
-    ridx = prm.route_idx + (i64)bh * prm.Cq * prm.Ck + r0;
-    nroute = r1 - r0;
-  } else {
-    row0 = blockIdx.x * kTile;
-    nrows = min(kTile, prm.N - row0);
-    nroute = 1;
-  }
+  if (misc[3] || none) return;
+  const int row0 = item.x, nrows = item.w >> 16, nroute = item.w & 0xFFFF;
   const bool dup = prm.sparse && nrows <= kTile / 2;           // every row twice: lanes r and r + 64 (see the header)
   // destination rows of the tile, fetched now so that the epilogue does not wait for them
   int* dsts = reinterpret_cast<int*>(sm + SM::dst);
   if (tid < kTile) dsts[tid] = tid < nrows ? (prm.sparse ? prm.q_perm[(i64)bh * prm.N + row0 + tid] : row0 + tid) : -1;
 
   // ---- set-up: barriers, TMEM, key ranges ---------------------------------------------------
-  if (tid == 0) {
+  if (warp == 8 && lane == 0) {
     for (int i = 0; i < kNumBars; ++i)
       mbar_init(bar(i), (i == P_FULL || i == P_FULL + 1 || i == S_FREE || i == S_FREE + 1) ? 256 : 1);
-    misc[1] = 0; misc[2] = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   if (warp == 9) tmem_alloc(base + SM::misc, 512);
-  __syncthreads();
-  {
-    int boxes = 0;
+  if (warp == 10 && lane < 8) prefetch_map(lane < 4 ? &mapsK.m[lane] : &mapsV.m[lane - 4]);
+  int boxes = 0;
+  if (prm.sparse) {
+    const int* kvo = prm.kv_off + (i64)(bh / prm.kv_div) * (prm.Ck + 1);
+    const int* ridx = prm.route_idx + (i64)bh * prm.Cq * prm.Ck + item.z;
     for (int t = tid; t < nroute; t += kThreads) {
-      int start = 0, len = prm.N;
-      if (prm.sparse) { const int g = ridx[t]; start = kv_stage[g]; len = kv_stage[g + 1] - start; }
-      ranges[t] = make_int2(start, len);
-      boxes += (len + kSub - 1) / kSub;
+      const int g = ridx[t], start = kvo[g];
+      ranges[t] = make_int2(start, kvo[g + 1] - start);
     }
-    boxes = warp_sum(boxes);
-    if (lane == 0 && boxes) atomicAdd((int*)&misc[2], boxes);
+    boxes = item.y;
+  } else {
+    if (tid == 0) ranges[0] = make_int2(0, prm.N);
+    boxes = (prm.N + kSub - 1) / kSub;
   }
-  fence_async_smem();                        // the staged offsets were read from memory that the copies will overwrite
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = __shfl_sync(FULLW, (uint32_t)misc[0], 0);
-  const int total_boxes = __shfl_sync(FULLW, misc[2], 0);
+  const int total_boxes = __shfl_sync(FULLW, boxes, 0);
   const int n_tiles = (total_boxes + kSubPerTile - 1) / kSubPerTile;
   volatile int* abort_flag = &misc[1];
 
@@ -743,11 +727,10 @@ bool launch_attention_tc(const AttnArgs& a, cudaStream_t st) {
   Params p{};
   p.BH = a.BH; p.H = a.H; p.N = a.N; p.Cq = a.Cq; p.Ck = a.Ck; p.sparse = sparse; p.kv_div = kvd;
   p.scale_log2 = a.scale * 1.4426950408889634f;
-  p.q_off = a.q_off; p.kv_off = a.kv_off; p.route_ptr = a.route_ptr; p.route_idx = a.route_idx; p.q_perm = a.q_perm;
-  p.tile_off = a.tile_off;
+  p.kv_off = a.kv_off; p.route_idx = a.route_idx; p.q_perm = a.q_perm; p.items = a.items; p.n_items = a.n_items;
   p.O = (__nv_bfloat16*)a.O; for (int i = 0; i < 3; ++i) p.os[i] = a.os[i];
   p.O_sparse = a.O_sparse; p.O_lo = (__nv_bfloat16*)a.O_lo; p.err = a.err;
-  const int tiles = (a.N + kTile - 1) / kTile + (sparse ? a.Cq : 0);
+  const int tiles = sparse ? attention_tc_items(a.N, a.Cq) : (a.N + kTile - 1) / kTile;
   if (d == 128) k_attention_tc<128><<<dim3(tiles, a.BH), kThreads, kSmemBytes<128>, st>>>(mq, mq64, mk, mv, p);
   else k_attention_tc<64><<<dim3(tiles, a.BH), kThreads, kSmemBytes<64>, st>>>(mq, mq64, mk, mv, p);
   return true;

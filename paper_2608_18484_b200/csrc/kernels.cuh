@@ -104,9 +104,9 @@ struct AttnArgs {
   const void *Q, *K, *V;
   i64 qs[3], ks[3], vs[3];
   // sparse metadata (null for dense)
-  const int *q_off, *kv_off, *route_ptr, *route_idx, *q_perm, *tile_off;
+  const int *q_off, *kv_off, *route_ptr, *route_idx, *q_perm;
   int Cq, Ck;
-  const int4* items; const int* n_items;       // float32: the list of launch_f32_items
+  const int4* items; const int* n_items;       // the list of launch_f32_items or launch_tc_items
   int kv_div;                 // query heads per K/V head (grouped-query attention): K/V-side arrays are indexed by bh / kv_div; 0 = 1
   // epilogue
   void* O; i64 os[3];
@@ -115,8 +115,6 @@ struct AttnArgs {
   int* err;                   // device error word (may be null)
 };
 cudaError_t init_attention_simt();
-// tile_off [BH][Cq+1]: prefix of the tiles per query group; small_rem > 0 leaves out a last tile of at most small_rem rows
-void launch_tile_offsets(const int* q_off, int BH, int Cq, int tile_rows, int small_rem, int* tile_off, cudaStream_t st);
 // float32, sparse calls.  The list of CTAs (attention_f32_items entries, `keys` [BH][Cq]), made once the routes are known; part /
 // counter: workspace of attention_f32_part_floats floats and attention_f32_items ints.
 size_t attention_f32_items(int BH, int N, int Cq);
@@ -129,10 +127,12 @@ void launch_correction_f32(const float* A, const float* c, void* O, const i64* o
 // ---- attention_tc.cu (tcgen05 / TMEM / TMA; bf16, d = 64 or 128) -------------------------------------
 cudaError_t init_attention_tc();
 bool attention_tc_supported(const AttnArgs& a);
-// tile_off in `a` must have been built for 128-row tiles
+// block-sparse calls: items of launch_tc_items ([BH][attention_tc_items] entries, `boxes` [BH][Cq], n_items [BH]), made once the routes are known
+int attention_tc_items(int N, int Cq);
+void launch_tc_items(const int* q_off, const int* kv_off, const int* route_ptr, const int* route_idx, int BH, int N, int Cq, int Ck, int kv_div, int* boxes, int4* items,
+                     int* n_items, cudaStream_t st);
 bool launch_attention_tc(const AttnArgs& a, cudaStream_t st);
-// Query-group remainders of 1..kRemRows rows are left out of the 128-row kernel's tiles (tile offsets built with
-// small_rem = kRemRows) and handled by attention_packed.cu
+// Query-group remainders of 1..kRemRows rows are left out of the 128-row kernel's tiles and handled by attention_packed.cu
 constexpr int kRemRows = 32;
 // attention_packed.cu: those remainders, packed across groups into 128-row tiles that walk over all keys with
 // per-row route masks.  rem_pos / rem_grp [BH][N], rem_cnt [BH] are built from the query offsets and the routes once per

@@ -1,0 +1,40 @@
+"""Block-sparse bf16 attention on group sizes at the edges of its query tiles (remainders of at most 32 rows, at most 64 rows, one
+tile, two tiles and what is left of them) and of its key boxes and tiles (16 and 128 keys)."""
+import numpy as np
+import pytest
+import torch
+
+from oracle import sparsepr_oracle as orc
+from paper_2608_18484_b200 import binding as B
+from tests.gpu_util import assert_bf16_close, to_np
+
+pytestmark = pytest.mark.gpu
+
+SIZES = [1, 15, 16, 17, 32, 33, 0, 64, 65, 127, 128, 129, 160, 161, 255, 256, 257, 0, 288, 289, 384, 513, 2]
+
+
+@pytest.mark.parametrize("d", [64, 128])
+def test_row_and_key_counts(d):
+    rng = np.random.default_rng(d)
+    heads, N, C = 3, sum(SIZES), len(SIZES)
+    block = -(-N // C)
+    assert -(-N // block) == C
+    gen = torch.Generator(device="cuda").manual_seed(d)
+    Q, K, V = [torch.randn(1, heads, N, d, device="cuda", generator=gen).bfloat16() for _ in range(3)]
+    aQ, aK, ptr, idx = [], [], [], []
+    for _ in range(heads):
+        aQ.append(rng.permutation(np.repeat(np.arange(C), rng.permutation(SIZES))))
+        aK.append(rng.permutation(np.repeat(np.arange(C), rng.permutation(SIZES))))
+        full = int(np.argmax(np.bincount(aK[-1], minlength=C)))   # every group is routed to at least one group with keys
+        routes = [np.unique(np.append(rng.choice(C, size=n, replace=False), full)) for n in rng.permutation([C] + list(range(1, C)))]
+        ptr.append(np.concatenate([[0], np.cumsum([len(r) for r in routes])]))
+        idx.append(np.concatenate(routes))
+    kw = dict(block=block, density=0.5, n_sample=64, n_probe=0, mode=1, softmax_scale=d ** -0.5)
+    plan = B.sparsepr_plan_import(Q, K, V, dict(kv_assign=np.stack(aK), q_assign=np.stack(aQ), route_ptr=np.stack(ptr), route_idx=idx), **kw)
+    O, Osp = B.sparsepr_attend(plan, Q, K, V, return_sparse=True)
+    O2 = B.sparsepr_attend(plan, Q, K, V)                          # (without the float32 copy the output goes another way)
+    assert B.sparsepr_plan_stats(plan)["device_error"] == 0
+    for i in range(heads):
+        ref = orc.sparse_attention(to_np(Q[0, i]), to_np(K[0, i]), to_np(V[0, i]), aQ[i], aK[i], ptr[i], idx[i], d ** -0.5)
+        for out in (O[0, i], Osp[0, i], O2[0, i]):
+            assert_bf16_close(to_np(out), ref)                      # probabilities and output in bf16, sums in float32
