@@ -525,38 +525,46 @@ void launch_f32_items(const int* q_off, const int* kv_off, const int* route_ptr,
 
 // The 128-row tensor-core kernel: the tiles of a head, longest first (per head, not over all of them: tiles of one head run together
 // and share its keys in L2).  Every 128 rows of a group are a tile; a last tile of at most small_rem rows is left to the
-// remainder kernel.  Item: first row, boxes of 16 keys, place of the group's routes in the head's list, rows << 16 | routes.
+// remainder kernel.  Two lists: pairs of tiles of a group (none where cap_pairs is 0), and tiles left alone.  Item: first row, boxes of 16 keys, place of the
+// group's routes in the head's list, rows << 16 | routes.
 __global__ void __launch_bounds__(kItemBuckets) k_tc_items(const int* __restrict__ q_off, const int* __restrict__ route_ptr, const int* __restrict__ boxes, int Cq, int small_rem,
-                                                           int shift, int cap, int4* __restrict__ items, int* __restrict__ n_items) {
+                                                           int shift, int cap_pairs, int cap_single, int4* __restrict__ items, int* __restrict__ n_items) {
   __shared__ int hist[kItemBuckets];
   __shared__ int scratch[34];
-  const int bh = blockIdx.x;
+  const int bh = blockIdx.x, single = blockIdx.y;
   const int* qo = q_off + (i64)bh * (Cq + 1);
   const int* rp = route_ptr + (i64)bh * (Cq + 1);
+  int4* out = single ? items + (i64)gridDim.x * cap_pairs + (i64)bh * cap_single : items + (i64)bh * cap_pairs;
   hist[threadIdx.x] = 0;
   __syncthreads();
   int total = 0;
   for (int pass = 0; pass < 2; ++pass) {
     for (int a = threadIdx.x; a < Cq; a += kItemBuckets) {
-      const int first = qo[a], n = qo[a + 1] - first, rem = n % 128, tiles = n / 128 + (rem > small_rem ? 1 : 0), bx = boxes[(i64)bh * Cq + a];
-      if (tiles == 0) continue;
-      int at = atomicAdd(&hist[kItemBuckets - 1 - min(kItemBuckets - 1, bx >> shift)], tiles);
+      const int first = qo[a], all = qo[a + 1] - first, n = all - (all % 128 <= small_rem ? all % 128 : 0), bx = boxes[(i64)bh * Cq + a];
+      const int pairs = cap_pairs ? n / 256 + (n % 256 > 128 ? 1 : 0) : 0, alone = max(n - 256 * pairs, 0), mine = single ? (alone + 127) / 128 : pairs;
+      if (mine == 0) continue;
+      int at = atomicAdd(&hist[kItemBuckets - 1 - min(kItemBuckets - 1, bx >> shift)], mine);
       if (pass == 0) continue;
       const int r0 = rp[a], nr = rp[a + 1] - r0;
-      for (int t = 0; t < tiles; ++t, ++at) items[(i64)bh * cap + at] = make_int4(first + 128 * t, bx, r0, min(128, n - 128 * t) << 16 | nr);
+      const int size = single ? 128 : 256, from = single ? 256 * pairs : 0;
+      for (int t = 0; t < mine; ++t) out[at + t] = make_int4(first + from + size * t, bx, r0, min(size, n - from - size * t) << 16 | nr);
     }
     __syncthreads();
     if (pass == 0) total = block_exclusive_scan(hist, kItemBuckets, scratch);
   }
-  if (threadIdx.x == 0) n_items[bh] = total;
+  if (threadIdx.x == 0) n_items[single * gridDim.x + bh] = total;
 }
-int attention_tc_items(int N, int Cq) { return (N + 127) / 128 + Cq; }
+// Two tiles per CTA where one per CTA gives the SMs three rounds or more: a pair takes 1.6 times as long as one tile, so that with few tiles
+// it is better to have them on as many SMs.  (480p-like, 24 heads, 45 rounds: kernel 4350 us with tiles alone, 4240 with pairs; 2 heads of
+// 4770 tokens, half a round: call 1167 us with tiles alone, 1171 with pairs.)
+int attention_tc_pairs(int BH, int N) { return (i64)BH * N >= (i64)3 * sm_count() * 128 ? (N + 128) / 129 : 0; }      // (a pair has more than 128 rows)
+int attention_tc_singles(int BH, int N, int Cq) { return attention_tc_pairs(BH, N) ? Cq : (N + 127) / 128 + Cq; }
 void launch_tc_items(const int* q_off, const int* kv_off, const int* route_ptr, const int* route_idx, int BH, int N, int Cq, int Ck, int kv_div, int* boxes, int4* items,
                      int* n_items, cudaStream_t st) {
   k_route_keys<<<dim3((Cq + 31) / 32, BH), 1024, 0, st>>>(kv_off, route_ptr, route_idx, Cq, Ck, kv_div, 16, boxes);
   int shift = 0;
   while (((N + 15) / 16 + Ck) >> shift >= kItemBuckets) ++shift;
-  k_tc_items<<<BH, kItemBuckets, 0, st>>>(q_off, route_ptr, boxes, Cq, kRemRows, shift, attention_tc_items(N, Cq), items, n_items);
+  k_tc_items<<<dim3(BH, 2), kItemBuckets, 0, st>>>(q_off, route_ptr, boxes, Cq, kRemRows, shift, attention_tc_pairs(BH, N), attention_tc_singles(BH, N, Cq), items, n_items);
 }
 
 template <int D>

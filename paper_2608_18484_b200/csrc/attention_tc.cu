@@ -1,8 +1,8 @@
 // Block-sparse / dense attention on the sm_100a tensor cores (bf16, D = d = d_v = 64 or 128; at 64 the products are half
 // as long and the softmax threads, which set the pace, do the same work per score).
 //
-// One CTA processes one 128-row query tile (of one query group, Eq. 3; or of the whole
-// head for dense attention, Eq. 1).  Roles:
+// One CTA processes one 128-row query tile, or two of the same query group (of one query group, Eq. 3; or of the whole
+// head for dense attention, Eq. 1).  With one tile, roles:
 //   warps 0-7  softmax: warps w and w+4 share the 32 rows of TMEM quadrant w and split the
 //              128 scores of a row in two halves (keys 0-63 / 64-127 of the tile)
 //   warp  8    TMA producer of Q and the key tiles (+ tile meta ring)
@@ -23,6 +23,16 @@
 // this is why the two products have a thread each on different schedulers, why the producers issue few, large
 // copies, and why the barrier polls of a tile are grouped.
 // The reference maximum of a row moves only when it grows by more than 2^8 (then O is rescaled).
+// Two tiles (PAIR): the K and V tiles serve 256 rows, which halves the traffic from L2 (64 KB per key tile; all SMs together
+// read 9.1 to 10.4 TB/s from L2, 0.95 us per 64 KB and SM, and one tile per CTA takes 1.1 us per key tile).  Every tile has its
+// own four softmax warps, one row per thread, and its own issuer of both products; P takes the place of S (the
+// accumulators leave no other), so a tile alternates between the tensor cores and its softmax warps, while the other tile does
+// the opposite.  Bound by that chain: product 845 cycles (512 and what the other tile has queued), fetch and maximum 500,
+// exponentials 1200, P V and its completion 750; 3300 cycles per key tile for both, where one tile takes 2010.  The threads have
+// 224 registers (setmaxnreg).  One pair of eight by polynomial instead of three: a warp alone is short of issue slots, not of
+// the special-function unit (dense, 12 heads of 18944 tokens: 1726 us with three, 1662 with two, 1630 with one, 1644 with none).
+// Dense, 24 heads of 32760 tokens: 12.0 -> 10.1 ms (the clock falls to 1.6 GHz under the power limit); the same two tiles left
+// to themselves fall into step (3900 cycles per key tile).
 // Epilogue: O / l, stored as bf16 at the original token index (inverse permutation).  The residual correction of
 // Eq. 9 is a pass of its own (correction_tc.cu) so that the fit can overlap this kernel; for that pass the part of
 // every element that the bf16 rounding dropped is stored as a second bf16 word (O_lo), so that the corrected output
@@ -44,33 +54,36 @@ namespace spr {
 namespace tc {
 
 constexpr int kThreads = 384;
-constexpr int kTile = 128;            // query rows per CTA, keys per tile
+constexpr int kTile = 128;            // rows per query tile (one or two per CTA), keys per tile
 constexpr int kSub = 16;              // rows per TMA box of the K/V stream
 constexpr int kSubPerTile = kTile / kSub;
 constexpr uint32_t kHalfBytes = kTile * 128;          // one [128 rows x 64 bf16] swizzled block
 template <int D> constexpr uint32_t kTileBytes = (D / 64) * kHalfBytes;      // 32 KB at D = 128, 16 KB at D = 64
 constexpr uint32_t kSubBytes = kSub * 128;            // 2 KB per box
 constexpr int kPolyOf8 = 3;            // pairs of every 8 whose exponential is a polynomial on the FMA pipe
+constexpr int kPairPolyOf8 = 1;        // the same with two query tiles per CTA
 constexpr int kKStages = 2;            // K tiles in flight (consumed by Q K^T)
 constexpr int kVStages = 2;            // V tiles in flight (consumed by P V)
+constexpr int kSoftmaxRegs = 224, kOtherRegs = 56;     // registers per thread after the split: 128 (2 x 224 + 56) = the 384 x 168 of the launch
 
-template <int D> struct Smem {         // offsets from a 1024-byte aligned base
+template <int D, bool PAIR> struct Smem {         // offsets from a 1024-byte aligned base
   static constexpr uint32_t q = 0;
-  static constexpr uint32_t k = q + kTileBytes<D>;
+  static constexpr uint32_t k = q + (PAIR ? 2 : 1) * kTileBytes<D>;
   static constexpr uint32_t v = k + kKStages * kTileBytes<D>;
   static constexpr uint32_t ranges = v + kVStages * kTileBytes<D>;
   static constexpr uint32_t xchg = ranges + kMaxGroups * 8;     // float [2 tile parities][2 halves][128] row maxima; float [2][128] row sums
   static constexpr uint32_t meta = xchg + 6 * 128 * 4;            // uint2[8]: ring of per-tile box counts
   static constexpr uint32_t bars = meta + 8 * 8;                  // kNumBars mbarriers
   static constexpr uint32_t misc = bars + 32 * 8;                 // tmem base, abort flag, counters
-  static constexpr uint32_t dst = misc + 64;                      // int [128]: where the rows of this tile go (original token index)
-  static constexpr uint32_t total = dst + kTile * 4;
+  static constexpr uint32_t dst = misc + 64;                      // int per row: where the rows of this CTA go (original token index)
+  static constexpr uint32_t total = dst + (PAIR ? 2 : 1) * kTile * 4;
 };
-template <int D> constexpr size_t kSmemBytes = Smem<D>::total;                        // the dynamic segment is 1024-byte aligned and the only shared memory
+template <int D, bool PAIR> constexpr size_t kSmemBytes = Smem<D, PAIR>::total;                        // the dynamic segment is 1024-byte aligned and the only shared memory
 
 enum Bar { Q_FULL = 0, K_FULL = 1, K_EMPTY = K_FULL + kKStages, V_FULL = K_EMPTY + kKStages, V_EMPTY = V_FULL + kVStages,
            S_FULL = V_EMPTY + kVStages, S_FREE = S_FULL + 2, P_FULL = S_FREE + 2, P_EMPTY = P_FULL + 2, O_DONE = P_EMPTY + 2, META_FULL,
-           kNumBars = META_FULL + 8 };
+           // two query tiles x: P of the keys [0, 96) and [96, 128) is in tensor memory; P V is complete (P and O at rest)
+           P_PART = META_FULL + 8, PV_DONE = P_PART + 4, kNumBars = PV_DONE + 2 };
 static_assert(kNumBars <= 32, "barrier area");
 
 struct Params {
@@ -89,11 +102,12 @@ struct Maps { CUtensorMap m[4]; };      // the same tensor with boxes of 16, 32,
 
 __device__ __forceinline__ uint32_t pack_bf16(float a, float b) { return pack_bf16x2(a, b); }
 
-template <int D>
+template <int D, bool PAIR>
 __global__ void __launch_bounds__(kThreads, 1)
 k_attention_tc(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__ CUtensorMap mapQ64,
                const __grid_constant__ Maps mapsK, const __grid_constant__ Maps mapsV, Params prm) {
-  using SM = Smem<D>;
+  using SM = Smem<D, PAIR>;
+  constexpr int kRows = PAIR ? 2 * kTile : kTile;                          // query rows of a CTA
   constexpr int kHalves = D / 64;                                          // 64-column blocks of a row
   constexpr int kOc = D / 2;                                               // output columns of a thread
   extern __shared__ __align__(1024) unsigned char smem_raw[];
@@ -117,7 +131,7 @@ k_attention_tc(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__
   // 1446 us, now 1417; call with 16 heads of d = 64 and 17550 tokens 2540 us, now 2494.)
   // Once any CTA has recorded a timeout the remaining CTAs of the launch leave at once (also if the
   // shared-memory base is not aligned as the swizzled tiles require).
-  int4 item = make_int4((int)blockIdx.x * kTile, 0, 0, (min(kTile, prm.N - (int)blockIdx.x * kTile) << 16) | 1);
+  int4 item = make_int4((int)blockIdx.x * kRows, 0, 0, (min(kRows, prm.N - (int)blockIdx.x * kRows) << 16) | 1);
   bool none = false;
   if (prm.sparse) {
     none = (int)blockIdx.x >= prm.n_items[bh];                 // beyond this head's tiles
@@ -131,15 +145,16 @@ k_attention_tc(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__
   __syncthreads();
   if (misc[3] || none) return;
   const int row0 = item.x, nrows = item.w >> 16, nroute = item.w & 0xFFFF;
-  const bool dup = prm.sparse && nrows <= kTile / 2;           // every row twice: lanes r and r + 64 (see the header)
+  const bool dup = !PAIR && prm.sparse && nrows <= kTile / 2;           // every row twice: lanes r and r + 64 (see the header)
   // destination rows of the tile, fetched now so that the epilogue does not wait for them
   int* dsts = reinterpret_cast<int*>(sm + SM::dst);
-  if (tid < kTile) dsts[tid] = tid < nrows ? (prm.sparse ? prm.q_perm[(i64)bh * prm.N + row0 + tid] : row0 + tid) : -1;
+  if (tid < kRows) dsts[tid] = tid < nrows ? (prm.sparse ? prm.q_perm[(i64)bh * prm.N + row0 + tid] : row0 + tid) : -1;
 
   // ---- set-up: barriers, TMEM, key ranges ---------------------------------------------------
   if (warp == 8 && lane == 0) {
     for (int i = 0; i < kNumBars; ++i)
-      mbar_init(bar(i), (i == P_FULL || i == P_FULL + 1 || i == S_FREE || i == S_FREE + 1) ? 256 : 1);
+      mbar_init(bar(i), i >= S_FREE && i < P_EMPTY ? 256 : i >= P_PART && i < PV_DONE ? 128
+                        : PAIR && i >= K_EMPTY && i < S_FULL && (i < V_FULL || i >= V_EMPTY) ? 2 : 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   if (warp == 9) tmem_alloc(base + SM::misc, 512);
@@ -165,6 +180,8 @@ k_attention_tc(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__
   const int n_tiles = (total_boxes + kSubPerTile - 1) / kSubPerTile;
   volatile int* abort_flag = &misc[1];
 
+  if (warp >= 8) {
+  if constexpr (PAIR) asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kOtherRegs));
   if (warp == 8 || warp == 10) {
     // =========================== TMA producers ==========================================
     // warp 8 streams Q and the key tiles, warp 10 the value tiles.  All lanes of a producer walk
@@ -175,7 +192,7 @@ k_attention_tc(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__
       const int c2 = (prm.sparse ? bh : h) / prm.kv_div;       // K/V head (group-major copies: [BH / kv_div]; originals: [B][H / kv_div])
       if (is_k && lane == 0) {
         const int q2 = prm.sparse ? bh : h;
-        mbar_expect_tx(bar(Q_FULL), kTileBytes<D>);
+        mbar_expect_tx(bar(Q_FULL), kRows / kTile * kTileBytes<D>);
         if (dup) {
           // the same 64 rows into both halves of the tile (rows 64-127 of a [128 x 64] block start 8 KB in)
           for (int part = 0; part < 2; ++part) {
@@ -183,8 +200,9 @@ k_attention_tc(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__
               tma_load_4d(base + SM::q + c * kHalfBytes + part * (kHalfBytes / 2), &mapQ64, bar(Q_FULL), 64 * c, row0, q2, c3);
           }
         } else {
-          for (int c = 0; c < kHalves; ++c)
-            tma_load_4d(base + SM::q + c * kHalfBytes, &mapQ, bar(Q_FULL), 64 * c, row0, q2, c3);
+          for (int x = 0; x < kRows / kTile; ++x)
+            for (int c = 0; c < kHalves; ++c)
+              tma_load_4d(base + SM::q + x * kTileBytes<D> + c * kHalfBytes, &mapQ, bar(Q_FULL), 64 * c, row0 + x * kTile, q2, c3);
         }
       }
       const int nst = is_k ? kKStages : kVStages;
@@ -235,6 +253,51 @@ k_attention_tc(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__
           const uint32_t dst = buf0 + s * kTileBytes<D> + lane * kSubBytes;
 #pragma unroll
           for (int c = 0; c < kHalves; ++c) tma_load_4d(dst + c * kHalfBytes, &maps->m[my_k], bar(full0 + s), 64 * c, my_start, c2, c3);
+        }
+      }
+    }
+  } else if constexpr (PAIR) {
+    // =========================== two query tiles: issuer of both products of tile x (warps 9 and 11) =======
+    // TMEM columns: S_x [128 x, 128 x + 128), P_x over its first 64 once the scores are in registers, O_x [256 + 128 x, ... + D).
+    // (As below, the whole warp walks the tiles and one elected lane issues.)
+    if (n_tiles > 0) {
+      const int x = warp == 9 ? 0 : 1;
+      const uint32_t idesc_qk = idesc_bf16(0, 128), idesc_pv = idesc_bf16(1, D);
+      const uint64_t q_desc = smem_desc(base + SM::q + x * kTileBytes<D>, 16), k_desc = smem_desc(base + SM::k, 16), v_desc = smem_desc(base + SM::v, kHalfBytes);
+      const uint32_t sx = tmem + 128u * x, ox = tmem + 256u + 128u * x;
+      bool ok = __all_sync(FULLW, mbar_wait(bar(Q_FULL), 0, abort_flag));
+      for (int i = 0; i < n_tiles && ok; ++i) {
+        const int s = i & 1;
+        ok = mbar_wait(bar(K_FULL + s), (i >> 1) & 1, abort_flag);
+        if (i > 0) ok = ok && mbar_wait(bar(PV_DONE + x), (i - 1) & 1, abort_flag);     // P of tile i - 1 lies in the score columns
+        if (!__all_sync(FULLW, ok)) break;
+        tc_fence_after();
+        const uint64_t kd = k_desc + (uint64_t)(s * (kTileBytes<D> >> 4)), vd = v_desc + (uint64_t)(s * (kTileBytes<D> >> 4));
+        if (elect_one()) {
+#pragma unroll
+          for (int kk = 0; kk < D / 16; ++kk) {
+            const uint64_t koff = (uint64_t)((kk >> 2) * (kHalfBytes >> 4) + (kk & 3) * 2);     // compile-time constant
+            umma_bf16(sx, q_desc + koff, kd + koff, idesc_qk, kk > 0);
+          }
+          umma_commit(bar(K_EMPTY + s));
+          umma_commit(bar(S_FULL + x));
+        }
+        __syncwarp();
+        ok = mbar_wait(bar(META_FULL + (i & 7)), (i >> 3) & 1, abort_flag);
+        const int nsub = __shfl_sync(FULLW, (int)meta[i & 7].y, 0);
+        ok = ok && mbar_wait(bar(V_FULL + s), (i >> 1) & 1, abort_flag);
+#pragma unroll
+        for (int part = 0; part < 2; ++part) {
+          ok = __all_sync(FULLW, ok && mbar_wait(bar(P_PART + 2 * x + part), i & 1, abort_flag));   // these P in TMEM, O rescaled if needed
+          if (!ok) break;
+          tc_fence_after();
+          if (elect_one()) {
+#pragma unroll
+            for (int kk = part ? 6 : 0; kk < (part ? 8 : 6); ++kk)
+              if (kk < nsub) umma_bf16_ts(ox, sx + kk * 8, vd + (uint64_t)(kk * (kSubBytes >> 4)), idesc_pv, (i > 0 || kk > 0) ? 1u : 0u);
+            if (part == 1) { umma_commit(bar(V_EMPTY + s)); umma_commit(bar(PV_DONE + x)); }
+          }
+          __syncwarp();
         }
       }
     }
@@ -304,7 +367,143 @@ k_attention_tc(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__
       }
       if (ok && elect_one()) umma_commit(bar(O_DONE));
     }
-  } else if (warp < 8) {
+  }
+  } else if constexpr (PAIR) {
+    asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(kSoftmaxRegs));
+    // =========================== two query tiles: softmax ===================================
+    // Warps 4 x .. 4 x + 3 own tile x, a thread one row of it.
+    const int x = warp >> 2, row = (warp & 3) * 32 + lane;
+    const uint32_t s_addr = tmem + ((uint32_t)((warp & 3) * 32) << 16) + 128u * (uint32_t)x, o_addr = s_addr + 256u;
+    const float sc = prm.scale_log2;
+    float m_ref = -INFINITY, l = 0.f;
+    bool ok = true;
+    // The warps of the two tiles that share a scheduler take turns with their exponentials (barriers 1 + w and 5 + w: tile 0,
+    // tile 1 may go): left to themselves the tiles fall into step, and then wait for the tensor cores together and compete
+    // for the scheduler together.  Every turn is taken and passed on whatever happened.
+    const int turn_mine = 1 + warp, turn_other = 1 + (warp ^ 4);
+    if (x == 1) asm volatile("bar.arrive %0, 64;" ::"r"(turn_other) : "memory");
+    for (int i = 0; i < n_tiles; ++i) {
+      // the two barriers are polled back to back (their shared-memory round trips overlap)
+      const bool t_meta = mbar_try(bar(META_FULL + (i & 7)), (i >> 3) & 1), t_s = mbar_try(bar(S_FULL + x), i & 1);
+      if (!t_meta) ok = ok && mbar_wait(bar(META_FULL + (i & 7)), (i >> 3) & 1, abort_flag);
+      if (!t_s) ok = ok && mbar_wait(bar(S_FULL + x), i & 1, abort_flag);
+      ok = __all_sync(FULLW, ok);
+      float s[4][32];
+      float corr = 1.f, mneg = 0.f;
+      if (ok) {
+        tc_fence_after();
+        const uint2 mt = meta[i & 7];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) tmem_ld32_nowait(s_addr + 32 * q, s[q]);
+        tmem_ld_wait();
+        if (!(mt.x == 0xFFFFFFFFu && mt.y == 8u)) {              // (uniform)
+          // only the boxes that end a key range (or lie beyond the stream) have columns to mask
+#pragma unroll
+          for (int bx = 0; bx < 8; ++bx) {
+            const int lim = bx < (int)mt.y ? (int)((mt.x >> (4 * bx)) & 15u) : -1;      // last valid column of the box
+            if (lim != 15) {
+#pragma unroll
+              for (int c = 0; c < 16; ++c) s[bx >> 1][(bx & 1) * 16 + c] = (c <= lim) ? s[bx >> 1][(bx & 1) * 16 + c] : -INFINITY;
+            }
+          }
+        }
+        float m8[8];
+#pragma unroll
+        for (int c = 0; c < 8; ++c) m8[c] = -INFINITY;
+#pragma unroll
+        for (int q = 0; q < 4; ++q)
+#pragma unroll
+          for (int c = 0; c < 32; c += 2) m8[(c >> 1) & 7] = max3(m8[(c >> 1) & 7], s[q][c], s[q][c + 1]);
+        const float mx = max3(max3(m8[0], m8[1], m8[2]), max3(m8[3], m8[4], m8[5]), fmaxf(m8[6], m8[7]));
+        const bool move = (mx - m_ref) * sc > 8.f;               // true on the first tile (m_ref = -inf)
+        const float m_new = move ? mx : m_ref;
+        corr = move ? ex2((m_ref - m_new) * sc) : 1.f;           // 0 on the first tile
+        mneg = -m_new * sc;
+        m_ref = m_new;
+        if (i > 0 && __any_sync(FULLW, move)) {                  // rescale the rows of this warp (rare); the previous P V is complete: S_FULL says so
+#pragma unroll 1
+          for (int q = 0; q < D / 32; ++q) {
+            float t[32];
+            tmem_ld32(o_addr + q * 32, t);
+#pragma unroll
+            for (int c = 0; c < 32; ++c) t[c] *= corr;
+            tmem_st32(o_addr + q * 32, t);
+          }
+        }
+      }
+      asm volatile("bar.sync %0, 64;" ::"r"(turn_mine) : "memory");
+      if (ok) {
+        // probabilities, 32 at a time; P V starts on the first 96 while the others are computed
+        float2 ps2[2] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
+        const float2 sc2 = make_float2(sc, sc), mneg2 = make_float2(mneg, mneg);
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+          uint32_t w[16];
+#pragma unroll
+          for (int c = 0; c < 16; ++c) {
+            float2 e = __ffma2_rn(make_float2(s[q][2 * c], s[q][2 * c + 1]), sc2, mneg2);
+            if ((c & 7) < kPairPolyOf8) e = ex2_poly2(e);
+            else { e.x = ex2(e.x); e.y = ex2(e.y); }
+            ps2[c & 1] = __fadd2_rn(ps2[c & 1], e);
+            w[c] = pack_bf16(e.x, e.y);
+          }
+          tmem_st16u_nowait(s_addr + 16 * q, w);
+          if (q >= 2) {
+            tmem_st_wait();
+            tc_fence_before();
+            mbar_arrive(bar(P_PART + 2 * x + (q - 2)));
+          }
+        }
+        l = l * corr + ((ps2[0].x + ps2[0].y) + (ps2[1].x + ps2[1].y));
+      }
+      asm volatile("bar.arrive %0, 64;" ::"r"(turn_other) : "memory");
+    }
+    // ---- normalise, store ------------------------------------------------------------------------
+    if (n_tiles > 0) ok = __all_sync(FULLW, ok && mbar_wait(bar(PV_DONE + x), (n_tiles - 1) & 1, abort_flag));
+    const float inv = l > 0.f ? 1.f / l : 0.f;
+    const int rows = min(kTile, nrows - x * kTile);
+    const int* dst = dsts + x * kTile;
+    tc_fence_after();
+    // Coalesced stores, as below, but a warp stages and writes its own rows, one of the two words at a time, in the place
+    // of its query rows (the other tile may still be reading the rings); 16-byte pieces are permuted within a row by the
+    // row number, so that a quarter warp meets different banks both ways.
+    unsigned char* stage = sm + SM::q + x * kTileBytes<D>;
+    constexpr int kLpr = D / 8, kRpi = 32 / kLpr;                // pieces (lanes) per row, rows per step of a warp
+#pragma unroll 1
+    for (int word = 0; word < (prm.O_lo ? 2 : 1); ++word) {
+#pragma unroll 1
+      for (int q = 0; q < D / 32; ++q) {
+        float t[32];
+        if (ok && n_tiles > 0) tmem_ld32(o_addr + q * 32, t);    // (uniform)
+#pragma unroll
+        for (int c = 0; c < 32; ++c) t[c] = ok && n_tiles > 0 && inv != 0.f ? t[c] * inv : 0.f;
+        if (word == 0 && prm.O_sparse && ok && row < rows) {
+          float* sp = prm.O_sparse + ((i64)bh * prm.N + dst[row]) * D + q * 32;
+#pragma unroll
+          for (int c = 0; c < 32; c += 4) *reinterpret_cast<float4*>(sp + c) = make_float4(t[c], t[c + 1], t[c + 2], t[c + 3]);
+        }
+        if (word == 1) {
+#pragma unroll
+          for (int c = 0; c < 32; ++c) t[c] -= __bfloat162float(__float2bfloat16_rn(t[c]));     // what the rounding of the first word dropped
+        }
+#pragma unroll
+        for (int ch = 0; ch < 4; ++ch)
+          *reinterpret_cast<uint4*>(stage + row * 2 * D + (((q * 4 + ch) ^ (row & 7)) * 16)) =
+              make_uint4(pack_bf16(t[8 * ch], t[8 * ch + 1]), pack_bf16(t[8 * ch + 2], t[8 * ch + 3]), pack_bf16(t[8 * ch + 4], t[8 * ch + 5]), pack_bf16(t[8 * ch + 6], t[8 * ch + 7]));
+      }
+      __syncwarp();
+#pragma unroll 4
+      for (int it = 0; it < 32 / kRpi; ++it) {
+        const int r = (warp & 3) * 32 + kRpi * it + lane / kLpr, ch = lane % kLpr;
+        if (ok && r < rows) {
+          const uint4 vh = *reinterpret_cast<const uint4*>(stage + r * 2 * D + ((ch ^ (r & 7)) * 16));
+          __nv_bfloat16* op = word == 0 ? prm.O + b * prm.os[0] + h * prm.os[1] + (i64)dst[r] * prm.os[2] : prm.O_lo + ((i64)bh * prm.N + dst[r]) * D;
+          *reinterpret_cast<uint4*>(op + ch * 8) = vh;
+        }
+      }
+      __syncwarp();
+    }
+  } else {
     // =========================== softmax (warps 0-7) =======================================
     // Thread (half hh, quadrant wq, lane) owns the 64 scores of keys [64 hh, 64 hh + 64) of query row
     // 32 wq + lane; warps wq and wq + 4 meet at the named barrier 1 + wq to agree on the row maximum.
@@ -692,16 +891,20 @@ bool make_map(CUtensorMap* m, const void* ptr, int cols, int rows, int H, int B,
 }  // namespace tc
 
 cudaError_t init_attention_tc() {
-  const cudaError_t e = cudaFuncSetAttribute(tc::k_attention_tc<128>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)tc::kSmemBytes<128>);
-  if (e != cudaSuccess) return e;
-  return cudaFuncSetAttribute(tc::k_attention_tc<64>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)tc::kSmemBytes<64>);
+  cudaError_t e = cudaSuccess;
+  const auto set = [&](auto kernel, size_t bytes) { if (e == cudaSuccess) e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes); };
+  set(tc::k_attention_tc<128, false>, tc::kSmemBytes<128, false>);
+  set(tc::k_attention_tc<64, false>, tc::kSmemBytes<64, false>);
+  set(tc::k_attention_tc<128, true>, tc::kSmemBytes<128, true>);
+  set(tc::k_attention_tc<64, true>, tc::kSmemBytes<64, true>);
+  return e;
 }
 
 bool attention_tc_supported(const AttnArgs& a) {
   return a.dtype == SPARSEPR_BF16 && (a.d == 64 || a.d == 128) && tc::tma_available();
 }
 
-bool launch_attention_tc(const AttnArgs& a, cudaStream_t st) {
+bool launch_attention_tc(const AttnArgs& a, cudaStream_t st, bool pairs) {
   using namespace tc;
   const int d = a.d;
   CUtensorMap mq, mq64;
@@ -727,12 +930,24 @@ bool launch_attention_tc(const AttnArgs& a, cudaStream_t st) {
   Params p{};
   p.BH = a.BH; p.H = a.H; p.N = a.N; p.Cq = a.Cq; p.Ck = a.Ck; p.sparse = sparse; p.kv_div = kvd;
   p.scale_log2 = a.scale * 1.4426950408889634f;
-  p.kv_off = a.kv_off; p.route_idx = a.route_idx; p.q_perm = a.q_perm; p.items = a.items; p.n_items = a.n_items;
+  p.kv_off = a.kv_off; p.route_idx = a.route_idx; p.q_perm = a.q_perm; p.items = a.items + (pairs ? 0 : (i64)a.BH * attention_tc_pairs(a.BH, a.N)); p.n_items = a.n_items + (pairs ? 0 : a.BH);
   p.O = (__nv_bfloat16*)a.O; for (int i = 0; i < 3; ++i) p.os[i] = a.os[i];
   p.O_sparse = a.O_sparse; p.O_lo = (__nv_bfloat16*)a.O_lo; p.err = a.err;
-  const int tiles = sparse ? attention_tc_items(a.N, a.Cq) : (a.N + kTile - 1) / kTile;
-  if (d == 128) k_attention_tc<128><<<dim3(tiles, a.BH), kThreads, kSmemBytes<128>, st>>>(mq, mq64, mk, mv, p);
-  else k_attention_tc<64><<<dim3(tiles, a.BH), kThreads, kSmemBytes<64>, st>>>(mq, mq64, mk, mv, p);
+  const auto run = [&](auto kernel, int ctas, size_t bytes) { kernel<<<dim3(ctas, a.BH), kThreads, bytes, st>>>(mq, mq64, mk, mv, p); };
+  // Two query tiles per CTA for dense calls: a pair takes about 1.6 times as long as one tile, so that it pays unless the CTAs of one
+  // tile leave SMs idle (or fill their last round where the pairs do not): 8 heads of 4096 tokens, two rounds of tiles, one of pairs,
+  // 81 -> 72 us; 2 heads of 4770 tokens, one round of tiles, 49 us, which pairs on half the SMs would lengthen.
+  const int tiles = (a.N + kTile - 1) / kTile, sms = sm_count();
+  const auto rounds = [&](int per_head) { return ((i64)per_head * a.BH + sms - 1) / sms; };
+  if (sparse ? pairs : 100 * rounds(tiles) > 164 * rounds((tiles + 1) / 2)) {
+    const int ctas = sparse ? attention_tc_pairs(a.BH, a.N) : (tiles + 1) / 2;
+    if (d == 128) run(k_attention_tc<128, true>, ctas, kSmemBytes<128, true>);
+    else run(k_attention_tc<64, true>, ctas, kSmemBytes<64, true>);
+  } else {
+    const int ctas = sparse ? attention_tc_singles(a.BH, a.N, a.Cq) : tiles;
+    if (d == 128) run(k_attention_tc<128, false>, ctas, kSmemBytes<128, false>);
+    else run(k_attention_tc<64, false>, ctas, kSmemBytes<64, false>);
+  }
   return true;
 }
 

@@ -14,9 +14,10 @@ SIZES = [1, 15, 16, 17, 32, 33, 0, 64, 65, 127, 128, 129, 160, 161, 255, 256, 25
 
 
 @pytest.mark.parametrize("d", [64, 128])
-def test_row_and_key_counts(d):
+@pytest.mark.parametrize("heads", [3, 20], ids=["alone", "pairs"])     # few tiles: one per CTA; many: two tiles of a group per CTA
+def test_row_and_key_counts(heads, d):
     rng = np.random.default_rng(d)
-    heads, N, C = 3, sum(SIZES), len(SIZES)
+    N, C = sum(SIZES), len(SIZES)
     block = -(-N // C)
     assert -(-N // block) == C
     gen = torch.Generator(device="cuda").manual_seed(d)
@@ -34,7 +35,18 @@ def test_row_and_key_counts(d):
     O, Osp = B.sparsepr_attend(plan, Q, K, V, return_sparse=True)
     O2 = B.sparsepr_attend(plan, Q, K, V)                          # (without the float32 copy the output goes another way)
     assert B.sparsepr_plan_stats(plan)["device_error"] == 0
-    for i in range(heads):
+    for i in sorted({0, 1, heads - 1}):
         ref = orc.sparse_attention(to_np(Q[0, i]), to_np(K[0, i]), to_np(V[0, i]), aQ[i], aK[i], ptr[i], idx[i], d ** -0.5)
         for out in (O[0, i], Osp[0, i], O2[0, i]):
             assert_bf16_close(to_np(out), ref)                      # probabilities and output in bf16, sums in float32
+
+
+@pytest.mark.parametrize("heads,N", [(1, 257), (148, 129), (74, 384), (37, 1000)])
+def test_dense_pairs(heads, N):
+    """One and two query tiles per CTA, the second one full, ragged (one row) and empty: two where one per CTA
+    would make two rounds on 148 SMs and two make one."""
+    gen = torch.Generator(device="cuda").manual_seed(N)
+    Q, K, V = [torch.randn(1, heads, N, 128, device="cuda", generator=gen).bfloat16() for _ in range(3)]
+    O = B.sparsepr_dense(Q, K, V, 128 ** -0.5)
+    for i in sorted({0, heads - 1}):
+        assert_bf16_close(to_np(O[0, i]), orc.dense_attention(to_np(Q[0, i]), to_np(K[0, i]), to_np(V[0, i]), 128 ** -0.5))
