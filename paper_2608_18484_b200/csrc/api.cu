@@ -184,9 +184,9 @@ struct SideSet {
   // probe rows and fit next to the block-sparse kernel), forked and joined with the two events
   cudaStream_t side = nullptr;
   cudaEvent_t ev_fork = nullptr, ev_join = nullptr;
-  // third stream: the remainder kernel beside the 128-row kernel
+  // third stream: the routing beside the gathers; the remainder kernel and the paired tiles beside the single ones
   cudaStream_t side2 = nullptr;
-  cudaEvent_t ev_join2 = nullptr;
+  cudaEvent_t ev_join2 = nullptr, ev_route = nullptr;
 };
 namespace {
 std::mutex g_side_mu;
@@ -212,11 +212,13 @@ SideSet* acquire_side_set() {
   if (cudaStreamCreateWithPriority(&s->side, cudaStreamNonBlocking, prio_hi) != cudaSuccess ||
       cudaStreamCreateWithPriority(&s->side2, cudaStreamNonBlocking, prio_hi) != cudaSuccess ||
       cudaEventCreateWithFlags(&s->ev_join2, cudaEventDisableTiming) != cudaSuccess ||
+      cudaEventCreateWithFlags(&s->ev_route, cudaEventDisableTiming) != cudaSuccess ||
       cudaEventCreateWithFlags(&s->ev_fork, cudaEventDisableTiming) != cudaSuccess ||
       cudaEventCreateWithFlags(&s->ev_join, cudaEventDisableTiming) != cudaSuccess) {
     if (s->ev_fork) cudaEventDestroy(s->ev_fork);
     if (s->ev_join) cudaEventDestroy(s->ev_join);
     if (s->ev_join2) cudaEventDestroy(s->ev_join2);
+    if (s->ev_route) cudaEventDestroy(s->ev_route);
     if (s->side) cudaStreamDestroy(s->side);
     if (s->side2) cudaStreamDestroy(s->side2);
     delete s;
@@ -236,14 +238,14 @@ struct sparsepr_plan_s {
   cudaStream_t stream;
   SideSet* set = nullptr;
   cudaStream_t side = nullptr, side2 = nullptr;          // aliases of the set's members
-  cudaEvent_t ev_fork = nullptr, ev_join = nullptr, ev_join2 = nullptr;
-  // the probe selection of the plan call may still run on `side` when the call returns: the first attend call
-  // orders it (its probe work follows on the same stream and is joined there); statistics, export and the
-  // destructor wait for it themselves
+  cudaEvent_t ev_fork = nullptr, ev_join = nullptr, ev_join2 = nullptr, ev_route = nullptr;
+  // the probe selection of the plan call may still run on `side` when the call returns, and the routing on `side2`: the first
+  // attend call orders the former (its probe work follows on the same stream and is joined there), every attend call
+  // waits for ev_route; statistics, export and the destructor wait for both themselves
   mutable bool side_pending = false;
   bool imported = false;                                  // built by sparsepr_plan_import: no partition stages ran
   ~sparsepr_plan_s() {
-    if (side && side_pending) cudaStreamSynchronize(side);
+    if (side && side_pending) { cudaStreamSynchronize(side); cudaStreamSynchronize(side2); }
     release_side_set(set);
   }
   // device state (all inside the caller's plan workspace)
@@ -498,7 +500,7 @@ static sparsepr_status_t make_plan(const sparsepr_shape_t* shape, const sparsepr
   p->set = acquire_side_set();
   if (!p->set) { delete p; return SPARSEPR_ERR_CUDA; }
   p->side = p->set->side; p->side2 = p->set->side2;
-  p->ev_fork = p->set->ev_fork; p->ev_join = p->set->ev_join; p->ev_join2 = p->set->ev_join2;
+  p->ev_fork = p->set->ev_fork; p->ev_join = p->set->ev_join; p->ev_join2 = p->set->ev_join2; p->ev_route = p->set->ev_route;
   Carver c(workspace);
   carve_plan(c, r, p);
   *out = p;
@@ -583,18 +585,27 @@ static sparsepr_status_t plan_impl(const sparsepr_shape_t* shape, const sparsepr
   launch_group_sort(p->a_Q, r.BH, r.N, r.Cq, p->q_perm, p->q_inv, p->q_off, p->err, st);
   launch_group_means(r.dtype, Q, r.qs, r.BH, r.H, p->q_perm, p->q_off, r.N, r.Cq, r.d, p->theta, p->nq, st);
   tm.mark(SPARSEPR_STAGE_QUERY_PERMUTE);
-  // probes and routes; without a profile the probe selection runs beside the routing
-  const bool overlap = prof == nullptr && r.M > 0;
-  cudaStream_t ps = st;
-  if (overlap) { fork_side(p, st); ps = p->side; }
+  // Probes and routes.  Without a profile both leave the caller's stream: the routes (one CTA per head for most of the time) run
+  // beside the gathers of the attend call that follows, which orders itself behind them by ev_route, and beside the probe
+  // selection, which is not needed before the probe rows.
+  const bool beside = prof == nullptr;
+  cudaStream_t ps = st, rs = st;
+  const auto cell_scores = [&] { launch_cell_scores(p->theta, p->kappa, p->nq, p->nk, r.BH, r.Cq, r.Ck, r.d, r.scale, p->score, r.G, rs); };
+  if (beside) {
+    fork_side(p, st);
+    cudaStreamWaitEvent(p->side2, p->ev_fork, 0);
+    ps = p->side; rs = p->side2;
+    cell_scores();
+  }
   if (r.M > 0)
     launch_probe_select(p->phi, r.RQ, r.fQ, p->q_perm, p->q_off, p->nq, r.BH, r.N, r.Cq, r.M, p->probe_dist, p->probe_idx, p->probe_w, ps);
   tm.mark(SPARSEPR_STAGE_PROBE_SELECT);
-  launch_cell_scores(p->theta, p->kappa, p->nq, p->nk, r.BH, r.Cq, r.Ck, r.d, r.scale, p->score, r.G, st);
+  if (!beside) cell_scores();
   launch_route_select(p->score, p->nq, p->nk, r.BH, r.Cq, r.Ck, pair_budget(r), r.density >= 1.0f, p->route_ptr,
-                      p->route_idx, p->rstate, nullptr, r.G, st);
-  launch_tiles(p, st);
-  if (overlap) p->side_pending = true;          // not joined here: the probes are not needed before the attend call
+                      p->route_idx, p->rstate, nullptr, r.G, rs);
+  launch_tiles(p, rs);
+  cudaEventRecord(p->ev_route, rs);
+  p->side_pending = beside;                     // not joined here: neither is needed before the attend call
   tm.mark(SPARSEPR_STAGE_ROUTE);
   tm.finish();
   if (!launch_ok()) { delete p; return SPARSEPR_ERR_CUDA; }
@@ -661,6 +672,7 @@ sparsepr_status_t sparsepr_plan_import(const sparsepr_shape_t* shape, const spar
   k_sizes_from_off<<<dim3((r.Cq + 255) / 256, r.BH), 256, 0, st>>>(p->q_off, r.Cq, p->nq);
   launch_count_pairs(p->q_off, p->kv_off, p->route_ptr, p->route_idx, r.BH, r.Cq, r.Ck, p->rstate, r.G, st);
   launch_tiles(p, st);
+  cudaEventRecord(p->ev_route, st);
   if (!launch_ok() || cudaStreamSynchronize(st) != cudaSuccess) { delete p; return SPARSEPR_ERR_CUDA; }
   *out = p;
   return SPARSEPR_OK;
@@ -686,6 +698,7 @@ static sparsepr_status_t attend_impl(const sparsepr_plan_t* p, const void* Q, co
   launch_gather_rows(r.dtype, Q, r.qs, r.BH, r.H, p->q_perm, r.N, r.d, w.Qg, st);
   launch_gather_rows(r.dtype, K, r.ks, r.BHkv, r.Hkv, p->kv_perm, r.N, r.d, w.Kg, st);
   launch_gather_rows(r.dtype, V, r.vs, r.BHkv, r.Hkv, p->kv_perm, r.N, r.d, w.Vg, st);
+  cudaStreamWaitEvent(st, p->ev_route, 0);
   tm.mark(SPARSEPR_STAGE_GATHER);
   const bool fitted = r.mode == 0 && r.M > 0;
   AttnArgs aa{};
@@ -729,12 +742,12 @@ static sparsepr_status_t attend_impl(const sparsepr_plan_t* p, const void* Q, co
   if (tensor) {
     // with a correction to follow, the block-sparse kernels also store what the bf16 rounding of O dropped
     if (fitted) aa.O_lo = w.Olo;
-    // the packed remainder tiles are few and long, the 128-row tiles many and short: they share the GPU instead of
-    // running one after the other (also in a profiled call: both belong to the ATTENTION stage)
+    // the packed remainder tiles are few and long, then come the pairs of tiles and the tiles alone, many and short: they share the GPU
+    // instead of running one after the other (also in a profiled call: all belong to the ATTENTION stage)
     if (!overlap) cudaEventRecord(p->ev_fork, st);                // (with the probes' overlap the event is recorded already)
     cudaStreamWaitEvent(p->side2, p->ev_fork, 0);
-    if (attention_tc_pairs(r.BH, r.N) && !launch_attention_tc(aa, p->side2, true)) return SPARSEPR_ERR_CUDA;
     if (!launch_attention_packed(aa, p->rem_pos, p->rem_grp, p->rem_cnt, p->side2)) return SPARSEPR_ERR_CUDA;
+    if (attention_tc_pairs(r.BH, r.N) && !launch_attention_tc(aa, p->side2, true)) return SPARSEPR_ERR_CUDA;
     if (!launch_attention_tc(aa, st)) return SPARSEPR_ERR_CUDA;
     cudaEventRecord(p->ev_join2, p->side2);
     cudaStreamWaitEvent(st, p->ev_join2, 0);
@@ -803,7 +816,7 @@ sparsepr_status_t sparsepr_dense(const sparsepr_shape_t* shape, float softmax_sc
 
 sparsepr_status_t sparsepr_plan_device_error(const sparsepr_plan_t* p, int32_t* device_error) {
   if (!p || !device_error) return SPARSEPR_ERR_INVALID_ARG;
-  if (cudaStreamSynchronize(p->stream) != cudaSuccess || (p->side && cudaStreamSynchronize(p->side) != cudaSuccess)) return SPARSEPR_ERR_CUDA;
+  if (cudaStreamSynchronize(p->stream) != cudaSuccess || (p->side && (cudaStreamSynchronize(p->side) != cudaSuccess || cudaStreamSynchronize(p->side2) != cudaSuccess))) return SPARSEPR_ERR_CUDA;
   int errw = 0;
   if (cudaMemcpy(&errw, p->err, sizeof(errw), cudaMemcpyDeviceToHost) != cudaSuccess) return SPARSEPR_ERR_CUDA;
   *device_error = errw;
@@ -813,7 +826,7 @@ sparsepr_status_t sparsepr_plan_device_error(const sparsepr_plan_t* p, int32_t* 
 sparsepr_status_t sparsepr_plan_stats(const sparsepr_plan_t* p, sparsepr_stats_t* out) {
   if (!p || !out) return SPARSEPR_ERR_INVALID_ARG;
   const Resolved& r = p->r;
-  if (cudaStreamSynchronize(p->stream) != cudaSuccess || (p->side && cudaStreamSynchronize(p->side) != cudaSuccess)) return SPARSEPR_ERR_CUDA;
+  if (cudaStreamSynchronize(p->stream) != cudaSuccess || (p->side && (cudaStreamSynchronize(p->side) != cudaSuccess || cudaStreamSynchronize(p->side2) != cudaSuccess))) return SPARSEPR_ERR_CUDA;
   std::memset(out, 0, sizeof(*out));
   std::vector<RouteState> rs(r.BH);
   std::vector<int> qo((size_t)r.BH * (r.Cq + 1)), ko((size_t)r.BHkv * (r.Ck + 1)), rp((size_t)r.BH * (r.Cq + 1));
@@ -909,7 +922,7 @@ sparsepr_status_t sparsepr_plan_stats(const sparsepr_plan_t* p, sparsepr_stats_t
 sparsepr_status_t sparsepr_plan_export(const sparsepr_plan_t* p, sparsepr_plan_host_t* o) {
   if (!p || !o) return SPARSEPR_ERR_INVALID_ARG;
   const Resolved& r = p->r;
-  if (cudaStreamSynchronize(p->stream) != cudaSuccess || (p->side && cudaStreamSynchronize(p->side) != cudaSuccess)) return SPARSEPR_ERR_CUDA;
+  if (cudaStreamSynchronize(p->stream) != cudaSuccess || (p->side && (cudaStreamSynchronize(p->side) != cudaSuccess || cudaStreamSynchronize(p->side2) != cudaSuccess))) return SPARSEPR_ERR_CUDA;
   const size_t BH = r.BH, N = r.N;
   bool ok = true;
   auto cp = [&](void* dst, const void* src, size_t bytes) { if (dst && bytes) ok &= cudaMemcpy(dst, src, bytes, cudaMemcpyDeviceToHost) == cudaSuccess; };
@@ -931,7 +944,7 @@ sparsepr_status_t sparsepr_plan_export_features(const sparsepr_plan_t* p, sparse
   if (!p || !o) return SPARSEPR_ERR_INVALID_ARG;
   if (p->imported) return SPARSEPR_ERR_UNSUPPORTED;          // an imported plan never computed them
   const Resolved& r = p->r;
-  if (cudaStreamSynchronize(p->stream) != cudaSuccess || (p->side && cudaStreamSynchronize(p->side) != cudaSuccess)) return SPARSEPR_ERR_CUDA;
+  if (cudaStreamSynchronize(p->stream) != cudaSuccess || (p->side && (cudaStreamSynchronize(p->side) != cudaSuccess || cudaStreamSynchronize(p->side2) != cudaSuccess))) return SPARSEPR_ERR_CUDA;
   const size_t BH = r.BH, N = r.N, d = r.d;
   bool ok = true;
   auto cp = [&](void* dst, const void* src, size_t bytes) { if (dst && bytes) ok &= cudaMemcpy(dst, src, bytes, cudaMemcpyDeviceToHost) == cudaSuccess; };

@@ -417,49 +417,61 @@ void launch_route_select(const float* score, const int* nq, const int* nk, int B
 }
 
 // =============================================================================
-// Probe selection, Algorithm A.1.  Kernel 1 (one warp per query group): centroid
+// Probe selection, Algorithm A.1.  Kernel 1 (one CTA per query group): centroid
 // c_a of the group in phi_Q space and the distance d_i of every member, stored at
 // the member's group-major position.  Kernel 2 (one CTA per head): round t takes,
 // from every group that still has rows, the unpicked row with the smallest
 // (d_i, i); groups are visited in ascending id; stops at M rows.  Then the
 // coverage weights w_p = |G_a| / m_a (Appendix A.2).
 // =============================================================================
+// k_probe_dist: one CTA per query group, bound by the latency of the gathered rows.  (One warp per group walked its rows twice, eight at
+// a time, and the largest group set the duration: 343 us beside the cell scores at 480p-like size with 24 heads, now 192 us;
+// whole calls: 2 heads of 4096 float32 tokens 1075 -> 1008 us, 2 heads of 4770 bf16 tokens 1171 -> 1140 us.)  Eight warps fetch 64
+// rows at once; the sums keep the order of the rows (a column is summed by one thread), and a distance is formed by one warp as
+// before, so that the result is the same bit for bit.
+constexpr int kPdRows = 64, kPdCols = 128;
 __global__ void __launch_bounds__(256) k_probe_dist(const float* __restrict__ phi, int ldphi, int r,
                                                     const int* __restrict__ perm, const int* __restrict__ off, int N,
                                                     int C, double* __restrict__ dist) {
-  const int bh = blockIdx.y;
-  const int g = blockIdx.x * 8 + (threadIdx.x >> 5);
-  if (g >= C) return;
-  const int lane = threadIdx.x & 31;
+  __shared__ float rows[kPdRows][kPdCols];
+  __shared__ double centre[kPdCols];
+  const int bh = blockIdx.y, g = blockIdx.x, tid = threadIdx.x, w = tid >> 5, lane = tid & 31;
   const int p0 = off[(i64)bh * (C + 1) + g], p1 = off[(i64)bh * (C + 1) + g + 1];
   if (p1 <= p0) return;
   const float* ph = phi + (i64)bh * N * ldphi;
   const int* pm = perm + (i64)bh * N;
-  // lane owns columns lane, lane + 32, ... (up to four: 128 columns for a semantic query partition); the rows are
-  // read eight at a time (the loads are independent, the sums keep their order)
+  // lane owns columns lane, lane + 32, ... (up to four: 128 columns for a semantic query partition)
   constexpr int kCols = 4;
   bool has[kCols];
-  double cen[kCols];
 #pragma unroll
-  for (int j = 0; j < kCols; ++j) { has[j] = lane + 32 * j < r; cen[j] = 0.0; }
-  for (int p = p0; p < p1; p += 8) {
+  for (int j = 0; j < kCols; ++j) has[j] = lane + 32 * j < r;
+  double sum = 0.0;                                                // column tid (tid < r)
+  for (int p = p0; p < p1; p += kPdRows) {
     float x[8][kCols];
 #pragma unroll
     for (int q = 0; q < 8; ++q) {
-      const float* row = ph + (i64)pm[min(p + q, p1 - 1)] * ldphi;
+      const float* row = ph + (i64)pm[min(p + 8 * w + q, p1 - 1)] * ldphi;
 #pragma unroll
       for (int j = 0; j < kCols; ++j) x[q][j] = has[j] ? row[lane + 32 * j] : 0.f;
     }
+    __syncthreads();                                               // the rows before have been summed
 #pragma unroll
     for (int q = 0; q < 8; ++q)
-      if (p + q < p1) {
 #pragma unroll
-        for (int j = 0; j < kCols; ++j) if (has[j]) cen[j] += (double)x[q][j];
-      }
+      for (int j = 0; j < kCols; ++j) if (has[j]) rows[8 * w + q][lane + 32 * j] = x[q][j];
+    __syncthreads();
+    if (tid < r) {
+      const int n = min(kPdRows, p1 - p);
+#pragma unroll 8
+      for (int q = 0; q < n; ++q) sum += (double)rows[q][tid];
+    }
   }
+  if (tid < r) centre[tid] = sum / (double)(p1 - p0);
+  __syncthreads();
+  double cen[kCols];
 #pragma unroll
-  for (int j = 0; j < kCols; ++j) cen[j] /= (double)(p1 - p0);
-  for (int p = p0; p < p1; p += 8) {
+  for (int j = 0; j < kCols; ++j) cen[j] = has[j] ? centre[lane + 32 * j] : 0.0;
+  for (int p = p0 + 8 * w; p < p1; p += kPdRows) {
     float x[8][kCols];
 #pragma unroll
     for (int q = 0; q < 8; ++q) {
@@ -568,8 +580,7 @@ cudaError_t init_routing() {
 void launch_probe_select(const float* phiQ, int ldphi, int r, const int* q_perm, const int* q_off, const int* nq, int BH,
                          int N, int Cq, int M, double* dist_scratch, int* probe_idx, float* probe_w, cudaStream_t st) {
   (void)nq;
-  dim3 grid((Cq + 7) / 8, BH);
-  k_probe_dist<<<grid, 256, 0, st>>>(phiQ, ldphi, r, q_perm, q_off, N, Cq, dist_scratch);
+  k_probe_dist<<<dim3(Cq, BH), 256, 0, st>>>(phiQ, ldphi, r, q_perm, q_off, N, Cq, dist_scratch);
   k_probe_pick<<<BH, 1024, probe_smem(Cq, M), st>>>(dist_scratch, q_perm, q_off, N, Cq, M, probe_idx, probe_w);
 }
 
