@@ -8,39 +8,44 @@
 // (M < d_v) and a small ridge the fitted map can have a norm of ~10, and one word of A then costs up to 0.012 of
 // the 0.02 that the output may differ from the oracle (the products are X_h A_h + X_l A_h + X_h A_l; X_l A_l is
 // below 2^-17 of the result).
-// The pass is bandwidth bound: each 128-row tile is read once (4 D bytes per row) and written once (2 D).
-// A CTA takes TWO consecutive row tiles of a head (the map is loaded once for both, 64 KB at D = 128, and all loads
-// of the CTA are issued up front: 192 KB in flight per SM at D = 128).
-//   warps 0-3  one thread per row of tile 0: X A from TMEM, X from the two swizzled tiles, + c, store; warps 4-7: tile 1
-//   warp  8    TMA loads (2 x (X_h, X_l), A_h^T, A_l^T), 3 D / 16 tcgen05.mma per tile, TMEM owner
+// The pass is bandwidth bound: each 128-row tile is read once (4 D bytes per row) and written once (2 D), 93 us at the copy rate for
+// 24 heads of 32760 rows.  One CTA per SM walks a run of consecutive tiles, of one head mostly, whose map stays in shared
+// memory; two tiles are in work, so that the loads of one, the products (24 instructions, 0.8 us) and the epilogue of the other
+// overlap, and the result leaves as a bulk store of the whole tile from the place of X_h.  (A CTA per two tiles, which loaded,
+// multiplied and stored, row by row, one after the other: 194 us; now 112.)
+//   warps 0-7  warps w and w + 4: 32 rows, half of the columns each: X A from TMEM, X from the two swizzled tiles, + c, back to X_h
+//   warp  8    TMA loads (X_h, X_l of a tile; A_h^T, A_l^T when the head changes)
+//   warp  9    3 D / 16 tcgen05.mma per tile, TMEM owner
 // Every mbarrier wait is bounded; on expiry the CTA records SPARSEPR_ERR_TIMEOUT and leaves.
 #include <cuda.h>
+#include <algorithm>
 #include "kernels.cuh"
 #include "tc_common.cuh"
 
 namespace spr {
 namespace tc {
 
-constexpr int kCorrThreads = 288;
+constexpr int kCorrThreads = 320;
 constexpr int kCorrTile = 128;
 constexpr uint32_t kCorrHalf = kCorrTile * 128;      // one [128 rows x 64 bf16] swizzled block
 template <int D> constexpr uint32_t kCorrTileBytes = (D / 64) * kCorrHalf;
 template <int D> constexpr uint32_t kCorrMapHalf = D * 128;                   // [D rows x 64 bf16]
 template <int D> struct CorrSmem {
-  static constexpr uint32_t xh = 0;                        // tile u at xh + 2 u kCorrTileBytes<D>, its second words one tile further
+  static constexpr uint32_t xh = 0;                        // stage u at xh + 2 u kCorrTileBytes<D>, its second words one tile further
   static constexpr uint32_t xl = xh + kCorrTileBytes<D>;
   static constexpr uint32_t a = xh + 4 * kCorrTileBytes<D>;
   static constexpr uint32_t al = a + (D / 64) * kCorrMapHalf<D>;
-  static constexpr uint32_t bars = al + (D / 64) * kCorrMapHalf<D>;    // full[2], done[2]
-  static constexpr uint32_t misc = bars + 32;
+  static constexpr uint32_t bars = al + (D / 64) * kCorrMapHalf<D>;
+  static constexpr uint32_t misc = bars + 72;
   static constexpr uint32_t total = misc + 16;
 };
 static_assert(CorrSmem<128>::total <= 227 * 1024, "shared memory");
 
+// a stage is loaded; stored and free; multiplied (product u in TMEM); the product has been read; the map is loaded
+enum CorrBar { C_FULL = 0, C_EMPTY = 2, C_DONE = 4, C_READ = 6, C_MAP = 8, kCorrBars };
 struct CorrParams {
-  int H, N;
+  int BH, H, N;
   const float* c;                  // [BH][D]
-  __nv_bfloat16* O; i64 os[3];
   int* err;
 };
 
@@ -51,55 +56,74 @@ k_correction_tc(const __grid_constant__ CUtensorMap mapO, const __grid_constant_
   using SM = CorrSmem<D>;
   constexpr int kHalves = D / 64;
   constexpr uint32_t kMapHalf = kCorrMapHalf<D>;
+  constexpr uint32_t FULLW = 0xffffffffu;
   extern __shared__ __align__(1024) unsigned char smem_raw[];
   const uint32_t base = smem_u32(smem_raw);
   volatile int* misc = reinterpret_cast<volatile int*>(smem_raw + SM::misc);   // [0] tmem base, [1] abort, [2] skip
-  const uint32_t bar_full = base + SM::bars, bar_done = bar_full + 16;       // [2] each
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const int bh = blockIdx.y, b = bh / prm.H, h = bh % prm.H;
+  const auto bar = [&](int i) { return base + SM::bars + 8u * i; };
+  const int tid = threadIdx.x, warp = __shfl_sync(FULLW, tid >> 5, 0), lane = tid & 31;
   const int n_tiles = (prm.N + kCorrTile - 1) / kCorrTile;
-  const int tile0 = blockIdx.x * 2;
-  const int nt = min(2, n_tiles - tile0);
+  const i64 total = (i64)prm.BH * n_tiles;
+  const int g0 = (int)(total * blockIdx.x / gridDim.x), count = (int)(total * (blockIdx.x + 1) / gridDim.x) - g0;    // this CTA's tiles
   if (tid == 0) {
     misc[2] = (prm.err != nullptr && *reinterpret_cast<volatile int*>(prm.err) == SPARSEPR_ERR_TIMEOUT) || (base & 1023u) != 0;
     if ((base & 1023u) != 0) set_error(prm.err, SPARSEPR_ERR_CUDA);
-    for (int i = 0; i < 2; ++i) { mbar_init(bar_full + 8 * i, 1); mbar_init(bar_done + 8 * i, 1); }
+    for (int i = 0; i < kCorrBars; ++i) mbar_init(bar(i), i >= C_READ && i < C_MAP ? 256 : 1);
     misc[1] = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   __syncthreads();
   if (misc[2]) return;
-  if (warp == 8) tmem_alloc(base + SM::misc, 256);
+  if (warp == 9) tmem_alloc(base + SM::misc, 256);
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
-  const uint32_t tmem = (uint32_t)misc[0];
+  const uint32_t tmem = __shfl_sync(FULLW, (uint32_t)misc[0], 0);
   volatile int* abort_flag = &misc[1];
 
   if (warp == 8) {
-    if (lane == 0) {
-      // every load of the CTA first: tile 0 with the map, then tile 1
-      for (int u = 0; u < nt; ++u) {
-        const uint32_t bf = bar_full + 8 * u, xb = base + SM::xh + u * 2 * kCorrTileBytes<D>;
-        const int row0 = (tile0 + u) * kCorrTile;
-        mbar_expect_tx(bf, 2 * kCorrTileBytes<D> + (u == 0 ? 2 * kHalves * kMapHalf : 0));
+    int head = -1;
+    for (int k = 0; k < count; ++k) {
+      const int u = k & 1, bh = (g0 + k) / n_tiles, row0 = ((g0 + k) % n_tiles) * kCorrTile;
+      if (!__all_sync(FULLW, mbar_wait(bar(C_EMPTY + u), ((k >> 1) & 1) ^ 1, abort_flag))) break;     // (the first pass completes at once)
+      if (lane == 0) {
+        const uint32_t xb = base + SM::xh + u * 2 * kCorrTileBytes<D>;
+        mbar_expect_tx(bar(C_FULL + u), 2 * kCorrTileBytes<D>);
         for (int c = 0; c < kHalves; ++c) {
-          tma_load_4d(xb + c * kCorrHalf, &mapO, bf, 64 * c, row0, h, b);
-          tma_load_4d(xb + kCorrTileBytes<D> + c * kCorrHalf, &mapL, bf, 64 * c, row0, bh, 0);
-          if (u == 0) {
-            tma_load_4d(base + SM::a + c * kMapHalf, &mapA, bf, 64 * c, 0, bh, 0);
-            tma_load_4d(base + SM::al + c * kMapHalf, &mapA, bf, 64 * c, 0, gridDim.y + bh, 0);      // the second words follow the first ones
-          }
+          tma_load_4d(xb + c * kCorrHalf, &mapO, bar(C_FULL + u), 64 * c, row0, bh % prm.H, bh / prm.H);
+          tma_load_4d(xb + kCorrTileBytes<D> + c * kCorrHalf, &mapL, bar(C_FULL + u), 64 * c, row0, bh, 0);
         }
       }
-      const uint64_t ad = smem_desc(base + SM::a, 16), ald = smem_desc(base + SM::al, 16);
-      const uint32_t idesc = idesc_bf16(0, D);
-      for (int u = 0; u < nt; ++u) {
-        if (!mbar_wait(bar_full + 8 * u, 0, abort_flag)) break;
-        tc_fence_after();
-        const uint64_t hd = smem_desc(base + SM::xh + u * 2 * kCorrTileBytes<D>, 16);
-        const uint64_t ld = smem_desc(base + SM::xl + u * 2 * kCorrTileBytes<D>, 16);
-        const uint32_t d = tmem + 128u * u;
+      __syncwarp();
+      if (bh != head) {                                          // the products with the map before must be complete
+        if (k > 0 && !__all_sync(FULLW, mbar_wait(bar(C_DONE + (u ^ 1)), ((k - 1) >> 1) & 1, abort_flag))) break;
+        head = bh;
+        if (lane == 0) {
+          mbar_expect_tx(bar(C_MAP), 2 * kHalves * kMapHalf);
+          for (int c = 0; c < kHalves; ++c) {
+            tma_load_4d(base + SM::a + c * kMapHalf, &mapA, bar(C_MAP), 64 * c, 0, bh, 0);
+            tma_load_4d(base + SM::al + c * kMapHalf, &mapA, bar(C_MAP), 64 * c, 0, prm.BH + bh, 0);    // the second words follow the first ones
+          }
+        }
+        __syncwarp();
+      }
+    }
+  } else if (warp == 9) {
+    // (the whole warp walks the tiles and one elected lane issues: see attention_tc.cu)
+    const uint64_t ad = smem_desc(base + SM::a, 16), ald = smem_desc(base + SM::al, 16);
+    const uint32_t idesc = idesc_bf16(0, D);
+    int head = -1, maps = 0;
+    bool ok = true;
+    for (int k = 0; k < count && ok; ++k) {
+      const int u = k & 1, bh = (g0 + k) / n_tiles;
+      if (bh != head) { ok = mbar_wait(bar(C_MAP), maps & 1, abort_flag); head = bh; ++maps; }
+      ok = ok && mbar_wait(bar(C_READ + u), ((k >> 1) & 1) ^ 1, abort_flag);
+      ok = __all_sync(FULLW, ok && mbar_wait(bar(C_FULL + u), (k >> 1) & 1, abort_flag));
+      if (!ok) break;
+      tc_fence_after();
+      const uint64_t hd = smem_desc(base + SM::xh + u * 2 * kCorrTileBytes<D>, 16), ld = smem_desc(base + SM::xl + u * 2 * kCorrTileBytes<D>, 16);
+      const uint32_t d = tmem + 128u * u;
+      if (elect_one()) {
 #pragma unroll
         for (int kk = 0; kk < D / 16; ++kk) {
           const uint64_t koff = (uint64_t)((kk >> 2) * (kCorrHalf >> 4) + (kk & 3) * 2), aoff = (uint64_t)((kk >> 2) * (kMapHalf >> 4) + (kk & 3) * 2);
@@ -115,25 +139,27 @@ k_correction_tc(const __grid_constant__ CUtensorMap mapO, const __grid_constant_
           const uint64_t koff = (uint64_t)((kk >> 2) * (kCorrHalf >> 4) + (kk & 3) * 2), aoff = (uint64_t)((kk >> 2) * (kMapHalf >> 4) + (kk & 3) * 2);
           umma_bf16(d, hd + koff, ald + aoff, idesc, 1);
         }
-        umma_commit(bar_done + 8 * u);
+        umma_commit(bar(C_DONE + u));
       }
+      __syncwarp();
     }
   } else {
-    // ---- epilogue: one thread per row; warps 0-3 take tile 0, warps 4-7 tile 1 ---------------------------------
-    const int row = (warp & 3) * 32 + lane;
-    const float* cv = prm.c + (i64)bh * D;
-    for (int u = warp >> 2; u < nt; u += 2) {
-      const bool ok = __all_sync(0xffffffffu, mbar_wait(bar_done + 8 * u, 0, abort_flag));
-      if (!ok) break;
+    // ---- epilogue: a thread takes half the columns of a row -----------------------------------------------------
+    const int wq = warp & 3, hh = warp >> 2, row = wq * 32 + lane;
+    bool ok = true;
+    for (int k = 0; k < count; ++k) {
+      const int u = k & 1, bh = (g0 + k) / n_tiles, row0 = ((g0 + k) % n_tiles) * kCorrTile;
+      ok = __all_sync(FULLW, ok && mbar_wait(bar(C_DONE + u), (k >> 1) & 1, abort_flag));
       tc_fence_after();
-      const int row0 = (tile0 + u) * kCorrTile;
-      __nv_bfloat16* op = prm.O + b * prm.os[0] + h * prm.os[1] + (i64)(row0 + row) * prm.os[2];
-      const unsigned char* hrow = smem_raw + SM::xh + u * 2 * kCorrTileBytes<D> + row * 128;
-      const unsigned char* lrow = smem_raw + SM::xl + u * 2 * kCorrTileBytes<D> + row * 128;
+      const float* cv = prm.c + (i64)bh * D;
+      unsigned char* hrow = smem_raw + SM::xh + u * 2 * kCorrTileBytes<D> + row * 128;
+      const unsigned char* lrow = hrow + kCorrTileBytes<D>;
 #pragma unroll
-      for (int q = 0; q < D / 32; ++q) {
+      for (int q2 = 0; q2 < D / 64; ++q2) {
+        if (!ok) break;
+        const int q = hh * (D / 64) + q2;
         float t[32];
-        tmem_ld32(tmem + ((uint32_t)((warp & 3) * 32) << 16) + 128u * u + q * 32, t);
+        tmem_ld32(tmem + ((uint32_t)(wq * 32) << 16) + 128u * u + q * 32, t);
 #pragma unroll
         for (int ch = 0; ch < 4; ++ch) {
           const int j = (q & 1) * 4 + ch;                                // 16-byte chunk of the 128-byte row
@@ -142,17 +168,27 @@ k_correction_tc(const __grid_constant__ CUtensorMap mapO, const __grid_constant_
           const uint4 rl = *reinterpret_cast<const uint4*>(lrow + so);
           const __nv_bfloat162* hp = reinterpret_cast<const __nv_bfloat162*>(&rh);
           const __nv_bfloat162* lp = reinterpret_cast<const __nv_bfloat162*>(&rl);
-          float v8[8];
+          uint32_t w[4];
 #pragma unroll
-          for (int k = 0; k < 4; ++k) {
-            const float2 fh = __bfloat1622float2(hp[k]), fl = __bfloat1622float2(lp[k]);
-            const int col = q * 32 + ch * 8 + 2 * k;
-            v8[2 * k] = (fh.x + fl.x) + t[ch * 8 + 2 * k] + cv[col];
-            v8[2 * k + 1] = (fh.y + fl.y) + t[ch * 8 + 2 * k + 1] + cv[col + 1];
+          for (int e = 0; e < 4; ++e) {
+            const float2 fh = __bfloat1622float2(hp[e]), fl = __bfloat1622float2(lp[e]);
+            const int col = q * 32 + ch * 8 + 2 * e;
+            w[e] = pack_bf16x2((fh.x + fl.x) + t[ch * 8 + 2 * e] + cv[col], (fh.y + fl.y) + t[ch * 8 + 2 * e + 1] + cv[col + 1]);
           }
-          if (row0 + row < prm.N) store8(op + q * 32 + ch * 8, v8);
+          *reinterpret_cast<uint4*>(hrow + so) = make_uint4(w[0], w[1], w[2], w[3]);
         }
       }
+      tc_fence_before();
+      mbar_arrive(bar(C_READ + u));
+      fence_async_smem();                                                // the copy below reads what was written above
+      asm volatile("bar.sync 1, 256;" ::: "memory");                     // (passed whatever happened)
+      if (tid == 0 && ok) {                                                    // rows past the end of the tensor are not written
+        const uint32_t xb = base + SM::xh + u * 2 * kCorrTileBytes<D>;
+        for (int c = 0; c < kHalves; ++c) tma_store_4d(&mapO, xb + c * kCorrHalf, 64 * c, row0, bh % prm.H, bh / prm.H);
+        bulk_store_wait_read();
+        mbar_arrive(bar(C_EMPTY + u));
+      }
+      __syncwarp();
     }
   }
   tc_fence_before();
@@ -162,7 +198,7 @@ k_correction_tc(const __grid_constant__ CUtensorMap mapO, const __grid_constant_
     if (tid == 0) set_error(prm.err, SPARSEPR_ERR_TIMEOUT);
     __syncthreads();
   }
-  if (warp == 8) {
+  if (warp == 9) {
     tc_fence_after();
     tmem_dealloc(tmem, 256);
   }
@@ -205,9 +241,8 @@ bool launch_correction_tc(const float* c, const __nv_bfloat16* At, const void* O
       !make_map(&ma, At, d, d, 2 * BH, 1, 0, (i64)d * d, d, d))
     return false;
   CorrParams p{};
-  p.H = H; p.N = N; p.c = c; p.O = (__nv_bfloat16*)O; p.err = err;
-  for (int i = 0; i < 3; ++i) p.os[i] = os[i];
-  const dim3 grid(((N + kCorrTile - 1) / kCorrTile + 1) / 2, BH);
+  p.BH = BH; p.H = H; p.N = N; p.c = c; p.err = err;
+  const int grid = (int)std::min<i64>(sm_count(), (i64)BH * ((N + kCorrTile - 1) / kCorrTile));
   if (d == 128) k_correction_tc<128><<<grid, kCorrThreads, CorrSmem<128>::total, st>>>(mo, ml, ma, p);
   else k_correction_tc<64><<<grid, kCorrThreads, CorrSmem<64>::total, st>>>(mo, ml, ma, p);
   return true;
