@@ -508,7 +508,7 @@ def main():
         # float32 path: FP32 CUDA cores, 148 SMs x 128 lanes x 2 flop x max SM clock
         sm_max = (clocks or {}).get("sm_max_mhz") or 1965.0
         peak_alu = 148 * 128 * 2 * sm_max * 1e6 / 1e12
-        roofline = {"kernel": "k_attention_simt (block-sparse)", "bound": "alu", "achieved": achieved,
+        roofline = {"kernel": "k_attention_f32_sparse", "bound": "alu", "achieved": achieved,
                     "peak": peak_alu, "unit": "TFLOP/s", "frac": achieved / peak_alu, "traffic": None,
                     "peak_source": "derived: 148 SM x 128 FP32 lanes x 2 x %.0f MHz" % sm_max,
                     "issued_tflops": issued / (attn_ms * 1e-3) / 1e12}
