@@ -28,7 +28,8 @@
 // own four softmax warps, one row per thread, and its own issuer of both products; P takes the place of S (the
 // accumulators leave no other), so a tile alternates between the tensor cores and its softmax warps, while the other tile does
 // the opposite.  Bound by that chain: product 845 cycles (512 and what the other tile has queued), fetch and maximum 500,
-// exponentials 1200, P V and its completion 750; 3300 cycles per key tile for both, where one tile takes 2010.  The threads have
+// exponentials 1200, P V and its completion 750 (with three pairs of eight by polynomial); 3300 cycles per key tile for both, where one
+// tile takes 2010.  The threads have
 // 224 registers (setmaxnreg).  One pair of eight by polynomial instead of three: a warp alone is short of issue slots, not of
 // the special-function unit (dense, 12 heads of 18944 tokens: 1726 us with three, 1662 with two, 1630 with one, 1644 with none).
 // Dense, 24 heads of 32760 tokens: 12.0 -> 10.1 ms (the clock falls to 1.6 GHz under the power limit); the same two tiles left
