@@ -15,8 +15,8 @@
 //              boxes (tiles of 128 keys, every box inside one group), and publishes the group of every box;
 //   warp  10   V producer
 //   warp  9    issues Q K^T (one thread); owns the TMEM allocation;  warp 11 issues P V (one thread)
-// TMEM: S_0 [0,128), S_1 [128,256), P [256,320), O [320,320+D), Q [448,448+D/2); both products take their A
-// operand from tensor memory.  Reference maxima move lazily (growth beyond 2^8), as in the 128-row kernel.
+// TMEM: S_0 [0,128), S_1 [128,256), P [256,320), O [320,320+D), Q [448,448+D/2); D = 64: second words of P (see the
+// 128-row kernel) [384,448).  Both products take their A operand from tensor memory.  Reference maxima move lazily (growth beyond 2^8), as in the 128-row kernel.
 // Every mbarrier wait is bounded; on expiry the CTA records SPARSEPR_ERR_TIMEOUT and leaves.
 #include <cuda.h>
 #include "kernels.cuh"
@@ -28,6 +28,7 @@ namespace packed {
 
 constexpr int kThreads = 384;
 constexpr int kPolyOf8 = 3;                           // pairs of every 8 whose exponential is a polynomial on the FMA pipe
+template <int D> constexpr bool kTwoWords = D == 64;  // P as two bf16 words, every exponential ex2.approx
 constexpr int kTile = 128;
 constexpr int kSub = 16;                               // rows per TMA box of the K/V stream
 constexpr int kSubPerTile = kTile / kSub;
@@ -258,8 +259,10 @@ k_attention_packed(const __grid_constant__ Maps mapsK, const __grid_constant__ M
         if (elect_one()) {
 #pragma unroll
           for (int kk = 0; kk < kSubPerTile; ++kk)
-            if (kk < nsub)
-              umma_bf16_ts(tmem + 320u, tmem + 256u + kk * 8, vd + (uint64_t)(kk * (kSubBytes >> 4)), idesc_pv, (i > 0 || kk > 0) ? 1u : 0u);
+            if (kk < nsub) {
+              umma_bf16_ts(tmem + 320u, tmem + 256u + kk * 8, vd + (uint64_t)(kk * (kSubBytes >> 4)), idesc_pv, (!kTwoWords<D> && i > 0) || kk > 0 ? 1u : 0u);
+              if constexpr (kTwoWords<D>) umma_bf16_ts(tmem + 320u, tmem + 384u + kk * 8, vd + (uint64_t)(kk * (kSubBytes >> 4)), idesc_pv, 1u);
+            }
           umma_commit(bar(V_EMPTY + s));
           umma_commit(bar(P_EMPTY));
         }
@@ -297,6 +300,14 @@ k_attention_packed(const __grid_constant__ Maps mapsK, const __grid_constant__ M
       mbar_arrive(bar(Q_FULL));
     }
     float m_ref = -INFINITY, l = 0.f;
+    float oa[kTwoWords<D> ? kOc : 1];                          // D = 64: sum of the tiles but the last, whose share lies in tensor memory
+#pragma unroll
+    for (float& v : oa) v = 0.f;
+    auto take = [&](float f) {
+      float t[32];
+      tmem_ld32(o_addr, t);
+      add_share(oa, t, f, f, __all_sync(FULL, f == 1.f));
+    };
     bool ok = true;
     for (int i = 0; i < n_tiles; ++i) {
       // the barriers of this tile are polled back to back (their shared-memory round trips overlap)
@@ -365,7 +376,7 @@ k_attention_packed(const __grid_constant__ Maps mapsK, const __grid_constant__ M
       // the tensor cores still work on the previous tile.
       bool p_free = i == 0;
       if (!__all_sync(FULL, ok)) { ok = false; continue; }
-      if (i > 0 && __any_sync(FULL, rescale)) {
+      if (!kTwoWords<D> && i > 0 && __any_sync(FULL, rescale)) {
         ok = __all_sync(FULL, mbar_wait(bar(P_EMPTY), (i - 1) & 1, abort_flag));
         if (!ok) continue;
         p_free = true;
@@ -379,7 +390,7 @@ k_attention_packed(const __grid_constant__ Maps mapsK, const __grid_constant__ M
           tmem_st32(o_addr + q * 32, t);
         }
       }
-      // exponentials: kPolyOf8 of every 8 pairs on the FMA pipe, the others on the special-function unit;
+      // exponentials: kPolyOf8 of every 8 pairs on the FMA pipe (D = 64: none), the others on the special-function unit;
       // masked columns give exactly 0 on both.  A box that no row of this warp routes to (a warp holds the
       // remainders of few query groups, and a group routes to a fraction of the K/V groups) is all zeros:
       // its exponentials are skipped for the whole warp.
@@ -394,7 +405,7 @@ k_attention_packed(const __grid_constant__ Maps mapsK, const __grid_constant__ M
 #pragma unroll
           for (int q = bx * 8; q < bx * 8 + 8; ++q) {
             float2 x = __ffma2_rn(make_float2(s[2 * q], s[2 * q + 1]), sc2, mneg2);
-            if ((q & 7) < kPolyOf8) x = ex2_poly2(x);
+            if (!kTwoWords<D> && (q & 7) < kPolyOf8) x = ex2_poly2(x);
             else { x.x = ex2(x.x); x.y = ex2(x.y); }
             s[2 * q] = x.x; s[2 * q + 1] = x.y;
             ps2[q & 1] = __fadd2_rn(ps2[q & 1], x);
@@ -410,8 +421,14 @@ k_attention_packed(const __grid_constant__ Maps mapsK, const __grid_constant__ M
           ok = __all_sync(FULL, mbar_wait(bar(P_EMPTY), (i - 1) & 1, abort_flag));
           if (!ok) continue;
           tc_fence_after();
+          if constexpr (kTwoWords<D>) take(rescale ? corr : 1.f);
         }
         tmem_st32u(p_addr, w);
+        if constexpr (kTwoWords<D>) {
+#pragma unroll
+          for (int c = 0; c < 32; ++c) w[c] = pack_bf16x2_rest(s[2 * c], s[2 * c + 1], w[c]);
+          tmem_st32u(p_addr + 128u, w);
+        }
       }
       tc_fence_before();
       mbar_arrive(bar(P_FULL));
@@ -428,6 +445,11 @@ k_attention_packed(const __grid_constant__ Maps mapsK, const __grid_constant__ M
 #pragma unroll
       for (int c = 0; c < kOc; ++c) o[c] = 0.f;
       if (n_tiles > 0) {
+        if constexpr (kTwoWords<D>) {
+          take(1.f);
+#pragma unroll
+          for (int c = 0; c < kOc; ++c) o[c] = inv != 0.f ? oa[c] * inv : 0.f;
+        } else
 #pragma unroll
         for (int q = 0; q < kOc / 32; ++q) {
           float t[32];

@@ -1,5 +1,9 @@
-// Block-sparse / dense attention on the sm_100a tensor cores (bf16, D = d = d_v = 64 or 128; at 64 the products are half
-// as long and the softmax threads, which set the pace, do the same work per score).
+// Block-sparse / dense attention on the sm_100a tensor cores (bf16, D = d = d_v = 64 or 128).  At D = 64 the probabilities keep the
+// float32 precision that the CUDA-core kernels of this head dimension gave them: they enter P V as two bf16 words (two products, as
+// long together as the one at D = 128; tensor memory has the room), every exponential takes ex2.approx, and the product of a key
+// tile is a sum of its own that the softmax threads add up in float32 (the accumulator of the tensor cores drops what does not fit
+// when a term is added: 1.0e-5 with one running sum).  Error of the hard-drop rows against float64 at 17550 tokens: 4.8e-7; with one
+// word 2.0e-4, of the CUDA-core kernels 1.2e-6.  Attention stage of 16 such heads: 1.12 ms (one word 0.90, CUDA cores 12.2).
 //
 // One CTA processes one 128-row query tile, or two of the same query group (of one query group, Eq. 3; or of the whole
 // head for dense attention, Eq. 1).  With one tile, roles:
@@ -17,7 +21,7 @@
 //                        runs two tiles ahead of the softmax
 //   P_b = exp2(.)        softmax threads: tcgen05.ld their half row of S_b, row maximum (the two halves meet
 //                        through shared memory), bf16 P to TMEM columns of its own (two buffers as well);
-//                        3 of every 8 exponentials are a cubic on the FMA pipe, the others use ex2.approx
+//                        3 of every 8 exponentials are a cubic on the FMA pipe, the others use ex2.approx (D = 64: all of them)
 //   O  += P V_i          tcgen05.mma with the A operand read from TMEM; O stays in TMEM
 // A single issuing thread shares its warp scheduler with two softmax warps that rarely leave it an issue slot:
 // this is why the two products have a thread each on different schedulers, why the producers issue few, large
@@ -63,6 +67,7 @@ template <int D> constexpr uint32_t kTileBytes = (D / 64) * kHalfBytes;      // 
 constexpr uint32_t kSubBytes = kSub * 128;            // 2 KB per box
 constexpr int kPolyOf8 = 3;            // pairs of every 8 whose exponential is a polynomial on the FMA pipe
 constexpr int kPairPolyOf8 = 1;        // the same with two query tiles per CTA
+template <int D> constexpr bool kTwoWords = D == 64;   // P as two bf16 words
 constexpr int kKStages = 2;            // K tiles in flight (consumed by Q K^T)
 constexpr int kVStages = 2;            // V tiles in flight (consumed by P V)
 constexpr int kSoftmaxRegs = 224, kOtherRegs = 56;     // registers per thread after the split: 128 (2 x 224 + 56) = the 384 x 168 of the launch
@@ -259,7 +264,8 @@ k_attention_tc(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__
     }
   } else if constexpr (PAIR) {
     // =========================== two query tiles: issuer of both products of tile x (warps 9 and 11) =======
-    // TMEM columns: S_x [128 x, 128 x + 128), P_x over its first 64 once the scores are in registers, O_x [256 + 128 x, ... + D).
+    // TMEM columns: S_x [128 x, 128 x + 128), P_x over its first 64 (second words: over the others) once the scores are in registers,
+    // O_x [256 + 128 x, ... + D).
     // (As below, the whole warp walks the tiles and one elected lane issues.)
     if (n_tiles > 0) {
       const int x = warp == 9 ? 0 : 1;
@@ -295,7 +301,10 @@ k_attention_tc(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__
           if (elect_one()) {
 #pragma unroll
             for (int kk = part ? 6 : 0; kk < (part ? 8 : 6); ++kk)
-              if (kk < nsub) umma_bf16_ts(ox, sx + kk * 8, vd + (uint64_t)(kk * (kSubBytes >> 4)), idesc_pv, (i > 0 || kk > 0) ? 1u : 0u);
+              if (kk < nsub) {
+                umma_bf16_ts(ox, sx + kk * 8, vd + (uint64_t)(kk * (kSubBytes >> 4)), idesc_pv, (!kTwoWords<D> && i > 0) || kk > 0 ? 1u : 0u);
+                if constexpr (kTwoWords<D>) umma_bf16_ts(ox, sx + 64u + kk * 8, vd + (uint64_t)(kk * (kSubBytes >> 4)), idesc_pv, 1u);
+              }
             if (part == 1) { umma_commit(bar(V_EMPTY + s)); umma_commit(bar(PV_DONE + x)); }
           }
           __syncwarp();
@@ -304,7 +313,10 @@ k_attention_tc(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__
     }
   } else if (warp == 9) {
     // =========================== Q K^T issuer ============================================
-    // TMEM columns: S_0 [0,128), S_1 [128,256), P_0 [256,320) and P_1 [448,512) (two bf16 per column), O [320,320+D).
+    // TMEM columns: S_0 [0,128), S_1 [128,256), P_0 [256,320) and P_1 [448,512) (two bf16 per column), O [320,320+D); D = 64: O_0 [320,384),
+    // O_1 [384,448), of tiles in turn.  The second words
+    // of P_b take the place of its scores: a thread's 32 columns of them lie over the 64 scores that only it reads, so the next
+    // product into the buffer waits for P V instead of the scores' way into registers (the products still run a tile ahead).
     // The two products are issued by two threads on different warp schedulers: an issuing thread shares its
     // scheduler with two softmax warps that rarely leave it a slot, and the score tile two steps ahead must not
     // queue behind the P V of the current one.
@@ -320,8 +332,8 @@ k_attention_tc(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__
       bool ok = __all_sync(FULLW, mbar_wait(bar(Q_FULL), 0, abort_flag));
       for (int i = 0; i < n_tiles && ok; ++i) {
         const int s = i % kKStages;
-        // score buffer i mod 2 is free once every softmax thread holds tile i - 2 in registers
-        if (i >= 2) ok = mbar_wait(bar(S_FREE + (i & 1)), ((i - 2) >> 1) & 1, abort_flag);
+        // score buffer i mod 2 is free once every softmax thread holds tile i - 2 in registers (second words: once they are consumed)
+        if (i >= 2) ok = mbar_wait(bar((kTwoWords<D> ? P_EMPTY : S_FREE) + (i & 1)), ((i - 2) >> 1) & 1, abort_flag);
         ok = __all_sync(FULLW, ok && mbar_wait(bar(K_FULL + s), (i / kKStages) & 1, abort_flag));
         if (!ok) break;
         tc_fence_after();
@@ -353,14 +365,17 @@ k_attention_tc(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__
         ok = __all_sync(FULLW, ok && mbar_wait(bar(P_FULL + (i & 1)), (i >> 1) & 1, abort_flag));   // P(i) in TMEM, O rescaled if needed
         if (!ok) break;
         tc_fence_after();
-        const uint32_t d = tmem + 320u;
+        const uint32_t d = tmem + 320u + (kTwoWords<D> ? (uint32_t)(i & 1) * 64u : 0u);
         const uint32_t pa = tmem + ((i & 1) ? 448u : 256u);
         const uint64_t vd = v_desc0 + (uint64_t)(s * (kTileBytes<D> >> 4));
         if (elect_one()) {
 #pragma unroll
           for (int kk = 0; kk < kSubPerTile; ++kk)
-            if (kk < nsub)
-              umma_bf16_ts(d, pa + kk * 8, vd + (uint64_t)(kk * (kSubBytes >> 4)), idesc_pv, (i > 0 || kk > 0) ? 1u : 0u);
+            if (kk < nsub) {
+              umma_bf16_ts(d, pa + kk * 8, vd + (uint64_t)(kk * (kSubBytes >> 4)), idesc_pv, (!kTwoWords<D> && i > 0) || kk > 0 ? 1u : 0u);
+              if constexpr (kTwoWords<D>)
+                umma_bf16_ts(d, tmem + (uint32_t)(i & 1) * 128u + (kk >> 2) * 64 + (kk & 3) * 8, vd + (uint64_t)(kk * (kSubBytes >> 4)), idesc_pv, 1u);
+            }
           umma_commit(bar(V_EMPTY + s));
           umma_commit(bar(P_EMPTY + (i & 1)));
         }
@@ -377,6 +392,17 @@ k_attention_tc(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__
     const uint32_t s_addr = tmem + ((uint32_t)((warp & 3) * 32) << 16) + 128u * (uint32_t)x, o_addr = s_addr + 256u;
     const float sc = prm.scale_log2;
     float m_ref = -INFINITY, l = 0.f;
+    float oa[kTwoWords<D> ? D : 1];                              // the row's sum of the tiles before (D = 64)
+#pragma unroll
+    for (float& v : oa) v = 0.f;
+    auto take = [&] {                                            // ... plus the last one's share
+#pragma unroll
+      for (int q = 0; q < D / 32; ++q) {
+        float t[32];
+        tmem_ld32(o_addr + q * 32, t);
+        add_share(oa + q * 32, t, 1.f, 1.f, true);
+      }
+    };
     bool ok = true;
     // The warps of the two tiles that share a scheduler take turns with their exponentials (barriers 1 + w and 5 + w: tile 0,
     // tile 1 may go): left to themselves the tiles fall into step, and then wait for the tensor cores together and compete
@@ -394,6 +420,7 @@ k_attention_tc(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__
       if (ok) {
         tc_fence_after();
         const uint2 mt = meta[i & 7];
+        if constexpr (kTwoWords<D>) { if (i > 0) take(); }       // (the previous P V is complete: S_FULL says so)
 #pragma unroll
         for (int q = 0; q < 4; ++q) tmem_ld32_nowait(s_addr + 32 * q, s[q]);
         tmem_ld_wait();
@@ -422,6 +449,10 @@ k_attention_tc(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__
         mneg = -m_new * sc;
         m_ref = m_new;
         if (i > 0 && __any_sync(FULLW, move)) {                  // rescale the rows of this warp (rare); the previous P V is complete: S_FULL says so
+          if constexpr (kTwoWords<D>) {
+#pragma unroll
+            for (float& v : oa) v *= corr;
+          } else
 #pragma unroll 1
           for (int q = 0; q < D / 32; ++q) {
             float t[32];
@@ -439,16 +470,18 @@ k_attention_tc(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__
         const float2 sc2 = make_float2(sc, sc), mneg2 = make_float2(mneg, mneg);
 #pragma unroll
         for (int q = 0; q < 4; ++q) {
-          uint32_t w[16];
+          uint32_t w[16], wl[kTwoWords<D> ? 16 : 1];
 #pragma unroll
           for (int c = 0; c < 16; ++c) {
             float2 e = __ffma2_rn(make_float2(s[q][2 * c], s[q][2 * c + 1]), sc2, mneg2);
-            if ((c & 7) < kPairPolyOf8) e = ex2_poly2(e);
+            if (!kTwoWords<D> && (c & 7) < kPairPolyOf8) e = ex2_poly2(e);
             else { e.x = ex2(e.x); e.y = ex2(e.y); }
             ps2[c & 1] = __fadd2_rn(ps2[c & 1], e);
             w[c] = pack_bf16(e.x, e.y);
+            if constexpr (kTwoWords<D>) wl[c] = pack_bf16x2_rest(e.x, e.y, w[c]);
           }
           tmem_st16u_nowait(s_addr + 16 * q, w);
+          if constexpr (kTwoWords<D>) tmem_st16u_nowait(s_addr + 64 + 16 * q, wl);
           if (q >= 2) {
             tmem_st_wait();
             tc_fence_before();
@@ -465,6 +498,7 @@ k_attention_tc(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__
     const int rows = min(kTile, nrows - x * kTile);
     const int* dst = dsts + x * kTile;
     tc_fence_after();
+    if constexpr (kTwoWords<D>) { if (ok && n_tiles > 0) take(); }   // (uniform)
     // Coalesced stores, as below, but a warp stages and writes its own rows, one of the two words at a time, in the place
     // of its query rows (the other tile may still be reading the rings); 16-byte pieces are permuted within a row by the
     // row number, so that a quarter warp meets different banks both ways.
@@ -472,10 +506,15 @@ k_attention_tc(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__
     constexpr int kLpr = D / 8, kRpi = 32 / kLpr;                // pieces (lanes) per row, rows per step of a warp
 #pragma unroll 1
     for (int word = 0; word < (prm.O_lo ? 2 : 1); ++word) {
-#pragma unroll 1
+#pragma unroll (kTwoWords<D> ? D / 32 : 1)
       for (int q = 0; q < D / 32; ++q) {
         float t[32];
-        if (ok && n_tiles > 0) tmem_ld32(o_addr + q * 32, t);    // (uniform)
+        if constexpr (kTwoWords<D>) {
+#pragma unroll
+          for (int c = 0; c < 32; ++c) t[c] = oa[q * 32 + c];
+        } else {
+          if (ok && n_tiles > 0) tmem_ld32(o_addr + q * 32, t);  // (uniform)
+        }
 #pragma unroll
         for (int c = 0; c < 32; ++c) t[c] = ok && n_tiles > 0 && inv != 0.f ? t[c] * inv : 0.f;
         if (word == 0 && prm.O_sparse && ok && row < rows) {
@@ -517,6 +556,19 @@ k_attention_tc(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__
     float m_ref = -INFINITY, l = 0.f;
     bool ok = true;
     const float sc = prm.scale_log2;
+    // D = 64: sum of the tiles but the last two, whose shares lie in tensor memory; corr_prev: the rescaling since the one before the last
+    float oa[kTwoWords<D> ? kOc : 1], corr_prev = 1.f;
+#pragma unroll
+    for (float& v : oa) v = 0.f;
+    auto take = [&](int i, float fo, float ft) {                 // the share of tile i
+      float t[32];
+      tmem_ld32(o_addr + (uint32_t)(i & 1) * 64u, t);
+      add_share(oa, t, fo, ft, __all_sync(FULL, fo == 1.f && ft == 1.f));
+    };
+    auto take_last = [&] {
+      if (n_tiles > 1) take(n_tiles - 2, 1.f, corr_prev);
+      take(n_tiles - 1, 1.f, 1.f);
+    };
     // the finished output columns [kOc hh, kOc hh + kOc) of tile row r: bf16 at the original token index, the part that
     // the rounding dropped as a second word, float32 on request
     auto store_row = [&](int r, const float (&o)[kOc]) {
@@ -573,8 +625,10 @@ k_attention_tc(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__
           const uint2 mt = meta[i & 7];
           tmem_ld32_nowait(tmem + lane_addr + (uint32_t)(i & 1) * 128u + (uint32_t)cb, s);
           tmem_ld_wait();
-          tc_fence_before();
-          mbar_arrive(bar(S_FREE + (i & 1)));                       // the scores are in registers
+          if constexpr (!kTwoWords<D>) {
+            tc_fence_before();
+            mbar_arrive(bar(S_FREE + (i & 1)));                     // the scores are in registers
+          }
           if (!(mt.x == 0xFFFFFFFFu && mt.y == 8u)) {
 #pragma unroll
             for (int bx = 0; bx < 2; ++bx) {
@@ -609,7 +663,10 @@ k_attention_tc(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__
           tc_fence_after();
         }
         if (!ok) continue;
-        if (i > 0 && __any_sync(FULL, move)) {                   // rescale this half of the lane's accumulator (rare)
+        if constexpr (kTwoWords<D>) {
+          if (i > 1) take(i - 2, corr, corr_prev * corr);        // (its product is complete: P_EMPTY says so)
+          corr_prev = corr;
+        } else if (i > 0 && __any_sync(FULL, move)) {            // rescale this half of the lane's accumulator (rare)
           ok = __all_sync(FULL, mbar_wait(bar(P_EMPTY + ((i - 1) & 1)), ((i - 1) >> 1) & 1, abort_flag));
           if (!ok) continue;
           tc_fence_after();
@@ -627,7 +684,7 @@ k_attention_tc(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__
 #pragma unroll
         for (int q = 0; q < 16; ++q) {
           float2 x = __ffma2_rn(make_float2(s[2 * q], s[2 * q + 1]), sc2, mneg2);
-          if ((q & 7) < kPolyOf8) x = ex2_poly2(x);
+          if (!kTwoWords<D> && (q & 7) < kPolyOf8) x = ex2_poly2(x);
           else { x.x = ex2(x.x); x.y = ex2(x.y); }
           s[2 * q] = x.x; s[2 * q + 1] = x.y;
           ps2[q & 1] = __fadd2_rn(ps2[q & 1], x);
@@ -642,6 +699,13 @@ k_attention_tc(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__
           const uint32_t pa = p_addr0 + (uint32_t)(i & 1) * 192u;
           tmem_st16u_nowait(pa + 16u * (uint32_t)u, w);
           tmem_st16u_nowait(pa + 16u * (uint32_t)(1 - u), z);
+          if constexpr (kTwoWords<D>) {
+#pragma unroll
+            for (int c = 0; c < 16; ++c) w[c] = pack_bf16x2_rest(s[2 * c], s[2 * c + 1], w[c]);
+            const uint32_t pl = tmem + lane_addr + (uint32_t)(i & 1) * 128u + (uint32_t)hh * 64u;
+            tmem_st16u_nowait(pl + 16u * (uint32_t)u, w);
+            tmem_st16u_nowait(pl + 16u * (uint32_t)(1 - u), z);
+          }
           tmem_st_wait();
         }
         tc_fence_before();
@@ -655,6 +719,11 @@ k_attention_tc(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__
       for (int c = 0; c < kOc; ++c) o[c] = 0.f;
       if (ok && n_tiles > 0) {
         tc_fence_after();
+        if constexpr (kTwoWords<D>) {
+          take_last();
+#pragma unroll
+          for (int c = 0; c < kOc; ++c) o[c] = oa[c];
+        } else
 #pragma unroll
         for (int q = 0; q < kOc / 32; ++q) {
           float t[32];
@@ -700,8 +769,10 @@ k_attention_tc(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__
         tmem_ld32_nowait(s_addr, *reinterpret_cast<float(*)[32]>(&s[0]));
         tmem_ld32_nowait(s_addr + 32, *reinterpret_cast<float(*)[32]>(&s[32]));
         tmem_ld_wait();
-        tc_fence_before();
-        mbar_arrive(bar(S_FREE + (i & 1)));                         // the scores are in registers
+        if constexpr (!kTwoWords<D>) {
+          tc_fence_before();
+          mbar_arrive(bar(S_FREE + (i & 1)));                       // the scores are in registers
+        }
         if (!(mt.x == 0xFFFFFFFFu && mt.y == 8u)) {
           // only the boxes that end a key range (or lie beyond the stream) have columns to mask; the test is uniform
 #pragma unroll
@@ -738,7 +809,10 @@ k_attention_tc(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__
         tc_fence_after();
       }
       if (!ok) continue;                                         // warp-uniform; the pair barrier above has been passed
-      if (i > 0 && __any_sync(FULL, move)) {                     // rescale this half of the warp's O rows (rare)
+      if constexpr (kTwoWords<D>) {
+        if (i > 1) take(i - 2, corr, corr_prev * corr);          // (its product is complete: P_EMPTY says so)
+        corr_prev = corr;
+      } else if (i > 0 && __any_sync(FULL, move)) {              // rescale this half of the warp's O rows (rare)
         // O must be at rest: the product of the previous tile has to be complete as well
         ok = __all_sync(FULL, mbar_wait(bar(P_EMPTY + ((i - 1) & 1)), ((i - 1) >> 1) & 1, abort_flag));
         if (!ok) continue;
@@ -758,7 +832,7 @@ k_attention_tc(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__
 #pragma unroll
       for (int q = 0; q < 32; ++q) {
         float2 x = __ffma2_rn(make_float2(s[2 * q], s[2 * q + 1]), sc2, mneg2);
-        if ((q & 7) < kPolyOf8) x = ex2_poly2(x);
+        if (!kTwoWords<D> && (q & 7) < kPolyOf8) x = ex2_poly2(x);
         else { x.x = ex2(x.x); x.y = ex2(x.y); }
         s[2 * q] = x.x; s[2 * q + 1] = x.y;
         ps2[q & 1] = __fadd2_rn(ps2[q & 1], x);
@@ -770,6 +844,11 @@ k_attention_tc(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__
 #pragma unroll
         for (int c = 0; c < 32; ++c) w[c] = pack_bf16(s[2 * c], s[2 * c + 1]);
         tmem_st32u(p_addr0 + (uint32_t)(i & 1) * 192u, w);
+        if constexpr (kTwoWords<D>) {
+#pragma unroll
+          for (int c = 0; c < 32; ++c) w[c] = pack_bf16x2_rest(s[2 * c], s[2 * c + 1], w[c]);
+          tmem_st32u(tmem + lane_addr + (uint32_t)(i & 1) * 128u + (uint32_t)hh * 64u, w);
+        }
       }
       tc_fence_before();
       mbar_arrive(bar(P_FULL + (i & 1)));
@@ -786,6 +865,11 @@ k_attention_tc(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__
     for (int c = 0; c < kOc; ++c) o[c] = 0.f;
     if (ok && n_tiles > 0) {
       tc_fence_after();
+      if constexpr (kTwoWords<D>) {
+        take_last();
+#pragma unroll
+        for (int c = 0; c < kOc; ++c) o[c] = inv != 0.f ? oa[c] * inv : 0.f;
+      } else
 #pragma unroll
       for (int q = 0; q < kOc / 32; ++q) {
         float t[32];

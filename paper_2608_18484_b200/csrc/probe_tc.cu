@@ -12,7 +12,9 @@
 //   warp  10   tcgen05.mma issuer, owns TMEM
 // TMEM: S0 [0,128), S1 [128,256), O_S [256,256+D), O_U [384,384+D).  The exponentials of a tile
 // are written back over its score buffer as bf16: retained weights in columns [0,64),
-// omitted weights in [64,128); the two P V products read them from TMEM.
+// omitted weights in [64,128); the two P V products read them from TMEM.  D = 64: weights as two bf16 words (see
+// attention_tc.cu), the second ones in [320,384) (retained) and [448,512) (omitted), free once the products of the tile
+// before are complete.
 #include "kernels.cuh"
 #include "tc_common.cuh"
 
@@ -60,6 +62,7 @@ k_probe_rows_tc(const __grid_constant__ CUtensorMap mapQ, const __grid_constant_
                 const __grid_constant__ CUtensorMap mapV, PbParams prm) {
   using SM = PbSmem<D>;
   constexpr int kHalves = D / 64, kOc = D / 2;                             // 64-column blocks of a row; output columns of a thread
+  constexpr bool kTwoWords = D == 64;                                      // weights as two bf16 words
   extern __shared__ __align__(1024) unsigned char smem_raw[];
   const uint32_t base = smem_u32(smem_raw);
   unsigned char* sm = smem_raw;
@@ -203,10 +206,12 @@ k_probe_rows_tc(const __grid_constant__ CUtensorMap mapQ, const __grid_constant_
 #pragma unroll
           for (int which = 0; which < 2; ++which)               // retained weights -> O_S, omitted -> O_U
 #pragma unroll
-            for (int kk = 0; kk < 8; ++kk)
-              umma_bf16_ts(tmem + 256u + which * 128u, pbuf + which * 64u + kk * 8, vd + (uint64_t)(kk * 128), idesc_pv, (i > 0 || kk > 0) ? 1u : 0u);
+            for (int kk = 0; kk < 8; ++kk) {
+              umma_bf16_ts(tmem + 256u + which * 128u, pbuf + which * 64u + kk * 8, vd + (uint64_t)(kk * 128), idesc_pv, (!kTwoWords && i > 0) || kk > 0 ? 1u : 0u);
+              if constexpr (kTwoWords) umma_bf16_ts(tmem + 256u + which * 128u, tmem + 320u + which * 128u + kk * 8, vd + (uint64_t)(kk * 128), idesc_pv, 1u);
+            }
           umma_commit(bar(PV_EMPTY + s));
-          umma_commit(bar(PT_DONE));                            // O_S / O_U hold every tile up to i
+          umma_commit(bar(PT_DONE));                            // O_S / O_U hold every tile up to i (D = 64: this one)
         }
         __syncwarp();
       }
@@ -223,6 +228,18 @@ k_probe_rows_tc(const __grid_constant__ CUtensorMap mapQ, const __grid_constant_
     float* xmax = reinterpret_cast<float*>(sm + SM::xchg);             // [parity][half][state][row]
     float* xsum = xmax + 8 * 128;                                          // [half][state][row]
     float mS = -INFINITY, mU = -INFINITY, lS = 0.f, lU = 0.f;
+    float oa[kTwoWords ? 2 : 1][kTwoWords ? 32 : 1];           // D = 64: both sums of the tiles but the last, whose share lies in tensor memory
+#pragma unroll
+    for (auto& o : oa) for (float& v : o) v = 0.f;
+    auto take = [&](float fS, float fU) {
+#pragma unroll
+      for (int which = 0; which < 2; ++which) {
+        const float f = which ? fU : fS;
+        float t[32];
+        tmem_ld32(tmem + lane_addr + 256u + which * 128u + (uint32_t)(hh * kOc), t);
+        add_share(oa[which], t, f, f, __all_sync(FULL, f == 1.f));
+      }
+    };
     bool ok = true;
     int pos = p_begin, i = 0;
     for (; pos < p_end; ++i) {
@@ -287,7 +304,10 @@ k_probe_rows_tc(const __grid_constant__ CUtensorMap mapQ, const __grid_constant_
       // the accumulators are stable once the previous P V products have completed
       if (i > 0) ok = __all_sync(FULL, ok && mbar_wait(bar(PT_DONE), (i - 1) & 1, abort_flag));
       if (!ok) break;
-      if (i > 0 && __any_sync(FULL, moveS || moveU)) {           // rescale this half of the O_S / O_U rows (rare)
+      if constexpr (kTwoWords) {
+        tc_fence_after();
+        if (i > 0) take(cS, cU);
+      } else if (i > 0 && __any_sync(FULL, moveS || moveU)) {    // rescale this half of the O_S / O_U rows (rare)
         tc_fence_after();
 #pragma unroll
         for (int q = 0; q < 2 * (kOc / 32); ++q) {
@@ -303,35 +323,35 @@ k_probe_rows_tc(const __grid_constant__ CUtensorMap mapQ, const __grid_constant_
       }
       const float nS = mS > -INFINITY ? -mS * sc : 0.f, nU = mU > -INFINITY ? -mU * sc : 0.f;
       float sumS = 0.f, sumU = 0.f;
-      // exponentials, packed in place: afterwards s[2j] holds the bf16 pair of retained weights of
-      // columns (2j, 2j+1) of this half and s[2j+1] the pair of omitted weights
+      // exponentials, 32 columns at a time: bf16 pairs of the retained and of the omitted weights (and their second words)
 #pragma unroll
-      for (int j = 0; j < 32; ++j) {
-        float eS[2], eU[2];
+      for (int half = 0; half < 2; ++half) {
 #pragma unroll
-        for (int u = 0; u < 2; ++u) {
-          const int c = 2 * j + u;
-          const bool r = (ret[c >> 5] >> (c & 31)) & 1u;
-          const float e = ex2(fmaf(s[c], sc, r ? nS : nU));     // masked columns: exp2(-inf) = 0
-          eS[u] = r ? e : 0.f;
-          eU[u] = r ? 0.f : e;
-          sumS += eS[u];
-          sumU += eU[u];
+        for (int j = 0; j < 32; ++j) {
+          const bool r = (ret[half] >> j) & 1u;
+          const float e = ex2(fmaf(s[32 * half + j], sc, r ? nS : nU));     // masked columns: exp2(-inf) = 0
+          sumS += r ? e : 0.f;
+          sumU += r ? 0.f : e;
+          s[32 * half + j] = e;
         }
-        s[2 * j] = __uint_as_float(pack_bf16x2(eS[0], eS[1]));
-        s[2 * j + 1] = __uint_as_float(pack_bf16x2(eU[0], eU[1]));
+        const uint32_t at = 32u * (uint32_t)hh + 16u * (uint32_t)half;      // keys [64 hh + 32 half, ... + 32)
+#pragma unroll
+        for (int which = 0; which < 2; ++which) {
+          const unsigned on = which ? ~ret[half] : ret[half];
+          uint32_t w[16], x[kTwoWords ? 16 : 1];
+#pragma unroll
+          for (int j = 0; j < 16; ++j) {
+            const float e0 = (on >> (2 * j)) & 1u ? s[32 * half + 2 * j] : 0.f, e1 = (on >> (2 * j + 1)) & 1u ? s[32 * half + 2 * j + 1] : 0.f;
+            w[j] = pack_bf16x2(e0, e1);
+            if constexpr (kTwoWords) x[j] = pack_bf16x2_rest(e0, e1, w[j]);
+          }
+          tmem_st16u_nowait(s_addr + 64u * which + at, w);
+          if constexpr (kTwoWords) tmem_st16u_nowait(tmem + lane_addr + 320u + 128u * which + at, x);
+        }
       }
+      tmem_st_wait();
       lS = lS * cS + sumS;
       lU = lU * cU + sumU;
-      {
-        uint32_t w[32];
-#pragma unroll
-        for (int c = 0; c < 32; ++c) w[c] = __float_as_uint(s[2 * c]);
-        tmem_st32u(s_addr + 32 * hh, w);                        // retained weights of keys [64 hh, 64 hh + 64)
-#pragma unroll
-        for (int c = 0; c < 32; ++c) w[c] = __float_as_uint(s[2 * c + 1]);
-        tmem_st32u(s_addr + 64 + 32 * hh, w);                   // omitted weights
-      }
       tc_fence_before();
       mbar_arrive(bar(PP_FULL + (i & 1)));
     }
@@ -351,6 +371,17 @@ k_probe_rows_tc(const __grid_constant__ CUtensorMap mapQ, const __grid_constant_
     }
     if (ok && any) {
       tc_fence_after();
+      if constexpr (kTwoWords) {
+        take(1.f, 1.f);
+        if (row < nrows) {
+#pragma unroll
+          for (int which = 0; which < 2; ++which) {
+            float* out = prm.partial + ((((i64)bh * prm.n_split + split) * prm.M + m0 + row) * 2 + which) * (D + 2) + 2 + hh * kOc;
+#pragma unroll
+            for (int c = 0; c < 32; ++c) out[c] = oa[which][c];
+          }
+        }
+      } else
 #pragma unroll
       for (int q = 0; q < 2 * (kOc / 32); ++q) {                // this half's columns of O_S, then of O_U
         constexpr int kQ = kOc / 32;

@@ -162,6 +162,22 @@ __device__ __forceinline__ uint32_t pack_bf16x2(float a, float b) {      // a in
   __nv_bfloat162 h = __floats2bfloat162_rn(a, b);
   return *reinterpret_cast<uint32_t*>(&h);
 }
+// what the rounding of (a, b) to the pair `hi` dropped, as a second bf16 pair
+__device__ __forceinline__ uint32_t pack_bf16x2_rest(float a, float b, uint32_t hi) {
+  return pack_bf16x2(a - __uint_as_float(hi << 16), b - __uint_as_float(hi & 0xFFFF0000u));
+}
+// o <- o fo + t ft for a tile's share t of an accumulator row; fo = ft = 1 in the whole warp when `plain`
+template <int kN> __device__ __forceinline__ void add_share(float* o, const float (&t)[kN], float fo, float ft, bool plain) {
+  if (!plain) {
+#pragma unroll
+    for (int c = 0; c < kN; ++c) o[c] *= fo;
+  }
+#pragma unroll
+  for (int c = 0; c < kN; c += 2) {
+    const float2 u = __ffma2_rn(make_float2(t[c], t[c + 1]), make_float2(ft, ft), make_float2(o[c], o[c + 1]));
+    o[c] = u.x; o[c + 1] = u.y;
+  }
+}
 __device__ __forceinline__ float ex2(float x) {
   float y;
   asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));

@@ -1,6 +1,6 @@
 """bf16 tensors with head dimension 64 on the tensor-core kernels: full tiles, doubled and packed group remainders, probe
 slices, the two-word correction and the projections, against the oracle on the oracle's own plan (outputs) and through the
-GPU's own plan (links); tolerances as for d = 128, where the arithmetic is the same."""
+GPU's own plan (links); tolerances as for d = 128 where the output is bf16.  Probabilities, sums and features are float32 here."""
 import pytest
 import torch
 
@@ -37,6 +37,23 @@ def test_attend_d64(name, wl, mode):
         assert_bf16_close(to_np(Osp[0, i]), O_sp)
         assert_bf16_close(to_np(O[0, i]), O_hat)
         assert_bf16_close(to_np(O2[0, i]), O_hat)
+
+
+@pytest.mark.parametrize("name,wl", CASES, ids=[c[0] for c in CASES])
+def test_float32_inside_d64(name, wl):
+    """Hard-drop rows and features before any rounding to bf16.  Rows: probabilities in two bf16 words (2^-18) of exponentials good to
+    2^-22, sums in float32: 2e-6 (one bf16 word: 2e-4).  Features: three words of F, float32 sums: 2^-23 in the 2-norm, and a fifth."""
+    host, (Qd, Kd, Vd) = heads_to_device(wl, [0, 1])
+    kw = dict(density=wl.density, block=wl.block, n_sample=wl.n_sample, n_probe=wl.n_probe, softmax_scale=1.0, mode=1)
+    prm = orc.default_params(**kw)
+    plans = oracle_plans(host, prm)
+    C = -(-wl.N // wl.block)
+    _, Osp = B.sparsepr_attend(B.sparsepr_plan_import(Qd, Kd, Vd, plans_to_host(plans, C, C), **kw), Qd, Kd, Vd, return_sparse=True)
+    feat = B.sparsepr_plan_export_features(B.sparsepr_plan(Qd, Kd, Vd, **kw), fields=("F_Q", "phi_Q"))
+    for i, (Q, K, V) in enumerate(host):
+        _, O_sp, _ = orc.attend_head(Q, K, V, plans[i], prm)
+        assert orc.rel_l2(to_np(Osp[0, i]), O_sp) <= 2e-6
+        assert orc.rel_l2(feat["phi_Q"][i], orc.query_response(Q, feat["F_Q"][i])) <= 1.4e-7
 
 
 def test_plan_d64():
