@@ -366,7 +366,7 @@ void carve_attend(Carver& c, const Resolved& r, AttendWs* w) {
   float* X = c.take<float>(BH * M1 * d); float* Dn = c.take<float>(BH * M1 * d);
   float* A = c.take<float>(BH * d * d); float* cc = c.take<float>(BH * d);
   float* Psi = c.take<float>(BH * d * d);
-  __nv_bfloat16* At = c.take<__nv_bfloat16>(2 * BH * d * d);   // the correction map as two bf16 words
+  __nv_bfloat16* At = c.take<__nv_bfloat16>(map_words(r.d) * BH * d * d);   // the correction map as bf16 words
   const bool f32 = r.dtype == SPARSEPR_F32;
   float* fpart = c.take<float>(f32 ? attention_f32_part_floats(r.BH, r.N, r.Cq, r.d) : 0);
   int* fcount = c.take<int>(f32 ? attention_f32_items(r.BH, r.N, r.Cq) : 0);

@@ -70,7 +70,7 @@ struct Params {
   const __nv_bfloat16* Qg;                     // [BH][N][D] group-major
   __nv_bfloat16* O; i64 os[3];
   float* O_sparse;
-  __nv_bfloat16* O_lo;             // optional [BH][N][D]: o - bf16(o), original order (second word for the correction pass)
+  __nv_bfloat16* O_lo;             // optional [BH][N][D], original order: second word for the correction pass (see attention_tc.cu)
   int* err;
 };
 
@@ -462,14 +462,24 @@ k_attention_packed(const __grid_constant__ Maps mapsK, const __grid_constant__ M
         const int dst = prm.q_perm[(i64)bh * prm.N + my_pos];
         const int b = bh / prm.H, h = bh % prm.H;
         __nv_bfloat16* op = prm.O + b * prm.os[0] + h * prm.os[1] + (i64)dst * prm.os[2] + hh * kOc;
+        if (kTwoWords<D> && prm.O_lo) {                        // the two halves of the float32 value
+          __nv_bfloat16* lp = prm.O_lo + ((i64)bh * prm.N + dst) * D + hh * kOc;
 #pragma unroll
-        for (int ch = 0; ch < kOc / 8; ++ch) {
-          float v8[8];
+          for (int ch = 0; ch < kOc / 8; ++ch) {
+            const float* v = o + ch * 8;
+            *reinterpret_cast<uint4*>(op + ch * 8) = make_uint4(upper_halves(v[0], v[1]), upper_halves(v[2], v[3]), upper_halves(v[4], v[5]), upper_halves(v[6], v[7]));
+            *reinterpret_cast<uint4*>(lp + ch * 8) = make_uint4(lower_halves(v[0], v[1]), lower_halves(v[2], v[3]), lower_halves(v[4], v[5]), lower_halves(v[6], v[7]));
+          }
+        } else {
 #pragma unroll
-          for (int k = 0; k < 8; ++k) v8[k] = o[ch * 8 + k];
-          store8(op + ch * 8, v8);
+          for (int ch = 0; ch < kOc / 8; ++ch) {
+            float v8[8];
+#pragma unroll
+            for (int k = 0; k < 8; ++k) v8[k] = o[ch * 8 + k];
+            store8(op + ch * 8, v8);
+          }
         }
-        if (prm.O_lo) {                                        // what the bf16 rounding above dropped
+        if (!kTwoWords<D> && prm.O_lo) {                       // what the bf16 rounding above dropped
           __nv_bfloat16* lp = prm.O_lo + ((i64)bh * prm.N + dst) * D + hh * kOc;
 #pragma unroll
           for (int ch = 0; ch < kOc / 8; ++ch) {

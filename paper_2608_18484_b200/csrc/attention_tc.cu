@@ -41,7 +41,7 @@
 // Epilogue: O / l, stored as bf16 at the original token index (inverse permutation).  The residual correction of
 // Eq. 9 is a pass of its own (correction_tc.cu) so that the fit can overlap this kernel; for that pass the part of
 // every element that the bf16 rounding dropped is stored as a second bf16 word (O_lo), so that the corrected output
-// is, in effect, rounded to bf16 only once.
+// is, in effect, rounded to bf16 only once.  D = 64: the two words are the halves of the float32 value itself.
 // A tile with at most 64 valid rows (the remainder of a query group) holds every row TWICE, at lanes r and r + 64:
 // the softmax threads of lanes 64-127 would otherwise spend a full tile's worth of exponentials on rows that do not
 // exist (the loop is bound by the throughput of those instructions).  The four threads that then sit on a row (two
@@ -100,7 +100,7 @@ struct Params {
   const int4* items; const int* n_items;       // block-sparse: the tiles of a head (launch_tc_items)
   __nv_bfloat16* O; i64 os[3];
   float* O_sparse;
-  __nv_bfloat16* O_lo;             // optional [BH][N][D]: o - bf16(o), original order (second word for the correction pass)
+  __nv_bfloat16* O_lo;             // optional [BH][N][D], original order: second word for the correction pass, o - bf16(o); D = 64: lower half of float32 o
   int* err;
 };
 
@@ -522,6 +522,19 @@ k_attention_tc(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__
 #pragma unroll
           for (int c = 0; c < 32; c += 4) *reinterpret_cast<float4*>(sp + c) = make_float4(t[c], t[c + 1], t[c + 2], t[c + 3]);
         }
+        if (kTwoWords<D> && prm.O_lo) {
+#pragma unroll
+          for (int ch = 0; ch < 4; ++ch) {
+            uint32_t h[4];
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+              const float a0 = t[8 * ch + 2 * k], a1 = t[8 * ch + 2 * k + 1];
+              h[k] = word ? lower_halves(a0, a1) : upper_halves(a0, a1);
+            }
+            *reinterpret_cast<uint4*>(stage + row * 2 * D + (((q * 4 + ch) ^ (row & 7)) * 16)) = make_uint4(h[0], h[1], h[2], h[3]);
+          }
+          continue;
+        }
         if (word == 1) {
 #pragma unroll
           for (int c = 0; c < 32; ++c) t[c] -= __bfloat162float(__float2bfloat16_rn(t[c]));     // what the rounding of the first word dropped
@@ -574,14 +587,24 @@ k_attention_tc(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__
     auto store_row = [&](int r, const float (&o)[kOc]) {
       const int dst = prm.sparse ? prm.q_perm[(i64)bh * prm.N + row0 + r] : row0 + r;
       __nv_bfloat16* op = prm.O + b * prm.os[0] + h * prm.os[1] + (i64)dst * prm.os[2] + hh * kOc;
+      if (kTwoWords<D> && prm.O_lo) {                          // the two halves of the float32 value
+        __nv_bfloat16* lp = prm.O_lo + ((i64)bh * prm.N + dst) * D + hh * kOc;
 #pragma unroll
-      for (int ch = 0; ch < kOc / 8; ++ch) {
-        float v8[8];
+        for (int ch = 0; ch < kOc / 8; ++ch) {
+          const float* v = o + ch * 8;
+          *reinterpret_cast<uint4*>(op + ch * 8) = make_uint4(upper_halves(v[0], v[1]), upper_halves(v[2], v[3]), upper_halves(v[4], v[5]), upper_halves(v[6], v[7]));
+          *reinterpret_cast<uint4*>(lp + ch * 8) = make_uint4(lower_halves(v[0], v[1]), lower_halves(v[2], v[3]), lower_halves(v[4], v[5]), lower_halves(v[6], v[7]));
+        }
+      } else {
 #pragma unroll
-        for (int k = 0; k < 8; ++k) v8[k] = o[ch * 8 + k];
-        store8(op + ch * 8, v8);
+        for (int ch = 0; ch < kOc / 8; ++ch) {
+          float v8[8];
+#pragma unroll
+          for (int k = 0; k < 8; ++k) v8[k] = o[ch * 8 + k];
+          store8(op + ch * 8, v8);
+        }
       }
-      if (prm.O_lo) {                                          // what the bf16 rounding above dropped
+      if (!kTwoWords<D> && prm.O_lo) {                         // what the bf16 rounding above dropped
         __nv_bfloat16* lp = prm.O_lo + ((i64)bh * prm.N + dst) * D + hh * kOc;
 #pragma unroll
         for (int ch = 0; ch < kOc / 8; ++ch) {
@@ -898,6 +921,7 @@ k_attention_tc(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__
 #pragma unroll
           for (int k = 0; k < 4; ++k) {
             const float a0 = o[ch * 8 + 2 * k], a1 = o[ch * 8 + 2 * k + 1];
+            if (kTwoWords<D> && prm.O_lo) { wh[k] = upper_halves(a0, a1); wl[k] = lower_halves(a0, a1); continue; }
             wh[k] = pack_bf16(a0, a1);
             wl[k] = pack_bf16(a0 - __bfloat162float(__float2bfloat16_rn(a0)), a1 - __bfloat162float(__float2bfloat16_rn(a1)));
           }

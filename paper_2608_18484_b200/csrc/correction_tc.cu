@@ -4,7 +4,11 @@
 // on a second stream while those kernels are busy.  The block-sparse kernels hand over the hard-drop rows X = O^sp
 // as two bf16 words, X = X_h + X_l: X_h is what they stored in O, X_l the part that rounding dropped (2^-17
 // relative together), so that the corrected output is rounded to bf16 once -- a one-word hand-over rounds twice,
-// which shows in the largest elements.  A enters the product as two bf16 words as well, A = A_h + A_l: with few probes
+// which shows in the largest elements.  At D = 64, where the fused pass of the CUDA-core kernels had X and A in float32, the words
+// are the two halves of float32 X; the epilogue warps first make the other two bf16 words of the product out of them (three words hold
+// all of X) and then add X itself; A enters in three words too, with the six products that reach float32.  (Share of the outputs
+// that are not the rounded float64 value at 1333 tokens and 130 probes, ridge 10: 1.3e-3; with two words each 2.9e-3 and up, with
+// probabilities in bf16 besides 0.23; fused float32 pass 6e-4.  44 us instead of 32 for 16 heads of 17550 rows.)  A enters the product as two bf16 words as well, A = A_h + A_l: with few probes
 // (M < d_v) and a small ridge the fitted map can have a norm of ~10, and one word of A then costs up to 0.012 of
 // the 0.02 that the output may differ from the oracle (the products are X_h A_h + X_l A_h + X_h A_l; X_l A_l is
 // below 2^-17 of the result).
@@ -13,9 +17,9 @@
 // memory; two tiles are in work, so that the loads of one, the products (24 instructions, 0.8 us) and the epilogue of the other
 // overlap, and the result leaves as a bulk store of the whole tile from the place of X_h.  (A CTA per two tiles, which loaded,
 // multiplied and stored, row by row, one after the other: 194 us; now 112.)
-//   warps 0-7  warps w and w + 4: 32 rows, half of the columns each: X A from TMEM, X from the two swizzled tiles, + c, back to X_h
-//   warp  8    TMA loads (X_h, X_l of a tile; A_h^T, A_l^T when the head changes)
-//   warp  9    3 D / 16 tcgen05.mma per tile, TMEM owner
+//   warps 0-7  warps w and w + 4: 32 rows, half of the columns each: (D = 64: words of X,) X A from TMEM, X from the two swizzled tiles, + c, back to X_h
+//   warp  8    TMA loads (X_h, X_l of a tile; the words of A^T when the head changes)
+//   warp  9    3 D / 16 (D = 64: 6 D / 16) tcgen05.mma per tile, TMEM owner
 // Every mbarrier wait is bounded; on expiry the CTA records SPARSEPR_ERR_TIMEOUT and leaves.
 #include <cuda.h>
 #include <algorithm>
@@ -34,15 +38,16 @@ template <int D> struct CorrSmem {
   static constexpr uint32_t xh = 0;                        // stage u at xh + 2 u kCorrTileBytes<D>, its second words one tile further
   static constexpr uint32_t xl = xh + kCorrTileBytes<D>;
   static constexpr uint32_t a = xh + 4 * kCorrTileBytes<D>;
-  static constexpr uint32_t al = a + (D / 64) * kCorrMapHalf<D>;
-  static constexpr uint32_t bars = al + (D / 64) * kCorrMapHalf<D>;
-  static constexpr uint32_t misc = bars + 72;
+  static constexpr uint32_t map_bytes = (D / 64) * kCorrMapHalf<D>;             // one word of A^T
+  static constexpr uint32_t xc = a + map_words(D) * map_bytes;                  // D = 64: second and third words of X, [2 stages][2]
+  static constexpr uint32_t bars = xc + (D == 64 ? 4 * kCorrTileBytes<D> : 0);
+  static constexpr uint32_t misc = bars + 88;
   static constexpr uint32_t total = misc + 16;
 };
 static_assert(CorrSmem<128>::total <= 227 * 1024, "shared memory");
 
-// a stage is loaded; stored and free; multiplied (product u in TMEM); the product has been read; the map is loaded
-enum CorrBar { C_FULL = 0, C_EMPTY = 2, C_DONE = 4, C_READ = 6, C_MAP = 8, kCorrBars };
+// a stage is loaded; stored and free; multiplied (product u in TMEM); the product has been read; the words of X are made; the map is loaded
+enum CorrBar { C_FULL = 0, C_EMPTY = 2, C_DONE = 4, C_READ = 6, C_CONV = 8, C_MAP = 10, kCorrBars };
 struct CorrParams {
   int BH, H, N;
   const float* c;                  // [BH][D]
@@ -56,6 +61,7 @@ k_correction_tc(const __grid_constant__ CUtensorMap mapO, const __grid_constant_
   using SM = CorrSmem<D>;
   constexpr int kHalves = D / 64;
   constexpr uint32_t kMapHalf = kCorrMapHalf<D>;
+  constexpr bool kHalvesOfX = D == 64;                           // X_h and the tile beside it are the halves of float32 X
   constexpr uint32_t FULLW = 0xffffffffu;
   extern __shared__ __align__(1024) unsigned char smem_raw[];
   const uint32_t base = smem_u32(smem_raw);
@@ -68,7 +74,7 @@ k_correction_tc(const __grid_constant__ CUtensorMap mapO, const __grid_constant_
   if (tid == 0) {
     misc[2] = (prm.err != nullptr && *reinterpret_cast<volatile int*>(prm.err) == SPARSEPR_ERR_TIMEOUT) || (base & 1023u) != 0;
     if ((base & 1023u) != 0) set_error(prm.err, SPARSEPR_ERR_CUDA);
-    for (int i = 0; i < kCorrBars; ++i) mbar_init(bar(i), i >= C_READ && i < C_MAP ? 256 : 1);
+    for (int i = 0; i < kCorrBars; ++i) mbar_init(bar(i), i >= C_READ && i < C_MAP ? 256 : 1);     // C_READ, C_CONV
     misc[1] = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
@@ -99,18 +105,16 @@ k_correction_tc(const __grid_constant__ CUtensorMap mapO, const __grid_constant_
         if (k > 0 && !__all_sync(FULLW, mbar_wait(bar(C_DONE + (u ^ 1)), ((k - 1) >> 1) & 1, abort_flag))) break;
         head = bh;
         if (lane == 0) {
-          mbar_expect_tx(bar(C_MAP), 2 * kHalves * kMapHalf);
-          for (int c = 0; c < kHalves; ++c) {
-            tma_load_4d(base + SM::a + c * kMapHalf, &mapA, bar(C_MAP), 64 * c, 0, bh, 0);
-            tma_load_4d(base + SM::al + c * kMapHalf, &mapA, bar(C_MAP), 64 * c, 0, prm.BH + bh, 0);    // the second words follow the first ones
-          }
+          mbar_expect_tx(bar(C_MAP), map_words(D) * SM::map_bytes);
+          for (int w = 0; w < map_words(D); ++w)
+            for (int c = 0; c < kHalves; ++c) tma_load_4d(base + SM::a + w * SM::map_bytes + c * kMapHalf, &mapA, bar(C_MAP), 64 * c, 0, w * prm.BH + bh, 0);
         }
         __syncwarp();
       }
     }
   } else if (warp == 9) {
     // (the whole warp walks the tiles and one elected lane issues: see attention_tc.cu)
-    const uint64_t ad = smem_desc(base + SM::a, 16), ald = smem_desc(base + SM::al, 16);
+    const uint64_t ad = smem_desc(base + SM::a, 16);
     const uint32_t idesc = idesc_bf16(0, D);
     int head = -1, maps = 0;
     bool ok = true;
@@ -118,26 +122,32 @@ k_correction_tc(const __grid_constant__ CUtensorMap mapO, const __grid_constant_
       const int u = k & 1, bh = (g0 + k) / n_tiles;
       if (bh != head) { ok = mbar_wait(bar(C_MAP), maps & 1, abort_flag); head = bh; ++maps; }
       ok = ok && mbar_wait(bar(C_READ + u), ((k >> 1) & 1) ^ 1, abort_flag);
-      ok = __all_sync(FULLW, ok && mbar_wait(bar(C_FULL + u), (k >> 1) & 1, abort_flag));
+      ok = __all_sync(FULLW, ok && mbar_wait(bar((kHalvesOfX ? C_CONV : C_FULL) + u), (k >> 1) & 1, abort_flag));
       if (!ok) break;
       tc_fence_after();
-      const uint64_t hd = smem_desc(base + SM::xh + u * 2 * kCorrTileBytes<D>, 16), ld = smem_desc(base + SM::xl + u * 2 * kCorrTileBytes<D>, 16);
+      const uint64_t hd = smem_desc(base + SM::xh + u * 2 * kCorrTileBytes<D>, 16);
+      const uint64_t ld = smem_desc(base + (kHalvesOfX ? SM::xc + u * 2 * kCorrTileBytes<D> : SM::xl + u * 2 * kCorrTileBytes<D>), 16);
       const uint32_t d = tmem + 128u * u;
       if (elect_one()) {
+        auto product = [&](uint64_t xd, int word, bool first) {          // (X A)[m][n] = sum_k X[m][k] At[n][k]
+          const uint64_t wd = ad + (uint64_t)(word * (SM::map_bytes >> 4));
 #pragma unroll
-        for (int kk = 0; kk < D / 16; ++kk) {
-          const uint64_t koff = (uint64_t)((kk >> 2) * (kCorrHalf >> 4) + (kk & 3) * 2), aoff = (uint64_t)((kk >> 2) * (kMapHalf >> 4) + (kk & 3) * 2);
-          umma_bf16(d, hd + koff, ad + aoff, idesc, kk > 0);             // (X A)[m][n] = sum_k X[m][k] At[n][k]
-        }
-#pragma unroll
-        for (int kk = 0; kk < D / 16; ++kk) {
-          const uint64_t koff = (uint64_t)((kk >> 2) * (kCorrHalf >> 4) + (kk & 3) * 2), aoff = (uint64_t)((kk >> 2) * (kMapHalf >> 4) + (kk & 3) * 2);
-          umma_bf16(d, ld + koff, ad + aoff, idesc, 1);
-        }
-#pragma unroll
-        for (int kk = 0; kk < D / 16; ++kk) {
-          const uint64_t koff = (uint64_t)((kk >> 2) * (kCorrHalf >> 4) + (kk & 3) * 2), aoff = (uint64_t)((kk >> 2) * (kMapHalf >> 4) + (kk & 3) * 2);
-          umma_bf16(d, hd + koff, ald + aoff, idesc, 1);
+          for (int kk = 0; kk < D / 16; ++kk) {
+            const uint64_t koff = (uint64_t)((kk >> 2) * (kCorrHalf >> 4) + (kk & 3) * 2), aoff = (uint64_t)((kk >> 2) * (kMapHalf >> 4) + (kk & 3) * 2);
+            umma_bf16(d, xd + koff, wd + aoff, idesc, !first || kk > 0);
+          }
+        };
+        if constexpr (kHalvesOfX) {                                      // smallest first
+          product(hd, 2, true);
+          product(ld, 1, false);
+          product(ld + (uint64_t)(kCorrTileBytes<D> >> 4), 0, false);
+          product(hd, 1, false);
+          product(ld, 0, false);
+          product(hd, 0, false);
+        } else {
+          product(hd, 0, true);
+          product(ld, 0, false);
+          product(hd, 1, false);
         }
         umma_commit(bar(C_DONE + u));
       }
@@ -149,6 +159,31 @@ k_correction_tc(const __grid_constant__ CUtensorMap mapO, const __grid_constant_
     bool ok = true;
     for (int k = 0; k < count; ++k) {
       const int u = k & 1, bh = (g0 + k) / n_tiles, row0 = ((g0 + k) % n_tiles) * kCorrTile;
+      if constexpr (kHalvesOfX) {
+        ok = __all_sync(FULLW, ok && mbar_wait(bar(C_FULL + u), (k >> 1) & 1, abort_flag));
+        if (ok) {
+#pragma unroll
+          for (int ch = 0; ch < 4; ++ch) {
+            const uint32_t at = row * 128 + (((hh * 4 + ch) ^ (row & 7)) << 4);
+            const uint4 rh = *reinterpret_cast<const uint4*>(smem_raw + SM::xh + u * 2 * kCorrTileBytes<D> + at);
+            const uint4 rl = *reinterpret_cast<const uint4*>(smem_raw + SM::xl + u * 2 * kCorrTileBytes<D> + at);
+            const uint32_t h[4] = {rh.x, rh.y, rh.z, rh.w}, l[4] = {rl.x, rl.y, rl.z, rl.w};
+            uint32_t w[4], w2[4];
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+              const float r0 = __uint_as_float(__byte_perm(l[e], h[e], 0x5410)) - __uint_as_float(h[e] << 16);
+              const float r1 = __uint_as_float(__byte_perm(l[e], h[e], 0x7632)) - __uint_as_float(h[e] & 0xFFFF0000u);
+              w[e] = pack_bf16x2(r0, r1);
+              w2[e] = pack_bf16x2_rest(r0, r1, w[e]);
+            }
+            unsigned char* xw = smem_raw + SM::xc + u * 2 * kCorrTileBytes<D> + at;
+            *reinterpret_cast<uint4*>(xw) = make_uint4(w[0], w[1], w[2], w[3]);
+            *reinterpret_cast<uint4*>(xw + kCorrTileBytes<D>) = make_uint4(w2[0], w2[1], w2[2], w2[3]);
+          }
+          fence_async_smem();                                            // the product reads what was written
+          mbar_arrive(bar(C_CONV + u));
+        }
+      }
       ok = __all_sync(FULLW, ok && mbar_wait(bar(C_DONE + u), (k >> 1) & 1, abort_flag));
       tc_fence_after();
       const float* cv = prm.c + (i64)bh * D;
@@ -171,9 +206,16 @@ k_correction_tc(const __grid_constant__ CUtensorMap mapO, const __grid_constant_
           uint32_t w[4];
 #pragma unroll
           for (int e = 0; e < 4; ++e) {
-            const float2 fh = __bfloat1622float2(hp[e]), fl = __bfloat1622float2(lp[e]);
+            float2 x;
+            if constexpr (kHalvesOfX) {
+              const uint32_t h = reinterpret_cast<const uint32_t*>(&rh)[e], l = reinterpret_cast<const uint32_t*>(&rl)[e];
+              x = make_float2(__uint_as_float(__byte_perm(l, h, 0x5410)), __uint_as_float(__byte_perm(l, h, 0x7632)));
+            } else {
+              const float2 fh = __bfloat1622float2(hp[e]), fl = __bfloat1622float2(lp[e]);
+              x = make_float2(fh.x + fl.x, fh.y + fl.y);
+            }
             const int col = q * 32 + ch * 8 + 2 * e;
-            w[e] = pack_bf16x2((fh.x + fl.x) + t[ch * 8 + 2 * e] + cv[col], (fh.y + fl.y) + t[ch * 8 + 2 * e + 1] + cv[col + 1]);
+            w[e] = pack_bf16x2(x.x + t[ch * 8 + 2 * e] + cv[col], x.y + t[ch * 8 + 2 * e + 1] + cv[col + 1]);
           }
           *reinterpret_cast<uint4*>(hrow + so) = make_uint4(w[0], w[1], w[2], w[3]);
         }
@@ -238,7 +280,7 @@ bool launch_correction_tc(const float* c, const __nv_bfloat16* At, const void* O
   CUtensorMap mo, ml, ma;
   if (!make_map(&mo, O, d, N, H, BH / H, os[0], os[1], os[2], kCorrTile) ||
       !make_map(&ml, O_lo, d, N, BH, 1, 0, (i64)N * d, d, kCorrTile) ||
-      !make_map(&ma, At, d, d, 2 * BH, 1, 0, (i64)d * d, d, d))
+      !make_map(&ma, At, d, d, map_words(d) * BH, 1, 0, (i64)d * d, d, d))
     return false;
   CorrParams p{};
   p.BH = BH; p.H = H; p.N = N; p.c = c; p.err = err;

@@ -271,8 +271,8 @@ __global__ void __launch_bounds__(512, 1) k_fit_solve(FitArgs a) {
 }
 
 // T = B Psi (d x r); A = diag(1/s_x) T Psi^T; c = mu_R - mu_x A.  float64 throughout.  Grid (d / 16 + 1, heads): CTA x
-// owns 16 rows of A; the last one forms c = mu_R - ((mu_x / s_x) B) Psi Psi^T.  With `At` the map is also written as the
-// two bf16 words the correction pass multiplies with: At [2][BH][n][k], first words, then what their rounding dropped.
+// owns 16 rows of A; the last one forms c = mu_R - ((mu_x / s_x) B) Psi Psi^T.  With `At` the map is also written as the two
+// (d = 64: three) bf16 words the correction pass multiplies with: At [words][BH][n][k], first words, then what their rounding dropped.
 // (One CTA per head: 132 us at two heads of d = 128, 630 us beside the attention kernels at 24 heads; now 25 and 125 us.)
 constexpr int kCompRows = 16;
 __global__ void __launch_bounds__(256) k_fit_compose(FitArgs a, int r) {
@@ -293,7 +293,10 @@ __global__ void __launch_bounds__(256) k_fit_compose(FitArgs a, int r) {
     if (Ah) {
       const __nv_bfloat16 hb = __float2bfloat16_rn(x);
       Ah[(i64)j * d + i] = hb;
-      Al[(i64)j * d + i] = __float2bfloat16_rn(x - __bfloat162float(hb));
+      const float rest = x - __bfloat162float(hb);
+      const __nv_bfloat16 lb = __float2bfloat16_rn(rest);
+      Al[(i64)j * d + i] = lb;
+      if (d == 64) (Al + (i64)gridDim.y * d * d)[(i64)j * d + i] = __float2bfloat16_rn(rest - __bfloat162float(lb));
     }
   };
   if (sc[L.flag] != 0.0) {                 // no usable fit: the head falls back to hard drop

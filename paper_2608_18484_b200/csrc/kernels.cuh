@@ -111,7 +111,8 @@ struct AttnArgs {
   // epilogue
   void* O; i64 os[3];
   float* O_sparse;            // optional [BH][N][d] in original order
-  void* O_lo;                 // optional bf16 [BH][N][d] in original order: o - bf16(o) (tensor-core kernels only)
+  void* O_lo;                 // optional [BH][N][d] 16-bit words in original order (tensor-core kernels only): o - bf16(o) as bf16; d = 64: O and
+                              // O_lo take the upper and the lower half of float32 o
   int* err;                   // device error word (may be null)
 };
 cudaError_t init_attention_simt();
@@ -145,8 +146,9 @@ void launch_remainder_rows(const int* q_off, const int* route_ptr, const int* ro
 bool launch_attention_packed(const AttnArgs& a, const int* rem_pos, const int* rem_grp, const int* rem_cnt, cudaStream_t st);
 // one warp runs the bounded mbarrier wait into its limit (2^16 cycles) and records SPARSEPR_ERR_TIMEOUT in *err
 void launch_selftest_bounded_wait(int* err, cudaStream_t st);
-// correction_tc.cu: O <- X + X A + c in place, X = O + O_lo (two bf16 words, O_lo [BH][N][d] contiguous), d_v = d = 64 or 128;
-// At [2][BH][d][d]: A transposed, as two bf16 words (from the fit)
+// correction_tc.cu: O <- X + X A + c in place, X = O and O_lo as the block-sparse kernels store them, d_v = d = 64 or 128;
+// At [map_words(d)][BH][d][d]: A transposed, as bf16 words (from the fit)
+__host__ __device__ constexpr int map_words(int d) { return d == 64 ? 3 : 2; }
 cudaError_t init_correction_tc();
 bool launch_correction_tc(const float* c, const __nv_bfloat16* At, const void* O_lo, void* O, const i64* os, int BH,
                           int H, int N, int d, int* err, cudaStream_t st);
@@ -181,7 +183,7 @@ struct FitArgs {
   double* scratch;                     // see fit_scratch_doubles
   double* eig_ws;                      // eig_scratch_doubles(BH, d) doubles
   float *A, *c;                        // outputs [BH][d][d], [BH][d]
-  __nv_bfloat16* At;                   // optional output [2][BH][d][d]: A transposed, as two bf16 words (correction pass)
+  __nv_bfloat16* At;                   // optional output [map_words(d)][BH][d][d]: A transposed, as bf16 words (correction pass)
   float* Psi;                          // [BH][d][r] scratch
   int* err;
 };

@@ -166,6 +166,9 @@ __device__ __forceinline__ uint32_t pack_bf16x2(float a, float b) {      // a in
 __device__ __forceinline__ uint32_t pack_bf16x2_rest(float a, float b, uint32_t hi) {
   return pack_bf16x2(a - __uint_as_float(hi << 16), b - __uint_as_float(hi & 0xFFFF0000u));
 }
+// upper and lower 16 bits of two float32 (a in the low half): the float32 value itself in two 16-bit words
+__device__ __forceinline__ uint32_t upper_halves(float a, float b) { return __byte_perm(__float_as_uint(a), __float_as_uint(b), 0x7632); }
+__device__ __forceinline__ uint32_t lower_halves(float a, float b) { return __byte_perm(__float_as_uint(a), __float_as_uint(b), 0x5410); }
 // o <- o fo + t ft for a tile's share t of an accumulator row; fo = ft = 1 in the whole warp when `plain`
 template <int kN> __device__ __forceinline__ void add_share(float* o, const float (&t)[kN], float fo, float ft, bool plain) {
   if (!plain) {
