@@ -243,6 +243,7 @@ struct sparsepr_plan_s {
   // attend call orders the former (its probe work follows on the same stream and is joined there), every attend call
   // waits for ev_route; statistics, export and the destructor wait for both themselves
   mutable bool side_pending = false;
+  unsigned long long capture = 0;                         // the stream capture the plan was made in (0: none)
   bool imported = false;                                  // built by sparsepr_plan_import: no partition stages ran
   ~sparsepr_plan_s() {
     if (side && side_pending) { cudaStreamSynchronize(side); cudaStreamSynchronize(side2); }
@@ -512,6 +513,27 @@ void fork_side(const sparsepr_plan_s* p, cudaStream_t st) {
   cudaEventRecord(p->ev_fork, st);
   cudaStreamWaitEvent(p->side, p->ev_fork, 0);
 }
+// the stream capture `st` takes part in, 0 if none
+unsigned long long capture_of(cudaStream_t st) {
+  cudaStreamCaptureStatus status = cudaStreamCaptureStatusNone;
+  unsigned long long id = 0;
+  if (cudaStreamGetCaptureInfo(st, &status, &id) != cudaSuccess) { cudaGetLastError(); return 0; }
+  return status == cudaStreamCaptureStatusActive ? id : 0;
+}
+// Work of an attend call on `st` comes after the routes.  A captured wait can only name work of its own capture: an attend call
+// that is captured on a plan made before the capture waits for the plan here, on the host (the replays find it complete), and
+// one outside the capture of its plan is ordered by whoever launches the graph.
+bool wait_for_routes(const sparsepr_plan_s* p, cudaStream_t st) {
+  const unsigned long long cap = capture_of(st);
+  if (cap == p->capture) return cudaStreamWaitEvent(st, p->ev_route, 0) == cudaSuccess;
+  if (p->capture != 0) return true;
+  cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;      // the waits below concern no captured stream
+  cudaThreadExchangeStreamCaptureMode(&mode);
+  const bool ok = cudaEventSynchronize(p->ev_route) == cudaSuccess && (!p->side_pending || cudaStreamSynchronize(p->side) == cudaSuccess);
+  cudaThreadExchangeStreamCaptureMode(&mode);
+  if (ok) p->side_pending = false;
+  return ok;
+}
 // ... and `st` continues once the side stream's work is done
 void join_side(const sparsepr_plan_s* p, cudaStream_t st) {
   cudaEventRecord(p->ev_join, p->side);
@@ -534,6 +556,7 @@ static sparsepr_status_t plan_impl(const sparsepr_shape_t* shape, const sparsepr
   }
   cudaStream_t st = p->stream;
   cudaGetLastError();
+  p->capture = capture_of(st);
   cudaMemsetAsync(p->err, 0, 64 * sizeof(int), st);
   cudaMemsetAsync(p->maxabs, 0, r.BH * sizeof(unsigned), st);
   StageTimer tm(prof, st);
@@ -698,7 +721,7 @@ static sparsepr_status_t attend_impl(const sparsepr_plan_t* p, const void* Q, co
   launch_gather_rows(r.dtype, Q, r.qs, r.BH, r.H, p->q_perm, r.N, r.d, w.Qg, st);
   launch_gather_rows(r.dtype, K, r.ks, r.BHkv, r.Hkv, p->kv_perm, r.N, r.d, w.Kg, st);
   launch_gather_rows(r.dtype, V, r.vs, r.BHkv, r.Hkv, p->kv_perm, r.N, r.d, w.Vg, st);
-  cudaStreamWaitEvent(st, p->ev_route, 0);
+  if (!wait_for_routes(p, st)) return SPARSEPR_ERR_CUDA;
   tm.mark(SPARSEPR_STAGE_GATHER);
   const bool fitted = r.mode == 0 && r.M > 0;
   AttnArgs aa{};
