@@ -610,8 +610,9 @@ static sparsepr_status_t plan_impl(const sparsepr_shape_t* shape, const sparsepr
   tm.mark(SPARSEPR_STAGE_QUERY_PERMUTE);
   // Probes and routes.  Without a profile both leave the caller's stream: the routes (one CTA per head for most of the time) run
   // beside the gathers of the attend call that follows, which orders itself behind them by ev_route, and beside the probe
-  // selection, which is not needed before the probe rows.
-  const bool beside = prof == nullptr;
+  // selection, which is not needed before the probe rows.  A plan without probes stays on the caller's stream: whoever
+  // synchronises that has all of it, and destroying it waits for nothing.
+  const bool beside = prof == nullptr && r.M > 0;
   cudaStream_t ps = st, rs = st;
   const auto cell_scores = [&] { launch_cell_scores(p->theta, p->kappa, p->nq, p->nk, r.BH, r.Cq, r.Ck, r.d, r.scale, p->score, r.G, rs); };
   if (beside) {

@@ -15,6 +15,21 @@ from tests.gpu_util import heads_to_device, to_np
 
 pytestmark = pytest.mark.gpu
 
+
+@pytest.mark.parametrize("kw", [dict(n_probe=0), dict(n_probe=32, mode=1)], ids=["no-probes", "hard"])
+def test_destroying_a_plan_without_probes_waits_for_nothing(kw):
+    Q = torch.randn(1, 2, 1024, 64, device="cuda")
+    kw = dict(kw, density=0.3, block=64, n_sample=64, softmax_scale=1.0)
+    B.sparsepr_plan(Q, Q, Q, **kw)                               # everything set up
+    torch.cuda.synchronize()
+    torch.cuda._sleep(1 << 30)                                   # half a second of the GPU
+    done = torch.cuda.Event()
+    plan = B.sparsepr_plan(Q, Q, Q, **kw)
+    done.record()
+    del plan
+    assert not done.query()
+    torch.cuda.synchronize()
+
 CASES = [("tiny-f32", W.TINY), ("480p-like-bf16", W.VIDEO_480P.scaled(grid=(3, 30, 52), H=2, n_probe=64))]
 
 
