@@ -243,6 +243,7 @@ struct sparsepr_plan_s {
   // attend call orders the former (its probe work follows on the same stream and is joined there), every attend call
   // waits for ev_route; statistics, export and the destructor wait for both themselves
   mutable bool side_pending = false;
+  mutable std::mutex attend_mu;                           // attend calls of several threads share the streams and events: one at a time is queued
   unsigned long long capture = 0;                         // the stream capture the plan was made in (0: none)
   bool imported = false;                                  // built by sparsepr_plan_import: no partition stages ran
   ~sparsepr_plan_s() {
@@ -717,6 +718,7 @@ static sparsepr_status_t attend_impl(const sparsepr_plan_t* p, const void* Q, co
   Carver c(workspace);
   carve_attend(c, r, &w);
   cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
+  std::unique_lock<std::mutex> lock(p->attend_mu);
   cudaGetLastError();
   StageTimer tm(prof, st);
   launch_gather_rows(r.dtype, Q, r.qs, r.BH, r.H, p->q_perm, r.N, r.d, w.Qg, st);
@@ -788,6 +790,7 @@ static sparsepr_status_t attend_impl(const sparsepr_plan_t* p, const void* Q, co
   }
   if (fitted) launch_write_probe_rows(r.dtype, w.Dn, p->probe_idx, r.BH, r.H, r.M, r.d, O, r.os, st);
   tm.mark(SPARSEPR_STAGE_PROBE_WRITE);
+  lock.unlock();
   tm.finish();
   return launch_ok() ? SPARSEPR_OK : SPARSEPR_ERR_CUDA;
 }
