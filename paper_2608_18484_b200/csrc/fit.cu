@@ -10,9 +10,11 @@
 
 namespace spr {
 
-// scratch per head (doubles): Xb[M*d] Rb[M*d] G[d*d] B[d*d] S[d*d] mu_x[d] mu_R[d] s_x[d] wt[M] flag[1]
+// scratch per head (doubles): Xb[M*d] Rb[M*d] G[d*d] B[d*d] S[d*d] mu_x[d] mu_R[d] s_x[d] wt[M] flag[1] failed[1]
+// flag: no usable probes (k_fit_prepare); failed: a pivot of the elimination was not positive (the CTAs of k_fit_solve, all of
+// which find the same one)
 struct FitLayout {
-  size_t Xb, Rb, G, B, S, mu_x, mu_R, s_x, wt, flag, total;
+  size_t Xb, Rb, G, B, S, mu_x, mu_R, s_x, wt, flag, failed, total;
   __host__ __device__ FitLayout(int M, int d) {
     size_t o = 0;
     Xb = o; o += (size_t)M * d;
@@ -23,6 +25,7 @@ struct FitLayout {
     mu_x = o; o += d; mu_R = o; o += d; s_x = o; o += d;
     wt = o; o += M;
     flag = o; o += 1;
+    failed = o; o += 1;
     total = (o + 31) / 32 * 32;
   }
 };
@@ -52,7 +55,12 @@ __global__ void __launch_bounds__(kPrepCols * kPrepSlices) k_fit_prepare(FitArgs
   for (int p = tid; p < M; p += kNt) { sw += (double)w[p]; cnt += w[p] > 0.f ? 1.0 : 0.0; }
   sw = block_sum(sw, red);
   cnt = block_sum(cnt, red);
-  if (tid == 0 && blockIdx.x == 0) sc[L.flag] = (sw > 0.0 && cnt > 0.0) ? 0.0 : 1.0;
+  if (tid == 0 && blockIdx.x == 0) {
+    const bool usable = sw > 0.0 && cnt > 0.0;
+    sc[L.flag] = usable ? 0.0 : 1.0;
+    sc[L.failed] = 0.0;
+    if (!usable) set_error(a.err, SPARSEPR_ERR_NUMERIC);
+  }
   if (!(sw > 0.0)) sw = 1.0;
   const double inv_sw = 1.0 / sw;
   if (blockIdx.x == 0)
@@ -180,7 +188,7 @@ __global__ void __launch_bounds__(512, 1) k_fit_solve(FitArgs a) {
 #pragma unroll
     for (int c = 0; c < kRc; ++c) x[r][kGc + c] = (T)Bm[row * D + lane + 32 * c];
   }
-  if (sc[L.flag] != 0.0) return;                                 // uniform: no usable probes (set by k_fit_prepare)
+  if (sc[L.flag] != 0.0) return;                                 // uniform: no usable probes (nobody writes it here)
   bool bad = false;
   if (warp == 0) {
 #pragma unroll
@@ -221,7 +229,7 @@ __global__ void __launch_bounds__(512, 1) k_fit_solve(FitArgs a) {
     }
   }
   if (bad) {                                                     // uniform over the CTA: everyone saw every pivot
-    if (threadIdx.x == 0) { sc[L.flag] = 1.0; set_error(a.err, SPARSEPR_ERR_NUMERIC); }
+    if (threadIdx.x == 0) { sc[L.failed] = 1.0; set_error(a.err, SPARSEPR_ERR_NUMERIC); }
     return;
   }
   // back substitution: row k of the solution = y_k / pivot, once all rows below have been taken out of it
@@ -299,7 +307,7 @@ __global__ void __launch_bounds__(256) k_fit_compose(FitArgs a, int r) {
       if (d == 64) (Al + (i64)gridDim.y * d * d)[(i64)j * d + i] = __float2bfloat16_rn(rest - __bfloat162float(lb));
     }
   };
-  if (sc[L.flag] != 0.0) {                 // no usable fit: the head falls back to hard drop
+  if (sc[L.flag] != 0.0 || sc[L.failed] != 0.0) {                 // no usable fit: the head falls back to hard drop
     if (tail) { for (int j = tid; j < d; j += 256) cvec[j] = 0.f; }
     else for (int e = tid; e < kCompRows * d; e += 256) put(i0 + e % kCompRows, e / kCompRows, 0.f);
     return;
