@@ -364,14 +364,14 @@ void carve_attend(Carver& c, const Resolved& r, AttendWs* w) {
   // tensor-core probe kernel: one CTA per (128 probe rows, key slice), about one wave
   const int ns_tc = std::max(1, std::min(sm_count() / std::max(1, r.BH * (int)((M1 + 127) / 128)), std::max(1, r.N / 128 / 4)));
   float* partial = c.take<float>(probe_partial_floats(r.BH, std::max(ns, ns_tc), (int)M1, r.d));
-  __nv_bfloat16* Qp = c.take<__nv_bfloat16>(BH * M1 * d);
+  const bool f32 = r.dtype == SPARSEPR_F32;
+  __nv_bfloat16* Qp = c.take<__nv_bfloat16>(f32 ? 0 : BH * M1 * d);
   float* X = c.take<float>(BH * M1 * d); float* Dn = c.take<float>(BH * M1 * d);
   float* A = c.take<float>(BH * d * d); float* cc = c.take<float>(BH * d);
   float* Psi = c.take<float>(BH * d * d);
-  __nv_bfloat16* At = c.take<__nv_bfloat16>(map_words(r.d) * BH * d * d);   // the correction map as bf16 words
-  const bool f32 = r.dtype == SPARSEPR_F32;
-  float* fpart = c.take<float>(f32 ? attention_f32_part_floats(r.BH, r.N, r.Cq, r.d) : 0);
-  int* fcount = c.take<int>(f32 ? attention_f32_items(r.BH, r.N, r.Cq) : 0);
+  __nv_bfloat16* At = c.take<__nv_bfloat16>(f32 ? 0 : map_words(r.d) * BH * d * d);   // the correction map as bf16 words
+  float* fpart = c.take<float>(f32 ? attention_f32_part_floats(r.d) : 0);
+  int* fcount = c.take<int>(f32 ? attention_f32_slots() : 0);
   double* fit = c.take<double>(fit_scratch_doubles(r.BH, (int)M1, r.d));
   double* fit_eigws = c.take<double>(eig_scratch_doubles(r.BH, r.d));
   if (w) { w->fpart = fpart; w->fcount = fcount; w->Olo = Olo; w->Qg = Qg; w->Kg = Kg; w->Vg = Vg; w->partial = partial; w->X = X; w->Dn = Dn; w->A = A; w->c = cc; w->Psi = Psi; w->At = At; w->Qp = Qp; w->n_split_tc = ns_tc; w->fit = fit; w->fit_eigws = fit_eigws; w->n_split = ns; }

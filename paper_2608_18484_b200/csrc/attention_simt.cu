@@ -388,7 +388,7 @@ __global__ void __launch_bounds__(kFThreads, 2) k_attention_f32_dense(AttnArgs a
 // `chunk` key tiles; the items are issued in descending order of their work, so that no long one is left for the end.
 // Every part of a cut tile leaves (m, l, O) in `part`, and the CTA that finishes last (a counter per tile) adds them up in
 // the order of the parts.  The chunk is the smallest of the series 4, 6, 8, 12, 16, 24 ... that gives at most max_items items
-// (attention_f32_items): fine enough for a small list to fill the GPU, and for the kernels of the probes and the fit to find
+// (attention_f32_items) and max_slots parts of cut tiles (attention_f32_slots): fine enough for a small list to fill the GPU, and for the kernels of the probes and the fit to find
 // free slots beside a large one (they would wait for the longest items of the first wave), coarse enough that the parts
 // cost little.
 // keys of every group's routes, in boxes of `box` rows of which only the last of a range may be short
@@ -410,16 +410,16 @@ __device__ __forceinline__ int item_parts(int nt, int j) {                      
   const int c = item_chunk(j);
   return j < kChunks ? min(max((nt + c / 2) / c, 1), 255) : 1;
 }
-__global__ void __launch_bounds__(kItemBuckets) k_f32_items(const int* __restrict__ q_off, const int* __restrict__ keys, int BH, int Cq, int max_items, int shift,
-                                                            int4* __restrict__ items, int* __restrict__ n_items) {
+__global__ void __launch_bounds__(kItemBuckets) k_f32_items(const int* __restrict__ q_off, const int* __restrict__ keys, int BH, int Cq, int max_items, int max_slots,
+                                                            int shift, int4* __restrict__ items, int* __restrict__ n_items) {
   __shared__ int hist[kItemBuckets];
   __shared__ int scratch[34];
-  __shared__ int slots, sum[kChunks];
+  __shared__ int slots, sum[kChunks], cut[kChunks];
   hist[threadIdx.x] = 0;
   if (threadIdx.x == 0) slots = 0;
-  if (threadIdx.x < kChunks) sum[threadIdx.x] = 0;
+  if (threadIdx.x < kChunks) { sum[threadIdx.x] = 0; cut[threadIdx.x] = 0; }
   __syncthreads();
-  int n_of[kChunks] = {}, first, n, tiles, rows, nt;
+  int n_of[kChunks] = {}, n_cut[kChunks] = {}, first, n, tiles, rows, nt;
   auto group = [&](int e) {
     const int* qo = q_off + (i64)(e / Cq) * (Cq + 1) + e % Cq;
     first = qo[0]; n = qo[1] - first;
@@ -429,16 +429,16 @@ __global__ void __launch_bounds__(kItemBuckets) k_f32_items(const int* __restric
   for (int e = threadIdx.x; e < BH * Cq; e += kItemBuckets)
     if (group(e)) {
 #pragma unroll
-      for (int j = 0; j < kChunks; ++j) n_of[j] += tiles * item_parts(nt, j);
+      for (int j = 0; j < kChunks; ++j) { const int parts = item_parts(nt, j); n_of[j] += tiles * parts; n_cut[j] += parts > 1 ? tiles * parts : 0; }
     }
 #pragma unroll
   for (int j = 0; j < kChunks; ++j) {
-    const int v = __reduce_add_sync(0xffffffffu, n_of[j]);
-    if ((threadIdx.x & 31) == 0) atomicAdd(&sum[j], v);
+    const int v = __reduce_add_sync(0xffffffffu, n_of[j]), c = __reduce_add_sync(0xffffffffu, n_cut[j]);
+    if ((threadIdx.x & 31) == 0) { atomicAdd(&sum[j], v); atomicAdd(&cut[j], c); }
   }
   __syncthreads();
   int j = 0;
-  while (j < kChunks && sum[j] > max_items) ++j;
+  while (j < kChunks && (sum[j] > max_items || cut[j] > max_slots)) ++j;
   int total = 0;
   for (int pass = 0; pass < 2; ++pass) {
     for (int e = threadIdx.x; e < BH * Cq; e += kItemBuckets) {
@@ -514,13 +514,16 @@ void launch_correction_f32(const float* A, const float* c, void* O, const i64* o
 
 // Items of a list at most: four rounds of CTAs on every SM slot, and twice as many as tiles.
 size_t attention_f32_items(int BH, int N, int Cq) { return std::max((size_t)4 * 2 * sm_count(), (size_t)2 * BH * ((N + BM - 1) / BM + Cq)); }
-size_t attention_f32_part_floats(int BH, int N, int Cq, int d) { return attention_f32_items(BH, N, Cq) * BM * (d + 2); }
+// Partial states of cut tiles at most, 39 MB at d = 128 whatever the size.  (8 heads of 7161 tokens, 1360 tiles: 3335 us with 4 per SM, 3347
+// with 8, 3342 with 16, 3343 with as many as items, which were 1.2 GB of workspace at 24 heads of 32760 tokens.)
+size_t attention_f32_slots() { return (size_t)8 * sm_count(); }
+size_t attention_f32_part_floats(int d) { return attention_f32_slots() * BM * (d + 2); }
 void launch_f32_items(const int* q_off, const int* kv_off, const int* route_ptr, const int* route_idx, int BH, int N, int Cq, int Ck, int* keys, int4* items,
                       int* n_items, cudaStream_t st) {
   k_route_keys<<<dim3((Cq + 31) / 32, BH), 1024, 0, st>>>(kv_off, route_ptr, route_idx, Cq, Ck, 1, 1, keys);
   int shift = 0;
   while ((((N + BN - 1) / BN + 1) * 9) >> shift >= kItemBuckets) ++shift;
-  k_f32_items<<<1, kItemBuckets, 0, st>>>(q_off, keys, BH, Cq, (int)attention_f32_items(BH, N, Cq), shift, items, n_items);
+  k_f32_items<<<1, kItemBuckets, 0, st>>>(q_off, keys, BH, Cq, (int)attention_f32_items(BH, N, Cq), (int)attention_f32_slots(), shift, items, n_items);
 }
 
 // The 128-row tensor-core kernel: the tiles of a head, longest first (per head, not over all of them: tiles of one head run together
@@ -571,7 +574,7 @@ template <int D>
 static void attention_dispatch(const AttnArgs& a, float* part, int* counter, cudaStream_t st) {
   if (a.items) {
     const unsigned items = (unsigned)attention_f32_items(a.BH, a.N, a.Cq);
-    cudaMemsetAsync(counter, 0, items * sizeof(int), st);
+    cudaMemsetAsync(counter, 0, attention_f32_slots() * sizeof(int), st);
     k_attention_f32_sparse<D><<<items, kFThreads, F32Smem<D>::bytes, st>>>(a, part, counter);
   } else {
     k_attention_f32_dense<D><<<dim3((a.N + BM - 1) / BM, a.BH), kFThreads, F32Smem<D>::bytes, st>>>(a);

@@ -117,9 +117,10 @@ struct AttnArgs {
 };
 cudaError_t init_attention_simt();
 // float32, sparse calls.  The list of CTAs (attention_f32_items entries, `keys` [BH][Cq]), made once the routes are known; part /
-// counter: workspace of attention_f32_part_floats floats and attention_f32_items ints.
+// counter: workspace of attention_f32_part_floats floats and attention_f32_slots ints.
 size_t attention_f32_items(int BH, int N, int Cq);
-size_t attention_f32_part_floats(int BH, int N, int Cq, int d);
+size_t attention_f32_slots();
+size_t attention_f32_part_floats(int d);
 void launch_f32_items(const int* q_off, const int* kv_off, const int* route_ptr, const int* route_idx, int BH, int N, int Cq, int Ck, int* keys, int4* items,
                       int* n_items, cudaStream_t st);
 void launch_attention_f32(const AttnArgs& a, float* part, int* counter, cudaStream_t st);

@@ -1,5 +1,7 @@
 """Block-sparse float32 attention on group sizes at the edges of its row counts (8 rows per thread step, 64 rows per tile) and
 of its key tiles, with tiles whose keys are cut into parts (one head) and tiles that are not (40 heads)."""
+import ctypes
+
 import numpy as np
 import pytest
 import torch
@@ -40,3 +42,16 @@ def test_row_and_key_counts(heads, d):
         ref = orc.sparse_attention(to_np(Q[0, i]), to_np(K[0, i]), to_np(V[0, i]), aQ[i], aK[i], ptr[i], idx[i], d ** -0.5)
         # float32 sums of at most 1102 terms of mixed sign: 2^-24 sqrt(1102) = 2e-6 of their size
         assert orc.rel_l2(to_np(O[0, i]), ref) < 2e-6
+
+
+@pytest.mark.parametrize("H,N", [(8, 7161), (24, 32760)])
+def test_workspace_is_that_of_the_copies(H, N):
+    """The attend workspace of a large call: the group-major copies of Q, K and V, less than half as much again for
+    the probe rows and the fit, and a fixed number of partial states of cut tiles."""
+    s = B.Shape(B=1, H=H, N=N, d=128, dv=128, dtype=B.F32, Hkv=H)
+    for f in ("q_stride", "k_stride", "v_stride", "o_stride"):
+        getattr(s, f)[:] = [H * N * 128, N * 128, 128]
+    p = B.make_params(block=64, density=0.25, n_sample=128, n_probe=64)
+    copies = 3 * 4 * H * N * 128
+    need = B.lib().sparsepr_attend_workspace_bytes(ctypes.byref(s), ctypes.byref(p))
+    assert copies < need <= 1.4 * copies + 8 * 148 * 64 * 130 * 4      # (eight states of 64 rows per SM)
