@@ -747,8 +747,7 @@ static sparsepr_status_t attend_impl(const sparsepr_plan_t* p, const void* Q, co
     if (overlap) { fork_side(p, st); fs = p->side; }
     ProbeArgs pa{};
     pa.dtype = r.dtype; pa.BH = r.BH; pa.H = r.H; pa.N = r.N; pa.d = r.d; pa.M = r.M; pa.Ck = r.Ck; pa.Cq = r.Cq;
-    pa.n_split = w.n_split; pa.scale = r.scale; pa.Q = Q; pa.kv_div = r.G;
-    for (int i = 0; i < 3; ++i) pa.qs[i] = r.qs[i];
+    pa.n_split = w.n_split; pa.scale = r.scale; pa.Qg = w.Qg; pa.q_inv = p->q_inv; pa.kv_div = r.G;
     pa.Kg = w.Kg; pa.Vg = w.Vg; pa.probe_idx = p->probe_idx; pa.q_assign = p->a_Q; pa.kv_off = p->kv_off;
     pa.route_ptr = p->route_ptr; pa.route_idx = p->route_idx; pa.partial = w.partial; pa.X = w.X; pa.Dn = w.Dn;
     if (probe_tc_supported(pa)) {

@@ -603,11 +603,12 @@ __global__ void __launch_bounds__(256) k_probe_rows(ProbeArgs a) {
   const int words = (a.Ck + 31) / 32;
   int* kgrp = reinterpret_cast<int*>(bitmap + 64 * words);   // [64] K/V group of every tile key
   constexpr int OC = D / 16;
-  const int bh = blockIdx.z, b = bh / a.H, h = bh % a.H;
+  const int bh = blockIdx.z;
   const int m0 = blockIdx.y * BM, nrows = min(BM, a.M - m0);
   const int tid = threadIdx.x, ty = tid >> 4, tx = tid & 15;
   const int* pidx = a.probe_idx + (i64)bh * a.M + m0;
-  const T* Qb = (const T*)a.Q + b * a.qs[0] + h * a.qs[1];
+  const T* Qb = (const T*)a.Qg + (i64)bh * a.N * D;
+  const int* inv = a.q_inv + (i64)bh * a.N;
   const T* Kb = (const T*)a.Kg + (i64)bh * a.N * D;
   const T* Vb = (const T*)a.Vg + (i64)bh * a.N * D;
   const int* kvoff = a.kv_off + (i64)bh * (a.Ck + 1);
@@ -622,7 +623,7 @@ __global__ void __launch_bounds__(256) k_probe_rows(ProbeArgs a) {
     const int* ri = a.route_idx + (i64)bh * a.Cq * a.Ck;
     for (int t = rp[g] + (tid & 3); t < rp[g + 1]; t += 4) atomicOr(&bitmap[r * words + (ri[t] >> 5)], 1u << (ri[t] & 31));
   }
-  load_tile_transposed<T, D>(Qs, [&](int r) { return (r < nrows && pidx[r] >= 0) ? Qb + (i64)pidx[r] * a.qs[2] : (const T*)nullptr; });
+  load_tile_transposed<T, D>(Qs, [&](int r) { return (r < nrows && pidx[r] >= 0) ? Qb + (i64)inv[pidx[r]] * D : (const T*)nullptr; });
 
   // key positions of this split, in whole tiles
   const int tiles = (a.N + BN - 1) / BN;

@@ -158,7 +158,7 @@ struct ProbeArgs {
   int dtype, BH, H, N, d, M, Ck, Cq, n_split;
   int kv_div;                          // query heads per K/V head; Kg, Vg, kv_off are indexed by bh / kv_div
   float scale;
-  const void *Q; i64 qs[3];            // original layout (probe rows are gathered by index)
+  const void* Qg; const int* q_inv;    // group-major copy of Q and the place of every token in it (O may take the place of Q)
   const void *Kg, *Vg;                 // group-major [BH][N][d]
   const int *probe_idx, *q_assign, *kv_off, *route_ptr, *route_idx;
   float* partial;                      // [BH][n_split][M][2][d+2]

@@ -409,15 +409,15 @@ k_probe_rows_tc(const __grid_constant__ CUtensorMap mapQ, const __grid_constant_
 }
 
 // probe rows of Q gathered into a dense [BH][M][d] bf16 buffer (rows of missing probes are zero)
-__global__ void k_gather_probe_q(const __nv_bfloat16* __restrict__ Q, i64 sb, i64 sh, i64 sn, int H,
+__global__ void k_gather_probe_q(const __nv_bfloat16* __restrict__ Qg, const int* __restrict__ q_inv, int N,
                                  const int* __restrict__ probe_idx, int M, int d, __nv_bfloat16* __restrict__ out) {
-  const int bh = blockIdx.y, b = bh / H, h = bh % H;
+  const int bh = blockIdx.y;
   const int t = blockIdx.x * blockDim.x + threadIdx.x;          // d / 8 threads per row
   const int m = t / (d / 8), c = t % (d / 8) * 8;
   if (m >= M) return;
   const int pi = probe_idx[(i64)bh * M + m];
   uint4 v = make_uint4(0, 0, 0, 0);
-  if (pi >= 0) v = *reinterpret_cast<const uint4*>(Q + b * sb + h * sh + (i64)pi * sn + c);
+  if (pi >= 0) v = *reinterpret_cast<const uint4*>(Qg + ((i64)bh * N + q_inv[(i64)bh * N + pi]) * d + c);
   *reinterpret_cast<uint4*>(out + ((i64)bh * M + m) * d + c) = v;
 }
 
@@ -435,8 +435,7 @@ bool launch_probe_rows_tc(const ProbeArgs& a, __nv_bfloat16* Qp, int* err, cudaS
   const int kvd = a.kv_div < 1 ? 1 : a.kv_div;
   using namespace tc;
   const int d = a.d;
-  k_gather_probe_q<<<dim3((a.M * (d / 8) + 255) / 256, a.BH), 256, 0, st>>>((const __nv_bfloat16*)a.Q, a.qs[0], a.qs[1], a.qs[2], a.H,
-                                                                     a.probe_idx, a.M, d, Qp);
+  k_gather_probe_q<<<dim3((a.M * (d / 8) + 255) / 256, a.BH), 256, 0, st>>>((const __nv_bfloat16*)a.Qg, a.q_inv, a.N, a.probe_idx, a.M, d, Qp);
   CUtensorMap mq, mk, mv;
   if (!make_map(&mq, Qp, d, a.M, a.BH, 1, 0, (i64)a.M * d, d, 128) ||
       !make_map(&mk, a.Kg, d, a.N, a.BH / kvd, 1, 0, (i64)a.N * d, d, 128) ||

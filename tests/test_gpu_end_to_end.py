@@ -204,3 +204,16 @@ def test_feature_map_on_repeated_and_clustered_eigenvalues(d, dtype, tol, kind):
     # its sum is unique), and the squared norms are proportional to the eigenvalues
     assert abs(lam.sum() - lam_all[:rK].sum()) <= 10 * tol * lam_all[:rK].sum()
     assert np.allclose(np.diag(G), lam / lam.mean(), rtol=0, atol=20 * tol * np.diag(G).max())
+
+
+@pytest.mark.parametrize("which", [0, 1, 2], ids="QKV")
+@pytest.mark.parametrize("dtype,d", [(torch.float32, 64), (torch.float32, 128), (torch.bfloat16, 64), (torch.bfloat16, 128)], ids=["f32-64", "f32-128", "bf16-64", "bf16-128"])
+def test_output_in_the_place_of_an_input(dtype, d, which):
+    """Everything that reads Q, K and V takes the group-major copies, also what runs beside the kernels that write O."""
+    gen = torch.Generator(device="cuda").manual_seed(d)
+    X = [(torch.randn(1, 16, 4096, d, generator=gen, device="cuda") * d ** -0.25).to(dtype) for _ in range(3)]
+    plan = B.sparsepr_plan(*X, block=64, density=0.3, n_sample=64, n_probe=1024, softmax_scale=1.0)
+    ref = B.sparsepr_attend(plan, *X)
+    for _ in range(3):
+        Y = [x.clone() for x in X]
+        assert torch.equal(B.sparsepr_attend(plan, *Y, out=Y[which]), ref)
