@@ -345,9 +345,11 @@ k_kmeans_assign_tc(const __grid_constant__ CUtensorMap mapXh, const __grid_const
       if (ok && mine) {
         // Bound on |computed score - true score|.  A bf16 rounding is off by at most 2^-8 relative, so the words of x and
         // of 2 mu leave 2^-16 each and the dropped product xl.ml another 2^-16 of 2 |x| |mu|: 9.2e-5 in all.  Accumulation
-        // in fp32: 13 steps that add 17 terms, each aligned to the largest and cut at 2^-24 of it, which is at most
-        // 2 |x| |mu| + |mu|^2: 1.4e-5 of that.
-        const float E = 1.25e-4f * xn * mm + 1.5e-5f * mm * mm;
+        // in fp32: 13 steps that add 17 terms, the largest at most 2 |x| |mu| + |mu|^2.  How the unit aligns them is not documented;
+        // a sum delivered in float32 keeps at least that format's places below the largest term, so each term is allowed to lose 2^-23
+        // of it: 2.7e-5.  (Measured with words at their worst, cancelling terms and terms just below the last place of a large one:
+        // at most 7e-7 of it, and 0.07 of E in all.)
+        const float E = 1.5e-4f * xn * mm + 2.7e-5f * mm * mm;
         decided = second - best > 2.f * E;
         if (decided) {
           moved = old_a != bi;

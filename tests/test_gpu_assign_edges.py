@@ -24,6 +24,27 @@ def test_assign_at_the_edges(n, C, r):
     assert np.array_equal(a, orc.kmeans_assign(X, mu))
 
 
+@pytest.mark.parametrize("r", [16, 48, 64])
+def test_assign_where_the_scores_are_least_exact(r):
+    """Decisions against float64 on rows whose scores lose most: large norms with small differences, terms that cancel, words of the
+    split at their worst, terms just below the last place of a large one, and centroid pairs that lie nearly alike about the rows."""
+    rng = np.random.default_rng(r)
+    n, C = 3000, 150
+    N = lambda *s: rng.normal(size=s)
+    worst = 1 + 2.0 ** -8 - 2.0 ** -17
+    small = lambda k: np.concatenate([np.ones((k, 1)), 2.0 ** -11 * (1 + rng.random((k, r - 1)))], 1)
+    mid = N(C // 2, r)
+    off = 1e-4 * N(C // 2, r)
+    cases = [(N(n, r) + 100 / r ** 0.5, N(C, r) + 100 / r ** 0.5),
+             (np.sign(N(n, r)) * worst * 2.0 ** rng.integers(-6, 7, (n, r)), np.sign(N(C, r)) * worst * 2.0 ** rng.integers(-6, 7, (C, r))),
+             (small(n), -small(C)), (100 * N(n, r), 1e-3 * N(C, r)), (1e-3 * N(n, r), 100 * N(C, r)),
+             (mid[rng.integers(0, C // 2, n)] + 1e-3 * N(n, r), np.concatenate([mid + off, mid - off]))]
+    for X, mu in cases:
+        X, mu = X.astype(np.float32), mu.astype(np.float32)
+        a = B.sparsepr_stage_assign(torch.from_numpy(X).cuda(), torch.from_numpy(mu).cuda()).cpu().numpy()
+        assert np.array_equal(a, orc.kmeans_assign(X, mu))
+
+
 @pytest.mark.parametrize("N,C,iters", [(1000, 130, 8), (2047, 128, 5), (4100, 300, 8)])
 def test_updated_sums_follow_the_definition(N, C, iters):
     """Query partition of a plan against Lloyd's iteration in float64 on the features the plan exports.  The centroids of the
