@@ -48,7 +48,7 @@ def test_assign_where_the_scores_are_least_exact(r):
 @pytest.mark.parametrize("N,C,iters", [(1000, 130, 8), (2047, 128, 5), (4100, 300, 8)])
 def test_updated_sums_follow_the_definition(N, C, iters):
     """Query partition of a plan against Lloyd's iteration in float64 on the features the plan exports.  The centroids of the
-    two differ by a float32 rounding (6e-8), which can only decide a near-tie otherwise: at most 0.5 % of the rows."""
+    two differ by a float32 rounding (6e-8), and one row in about a million is that near a tie: at most one row differs."""
     gen = torch.Generator(device="cuda").manual_seed(N)
     Q, K = [torch.randn(1, 2, N, 128, device="cuda", generator=gen).mul_(128 ** -0.25).bfloat16() for _ in range(2)]
     kw = dict(density=0.5, Ck=C, Cq=C, n_sample=64, n_probe=16, softmax_scale=1.0, kmeans_iters=iters)
@@ -58,4 +58,4 @@ def test_updated_sums_follow_the_definition(N, C, iters):
     phi = B.sparsepr_plan_export_features(plan, fields=("phi_Q",))["phi_Q"]
     for h in range(2):
         ref, _ = orc.kmeans(phi[h], C, orc.stride_sample(C, N, 0, orc.TAG_Q_INIT, h), iters)
-        assert (a[h] == ref).mean() >= 0.995, (a[h] == ref).mean()
+        assert (a[h] != ref).sum() <= 1, (a[h] != ref).sum()

@@ -50,3 +50,55 @@ def test_dense_pairs(heads, N):
     O = B.sparsepr_dense(Q, K, V, 128 ** -0.5)
     for i in sorted({0, heads - 1}):
         assert_bf16_close(to_np(O[0, i]), orc.dense_attention(to_np(Q[0, i]), to_np(K[0, i]), to_np(V[0, i]), 128 ** -0.5))
+
+
+def sms():
+    return torch.cuda.get_device_properties(0).multi_processor_count
+
+
+def bnhd(gen, B_, H, N, d):
+    return torch.randn(B_, N, H, d, device="cuda", generator=gen).bfloat16().transpose(1, 2)
+
+
+@pytest.mark.parametrize("d,group", [(64, 1), (128, 1), (128, 4)])
+@pytest.mark.parametrize("N", [129, 384, 1000])
+def test_dense_pairs_batched(N, d, group):
+    """Two query tiles per CTA with two batch entries, tensors stored as [B, N, H, d] and several query heads to a K/V head, on as
+    many heads as make more than one round of single tiles on this GPU."""
+    tiles = -(-N // 128)
+    H = -(-2 * sms() // (2 * tiles) // 4) * 4                        # two rounds of tiles (or a little more), one of pairs
+    gen = torch.Generator(device="cuda").manual_seed(N + d)
+    Q, K, V = bnhd(gen, 2, H, N, d), bnhd(gen, 2, H // group, N, d), bnhd(gen, 2, H // group, N, d)
+    O = B.sparsepr_dense(Q, K, V, d ** -0.5)
+    assert O.stride() == Q.stride()
+    for b, h in [(0, 0), (0, H - 1), (1, 1), (1, H // 2), (1, H - 1)]:
+        assert_bf16_close(to_np(O[b, h]), orc.dense_attention(to_np(Q[b, h]), to_np(K[b, h // group]), to_np(V[b, h // group]), d ** -0.5))
+
+
+@pytest.mark.parametrize("group", [1, 4])
+def test_pairs_batched(group):
+    """The list of pairs with two batch entries, [B, N, H, d] and grouped queries: enough rows for it on this GPU, three rounds of tiles."""
+    rng = np.random.default_rng(group)
+    N, C, d = sum(SIZES), len(SIZES), 128
+    H = -(-3 * sms() * 128 // (2 * N) // 4) * 4 + 4
+    gen = torch.Generator(device="cuda").manual_seed(group)
+    Q, K, V = bnhd(gen, 2, H, N, d), bnhd(gen, 2, H // group, N, d), bnhd(gen, 2, H // group, N, d)
+    aK = [rng.permutation(np.repeat(np.arange(C), rng.permutation(SIZES))) for _ in range(2 * H // group)]
+    aQ, ptr, idx = [], [], []
+    for i in range(2 * H):
+        aQ.append(rng.permutation(np.repeat(np.arange(C), rng.permutation(SIZES))))
+        full = int(np.argmax(np.bincount(aK[i // group], minlength=C)))
+        routes = [np.unique(np.append(rng.choice(C, size=n, replace=False), full)) for n in rng.permutation([C] + list(range(1, C)))]
+        ptr.append(np.concatenate([[0], np.cumsum([len(r) for r in routes])]))
+        idx.append(np.concatenate(routes))
+    kw = dict(block=-(-N // C), density=0.5, n_sample=64, n_probe=0, mode=1, softmax_scale=d ** -0.5)
+    plan = B.sparsepr_plan_import(Q, K, V, dict(kv_assign=np.stack(aK), q_assign=np.stack(aQ), route_ptr=np.stack(ptr), route_idx=idx), **kw)
+    O, Osp = B.sparsepr_attend(plan, Q, K, V, return_sparse=True)
+    O2 = B.sparsepr_attend(plan, Q, K, V)
+    assert B.sparsepr_plan_stats(plan)["device_error"] == 0
+    for i in [0, 1, H - 1, H, 2 * H - 1]:
+        b, h = divmod(i, H)
+        kv = (K[b, h // group], V[b, h // group])
+        ref = orc.sparse_attention(to_np(Q[b, h]), to_np(kv[0]), to_np(kv[1]), aQ[i], aK[i // group], ptr[i], idx[i], d ** -0.5)
+        for out in (O[b, h], Osp[b, h], O2[b, h]):
+            assert_bf16_close(to_np(out), ref)
