@@ -295,7 +295,7 @@ void carve_plan(Carver& c, const Resolved& r, sparsepr_plan_s* p) {
   float* score = c.take<float>(BH * (size_t)r.Cq * r.Ck);
   int* rptr = c.take<int>(BH * (r.Cq + 1)); int* ridx = c.take<int>(BH * (size_t)r.Cq * r.Ck);
   const bool f32 = r.dtype == SPARSEPR_F32;
-  int4* items = c.take<int4>(f32 ? attention_f32_items((int)BH, (int)N, r.Cq) : BH * (attention_tc_pairs((int)BH, (int)N) + attention_tc_singles((int)BH, (int)N, r.Cq)));
+  int4* items = c.take<int4>(f32 ? attention_f32_items((int)BH, (int)N, r.Cq) : BH * (attention_tc_pairs((int)BH, (int)N, r.d) + attention_tc_singles((int)BH, (int)N, r.Cq, r.d)));
   int* ikeys = c.take<int>(BH * r.Cq); int* icount = c.take<int>(f32 ? 1 : 2 * BH);
   RouteState* rs = c.take<RouteState>(BH);
   double* pd = c.take<double>(BH * N);
@@ -327,7 +327,7 @@ void launch_tiles(const sparsepr_plan_s* p, cudaStream_t st) {
   if (r.dtype == SPARSEPR_F32) {
     launch_f32_items(p->q_off, p->kv_off, p->route_ptr, p->route_idx, r.BH, r.N, r.Cq, r.Ck, p->item_keys, p->items, p->n_items, st);
   } else {
-    launch_tc_items(p->q_off, p->kv_off, p->route_ptr, p->route_idx, r.BH, r.N, r.Cq, r.Ck, r.G, p->item_keys, p->items, p->n_items, st);
+    launch_tc_items(p->q_off, p->kv_off, p->route_ptr, p->route_idx, r.BH, r.N, r.Cq, r.Ck, r.d, r.G, p->item_keys, p->items, p->n_items, st);
     launch_remainder_rows(p->q_off, p->route_ptr, p->route_idx, r.BH, r.Cq, r.Ck, r.N, p->rem_pos, p->rem_grp, p->rem_cnt, st);
   }
 }
@@ -772,7 +772,7 @@ static sparsepr_status_t attend_impl(const sparsepr_plan_t* p, const void* Q, co
     if (!overlap) cudaEventRecord(p->ev_fork, st);                // (with the probes' overlap the event is recorded already)
     cudaStreamWaitEvent(p->side2, p->ev_fork, 0);
     if (!launch_attention_packed(aa, p->rem_pos, p->rem_grp, p->rem_cnt, p->side2)) return SPARSEPR_ERR_CUDA;
-    if (attention_tc_pairs(r.BH, r.N) && !launch_attention_tc(aa, p->side2, true)) return SPARSEPR_ERR_CUDA;
+    if (attention_tc_pairs(r.BH, r.N, r.d) && !launch_attention_tc(aa, p->side2, true)) return SPARSEPR_ERR_CUDA;
     if (!launch_attention_tc(aa, st)) return SPARSEPR_ERR_CUDA;
     cudaEventRecord(p->ev_join2, p->side2);
     cudaStreamWaitEvent(st, p->ev_join2, 0);

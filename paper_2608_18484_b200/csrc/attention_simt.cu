@@ -557,17 +557,18 @@ __global__ void __launch_bounds__(kItemBuckets) k_tc_items(const int* __restrict
   }
   if (threadIdx.x == 0) n_items[single * gridDim.x + bh] = total;
 }
-// Two tiles per CTA where one per CTA gives the SMs three rounds or more: a pair takes 1.6 times as long as one tile, so that with few tiles
-// it is better to have them on as many SMs.  (480p-like, 24 heads, 45 rounds: kernel 4350 us with tiles alone, 4240 with pairs; 2 heads of
-// 4770 tokens, half a round: call 1167 us with tiles alone, 1171 with pairs.)
-int attention_tc_pairs(int BH, int N) { return (i64)BH * N >= (i64)3 * sm_count() * 128 ? (N + 128) / 129 : 0; }      // (a pair has more than 128 rows)
-int attention_tc_singles(int BH, int N, int Cq) { return attention_tc_pairs(BH, N) ? Cq : (N + 127) / 128 + Cq; }
-void launch_tc_items(const int* q_off, const int* kv_off, const int* route_ptr, const int* route_idx, int BH, int N, int Cq, int Ck, int kv_div, int* boxes, int4* items,
+// Two tiles per CTA where one per CTA gives the SMs 20 rounds or more (d = 64: 40): below, and above all where the longest tiles decide,
+// it is better to have the tiles on as many SMs.  Attend on a kept plan, us with tiles alone and with pairs: 8 heads of 9360 tokens (4
+// rounds) 233, 340; 12 of 9360 (6) 320, 371; 12 of 18720 (12) 895, 901; 8 of 49152 (21) 3795, 3767; 24 of 32760 (42) 4951, 4901; 40
+// of 75600 (160) 37950, 37220.  d = 64: 16 of 17550 (15) 1235, 1272; 16 of 35100 (30) 4253, 4286; 24 of 32760 (42) 3373, 3360.
+int attention_tc_pairs(int BH, int N, int d) { return (i64)BH * N >= (i64)(d == 128 ? 20 : 40) * sm_count() * 128 ? (N + 128) / 129 : 0; }      // (a pair has more than 128 rows)
+int attention_tc_singles(int BH, int N, int Cq, int d) { return attention_tc_pairs(BH, N, d) ? Cq : (N + 127) / 128 + Cq; }
+void launch_tc_items(const int* q_off, const int* kv_off, const int* route_ptr, const int* route_idx, int BH, int N, int Cq, int Ck, int d, int kv_div, int* boxes, int4* items,
                      int* n_items, cudaStream_t st) {
   k_route_keys<<<dim3((Cq + 31) / 32, BH), 1024, 0, st>>>(kv_off, route_ptr, route_idx, Cq, Ck, kv_div, 16, boxes);
   int shift = 0;
   while (((N + 15) / 16 + Ck) >> shift >= kItemBuckets) ++shift;
-  k_tc_items<<<dim3(BH, 2), kItemBuckets, 0, st>>>(q_off, route_ptr, boxes, Cq, kRemRows, shift, attention_tc_pairs(BH, N), attention_tc_singles(BH, N, Cq), items, n_items);
+  k_tc_items<<<dim3(BH, 2), kItemBuckets, 0, st>>>(q_off, route_ptr, boxes, Cq, kRemRows, shift, attention_tc_pairs(BH, N, d), attention_tc_singles(BH, N, Cq, d), items, n_items);
 }
 
 template <int D>

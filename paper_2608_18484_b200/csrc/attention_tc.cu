@@ -1039,21 +1039,23 @@ bool launch_attention_tc(const AttnArgs& a, cudaStream_t st, bool pairs) {
   Params p{};
   p.BH = a.BH; p.H = a.H; p.N = a.N; p.Cq = a.Cq; p.Ck = a.Ck; p.sparse = sparse; p.kv_div = kvd;
   p.scale_log2 = a.scale * 1.4426950408889634f;
-  p.kv_off = a.kv_off; p.route_idx = a.route_idx; p.q_perm = a.q_perm; p.items = a.items + (pairs ? 0 : (i64)a.BH * attention_tc_pairs(a.BH, a.N)); p.n_items = a.n_items + (pairs ? 0 : a.BH);
+  p.kv_off = a.kv_off; p.route_idx = a.route_idx; p.q_perm = a.q_perm; p.items = a.items + (pairs ? 0 : (i64)a.BH * attention_tc_pairs(a.BH, a.N, d)); p.n_items = a.n_items + (pairs ? 0 : a.BH);
   p.O = (__nv_bfloat16*)a.O; for (int i = 0; i < 3; ++i) p.os[i] = a.os[i];
   p.O_sparse = a.O_sparse; p.O_lo = (__nv_bfloat16*)a.O_lo; p.err = a.err;
   const auto run = [&](auto kernel, int ctas, size_t bytes) { kernel<<<dim3(ctas, a.BH), kThreads, bytes, st>>>(mq, mq64, mk, mv, p); };
-  // Two query tiles per CTA for dense calls: a pair takes about 1.6 times as long as one tile, so that it pays unless the CTAs of one
-  // tile leave SMs idle (or fill their last round where the pairs do not): 8 heads of 4096 tokens, two rounds of tiles, one of pairs,
-  // 81 -> 72 us; 2 heads of 4770 tokens, one round of tiles, 49 us, which pairs on half the SMs would lengthen.
+  // Two query tiles per CTA for dense calls: a pair takes about 1.6 times as long as one tile (D = 64, whose two words of P keep the
+  // tensor cores twice as long: 1.8 times), so that it pays unless the CTAs of one tile leave SMs idle (or fill their last round where
+  // the pairs do not).  8 heads of 4096 tokens, two rounds of tiles, one of pairs: 79 us with tiles alone, 66 with pairs (D = 64: 96, 86);
+  // 24 heads of 32760 tokens 12.7 ms, 11.0 (D = 64: 13.8, 13.3); 2 heads of 4770 tokens, one round of tiles, 49 us, which pairs on
+  // half the SMs would lengthen.
   const int tiles = (a.N + kTile - 1) / kTile, sms = sm_count();
   const auto rounds = [&](int per_head) { return ((i64)per_head * a.BH + sms - 1) / sms; };
-  if (sparse ? pairs : 100 * rounds(tiles) > 164 * rounds((tiles + 1) / 2)) {
-    const int ctas = sparse ? attention_tc_pairs(a.BH, a.N) : (tiles + 1) / 2;
+  if (sparse ? pairs : 100 * rounds(tiles) > (d == 128 ? 164 : 180) * rounds((tiles + 1) / 2)) {
+    const int ctas = sparse ? attention_tc_pairs(a.BH, a.N, d) : (tiles + 1) / 2;
     if (d == 128) run(k_attention_tc<128, true>, ctas, kSmemBytes<128, true>);
     else run(k_attention_tc<64, true>, ctas, kSmemBytes<64, true>);
   } else {
-    const int ctas = sparse ? attention_tc_singles(a.BH, a.N, a.Cq) : tiles;
+    const int ctas = sparse ? attention_tc_singles(a.BH, a.N, a.Cq, d) : tiles;
     if (d == 128) run(k_attention_tc<128, false>, ctas, kSmemBytes<128, false>);
     else run(k_attention_tc<64, false>, ctas, kSmemBytes<64, false>);
   }

@@ -131,9 +131,9 @@ cudaError_t init_attention_tc();
 bool attention_tc_supported(const AttnArgs& a);
 // block-sparse calls: items of launch_tc_items, made once the routes are known: lists of pairs of tiles [BH][attention_tc_pairs] and of
 // tiles alone [BH][attention_tc_singles], their lengths n_items [2][BH]; `boxes` [BH][Cq].  `pairs`: which list a launch takes
-int attention_tc_pairs(int BH, int N);
-int attention_tc_singles(int BH, int N, int Cq);
-void launch_tc_items(const int* q_off, const int* kv_off, const int* route_ptr, const int* route_idx, int BH, int N, int Cq, int Ck, int kv_div, int* boxes, int4* items,
+int attention_tc_pairs(int BH, int N, int d);
+int attention_tc_singles(int BH, int N, int Cq, int d);
+void launch_tc_items(const int* q_off, const int* kv_off, const int* route_ptr, const int* route_idx, int BH, int N, int Cq, int Ck, int d, int kv_div, int* boxes, int4* items,
                      int* n_items, cudaStream_t st);
 bool launch_attention_tc(const AttnArgs& a, cudaStream_t st, bool pairs = false);
 // Query-group remainders of 1..kRemRows rows are left out of the 128-row kernel's tiles and handled by attention_packed.cu

@@ -14,7 +14,7 @@ SIZES = [1, 15, 16, 17, 32, 33, 0, 64, 65, 127, 128, 129, 160, 161, 255, 256, 25
 
 
 @pytest.mark.parametrize("d", [64, 128])
-@pytest.mark.parametrize("heads", [3, 20], ids=["alone", "pairs"])     # few tiles: one per CTA; many: two tiles of a group per CTA
+@pytest.mark.parametrize("heads", [3, 20], ids=["few", "many"])
 def test_row_and_key_counts(heads, d):
     rng = np.random.default_rng(d)
     N, C = sum(SIZES), len(SIZES)
@@ -75,12 +75,13 @@ def test_dense_pairs_batched(N, d, group):
         assert_bf16_close(to_np(O[b, h]), orc.dense_attention(to_np(Q[b, h]), to_np(K[b, h // group]), to_np(V[b, h // group]), d ** -0.5))
 
 
-@pytest.mark.parametrize("group", [1, 4])
-def test_pairs_batched(group):
-    """The list of pairs with two batch entries, [B, N, H, d] and grouped queries: enough rows for it on this GPU, three rounds of tiles."""
+@pytest.mark.parametrize("d,group", [(64, 1), (128, 1), (128, 4)])
+def test_pairs_batched(d, group):
+    """The list of pairs with two batch entries, [B, N, H, d] and grouped queries: enough rows for it on this GPU, 20 rounds of tiles
+    (40 at d = 64)."""
     rng = np.random.default_rng(group)
-    N, C, d = sum(SIZES), len(SIZES), 128
-    H = -(-3 * sms() * 128 // (2 * N) // 4) * 4 + 4
+    N, C = sum(SIZES), len(SIZES)
+    H = -(-(20 if d == 128 else 40) * sms() * 128 // (2 * N) // 4) * 4 + 4
     gen = torch.Generator(device="cuda").manual_seed(group)
     Q, K, V = bnhd(gen, 2, H, N, d), bnhd(gen, 2, H // group, N, d), bnhd(gen, 2, H // group, N, d)
     aK = [rng.permutation(np.repeat(np.arange(C), rng.permutation(SIZES))) for _ in range(2 * H // group)]
