@@ -367,7 +367,7 @@ void carve_attend(Carver& c, const Resolved& r, AttendWs* w) {
   const bool f32 = r.dtype == SPARSEPR_F32;
   __nv_bfloat16* Qp = c.take<__nv_bfloat16>(f32 ? 0 : BH * M1 * d);
   float* X = c.take<float>(BH * M1 * d); float* Dn = c.take<float>(BH * M1 * d);
-  float* A = c.take<float>(BH * d * d); float* cc = c.take<float>(BH * d);
+  float* A = c.take<float>(f32 ? BH * d * d : 0); float* cc = c.take<float>(BH * d);
   float* Psi = c.take<float>(BH * d * d);
   __nv_bfloat16* At = c.take<__nv_bfloat16>(f32 ? 0 : map_words(r.d) * BH * d * d);   // the correction map as bf16 words
   float* fpart = c.take<float>(f32 ? attention_f32_part_floats(r.d) : 0);

@@ -279,7 +279,7 @@ __global__ void __launch_bounds__(512, 1) k_fit_solve(FitArgs a) {
 }
 
 // T = B Psi (d x r); A = diag(1/s_x) T Psi^T; c = mu_R - mu_x A.  float64 throughout.  Grid (d / 16 + 1, heads): CTA x
-// owns 16 rows of A; the last one forms c = mu_R - ((mu_x / s_x) B) Psi Psi^T.  With `At` the map is also written as the two
+// owns 16 rows of A; the last one forms c = mu_R - ((mu_x / s_x) B) Psi Psi^T.  With `At` the map is written as the two
 // (d = 64: three) bf16 words the correction pass multiplies with: At [words][BH][n][k], first words, then what their rounding dropped.
 // (One CTA per head: 132 us at two heads of d = 128, 630 us beside the attention kernels at 24 heads; now 25 and 125 us.)
 constexpr int kCompRows = 16;
@@ -297,8 +297,9 @@ __global__ void __launch_bounds__(256) k_fit_compose(FitArgs a, int r) {
   __nv_bfloat16* Ah = a.At ? a.At + (i64)bh * d * d : nullptr;
   __nv_bfloat16* Al = a.At ? a.At + ((i64)gridDim.y + bh) * d * d : nullptr;
   auto put = [&](int i, int j, float x) {
-    A[(i64)i * d + j] = x;
-    if (Ah) {
+    if (!Ah) {
+      A[(i64)i * d + j] = x;
+    } else {
       const __nv_bfloat16 hb = __float2bfloat16_rn(x);
       Ah[(i64)j * d + i] = hb;
       const float rest = x - __bfloat162float(hb);

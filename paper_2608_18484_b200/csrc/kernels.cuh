@@ -183,8 +183,8 @@ struct FitArgs {
   const float *X, *Dn, *w;             // [BH][M][d], [BH][M][d], [BH][M]
   double* scratch;                     // see fit_scratch_doubles
   double* eig_ws;                      // eig_scratch_doubles(BH, d) doubles
-  float *A, *c;                        // outputs [BH][d][d], [BH][d]
-  __nv_bfloat16* At;                   // optional output [map_words(d)][BH][d][d]: A transposed, as bf16 words (correction pass)
+  float *A, *c;                        // outputs [BH][d][d] (unless At is given), [BH][d]
+  __nv_bfloat16* At;                   // output in the place of A, [map_words(d)][BH][d][d]: A transposed, as bf16 words (correction pass)
   float* Psi;                          // [BH][d][r] scratch
   int* err;
 };
