@@ -102,20 +102,23 @@ class ClockSampler:
 
 
 # --------------------------------------------------------------------------------------
-def launches_per_call(T, fitted, tensor_path):
-    """Kernels of this library launched by one plan + attend call (memsets excluded)."""
-    if tensor_path:      # per side: init, first norms, split features; per iteration: assign, recheck; first sums; T-1 updates
-        kmeans = 2 + 1 + 2 * T + (1 if T > 1 else 0) + (T - 1)
-    else:                # init, first norms, T assignments, T-1 updates
-        kmeans = 2 + T + (T - 1)
-    # per side: Gram, eigen-solver (Householder, vectors, orthogonalisation, back-transformation, marked-matrix fallback), projection (+ split of
-    # the feature map), k-means, sort + means; then probes; route; list of tiles (2) + remainder rows
-    plan = 2 * (6 + (2 if tensor_path else 1) + kmeans + 2) + 2 + 2 + 3
+def pair_rounds(d):
+    """Rounds of 128-row tiles from which the block-sparse call has a launch of tile pairs (attention_tc_pairs)."""
+    return 20 if d == 128 else 40
+
+
+def launches_per_call(T, fitted, bf16, pairs):
+    """Kernels of this library launched by one plan + attend call (memsets excluded) of the method's own partition."""
+    # per side: init, first norms, split features; per iteration: assign, recheck; first sums; T-1 updates
+    kmeans = 2 + 1 + 2 * T + (1 if T > 1 else 0) + (T - 1)
+    # per side: Gram, eigen-solver (Householder, vectors, orthogonalisation, back-transformation, marked-matrix fallback), projection (bf16: + split
+    # of the feature map), k-means, sort + means; then probes; route; list of tiles (2), bf16: + remainder rows
+    plan = 2 * (6 + (2 if bf16 else 1) + kmeans + 2) + 2 + 2 + (3 if bf16 else 2)
     if not fitted:
         plan -= 2
-    attend = 3 + 1 + (1 if tensor_path else 0)       # gathers, attention (+ the packed-remainder kernel)
+    attend = 3 + 1 + (1 + (1 if pairs else 0) if bf16 else 0)       # gathers, attention (bf16: + the packed remainders, + pairs of tiles)
     if fitted:
-        attend += (3 if tensor_path else 2) + 9 + 1  # probe rows (+gather) + merge, fit (eigen-solver: five launches), probe write
+        attend += (3 if bf16 else 2) + 9 + 1         # probe rows (+gather) + merge, fit (eigen-solver: five launches), probe write
         attend += 1                                  # correction pass
     return plan + attend
 
@@ -486,9 +489,8 @@ def main():
     flops = 4.0 * wl.d * st["routed_pairs"]                       # QK^T and PV on executed pairs, all heads
     issued = 4.0 * wl.d * st["padded_tile_pairs"]
     achieved = flops / (attn_ms * 1e-3) / 1e12
-    tensor_path = wl.dtype == "bf16" and wl.d == 128
-    if tensor_path:
-        # tcgen05 kernel timed inside a long step: the sustained bf16 GEMM peak is the denominator
+    pairs = wl.dtype == "bf16" and wl.H * wl.N >= pair_rounds(wl.d) * 128 * torch.cuda.get_device_properties(dev).multi_processor_count
+    if wl.dtype == "bf16":
         # tcgen05 kernels timed inside a long step: the sustained bf16 GEMM peak is the denominator of `frac`; the
         # fraction of the burst peak (the fair one when the clocks stay at their maximum) is printed beside it
         traffic = NCU_DRAM_BYTES_PER_HEAD.get(wl.name)
@@ -532,7 +534,7 @@ def main():
                              "note": "the call as timed (side streams overlap); stage_ms come from a one-stream run"},
            "kmeans_passes": [st["kmeans_passes_kv"], st["kmeans_passes_q"]],
            "device_error": st["device_error"], "assign_rechecked_rows": st["assign_rechecked_rows"],
-           "gpu_launches": launches_per_call(params.kmeans_iters or 8, True, wl.dtype == "bf16" and wl.d == 128) * args.steps,
+           "gpu_launches": launches_per_call(params.kmeans_iters or 8, True, wl.dtype == "bf16", pairs) * args.steps,
            "warm_started_call": warm, "roofline": roofline, "clocks": clocks, "e2e": e2e}
     if not args.no_cpu_baseline and world == 1:
         def gpu_call(small, Q, K, V):
