@@ -31,10 +31,10 @@ if ROOT not in sys.path:
 METRIC = "sparsepr_attn_ms_per_call"
 UNIT = "ms/call"
 
-# DRAM read + write bytes per head of one launch of the two block-sparse kernels, from ncu captures of 6 heads
-# (capture-size rule) of the named workload; a workload without a capture reports null.
+# DRAM read + write bytes per head of one launch of each block-sparse kernel, from ncu captures of 12 heads of the named
+# workload (tiles alone, pairs of tiles, packed remainders); a workload without a capture reports null.
 NCU_DRAM_BYTES_PER_HEAD = {
-    "video-dit-480p-like": {"k_attention_tc": 36.39e6, "k_attention_packed": 20.39e6},
+    "video-dit-480p-like": {"k_attention_tc": 33.07e6, "k_attention_tc (pairs)": 25.69e6, "k_attention_packed": 31.81e6},
 }
 
 
@@ -494,13 +494,13 @@ def main():
         # tcgen05 kernels timed inside a long step: the sustained bf16 GEMM peak is the denominator of `frac`; the
         # fraction of the burst peak (the fair one when the clocks stay at their maximum) is printed beside it
         traffic = NCU_DRAM_BYTES_PER_HEAD.get(wl.name)
-        roofline = {"kernel": "k_attention_tc + k_attention_packed (block-sparse, tcgen05)", "bound": "tensor", "achieved": achieved,
+        roofline = {"kernel": "k_attention_tc (tiles alone and in pairs) + k_attention_packed (block-sparse, tcgen05)", "bound": "tensor", "achieved": achieved,
                     "peak": peaks["bf16_sustained"], "unit": "TFLOP/s", "frac": achieved / peaks["bf16_sustained"],
                     "frac_of_burst_peak": achieved / peaks["bf16_tflops"], "burst_peak": peaks["bf16_tflops"],
                     "sm_mhz_median": (clocks or {}).get("sm_mhz"),
                     "traffic": (sum(traffic.values()) * wl.H if traffic else None), "traffic_unit": "bytes",
-                    "traffic_source": ("ncu dram__bytes_read.sum + dram__bytes_write.sum of one launch of each of the two kernels, "
-                                       "captured at 6 heads of this workload, per head x H (heads are independent CTAs over "
+                    "traffic_source": ("ncu dram__bytes_read.sum + dram__bytes_write.sum of one launch of each of the three kernels, "
+                                       "captured at 12 heads of this workload, per head x H (heads are independent CTAs over "
                                        "disjoint memory)") if traffic else None,
                     "algorithmic_bytes": 4.0 * wl.H * wl.N * wl.d * 2,
                     "peak_source": peaks["source"] + " cuBLAS bf16, sustained",

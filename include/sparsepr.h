@@ -23,15 +23,22 @@
  *     points into the plan workspace; it is valid until the workspace is released
  *     or sparsepr_plan_destroy is called.  Process-wide state is limited to what is
  *     set up once and then reused: kernel attributes and the tensor-map encoder
- *     (first call), a pool of auxiliary streams and events (two streams and three
+ *     (first call), a pool of auxiliary streams and events (two streams and four
  *     events per plan alive at the same time, per device; created when the pool is
  *     empty, returned by sparsepr_plan_destroy, never freed), the SM count per
  *     device, and the scratch array of sparsepr_stage_assign_static.
  *   - All work is enqueued on `cuda_stream` (a cudaStream_t passed as void*)
  *     and is asynchronous, except the calls documented as synchronising.
+ *     sparsepr_attend orders itself behind the whole plan; under stream capture on
+ *     a plan that was made outside the capture it waits for that plan on the host.
+ *     Several threads may call sparsepr_attend on one plan, each with a workspace and
+ *     an output of its own.  O may take the place of Q, K or V in sparsepr_attend.
+ *   - Q, K and V are expected to be finite.  The bf16 kernels read the values of a routed
+ *     group in whole boxes of 16 rows, and those of many short query groups together, and
+ *     multiply what a row does not attend to by zero: a non-finite value there spreads.
  *   - Errors are return codes.  Argument errors are detected before anything
  *     is launched.  Conditions found on the device (non-finite input, a
- *     breakdown of the Cholesky factorisation, a bounded wait that ran out)
+ *     breakdown of the fit's elimination or probes without weight, a bounded wait that ran out)
  *     are recorded in a device error word that sparsepr_plan_stats reports.
  *     The word lives in the plan workspace and persists for the life of the plan;
  *     once a bounded wait has run out (SPARSEPR_ERR_TIMEOUT) the tensor-core
@@ -172,12 +179,11 @@ typedef struct {
  * *_PERMUTE = counting sort and group means; QUERY_METRIC = centroid Gram and its
  * eigen-decomposition; PROBE_SELECT; ROUTE = cell scores and selection.  Attend:
  * GATHER = group-major copies of Q, K, V; PROBE_ROWS = exact and hard-drop rows of
- * the probes; FIT = ridge fit and subspace; ATTENTION = block-sparse kernels (the 128-row
- * tiles and the packed group remainders, side by side on two streams);
- * CORRECTION = residual correction of Eq. 9 (zero where the block-sparse kernel applies
- * it in its epilogue); PROBE_WRITE.  DENSE = the dense entry point.  A call without a
- * profile runs PROBE_SELECT beside ROUTE and PROBE_ROWS + FIT beside ATTENTION on a second
- * stream, so its duration is less than the sum of the stages. */
+ * the probes; FIT = ridge fit and subspace; ATTENTION = block-sparse kernels (bf16: the 128-row
+ * tiles, alone and in pairs, and the packed group remainders, side by side on two streams);
+ * CORRECTION = residual correction of Eq. 9; PROBE_WRITE.  DENSE = the dense entry point.  A call
+ * without a profile runs ROUTE beside PROBE_SELECT and GATHER on streams of the plan's own, and
+ * PROBE_ROWS + FIT beside ATTENTION, so its duration is less than the sum of the stages. */
 enum {
   SPARSEPR_STAGE_KEY_METRIC = 0, SPARSEPR_STAGE_KEY_PROJECT, SPARSEPR_STAGE_KEY_KMEANS, SPARSEPR_STAGE_KEY_PERMUTE,
   SPARSEPR_STAGE_QUERY_METRIC, SPARSEPR_STAGE_QUERY_PROJECT, SPARSEPR_STAGE_QUERY_KMEANS, SPARSEPR_STAGE_QUERY_PERMUTE,
@@ -201,11 +207,12 @@ size_t sparsepr_attend_workspace_bytes(const sparsepr_shape_t* shape, const spar
  * probe set and routes of every head from Q and K (DEVICE, read only; V is not
  * read -- values never enter the partition features -- and may be NULL).
  * `workspace` is DEVICE memory of at least sparsepr_plan_workspace_bytes, 256-byte
- * aligned; the plan lives in it.  *out receives a HOST handle.  The probe selection may
- * still be running on a stream of the plan's own when the call returns: sparsepr_attend
- * orders its work behind it, sparsepr_plan_stats / _export / _destroy wait for it, so the
- * workspace may be released once sparsepr_plan_destroy has returned and the work queued on
- * `cuda_stream` is complete. */
+ * aligned; the plan lives in it.  *out receives a HOST handle.  Unless the plan has no probes,
+ * the probe selection, the routing and the lists of tiles may still be running on streams of
+ * the plan's own when the work queued on `cuda_stream` is complete: sparsepr_attend orders its work
+ * behind them, sparsepr_plan_stats / _export wait for them, and so does sparsepr_plan_destroy if no attend
+ * call came before.  The workspace may be released or used for something else once sparsepr_plan_destroy
+ * has returned and the work queued on `cuda_stream` and by the attend calls is complete. */
 sparsepr_status_t sparsepr_plan(const sparsepr_shape_t* shape, const sparsepr_params_t* params,
                                 const void* Q, const void* K, const void* V,
                                 void* workspace, size_t workspace_bytes, void* cuda_stream,
@@ -232,8 +239,9 @@ sparsepr_status_t sparsepr_plan_assignments(const sparsepr_plan_t* plan, const i
                                             const int32_t** q_assign);
 
 /* Stages 3-4 (Eq. 3, Eq. 8-10): O (DEVICE, written in original token order) from
- * Q, K, V (DEVICE) and a plan.  `workspace`: DEVICE, sparsepr_attend_workspace_bytes,
- * 256-byte aligned; its contents are scratch.  `O_sparse` (DEVICE, float32
+ * Q, K, V (DEVICE) and a plan.  `workspace`: DEVICE, sparsepr_attend_workspace_bytes (the group-major
+ * copies of Q, K and V; bf16 with probes: a second word of O; float32: up to 39 MB for tiles whose keys are
+ * cut into parts; the probe rows and the fit), 256-byte aligned; its contents are scratch.  `O_sparse` (DEVICE, float32
  * [B,H,N,dv] contiguous, may be NULL) additionally receives the uncorrected
  * hard-drop output O^sp in original order, for error reporting. */
 sparsepr_status_t sparsepr_attend(const sparsepr_plan_t* plan, const void* Q, const void* K, const void* V,
@@ -299,7 +307,7 @@ sparsepr_status_t sparsepr_plan_import(const sparsepr_shape_t* shape, const spar
                                        void* workspace, size_t workspace_bytes, void* cuda_stream,
                                        sparsepr_plan_t** out);
 
-/* Frees the HOST handle only. */
+/* Frees the HOST handle only (see sparsepr_plan for what it waits for). */
 void sparsepr_plan_destroy(sparsepr_plan_t* plan);
 
 /* ---- single stages, exposed so that the integer work can be checked bit for bit ---- */

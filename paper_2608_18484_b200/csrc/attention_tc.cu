@@ -31,13 +31,13 @@
 // read 9.1 to 10.4 TB/s from L2, 0.95 us per 64 KB and SM, and one tile per CTA takes 1.1 us per key tile).  Every tile has its
 // own four softmax warps, one row per thread, and its own issuer of both products; P takes the place of S (the
 // accumulators leave no other), so a tile alternates between the tensor cores and its softmax warps, while the other tile does
-// the opposite.  Bound by that chain: product 845 cycles (512 and what the other tile has queued), fetch and maximum 500,
-// exponentials 1200, P V and its completion 750 (with three pairs of eight by polynomial); 3300 cycles per key tile for both, where one
-// tile takes 2010.  The threads have
+// the opposite.  Bound by that chain; the account was taken while three pairs of eight went to the polynomial (one does now, 6 %
+// faster): product 845 cycles (512 and what the other tile has queued), fetch and maximum 500, exponentials 1200, P V and its
+// completion 750, 3300 cycles per key tile for both, where one tile takes 2010.  The threads have
 // 224 registers (setmaxnreg).  One pair of eight by polynomial instead of three: a warp alone is short of issue slots, not of
 // the special-function unit (dense, 12 heads of 18944 tokens: 1726 us with three, 1662 with two, 1630 with one, 1644 with none).
-// Dense, 24 heads of 32760 tokens: 12.0 -> 10.1 ms (the clock falls to 1.6 GHz under the power limit); the same two tiles left
-// to themselves fall into step (3900 cycles per key tile).
+// Dense, 24 heads of 32760 tokens, one call after the other: 12.7 -> 11.0 ms (the clock falls to 1.6 GHz under the power limit); the
+// same two tiles left to themselves fall into step (3900 cycles per key tile).
 // Epilogue: O / l, stored as bf16 at the original token index (inverse permutation).  The residual correction of
 // Eq. 9 is a pass of its own (correction_tc.cu) so that the fit can overlap this kernel; for that pass the part of
 // every element that the bf16 rounding dropped is stored as a second bf16 word (O_lo), so that the corrected output
