@@ -103,3 +103,24 @@ def test_pairs_batched(d, group):
         ref = orc.sparse_attention(to_np(Q[b, h]), to_np(kv[0]), to_np(kv[1]), aQ[i], aK[i // group], ptr[i], idx[i], d ** -0.5)
         for out in (O[b, h], Osp[b, h], O2[b, h]):
             assert_bf16_close(to_np(out), ref)
+
+
+@pytest.mark.parametrize("d", [64, 128])
+def test_pairs_with_correction(d):
+    """A fitted call whose tiles come in pairs, which hand their rows to the correction in two words, against calls on two heads of
+    it, whose tiles come alone.  d = 64: float32 up to the rounding, which then differs for few elements; d = 128: bf16 probabilities."""
+    N = 3100
+    H = -(-(20 if d == 128 else 40) * sms() * 128 // N) + 1
+    gen = torch.Generator(device="cuda").manual_seed(d)
+    Q, K, V = [torch.randn(1, H, N, d, device="cuda", generator=gen).mul_(d ** -0.25).bfloat16() for _ in range(3)]
+    kw = dict(Ck=8, Cq=8, density=0.5, n_sample=64, n_probe=16, softmax_scale=1.0, lam=10.0)     # groups of three tiles
+    plan = B.sparsepr_plan(Q, K, V, **kw)
+    O = B.sparsepr_attend(plan, Q, K, V)
+    assert B.sparsepr_plan_stats(plan)["device_error"] == 0
+    host = B.sparsepr_plan_export(plan)
+    for hs in ([0, 1], [H // 2, H - 1]):
+        q, k, v = [x[:, hs].contiguous() for x in (Q, K, V)]
+        O2 = B.sparsepr_attend(B.sparsepr_plan_import(q, k, v, {n: a[hs] for n, a in host.items()}, **kw), q, k, v)
+        assert_bf16_close(to_np(O[:, hs]), to_np(O2))
+        if d == 64:
+            assert (O[:, hs] != O2).double().mean() <= 5e-3
