@@ -240,7 +240,7 @@ sparsepr_status_t sparsepr_plan_assignments(const sparsepr_plan_t* plan, const i
 
 /* Stages 3-4 (Eq. 3, Eq. 8-10): O (DEVICE, written in original token order) from
  * Q, K, V (DEVICE) and a plan.  `workspace`: DEVICE, sparsepr_attend_workspace_bytes (the group-major
- * copies of Q, K and V; bf16 with probes: a second word of O; float32: up to 39 MB for tiles whose keys are
+ * copies of Q, K and V; bf16 with probes: a second word of O; float32: up to 79 MB for tiles whose keys are
  * cut into parts; the probe rows and the fit), 256-byte aligned; its contents are scratch.  `O_sparse` (DEVICE, float32
  * [B,H,N,dv] contiguous, may be NULL) additionally receives the uncorrected
  * hard-drop output O^sp in original order, for error reporting. */

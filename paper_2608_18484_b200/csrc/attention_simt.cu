@@ -514,9 +514,10 @@ void launch_correction_f32(const float* A, const float* c, void* O, const i64* o
 
 // Items of a list at most: four rounds of CTAs on every SM slot, and twice as many as tiles.
 size_t attention_f32_items(int BH, int N, int Cq) { return std::max((size_t)4 * 2 * sm_count(), (size_t)2 * BH * ((N + BM - 1) / BM + Cq)); }
-// Partial states of cut tiles at most, 39 MB at d = 128 whatever the size.  (8 heads of 7161 tokens, 1360 tiles: 3335 us with 4 per SM, 3347
-// with 8, 3342 with 16, 3343 with as many as items, which were 1.2 GB of workspace at 24 heads of 32760 tokens.)
-size_t attention_f32_slots() { return (size_t)8 * sm_count(); }
+// Partial states of cut tiles at most, 79 MB at d = 128 whatever the size.  (A drawn call of the float32 range: 2459 us with 8 per SM, 2433
+// with 16 and with 32; 8 heads of 7161 tokens: 3335 to 3347 us with 4, 8, 16 and as many as items, which were 1.2 GB of workspace at
+// 24 heads of 32760 tokens.)
+size_t attention_f32_slots() { return (size_t)16 * sm_count(); }
 size_t attention_f32_part_floats(int d) { return attention_f32_slots() * BM * (d + 2); }
 void launch_f32_items(const int* q_off, const int* kv_off, const int* route_ptr, const int* route_idx, int BH, int N, int Cq, int Ck, int* keys, int4* items,
                       int* n_items, cudaStream_t st) {
