@@ -514,8 +514,8 @@ void launch_correction_f32(const float* A, const float* c, void* O, const i64* o
 
 // Items of a list at most: four rounds of CTAs on every SM slot, and twice as many as tiles.
 size_t attention_f32_items(int BH, int N, int Cq) { return std::max((size_t)4 * 2 * sm_count(), (size_t)2 * BH * ((N + BM - 1) / BM + Cq)); }
-// Partial states of cut tiles at most, 79 MB at d = 128 whatever the size.  (A drawn call of the float32 range: 2459 us with 8 per SM, 2433
-// with 16 and with 32; 8 heads of 7161 tokens: 3335 to 3347 us with 4, 8, 16 and as many as items, which were 1.2 GB of workspace at
+// Partial states of cut tiles at most, 79 MB at d = 128 whatever the size.  (6 heads of 10224 tokens, d = 64: call 2459 us with 8 per SM, 2433
+// with 16 and with 32; 8 heads of 7161 tokens, d = 128: 3335 to 3347 us with 4, 8, 16 and as many as items, which were 1.2 GB of workspace at
 // 24 heads of 32760 tokens.)
 size_t attention_f32_slots() { return (size_t)16 * sm_count(); }
 size_t attention_f32_part_floats(int d) { return attention_f32_slots() * BM * (d + 2); }
