@@ -166,7 +166,7 @@ __global__ void __launch_bounds__(1024) k_route_select(const float* __restrict__
   else if (rem < 0) tstar = 1ull << 32;
   else {
     i64* whist = reinterpret_cast<i64*>(nqs + Cq + ((Cq + Ck) & 1));   // [nw][256], 8-byte aligned (see route_smem)
-    __shared__ i64 s_above;
+    __shared__ i64 s_above, s_hist[256];
     __shared__ int s_dstar;
     unsigned prefix = 0;
     i64 above = 0;                      // cost of the cells above the current bucket
@@ -217,15 +217,19 @@ __global__ void __launch_bounds__(1024) k_route_select(const float* __restrict__
         __syncwarp();
       }
       __syncthreads();
+      // the warps' histograms added up, a digit per thread (by one warp, eight digits per lane, this took most of a small call's time)
+      if (threadIdx.x < 256) {
+        i64 t = 0;
+#pragma unroll 8
+        for (int ww = 0; ww < 32; ++ww) t += whist[ww * 256 + threadIdx.x];
+        s_hist[threadIdx.x] = t;
+      }
+      __syncthreads();
       if (w == 0) {
         // lane l owns digits 8l .. 8l+7
         i64 loc[8], lsum = 0;
 #pragma unroll
-        for (int k = 0; k < 8; ++k) {
-          i64 t = 0;
-          for (int ww = 0; ww < nw; ++ww) t += whist[ww * 256 + lane * 8 + k];
-          loc[k] = t; lsum += t;
-        }
+        for (int k = 0; k < 8; ++k) { loc[k] = s_hist[lane * 8 + k]; lsum += loc[k]; }
         i64 suf = lsum;                                          // sum over lanes >= this lane
 #pragma unroll
         for (int o = 1; o < 32; o <<= 1) { const i64 t = __shfl_down_sync(0xffffffffu, suf, o); if (lane + o < 32) suf += t; }
