@@ -281,6 +281,8 @@ __global__ void __launch_bounds__(512, 1) k_fit_solve(FitArgs a) {
 // T = B Psi (d x r); A = diag(1/s_x) T Psi^T; c = mu_R - mu_x A.  float64 throughout.  Grid (d / 16 + 1, heads): CTA x
 // owns 16 rows of A; the last one forms c = mu_R - ((mu_x / s_x) B) Psi Psi^T.  With `At` the map is written as the two
 // (d = 64: three) bf16 words the correction pass multiplies with: At [words][BH][n][k], first words, then what their rounding dropped.
+// Bound by chains of float64 latencies: four columns of A per thread at a time, quotients and loads ahead of the chains (a call of two heads of
+// 4770 tokens 3 us shorter, 16 heads of 18000 tokens 10 us).
 // (One CTA per head: 132 us at two heads of d = 128, 630 us beside the attention kernels at 24 heads; now 25 and 125 us.)
 constexpr int kCompRows = 16;
 __global__ void __launch_bounds__(256) k_fit_compose(FitArgs a, int r) {
@@ -329,6 +331,7 @@ __global__ void __launch_bounds__(256) k_fit_compose(FitArgs a, int r) {
       for (int e = tid; e < kCompRows * r; e += 256) {
         const int i = e / r, t = e % r;
         double s0 = 0.0, s1 = 0.0;
+#pragma unroll 8
         for (int k = 0; k < d; k += 2) {
           s0 = fma(Bs[i * d + k], (double)Ps[k * ldp + t], s0);
           s1 = fma(Bs[i * d + k + 1], (double)Ps[(k + 1) * ldp + t], s1);
@@ -339,18 +342,33 @@ __global__ void __launch_bounds__(256) k_fit_compose(FitArgs a, int r) {
     }
     const int i = tid % kCompRows;         // one row per thread: consecutive lanes write consecutive entries of At
     const double rsx = 1.0 / sc[L.s_x + i0 + i];
-    for (int j = tid / kCompRows; j < d; j += 256 / kCompRows) {
-      double s = 0.0;
-      if (a.full_rank) s = Bs[i * d + j];  // every row of B lies in the row space of the probe residuals: B Psi Psi^T = B
-      else for (int t = 0; t < r; ++t) s = fma(Ts[i * r + t], (double)Ps[j * ldp + t], s);
-      put(i0 + i, j, (float)(s * rsx));
+    // four columns at a time: the sums over t are chains of float64 latencies (d / 16 is 4 or 8)
+    for (int j0 = tid / kCompRows; j0 < d; j0 += 4 * (256 / kCompRows)) {
+      double s[4] = {0.0, 0.0, 0.0, 0.0};
+      if (a.full_rank) {                   // every row of B lies in the row space of the probe residuals: B Psi Psi^T = B
+#pragma unroll
+        for (int u = 0; u < 4; ++u) s[u] = Bs[i * d + j0 + u * (256 / kCompRows)];
+      } else {
+#pragma unroll 4
+        for (int t = 0; t < r; ++t) {
+          const double x = Ts[i * r + t];
+#pragma unroll
+          for (int u = 0; u < 4; ++u) s[u] = fma(x, (double)Ps[(j0 + u * (256 / kCompRows)) * ldp + t], s[u]);
+        }
+      }
+#pragma unroll
+      for (int u = 0; u < 4; ++u) put(i0 + i, j0 + u * (256 / kCompRows), (float)(s[u] * rsx));
     }
     return;
   }
   // c: u = (mu_x / s_x) B by 256 / d parts of the rows, t = u Psi, c = mu_R - t Psi^T
   const int parts = 256 / d, part = tid / d, k = tid % d, per = d / parts;
+  double* ratio = Bs + 512;                // mu_x / s_x
+  if (tid < d) ratio[tid] = sc[L.mu_x + tid] / sc[L.s_x + tid];
+  __syncthreads();
   double u = 0.0;
-  for (int i = part * per; i < (part + 1) * per; ++i) u = fma(sc[L.mu_x + i] / sc[L.s_x + i], Bm[(size_t)i * d + k], u);
+#pragma unroll 16
+  for (int i = part * per; i < (part + 1) * per; ++i) u = fma(ratio[i], Bm[(size_t)i * d + k], u);
   Bs[part * d + k] = u;
   __syncthreads();
   if (tid < d) {
@@ -366,12 +384,14 @@ __global__ void __launch_bounds__(256) k_fit_compose(FitArgs a, int r) {
   }
   if (tid < r) {
     double t = 0.0;
+#pragma unroll 16
     for (int q = 0; q < d; ++q) t = fma(us[q], (double)Ps[q * ldp + tid], t);
     Ts[tid] = t;
   }
   __syncthreads();
   if (tid < d) {
     double s = 0.0;
+#pragma unroll 4
     for (int t = 0; t < r; ++t) s = fma(Ts[t], (double)Ps[tid * ldp + t], s);
     cvec[tid] = (float)(sc[L.mu_R + tid] - s);
   }
