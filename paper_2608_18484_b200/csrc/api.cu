@@ -270,16 +270,21 @@ struct sparsepr_plan_s {
 
 namespace {
 
+size_t plan_zero_ints(const Resolved& r) { return 64 + (size_t)r.BH * (2 + 2 * (r.T + 1) + 4); }
+
 void carve_plan(Carver& c, const Resolved& r, sparsepr_plan_s* p) {
   const size_t BH = r.BH, N = r.N, d = r.d;
-  int* err = c.take<int>(64);
+  // what a plan starts from zero, in one piece: error words, largest feature magnitudes and k-means counters of either side
+  int* err = c.take<int>(plan_zero_ints(r));
   int* recheck = err ? err + 1 : nullptr;
+  unsigned* maxabs = err ? reinterpret_cast<unsigned*>(err + 64) : nullptr;                        // [2 sides][BH]
+  int* km_changed = err ? err + 64 + 2 * BH : nullptr;
+  int* flagcnt = err ? km_changed + 2 * (size_t)(r.T + 1) * BH : nullptr;                          // per side two sets of per-head counters, used by alternate passes
   double* Mmat = c.take<double>(BH * d * d);
   double* lam = c.take<double>(BH * d);
   float* FK = c.take<float>(BH * d * r.rK);
   float* FQ = c.take<float>(BH * d * r.rQ);
   float* phi = c.take<float>(BH * N * r.Rmax);
-  unsigned* maxabs = c.take<unsigned>(BH);
   int* fx = c.take<int>(BH);
   float* mu = c.take<float>(BH * r.Cmax * r.Rmax);
   float* mu2 = c.take<float>(BH * r.Cmax);
@@ -306,8 +311,6 @@ void carve_plan(Carver& c, const Resolved& r, sparsepr_plan_s* p) {
   float* xnorm = c.take<float>(BH * N); int* flagged = c.take<int>(BH * N);
   __nv_bfloat16* Ft = c.take<__nv_bfloat16>(BH * (size_t)3 * 64 * 128);
   int* rem_pos = c.take<int>(f32 ? 0 : BH * N); int* rem_grp = c.take<int>(f32 ? 0 : BH * N); int* rem_cnt = c.take<int>(f32 ? 0 : BH);
-  int* km_changed = c.take<int>(2 * (size_t)(r.T + 1) * BH);
-  int* flagcnt = c.take<int>(2 * BH);                       // two sets of per-head counters, used by alternate passes
   double* eigws = c.take<double>(eig_scratch_doubles((int)BH, r.d));
   double* Mpool = c.take<double>(r.G > 1 ? (size_t)r.BHkv * d * d : 0);
   if (p) {
@@ -387,9 +390,11 @@ void run_kmeans(const sparsepr_plan_s* p, int r, int C, int tag, int* assign, co
   const int ld = round16(r);
   // changed[t][bh], t = 1..T: rows of head bh that changed group in pass t.  A pass that changes nothing proves the
   // fixed point, so the later passes of that head return at once (their result would be identical).
-  int* changed = p->km_changed + (tag == kTagQInit ? (size_t)(R.T + 1) * R.BH : 0);
-  cudaMemsetAsync(changed, 0, (size_t)(R.T + 1) * R.BH * sizeof(int), st);
-  launch_kmeans_init(p->phi, ld, nheads, R.N, r, C, R.seed, tag, tag == kTagQInit ? R.head_offset : R.head_offset / R.G, p->mu, p->sums, p->counts, p->maxabs, p->fx_shift, st);
+  const int side = tag == kTagQInit ? 1 : 0;
+  int* changed = p->km_changed + side * (size_t)(R.T + 1) * R.BH;
+  int* flagcnt = p->flagcnt + side * 2 * (size_t)R.BH;
+  const unsigned* maxabs = p->maxabs + side * (size_t)R.BH;
+  launch_kmeans_init(p->phi, ld, nheads, R.N, r, C, R.seed, tag, tag == kTagQInit ? R.head_offset : R.head_offset / R.G, p->mu, p->sums, p->counts, maxabs, p->fx_shift, st);
   const bool tcp = kmeans_tc_supported() && r <= kMaxRank;
   float* mumax = tcp ? nullptr : p->mumax;       // the tensor-core assignment derives the norm bound from ||mu||^2 itself
   // (with the tensor-core assignment the finalize step also writes the operands made of the centroids, and the sums
@@ -403,7 +408,6 @@ void run_kmeans(const sparsepr_plan_s* p, int r, int C, int tag, int* assign, co
   if (warm_prev) launch_kmeans_group_sums(p->phi, ld, nheads, R.N, r, C, warm_prev, p->sums, p->counts, p->fx_shift, st);
   finalize(warm_prev ? upd_mode : 0);
   if (tcp) launch_split_bf16(p->phi, ld, (i64)nheads * R.N, r, p->xh, p->xl, p->xnorm, st);
-  if (tcp) cudaMemsetAsync(p->flagcnt, 0, 2 * (size_t)R.BH * sizeof(int), st);
   for (int t = 1; t <= R.T; ++t) {
     const bool upd = t < R.T;
     const int* prev = t > 1 ? changed + (size_t)(t - 1) * R.BH : nullptr;
@@ -415,7 +419,7 @@ void run_kmeans(const sparsepr_plan_s* p, int r, int C, int tag, int* assign, co
       ka.assign = assign; ka.old = t > 1 ? assign : warm_prev;
       const bool first_sums = upd && ka.old == nullptr;        // nothing to update yet: formed from the whole assignment below
       ka.sums = upd && !first_sums ? p->sums : nullptr; ka.counts = p->counts; ka.fx_shift = p->fx_shift;
-      ka.flagged = p->flagged; ka.flag_count = p->flagcnt + (size_t)(t & 1) * R.BH; ka.flag_count_next = p->flagcnt + (size_t)((t + 1) & 1) * R.BH;
+      ka.flagged = p->flagged; ka.flag_count = flagcnt + (size_t)(t & 1) * R.BH; ka.flag_count_next = flagcnt + (size_t)((t + 1) & 1) * R.BH;
       ka.recheck_total = p->recheck; ka.err = p->err;
       ka.prev_changed = prev; ka.cur_changed = cur;
       launch_kmeans_assign_tc(ka, st);
@@ -558,8 +562,8 @@ static sparsepr_status_t plan_impl(const sparsepr_shape_t* shape, const sparsepr
   cudaStream_t st = p->stream;
   cudaGetLastError();
   p->capture = capture_of(st);
-  cudaMemsetAsync(p->err, 0, 64 * sizeof(int), st);
-  cudaMemsetAsync(p->maxabs, 0, r.BH * sizeof(unsigned), st);
+  cudaMemsetAsync(p->err, 0, plan_zero_ints(r) * sizeof(int), st);
+  unsigned* const maxabs_q = p->maxabs + r.BH;
   StageTimer tm(prof, st);
   // K/V partition: sampled-query metric -> F_K -> phi_K -> k-means (semantic variant: k-means on K itself)
   if (r.partition == SPARSEPR_PARTITION_SEMANTIC) {
@@ -589,18 +593,17 @@ static sparsepr_status_t plan_impl(const sparsepr_shape_t* shape, const sparsepr
   launch_group_means(r.dtype, K, r.ks, r.BHkv, r.Hkv, p->kv_perm, p->kv_off, r.N, r.Ck, r.d, p->kappa, p->nk, st);
   tm.mark(SPARSEPR_STAGE_KEY_PERMUTE);
   // query partition: centroid metric -> F_Q -> phi_Q -> k-means (other variants: k-means on Q itself)
-  cudaMemsetAsync(p->maxabs, 0, r.BH * sizeof(unsigned), st);
   if (r.partition != SPARSEPR_PARTITION_RESPONSE_COUPLED) {
     tm.mark(SPARSEPR_STAGE_QUERY_METRIC);
-    launch_raw_features(r.dtype, Q, r.qs, r.BH, r.H, r.N, r.d, p->phi, p->maxabs, p->err, st);
+    launch_raw_features(r.dtype, Q, r.qs, r.BH, r.H, r.N, r.d, p->phi, maxabs_q, p->err, st);
   } else {
     launch_centroid_gram(p->kappa, p->nk, r.BHkv, r.Ck, r.d, p->Mmat, st);
     launch_eig_top(p->Mmat, (i64)r.d * r.d, r.BHkv, r.d, r.rQ, 0, r.dtype == SPARSEPR_F32, p->FQ, p->lam, p->eigws, st);
     tm.mark(SPARSEPR_STAGE_QUERY_METRIC);
     if (project_tc_supported(r.dtype, r.d, r.rQ, r.qs)) {
-      if (!launch_project_tc(Q, r.qs, r.BH, r.H, r.N, r.d, r.rQ, p->FQ, true, r.eps_rms, p->phi, r.RQ, p->maxabs, p->Ft, p->err, st, r.G)) { delete p; return SPARSEPR_ERR_CUDA; }
+      if (!launch_project_tc(Q, r.qs, r.BH, r.H, r.N, r.d, r.rQ, p->FQ, true, r.eps_rms, p->phi, r.RQ, maxabs_q, p->Ft, p->err, st, r.G)) { delete p; return SPARSEPR_ERR_CUDA; }
     } else {
-      launch_project(r.dtype, Q, r.qs, r.BH, r.H, r.N, r.d, r.rQ, p->FQ, true, r.eps_rms, p->phi, r.RQ, p->maxabs, p->err, st);
+      launch_project(r.dtype, Q, r.qs, r.BH, r.H, r.N, r.d, r.rQ, p->FQ, true, r.eps_rms, p->phi, r.RQ, maxabs_q, p->err, st);
     }
   }
   tm.mark(SPARSEPR_STAGE_QUERY_PROJECT);
