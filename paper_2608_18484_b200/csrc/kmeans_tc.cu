@@ -483,8 +483,8 @@ __global__ void __launch_bounds__(256) k_assign_recheck_staged(const int* __rest
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) best32 = fminf(best32, __shfl_xor_sync(FULL, best32, o));
     const float thr = best32 * (1.f + 4.f * (float)(R + 4) * 5.9604645e-8f) + 1e-30f;
-    // candidates: normally one, and then the decision is made (float64 arithmetic is slow on this GPU: about 16
-    // cycles per warp instruction, 5 instructions per term)
+    // candidates: normally one, and then the decision is made (the definition is a chain of float64 additions, about 9 cycles per term,
+    // behind conversions)
     int ncand = 0, cand = -1;
     for (int c = lane; c < C; c += 32)                         // (never past C: with a NaN row thr is +inf, and so are the pad entries)
       if (d32[c] <= thr) { ++ncand; cand = c; }
