@@ -100,13 +100,16 @@ __global__ void __launch_bounds__(kPrepCols * kPrepSlices) k_fit_prepare(FitArgs
 // blockIdx.z selects G = Xb^T W Xb + lam I, B(rhs) = Xb^T W Rb, S = Rb^T W Rb; a CTA owns one kT x kT tile of it (of the
 // symmetric G and S only the tiles on and above the diagonal, mirrored), a thread a 4 x 4 or 2 x 2 block.
 // T = float for 16-bit tensors, double otherwise, with smaller tiles to spread it.
+// The eigen-solver wants S symmetric to the bit.  With the weight on one operand, (w r_i) r_j and (w r_j) r_i round differently, so inside a
+// diagonal tile, which a CTA forms in full, S_ij and S_ji become their mean.
 // (One CTA per matrix with 64 entries per thread and no operand reuse in registers: 94 us at M = 64, d = 128, two heads;
 // now 18 us, of which a part is the wait for the kernel before.)
 template <typename T> constexpr int kGramTile = sizeof(T) == 4 ? 64 : 32;
 template <typename T>
 __global__ void __launch_bounds__(256) k_fit_gram(FitArgs a) {
   constexpr int kT = kGramTile<T>, kPt = kT / 16, kRows = 32;
-  __shared__ __align__(16) T ls[kRows][kT], rs[kRows][kT];
+  __shared__ __align__(16) T stage[2 * kRows * kT > kT * (kT + 1) ? 2 * kRows * kT : kT * (kT + 1)];
+  T (*ls)[kT] = reinterpret_cast<T (*)[kT]>(stage), (*rs)[kT] = ls + kRows;    // weighted left and right operands
   const int bh = blockIdx.y, which = blockIdx.z, M = a.M, d = a.d;
   const int nt = d / kT, i0 = (blockIdx.x / nt) * kT, j0 = (blockIdx.x % nt) * kT;
   pdl_wait();
@@ -144,6 +147,20 @@ __global__ void __launch_bounds__(256) k_fit_gram(FitArgs a) {
 #pragma unroll
         for (int v = 0; v < kPt; ++v) acc[u][v] = fma(x[u], y[v], acc[u][v]);
     }
+  }
+  if (which == 2 && i0 == j0) {
+    T (*tile)[kT + 1] = reinterpret_cast<T (*)[kT + 1]>(stage);
+    __syncthreads();
+#pragma unroll
+    for (int u = 0; u < kPt; ++u)
+#pragma unroll
+      for (int v = 0; v < kPt; ++v) tile[ti + u][tj + v] = acc[u][v];
+    __syncthreads();
+#pragma unroll
+    for (int u = 0; u < kPt; ++u)
+#pragma unroll
+      for (int v = 0; v < kPt; ++v) out[(size_t)(i0 + ti + u) * d + j0 + tj + v] = 0.5 * ((double)acc[u][v] + (double)tile[tj + v][ti + u]);
+    return;
   }
 #pragma unroll
   for (int u = 0; u < kPt; ++u)
