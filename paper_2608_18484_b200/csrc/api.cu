@@ -270,7 +270,7 @@ struct sparsepr_plan_s {
 
 namespace {
 
-size_t plan_zero_ints(const Resolved& r) { return 64 + (size_t)r.BH * (2 + 2 * (r.T + 1) + 4); }
+size_t plan_zero_ints(const Resolved& r) { return 64 + (size_t)r.BH * (2 + 2 * ((size_t)r.T + 1) + 4); }
 
 void carve_plan(Carver& c, const Resolved& r, sparsepr_plan_s* p) {
   const size_t BH = r.BH, N = r.N, d = r.d;
@@ -279,7 +279,7 @@ void carve_plan(Carver& c, const Resolved& r, sparsepr_plan_s* p) {
   int* recheck = err ? err + 1 : nullptr;
   unsigned* maxabs = err ? reinterpret_cast<unsigned*>(err + 64) : nullptr;                        // [2 sides][BH]
   int* km_changed = err ? err + 64 + 2 * BH : nullptr;
-  int* flagcnt = err ? km_changed + 2 * (size_t)(r.T + 1) * BH : nullptr;                          // per side two sets of per-head counters, used by alternate passes
+  int* flagcnt = err ? km_changed + 2 * ((size_t)r.T + 1) * BH : nullptr;                          // per side two sets of per-head counters, used by alternate passes
   double* Mmat = c.take<double>(BH * d * d);
   double* lam = c.take<double>(BH * d);
   float* FK = c.take<float>(BH * d * r.rK);
@@ -391,7 +391,7 @@ void run_kmeans(const sparsepr_plan_s* p, int r, int C, int tag, int* assign, co
   // changed[t][bh], t = 1..T: rows of head bh that changed group in pass t.  A pass that changes nothing proves the
   // fixed point, so the later passes of that head return at once (their result would be identical).
   const int side = tag == kTagQInit ? 1 : 0;
-  int* changed = p->km_changed + side * (size_t)(R.T + 1) * R.BH;
+  int* changed = p->km_changed + side * ((size_t)R.T + 1) * R.BH;
   int* flagcnt = p->flagcnt + side * 2 * (size_t)R.BH;
   const unsigned* maxabs = p->maxabs + side * (size_t)R.BH;
   launch_kmeans_init(p->phi, ld, nheads, R.N, r, C, R.seed, tag, tag == kTagQInit ? R.head_offset : R.head_offset / R.G, p->mu, p->sums, p->counts, maxabs, p->fx_shift, st);

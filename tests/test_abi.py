@@ -102,3 +102,11 @@ def test_missing_library_fails_loudly(monkeypatch, tmp_path):
     monkeypatch.setattr(B, "LIB_PATH", str(tmp_path / "nope.so"))
     with pytest.raises(RuntimeError, match="no CPU or PyTorch fallback"):
         B.lib()
+
+
+def test_plan_workspace_counts_every_kmeans_pass(lib):
+    # two counters per head and pass, in 64-bit arithmetic up to the largest number of passes
+    sh = _shape()
+    size = {t: lib.sparsepr_plan_workspace_bytes(C.byref(sh), C.byref(B.make_params(kmeans_iters=t))) for t in (1 << 20, 1 << 30, (1 << 31) - 1)}
+    for t in size:
+        assert abs(size[t] - size[1 << 20] - 2 * 4 * 2 * (t - (1 << 20))) <= 512, t
