@@ -226,7 +226,9 @@ sparsepr_status_t sparsepr_plan(const sparsepr_shape_t* shape, const sparsepr_pa
  * start independent of the sign gauge of the eigenvectors behind the feature maps, which can change between calls.
  * params->kmeans_iters still counts the assignment passes, and fewer are needed (the benchmark's warm leg uses 2).
  * The arrays may live in an earlier plan's workspace (see sparsepr_plan_assignments); they are read by work queued
- * on `cuda_stream` and must stay valid until that work is complete. */
+ * on `cuda_stream` and must stay valid until that work is complete.  Once that plan is destroyed, `workspace` may be its
+ * workspace again if shape, partition variant, numbers of groups, rK and rQ are the same (kmeans_iters may differ): the new
+ * partition then takes the place of the old one.  The arrays must not overlap `workspace` in any other way. */
 sparsepr_status_t sparsepr_plan_warm(const sparsepr_shape_t* shape, const sparsepr_params_t* params,
                                      const void* Q, const void* K, const void* V,
                                      const int32_t* prev_kv_assign, const int32_t* prev_q_assign,

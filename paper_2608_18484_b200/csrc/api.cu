@@ -274,12 +274,6 @@ size_t plan_zero_ints(const Resolved& r) { return 64 + (size_t)r.BH * (2 + 2 * (
 
 void carve_plan(Carver& c, const Resolved& r, sparsepr_plan_s* p) {
   const size_t BH = r.BH, N = r.N, d = r.d;
-  // what a plan starts from zero, in one piece: error words, largest feature magnitudes and k-means counters of either side
-  int* err = c.take<int>(plan_zero_ints(r));
-  int* recheck = err ? err + 1 : nullptr;
-  unsigned* maxabs = err ? reinterpret_cast<unsigned*>(err + 64) : nullptr;                        // [2 sides][BH]
-  int* km_changed = err ? err + 64 + 2 * BH : nullptr;
-  int* flagcnt = err ? km_changed + 2 * ((size_t)r.T + 1) * BH : nullptr;                          // per side two sets of per-head counters, used by alternate passes
   double* Mmat = c.take<double>(BH * d * d);
   double* lam = c.take<double>(BH * d);
   float* FK = c.take<float>(BH * d * r.rK);
@@ -313,6 +307,14 @@ void carve_plan(Carver& c, const Resolved& r, sparsepr_plan_s* p) {
   int* rem_pos = c.take<int>(f32 ? 0 : BH * N); int* rem_grp = c.take<int>(f32 ? 0 : BH * N); int* rem_cnt = c.take<int>(f32 ? 0 : BH);
   double* eigws = c.take<double>(eig_scratch_doubles((int)BH, r.d));
   double* Mpool = c.take<double>(r.G > 1 ? (size_t)r.BHkv * d * d : 0);
+  // What a plan starts from zero, in one piece: error words, largest feature magnitudes and k-means counters of either side.  Its size depends
+  // on the number of k-means passes, hence its place behind the rest: a warm plan of fewer passes may be made in the workspace of the plan
+  // that seeds it, and its partition has to lie exactly where the seed lies (a row's former group is read before the new one is written).
+  int* err = c.take<int>(plan_zero_ints(r));
+  int* recheck = err ? err + 1 : nullptr;
+  unsigned* maxabs = err ? reinterpret_cast<unsigned*>(err + 64) : nullptr;                        // [2 sides][BH]
+  int* km_changed = err ? err + 64 + 2 * BH : nullptr;
+  int* flagcnt = err ? km_changed + 2 * ((size_t)r.T + 1) * BH : nullptr;                          // per side two sets of per-head counters, used by alternate passes
   if (p) {
     p->km_changed = km_changed; p->flagcnt = flagcnt; p->eigws = eigws; p->Mpool = Mpool; p->Ft = Ft; p->rem_pos = rem_pos; p->rem_grp = rem_grp; p->rem_cnt = rem_cnt;
     p->err = err; p->recheck = recheck; p->Mmat = Mmat; p->lam = lam; p->FK = FK; p->FQ = FQ; p->phi = phi;
