@@ -107,7 +107,10 @@ __device__ __forceinline__ void load_row_chunks(const unsigned* __restrict__ row
   }
 }
 
-__global__ void __launch_bounds__(1024) k_route_select(const float* __restrict__ score, const int* __restrict__ nq,
+constexpr int kRouteThreads = 1024, kRouteWarps = kRouteThreads / 32;
+static_assert(kRouteThreads >= 256, "a thread per digit adds up the warps' histograms");
+
+__global__ void __launch_bounds__(kRouteThreads) k_route_select(const float* __restrict__ score, const int* __restrict__ nq,
                                                        const int* __restrict__ nk, int Cq, int Ck, i64 budget,
                                                        int select_all, int* __restrict__ route_ptr,
                                                        int* __restrict__ route_idx, RouteState* __restrict__ state,
@@ -124,7 +127,8 @@ __global__ void __launch_bounds__(1024) k_route_select(const float* __restrict__
   __shared__ i64 s_last_tie;
   const int bh = blockIdx.x;
   const unsigned* u = reinterpret_cast<const unsigned*>(score) + (i64)bh * Cq * Ck;
-  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = blockDim.x >> 5;
+  constexpr int nw = kRouteWarps;
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   for (int b = threadIdx.x; b < Ck; b += blockDim.x) nks[b] = nk[(i64)(bh / kv_div) * Ck + b];
   for (int a = threadIdx.x; a < Cq; a += blockDim.x) nqs[a] = nq[(i64)bh * Cq + a];
   __syncthreads();
@@ -217,11 +221,12 @@ __global__ void __launch_bounds__(1024) k_route_select(const float* __restrict__
         __syncwarp();
       }
       __syncthreads();
-      // the warps' histograms added up, a digit per thread (by one warp, eight digits per lane, this took most of a small call's time)
+      // the warps' histograms added up, a digit per thread (by one warp, eight digits per lane, the whole kernel took 72 us at
+      // two heads of 38 groups and 61 at two of 64; now 38 and 36)
       if (threadIdx.x < 256) {
         i64 t = 0;
 #pragma unroll 8
-        for (int ww = 0; ww < 32; ++ww) t += whist[ww * 256 + threadIdx.x];
+        for (int ww = 0; ww < nw; ++ww) t += whist[ww * 256 + threadIdx.x];
         s_hist[threadIdx.x] = t;
       }
       __syncthreads();
@@ -387,8 +392,8 @@ __global__ void __launch_bounds__(1024) k_route_select(const float* __restrict__
   }
 }
 
-static size_t route_smem(int Cq, int Ck) {      // forced, cnt, nqs [Cq], nks [Ck] ints, then 32 x 256 int64 cost and int32 key histograms
-  return (size_t)(3 * Cq + Ck + ((Cq + Ck) & 1)) * sizeof(int) + (size_t)32 * 256 * (sizeof(long long) + sizeof(int));
+static size_t route_smem(int Cq, int Ck) {      // forced, cnt, nqs [Cq], nks [Ck] ints, then a warp's 256 int64 cost and int32 key counts
+  return (size_t)(3 * Cq + Ck + ((Cq + Ck) & 1)) * sizeof(int) + (size_t)kRouteWarps * 256 * (sizeof(long long) + sizeof(int));
 }
 // routed pairs and cells of given routes (used when a plan is imported)
 __global__ void __launch_bounds__(256) k_count_pairs(const int* __restrict__ q_off, const int* __restrict__ kv_off,
@@ -416,7 +421,7 @@ void launch_count_pairs(const int* q_off, const int* kv_off, const int* route_pt
 void launch_route_select(const float* score, const int* nq, const int* nk, int BH, int Cq, int Ck, i64 budget,
                          int select_all, int* route_ptr, int* route_idx, RouteState* state, i64* pairs_out,
                          int kv_div, cudaStream_t st) {
-  launch_pdl(k_route_select, dim3(BH), dim3(1024), route_smem(Cq, Ck), st, score, nq, nk, Cq, Ck, budget, select_all, route_ptr, route_idx,
+  launch_pdl(k_route_select, dim3(BH), dim3(kRouteThreads), route_smem(Cq, Ck), st, score, nq, nk, Cq, Ck, budget, select_all, route_ptr, route_idx,
              state, pairs_out, kv_div < 1 ? 1 : kv_div);
 }
 
