@@ -298,9 +298,9 @@ __global__ void __launch_bounds__(512, 1) k_fit_solve(FitArgs a) {
 // T = B Psi (d x r); A = diag(1/s_x) T Psi^T; c = mu_R - mu_x A.  float64 throughout.  Grid (d / 16 + 1, heads): CTA x
 // owns 16 rows of A; the last one forms c = mu_R - ((mu_x / s_x) B) Psi Psi^T.  With `At` the map is written as the two
 // (d = 64: three) bf16 words the correction pass multiplies with: At [words][BH][n][k], first words, then what their rounding dropped.
-// Bound by chains of float64 latencies: four columns of A per thread at a time, quotients and loads ahead of the chains (a call of two heads of
-// 4770 tokens 3 us shorter, 16 heads of 18000 tokens 10 us).
-// (One CTA per head: 132 us at two heads of d = 128, 630 us beside the attention kernels at 24 heads; now 25 and 125 us.)
+// Bound by chains of float64 latencies: four columns of A per thread at a time, quotients and loads ahead of the chains.
+// (One CTA per head: 132 us at two heads of d = 128, 630 us beside the attention kernels at 24 heads; spread, one column at a time: 25 and
+// 122 us; now 11 and 60 us.)
 constexpr int kCompRows = 16;
 __global__ void __launch_bounds__(256) k_fit_compose(FitArgs a, int r) {
   extern __shared__ __align__(16) double sm_comp[];
@@ -333,7 +333,8 @@ __global__ void __launch_bounds__(256) k_fit_compose(FitArgs a, int r) {
     return;
   }
   const double* Bm = sc + L.B;
-  double* Bs = sm_comp;                    // [16][d] rows of B; tail: [2][d] halves of u, then [d] u
+  double* Bs = sm_comp;                    // [16][d] rows of B; tail: 256 parts of u (256 / d of them [d]), then [d] u, then [d] mu_x / s_x
+  constexpr int kTailU = 256, kTailRatio = kTailU + 128;
   double* Ts = Bs + kCompRows * d;         // [16][r]
   float* Ps = reinterpret_cast<float*>(Ts + kCompRows * 64);   // [d][r + 1]
   const int ldp = r + 1;
@@ -380,7 +381,7 @@ __global__ void __launch_bounds__(256) k_fit_compose(FitArgs a, int r) {
   }
   // c: u = (mu_x / s_x) B by 256 / d parts of the rows, t = u Psi, c = mu_R - t Psi^T
   const int parts = 256 / d, part = tid / d, k = tid % d, per = d / parts;
-  double* ratio = Bs + 512;                // mu_x / s_x
+  double* ratio = Bs + kTailRatio;
   if (tid < d) ratio[tid] = sc[L.mu_x + tid] / sc[L.s_x + tid];
   __syncthreads();
   double u = 0.0;
@@ -391,10 +392,10 @@ __global__ void __launch_bounds__(256) k_fit_compose(FitArgs a, int r) {
   if (tid < d) {
     double t = Bs[tid];
     for (int q = 1; q < parts; ++q) t += Bs[q * d + tid];
-    Bs[256 + tid] = t;
+    Bs[kTailU + tid] = t;
   }
   __syncthreads();
-  const double* us = Bs + 256;
+  const double* us = Bs + kTailU;
   if (a.full_rank) {
     if (tid < d) cvec[tid] = (float)(sc[L.mu_R + tid] - us[tid]);
     return;
