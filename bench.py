@@ -107,20 +107,16 @@ def pair_rounds(d):
     return 20 if d == 128 else 40
 
 
-def launches_per_call(T, fitted, bf16, pairs):
-    """Kernels of this library launched by one plan + attend call (memsets excluded) of the method's own partition."""
-    # per side: init, first norms, split features; per iteration: assign, recheck; first sums; T-1 updates
-    kmeans = 2 + 1 + 2 * T + (1 if T > 1 else 0) + (T - 1)
-    # per side: Gram, eigen-solver (Householder, vectors, orthogonalisation, back-transformation, marked-matrix fallback), projection (bf16: + split
-    # of the feature map), k-means, sort + means; then probes; route; list of tiles (2), bf16: + remainder rows
-    plan = 2 * (6 + (2 if bf16 else 1) + kmeans + 2) + 2 + 2 + (3 if bf16 else 2)
-    if not fitted:
-        plan -= 2
-    attend = 3 + 1 + (1 + (1 if pairs else 0) if bf16 else 0)       # gathers, attention (bf16: + the packed remainders, + pairs of tiles)
-    if fitted:
-        attend += (3 if bf16 else 2) + 9 + 1         # probe rows (+gather) + merge, fit (eigen-solver: five launches), probe write
-        attend += 1                                  # correction pass
-    return plan + attend
+def launches_per_call(call):
+    """Kernels of this library that one plan + attend call launches (which they are depends on its sizes): counted by the profiler on a call
+    outside the timed region."""
+    import torch
+    from torch.profiler import ProfilerActivity, profile
+    torch.cuda.synchronize()
+    with profile(activities=[ProfilerActivity.CUDA]) as prof:
+        call()
+        torch.cuda.synchronize()
+    return sum(1 for e in prof.events() if e.device_type == torch.autograd.DeviceType.CUDA and "spr::" in e.name)
 
 
 def max_over_ranks(value, device, world):
@@ -534,7 +530,7 @@ def main():
                              "note": "the call as timed (side streams overlap); stage_ms come from a one-stream run"},
            "kmeans_passes": [st["kmeans_passes_kv"], st["kmeans_passes_q"]],
            "device_error": st["device_error"], "assign_rechecked_rows": st["assign_rechecked_rows"],
-           "gpu_launches": launches_per_call(params.kmeans_iters or 8, True, wl.dtype == "bf16", pairs) * args.steps,
+           "gpu_launches": launches_per_call(step) * args.steps,
            "warm_started_call": warm, "roofline": roofline, "clocks": clocks, "e2e": e2e}
     if not args.no_cpu_baseline and world == 1:
         def gpu_call(small, Q, K, V):

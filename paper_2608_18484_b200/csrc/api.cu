@@ -387,7 +387,7 @@ i64 pair_budget(const Resolved& r) {
   return std::max<i64>(total - (i64)r.M * r.N, 0);
 }
 
-void run_kmeans(const sparsepr_plan_s* p, int r, int C, int tag, int* assign, const int* warm_prev, int nheads, cudaStream_t st) {
+bool run_kmeans(const sparsepr_plan_s* p, int r, int C, int tag, int* assign, const int* warm_prev, int nheads, cudaStream_t st) {
   const Resolved& R = p->r;
   const int ld = round16(r);
   // changed[t][bh], t = 1..T: rows of head bh that changed group in pass t.  A pass that changes nothing proves the
@@ -396,7 +396,7 @@ void run_kmeans(const sparsepr_plan_s* p, int r, int C, int tag, int* assign, co
   int* changed = p->km_changed + side * ((size_t)R.T + 1) * R.BH;
   int* flagcnt = p->flagcnt + side * 2 * (size_t)R.BH;
   const unsigned* maxabs = p->maxabs + side * (size_t)R.BH;
-  launch_kmeans_init(p->phi, ld, nheads, R.N, r, C, R.seed, tag, tag == kTagQInit ? R.head_offset : R.head_offset / R.G, p->mu, p->sums, p->counts, maxabs, p->fx_shift, st);
+  launch_kmeans_init(p->phi, ld, nheads, R.N, r, C, R.seed, tag, tag == kTagQInit ? R.head_offset : R.head_offset / R.G, p->mu, p->sums, p->counts, maxabs, p->fx_shift, p->recheck, st);
   const bool tcp = kmeans_tc_supported() && r <= kMaxRank;
   float* mumax = tcp ? nullptr : p->mumax;       // the tensor-core assignment derives the norm bound from ||mu||^2 itself
   // (with the tensor-core assignment the finalize step also writes the operands made of the centroids, and the sums
@@ -408,6 +408,14 @@ void run_kmeans(const sparsepr_plan_s* p, int r, int C, int tag, int* assign, co
   };
   // warm start: the initial centroids become the means of the current features over the previous partition's groups
   if (warm_prev) launch_kmeans_group_sums(p->phi, ld, nheads, R.N, r, C, warm_prev, p->sums, p->counts, p->fx_shift, st);
+  if (tcp && kmeans_run_ctas(nheads, R.N, C, r) > 0) {
+    launch_split_bf16(p->phi, ld, (i64)nheads * R.N, r, p->xh, p->xl, p->xnorm, st);
+    KmeansRunArgs ka{};
+    ka.BH = nheads; ka.N = R.N; ka.C = C; ka.r = r; ka.R = ld; ka.T = R.T; ka.xh = p->xh; ka.xl = p->xl; ka.phi = p->phi; ka.ldphi = ld; ka.xnorm = p->xnorm;
+    ka.mu = p->mu; ka.from_sums = warm_prev != nullptr; ka.old = warm_prev; ka.assign = assign; ka.sums = p->sums; ka.counts = p->counts;
+    ka.fx_shift = p->fx_shift; ka.flagged = p->flagged; ka.recheck_total = p->recheck; ka.err = p->err; ka.changed = changed; ka.ld_changed = R.BH;
+    return launch_kmeans_run(ka, st);
+  }
   finalize(warm_prev ? upd_mode : 0);
   if (tcp) launch_split_bf16(p->phi, ld, (i64)nheads * R.N, r, p->xh, p->xl, p->xnorm, st);
   for (int t = 1; t <= R.T; ++t) {
@@ -424,7 +432,7 @@ void run_kmeans(const sparsepr_plan_s* p, int r, int C, int tag, int* assign, co
       ka.flagged = p->flagged; ka.flag_count = flagcnt + (size_t)(t & 1) * R.BH; ka.flag_count_next = flagcnt + (size_t)((t + 1) & 1) * R.BH;
       ka.recheck_total = p->recheck; ka.err = p->err;
       ka.prev_changed = prev; ka.cur_changed = cur;
-      launch_kmeans_assign_tc(ka, st);
+      if (!launch_kmeans_assign_tc(ka, st)) return false;
       if (first_sums) launch_kmeans_group_sums(p->phi, ld, nheads, R.N, r, C, assign, p->sums, p->counts, p->fx_shift, st);
     } else {
       if (!upd) cudaMemsetAsync(p->recheck, 0, sizeof(int), st);
@@ -433,6 +441,7 @@ void run_kmeans(const sparsepr_plan_s* p, int r, int C, int tag, int* assign, co
     }
     if (upd) finalize(upd_mode);
   }
+  return true;
 }
 
 // pads [n][r] rows to [n][R] with zeros
@@ -589,7 +598,7 @@ static sparsepr_status_t plan_impl(const sparsepr_shape_t* shape, const sparsepr
     }
   }
   tm.mark(SPARSEPR_STAGE_KEY_PROJECT);
-  run_kmeans(p, r.fK, r.Ck, kTagKvInit, p->a_K, warm_kv, r.BHkv, st);
+  if (!run_kmeans(p, r.fK, r.Ck, kTagKvInit, p->a_K, warm_kv, r.BHkv, st)) { delete p; return SPARSEPR_ERR_CUDA; }
   tm.mark(SPARSEPR_STAGE_KEY_KMEANS);
   launch_group_sort(p->a_K, r.BHkv, r.N, r.Ck, p->kv_perm, p->kv_inv, p->kv_off, p->err, st);
   launch_group_means(r.dtype, K, r.ks, r.BHkv, r.Hkv, p->kv_perm, p->kv_off, r.N, r.Ck, r.d, p->kappa, p->nk, st);
@@ -609,7 +618,7 @@ static sparsepr_status_t plan_impl(const sparsepr_shape_t* shape, const sparsepr
     }
   }
   tm.mark(SPARSEPR_STAGE_QUERY_PROJECT);
-  run_kmeans(p, r.fQ, r.Cq, kTagQInit, p->a_Q, warm_q, r.BH, st);
+  if (!run_kmeans(p, r.fQ, r.Cq, kTagQInit, p->a_Q, warm_q, r.BH, st)) { delete p; return SPARSEPR_ERR_CUDA; }
   tm.mark(SPARSEPR_STAGE_QUERY_KMEANS);
   launch_group_sort(p->a_Q, r.BH, r.N, r.Cq, p->q_perm, p->q_inv, p->q_off, p->err, st);
   launch_group_means(r.dtype, Q, r.qs, r.BH, r.H, p->q_perm, p->q_off, r.N, r.Cq, r.d, p->theta, p->nq, st);

@@ -28,7 +28,7 @@ void launch_project(int dtype, const void* X, const i64* xs, int BH, int H, int 
 void launch_raw_features(int dtype, const void* X, const i64* xs, int BH, int H, int N, int d, float* phi, unsigned* maxabs,
                          int* err, cudaStream_t st);
 void launch_kmeans_init(const float* phi, int ldphi, int BH, int N, int r, int C, u64 seed, int tag, int head0, float* mu,
-                        i64* sums, int* counts, const unsigned* maxabs_bits, int* fx_shift, cudaStream_t st);
+                        i64* sums, int* counts, const unsigned* maxabs_bits, int* fx_shift, int* recheck_total, cudaStream_t st);   // recheck_total: set to 0
 void launch_kmeans_group_sums(const float* phi, int ldphi, int BH, int N, int r, int C, const int* assign, i64* sums,
                              int* counts, const int* fx_shift, cudaStream_t st);
 // update: 1 = new centroids from the sums, which are then cleared; 2 = the same, sums and counts stay.  mh, ml, mw: operands
@@ -78,6 +78,25 @@ bool kmeans_tc_supported();
 void launch_split_bf16(const float* x, int ld, i64 rows, int r, __nv_bfloat16* hi, __nv_bfloat16* lo, float* norm,
                        cudaStream_t st);
 bool launch_kmeans_assign_tc(const KmeansTcArgs& a, cudaStream_t st);
+// All passes of the k-means in one kernel, a cluster of CTAs per head.  mu: the first centroids; from_sums: those of groups with rows are
+// the means that `sums` holds; old: the groups `sums` is over, or null (sums and counts are zero).  changed: rows of head bh that changed group in
+// pass t go to changed[t ld_changed + bh], which must be zero.  recheck_total: rows rechecked in the last pass are added.
+struct KmeansRunArgs {
+  int BH, N, C, r, R, T;
+  const __nv_bfloat16 *xh, *xl;
+  const float* phi; int ldphi;
+  const float* xnorm;
+  const float* mu;
+  bool from_sums;
+  const int* old;
+  int* assign;
+  i64* sums; int* counts; const int* fx_shift;
+  int *flagged, *recheck_total, *err;
+  int* changed; int ld_changed;
+};
+// CTAs per head that the kernel above would take, 0 where the passes are better launched one by one
+int kmeans_run_ctas(int BH, int N, int C, int r);
+bool launch_kmeans_run(const KmeansRunArgs& a, cudaStream_t st);
 
 // ---- routing.cu ---------------------------------------------------------------
 struct RouteState {      // per head, device

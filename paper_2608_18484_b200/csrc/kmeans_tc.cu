@@ -31,7 +31,8 @@
 // two words of the features 31), the passes of one run 62 to 168 us, 1.38 ms for 16 passes where the kernel that kept best,
 // second and index per score and formed the sums anew took 2.11 ms; 40 heads of 75600 rows, 591 centroids: 540 us per
 // pass (958).  The early passes, in which a third of the rows move, are bound by the atomics of the sums.
-#include "kernels.cuh"
+#include <mutex>
+#include "kmeans_sums.cuh"
 #include "tc_common.cuh"
 
 namespace spr {
@@ -106,6 +107,111 @@ __device__ __forceinline__ float min16(const float* s) {
   const float a = min3(s[0], s[1], s[2]), b = min3(s[3], s[4], s[5]), c = min3(s[6], s[7], s[8]), d = min3(s[9], s[10], s[11]);
   const float e = min3(s[12], s[13], s[14]);
   return fminf(min3(a, b, s[15]), min3(c, d, e));
+}
+
+// the scores of a row tile and a chunk: ||mu||^2 + x_h mu_h + x_h mu_l + x_l mu_h; one k-step = 16 columns = 32 bytes = 2 address units
+__device__ __forceinline__ void km_product(uint32_t d, uint64_t one_desc, uint64_t wd, uint64_t xh, uint64_t mh, int ksteps, uint32_t idesc) {
+  const uint64_t xl = xh + (uint64_t)(kXBytes >> 4), ml = mh + (uint64_t)(kMuBytes >> 4);
+  umma_bf16(d, one_desc, wd, idesc, 0);
+#pragma unroll
+  for (int kk = 0; kk < 4; ++kk)
+    if (kk < ksteps) {
+      umma_bf16(d, xh + 2 * kk, mh + 2 * kk, idesc, 1);
+      umma_bf16(d, xh + 2 * kk, ml + 2 * kk, idesc, 1);
+      umma_bf16(d, xl + 2 * kk, mh + 2 * kk, idesc, 1);
+    }
+}
+// The scan of a row's scores by one thread of each half of the columns
+struct KmScan {
+  float cls[16];                                               // minima over the column classes c mod 16
+  float gb = kKmFar, gs = kKmFar;                              // best and second best of the minima of 16 columns
+  int gi = 0;                                                  // index of the best (c / 16)
+  __device__ __forceinline__ KmScan() {
+#pragma unroll
+    for (int j = 0; j < 16; ++j) cls[j] = kKmFar;
+  }
+  __device__ __forceinline__ void group(float cm, int g) {
+    gs = fminf(gs, fmaxf(cm, gb));
+    gi = cm < gb ? g : gi;
+    gb = fminf(gb, cm);
+  }
+  // the scores of the centroids from c0 on in this warp's lanes of tensor memory; hh: which half of the columns is this warp's
+  __device__ __forceinline__ void chunk(uint32_t acc_addr, int c0, int C, int hh) {
+    const int ng = (min(kKmChunk, C - c0) + 15) >> 4;          // groups of 16 columns that hold centroids
+    const int ns = (ng + 1) >> 1, s_mid = (ns + 1) >> 1;       // 32-column steps; this warp's half of them
+    const int s1 = hh ? ns : s_mid;
+#pragma unroll 1
+    for (int st = hh ? s_mid : 0; st < s1; ++st) {
+      float t[32];
+      tmem_ld32(acc_addr + st * 32, t);
+      group(min16(t), (c0 >> 4) + 2 * st);
+      if (2 * st + 1 < ng) {                                   // uniform (the product wrote no columns beyond ng groups)
+        group(min16(t + 16), (c0 >> 4) + 2 * st + 1);
+#pragma unroll
+        for (int j = 0; j < 16; ++j) cls[j] = min3(cls[j], t[j], t[16 + j]);
+      } else {
+#pragma unroll
+        for (int j = 0; j < 16; ++j) cls[j] = fminf(cls[j], t[j]);
+      }
+    }
+  }
+  // best and second best score of the half and the centroid of the best: second best of the class minima (tournament) and the class of the best
+  __device__ __forceinline__ void result(float& best, float& second, int& bi) const {
+    float tb[8], ts[8];
+#pragma unroll
+    for (int j = 0; j < 8; ++j) { tb[j] = fminf(cls[2 * j], cls[2 * j + 1]); ts[j] = fmaxf(cls[2 * j], cls[2 * j + 1]); }
+#pragma unroll
+    for (int w = 4; w > 0; w >>= 1)
+#pragma unroll
+      for (int j = 0; j < w; ++j) {
+        const float hi = fmaxf(tb[j], tb[j + w]);
+        ts[j] = min3(hi, ts[j], ts[j + w]);
+        tb[j] = fminf(tb[j], tb[j + w]);
+      }
+    int cj = 0;
+#pragma unroll
+    for (int j = 1; j < 16; ++j) cj = cls[j] == tb[0] ? j : cj;
+    best = tb[0]; second = fminf(ts[0], gs);
+    bi = gi * 16 + cj;
+  }
+};
+// The results of the two halves of the columns meet: xc = this row's place of the first half, 128 floats per half, second best and index 1024
+// and 2048 floats behind
+__device__ __forceinline__ void km_exchange(float* xc, int hh, int barrier, float& best, float& second, int& bi) {
+  xc[hh * 128] = best; xc[1024 + hh * 128] = second; reinterpret_cast<int*>(xc)[2048 + hh * 128] = bi;
+  asm volatile("bar.sync %0, 64;" ::"r"(barrier) : "memory");
+  const float ob = xc[(hh ^ 1) * 128], os = xc[1024 + (hh ^ 1) * 128];
+  const int oi = reinterpret_cast<const int*>(xc)[2048 + (hh ^ 1) * 128];
+  second = min3(fmaxf(best, ob), second, os);
+  bi = ob < best ? oi : bi;
+  best = fminf(best, ob);
+}
+// Bound on |computed score - true score|.  A bf16 rounding is off by at most 2^-8 relative, so the words of x and
+// of 2 mu leave 2^-16 each and the dropped product xl.ml another 2^-16 of 2 |x| |mu|: 9.2e-5 in all.  Accumulation
+// in fp32: 13 steps that add 17 terms, the largest at most 2 |x| |mu| + |mu|^2.  How the unit aligns them is not documented;
+// a sum delivered in float32 keeps at least that format's places below the largest term, so each term is allowed to lose 2^-23
+// of it: 2.7e-5.  (Measured with words at their worst, cancelling terms and terms just below the last place of a large one:
+// at most 7e-7 of it, and 0.07 of E in all.)
+__device__ __forceinline__ float km_score_error(float xn, float mm) { return 1.5e-4f * xn * mm + 2.7e-5f * mm * mm; }
+// The rows of a warp's 32 that changed their group (bits of todo; phi: the first of the 32), four at a time: the latency of their features is the cost
+__device__ __forceinline__ void km_moves(unsigned todo, const float* phi, int ldphi, i64* sums, int* counts, int C, int R, int r, float scl,
+                                         int old_a, int bi, int lane) {
+  while (todo) {
+    int rr[4];
+    float2 x2[4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      rr[u] = todo ? __ffs(todo) - 1 : -1;
+      todo &= todo - 1;
+      x2[u] = make_float2(0.f, 0.f);
+      if (rr[u] >= 0 && 2 * lane < r)                          // (ldphi is a multiple of 16 and columns r..ldphi-1 hold zeros)
+        x2[u] = *reinterpret_cast<const float2*>(phi + (i64)rr[u] * ldphi + 2 * lane);
+    }
+#pragma unroll
+    for (int u = 0; u < 4; ++u)
+      if (rr[u] >= 0)
+        km_move(sums, counts, C, R, r, scl, x2[u], __shfl_sync(0xffffffffu, old_a, rr[u]), __shfl_sync(0xffffffffu, bi, rr[u]), lane);
+  }
 }
 
 __global__ void __launch_bounds__(kKmThreads, 1)
@@ -234,19 +340,11 @@ k_kmeans_assign_tc(const __grid_constant__ CUtensorMap mapXh, const __grid_const
           const uint32_t d = tm + (uint32_t)ab * kKmChunk;
           const uint32_t idesc = ch == n_chunks - 1 ? idesc_last : idesc_full;
           const uint64_t moff = (uint64_t)((ms * kMuStage) >> 4);
-          const uint64_t mh = m_desc0 + moff, ml = mh + (uint64_t)(kMuBytes >> 4), wd = w_desc0 + moff;
-          const uint64_t xh = x_desc0 + (uint64_t)((xs * 2 * kXBytes) >> 4), xl = xh + (uint64_t)(kXBytes >> 4);
+          const uint64_t mh = m_desc0 + moff, wd = w_desc0 + moff;
+          const uint64_t xh = x_desc0 + (uint64_t)((xs * 2 * kXBytes) >> 4);
           if (elect_one()) {
             if (have) {
-              // ||mu||^2 + x_h mu_h + x_h mu_l + x_l mu_h; one k-step = 16 columns = 32 bytes = 2 address units
-              umma_bf16(d, one_desc, wd, idesc, 0);
-#pragma unroll
-              for (int kk = 0; kk < 4; ++kk)
-                if (kk < ksteps) {
-                  umma_bf16(d, xh + 2 * kk, mh + 2 * kk, idesc, 1);
-                  umma_bf16(d, xh + 2 * kk, ml + 2 * kk, idesc, 1);
-                  umma_bf16(d, xl + 2 * kk, mh + 2 * kk, idesc, 1);
-                }
+              km_product(d, one_desc, wd, xh, mh, ksteps, idesc);
               umma_commit(bar(ACC_FULL + ab));
               if (ch == n_chunks - 1) umma_commit(bar(X_EMPTY + xs));
               if (!resident) umma_commit(bar(MU_EMPTY + ms));
@@ -272,84 +370,28 @@ k_kmeans_assign_tc(const __grid_constant__ CUtensorMap mapXh, const __grid_const
       const bool mine = row < prm.N && (lane >> 4) == hh;      // the two warps of a quadrant finish 16 of its rows each
       const float xn = mine ? prm.xnorm[gr] : 0.f;             // needed after the scores: fetched now
       const int old_a = (prm.old != nullptr && mine) ? prm.old[gr] : -1;
-      float cls[16];                                           // minima over the column classes c mod 16
-#pragma unroll
-      for (int j = 0; j < 16; ++j) cls[j] = kKmFar;
-      float gb = kKmFar, gs = kKmFar;                          // best and second best of the minima of 16 columns
-      int gi = 0;                                              // index of the best (c / 16)
+      KmScan scan;
       for (int ch = 0; ch < n_chunks; ++ch, ++k) {             // k: chunks of this group so far
         const int ab = 2 * grp + (k & 1);
         ok = __all_sync(FULL, ok && mbar_wait(bar(ACC_FULL + ab), (k >> 1) & 1, abort_flag));
         if (ok) {
           tc_fence_after();
           const uint32_t acc_addr = acc_addr0 + (uint32_t)(k & 1) * kKmChunk;
-          const int c0 = ch * kKmChunk;
-          const int ng = (min(kKmChunk, prm.C - c0) + 15) >> 4;    // groups of 16 columns that hold centroids
-          const int ns = (ng + 1) >> 1, s_mid = (ns + 1) >> 1;     // 32-column steps; this warp's half of them
-          const int s1 = hh ? ns : s_mid;
-#pragma unroll 1
-          for (int st = hh ? s_mid : 0; st < s1; ++st) {
-            float t[32];
-            tmem_ld32(acc_addr + st * 32, t);
-            auto group = [&](float cm, int g) {
-              gs = fminf(gs, fmaxf(cm, gb));
-              gi = cm < gb ? g : gi;
-              gb = fminf(gb, cm);
-            };
-            group(min16(t), (c0 >> 4) + 2 * st);
-            if (2 * st + 1 < ng) {                             // uniform (the product wrote no columns beyond ng groups)
-              group(min16(t + 16), (c0 >> 4) + 2 * st + 1);
-#pragma unroll
-              for (int j = 0; j < 16; ++j) cls[j] = min3(cls[j], t[j], t[16 + j]);
-            } else {
-#pragma unroll
-              for (int j = 0; j < 16; ++j) cls[j] = fminf(cls[j], t[j]);
-            }
-          }
+          scan.chunk(acc_addr, ch * kKmChunk, prm.C, hh);
           tc_fence_before();
         }
         __syncwarp();
         if (lane == 0) mbar_arrive(bar(ACC_EMPTY + ab));
       }
-      // second best of the class minima (tournament) and the class of the best
-      float tb[8], ts[8];
-#pragma unroll
-      for (int j = 0; j < 8; ++j) { tb[j] = fminf(cls[2 * j], cls[2 * j + 1]); ts[j] = fmaxf(cls[2 * j], cls[2 * j + 1]); }
-#pragma unroll
-      for (int w = 4; w > 0; w >>= 1)
-#pragma unroll
-        for (int j = 0; j < w; ++j) {
-          const float hi = fmaxf(tb[j], tb[j + w]);
-          ts[j] = min3(hi, ts[j], ts[j + w]);
-          tb[j] = fminf(tb[j], tb[j + w]);
-        }
-      int cj = 0;
-#pragma unroll
-      for (int j = 1; j < 16; ++j) cj = cls[j] == tb[0] ? j : cj;
-      float best = tb[0], second = fminf(ts[0], gs);
-      int bi = gi * 16 + cj;
-      {
-        // the two halves of the columns
-        float* xc = xb + ((grp * 2 + ((tl >> 1) & 1)) * 2) * 128 + wq * 32 + lane;
-        xc[hh * 128] = best; xc[1024 + hh * 128] = second; reinterpret_cast<int*>(xc)[2048 + hh * 128] = bi;
-        asm volatile("bar.sync %0, 64;" ::"r"(1 + grp * 4 + wq) : "memory");
-        const float ob = xc[(hh ^ 1) * 128], os = xc[1024 + (hh ^ 1) * 128];
-        const int oi = reinterpret_cast<const int*>(xc)[2048 + (hh ^ 1) * 128];
-        second = min3(fmaxf(best, ob), second, os);
-        bi = ob < best ? oi : bi;
-        best = fminf(best, ob);
-      }
+      float best, second;
+      int bi;
+      scan.result(best, second, bi);
+      km_exchange(xb + ((grp * 2 + ((tl >> 1) & 1)) * 2) * 128 + wq * 32 + lane, hh, 1 + grp * 4 + wq, best, second, bi);
       bi = min(bi, prm.C - 1);                               // (only rows of non-finite scores could point past C)
       // decide, or hand the row to the exact recheck
       bool decided = false, moved = false;
       if (ok && mine) {
-        // Bound on |computed score - true score|.  A bf16 rounding is off by at most 2^-8 relative, so the words of x and
-        // of 2 mu leave 2^-16 each and the dropped product xl.ml another 2^-16 of 2 |x| |mu|: 9.2e-5 in all.  Accumulation
-        // in fp32: 13 steps that add 17 terms, the largest at most 2 |x| |mu| + |mu|^2.  How the unit aligns them is not documented;
-        // a sum delivered in float32 keeps at least that format's places below the largest term, so each term is allowed to lose 2^-23
-        // of it: 2.7e-5.  (Measured with words at their worst, cancelling terms and terms just below the last place of a large one:
-        // at most 7e-7 of it, and 0.07 of E in all.)
-        const float E = 1.5e-4f * xn * mm + 2.7e-5f * mm * mm;
+        const float E = km_score_error(xn, mm);
         decided = second - best > 2.f * E;
         if (decided) {
           moved = old_a != bi;
@@ -364,26 +406,8 @@ k_kmeans_assign_tc(const __grid_constant__ CUtensorMap mapXh, const __grid_const
         if (lane == 0 && nmoved) atomicAdd(prm.cur_changed + bh, nmoved);
       }
       if (prm.sums) {
-        // rows that changed their group, four at a time (the latency of their features is the cost)
-        unsigned todo = __ballot_sync(FULL, decided && moved);
-        i64* sums = prm.sums + (i64)bh * prm.C * prm.R;
-        int* counts = prm.counts + (i64)bh * prm.C;
-        while (todo) {
-          int rr[4];
-          float2 x2[4];
-#pragma unroll
-          for (int u = 0; u < 4; ++u) {
-            rr[u] = todo ? __ffs(todo) - 1 : -1;
-            todo &= todo - 1;
-            x2[u] = make_float2(0.f, 0.f);
-            if (rr[u] >= 0 && 2 * lane < prm.r)              // (ldphi is a multiple of 16 and columns r..ldphi-1 hold zeros)
-              x2[u] = *reinterpret_cast<const float2*>(prm.phi + ((i64)bh * prm.N + rowbase + rr[u]) * prm.ldphi + 2 * lane);
-          }
-#pragma unroll
-          for (int u = 0; u < 4; ++u)
-            if (rr[u] >= 0)
-              km_move(sums, counts, prm.C, prm.R, prm.r, scl, x2[u], __shfl_sync(FULL, old_a, rr[u]), __shfl_sync(FULL, bi, rr[u]), lane);
-        }
+        km_moves(__ballot_sync(FULL, decided && moved), prm.phi + ((i64)bh * prm.N + rowbase) * prm.ldphi, prm.ldphi, prm.sums + (i64)bh * prm.C * prm.R,
+                 prm.counts + (i64)bh * prm.C, prm.C, prm.R, prm.r, scl, old_a, bi, lane);
       }
     }
   }
@@ -398,6 +422,84 @@ k_kmeans_assign_tc(const __grid_constant__ CUtensorMap mapXh, const __grid_const
     tc_fence_after();
     tmem_dealloc(tmem, 512);
   }
+}
+
+// Float32 distances of row x [R] to the centroids (rows LDM floats apart) into d32 [C rounded up to 32], by one warp: 32 kJ centroids at a time; returns the smallest
+template <int kJ>
+__device__ __forceinline__ float recheck_distances(const float* xs, const float* mu_s, int LDM, int C, int R, float* d32, int lane) {
+  const int Cp = (C + 31) & ~31;
+  float best32 = INFINITY;
+  for (int c0 = 0; c0 < C; c0 += 32 * kJ) {
+    // packed float32 arithmetic, two columns per instruction: (m - x)^2 summed in two partial sums per centroid
+    float2 acc[kJ];
+    const float* mrow[kJ];
+#pragma unroll
+    for (int j = 0; j < kJ; ++j) { acc[j] = make_float2(0.f, 0.f); mrow[j] = mu_s + (size_t)min(c0 + 32 * j + lane, C - 1) * LDM; }
+#pragma unroll 2
+    for (int k = 0; k < R; k += 4) {
+      const float4 xv = *reinterpret_cast<const float4*>(xs + k);
+      const float2 nx0 = make_float2(-xv.x, -xv.y), nx1 = make_float2(-xv.z, -xv.w);
+#pragma unroll
+      for (int j = 0; j < kJ; ++j) {
+        const float4 mv = *reinterpret_cast<const float4*>(mrow[j] + k);
+        const float2 d0 = __fadd2_rn(make_float2(mv.x, mv.y), nx0), d1 = __fadd2_rn(make_float2(mv.z, mv.w), nx1);
+        acc[j] = __ffma2_rn(d0, d0, acc[j]);
+        acc[j] = __ffma2_rn(d1, d1, acc[j]);
+      }
+    }
+#pragma unroll
+    for (int j = 0; j < kJ; ++j) {
+      const int c = c0 + 32 * j + lane;
+      if (c < Cp) {
+        const float d = c < C ? acc[j].x + acc[j].y : INFINITY;
+        d32[c] = d;
+        best32 = fminf(best32, d);
+      }
+    }
+  }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) best32 = fminf(best32, __shfl_xor_sync(0xffffffffu, best32, o));
+  return best32;
+}
+// The exact decision for one row by one warp (see the kernel below); x, centroids and the warp's scratch d32 in shared memory
+__device__ __forceinline__ int recheck_row(const float* xs, const float* mu_s, int LDM, int C, int R, float* d32, int lane) {
+  const unsigned FULL = 0xffffffffu;
+  const float best32 = C <= 64 ? recheck_distances<2>(xs, mu_s, LDM, C, R, d32, lane) : recheck_distances<8>(xs, mu_s, LDM, C, R, d32, lane);
+  const float thr = best32 * (1.f + 4.f * (float)(R + 4) * 5.9604645e-8f) + 1e-30f;
+  // candidates: normally one, and then the decision is made (the definition is a chain of float64 additions, about 9 cycles per term,
+  // behind conversions)
+  int ncand = 0, cand = -1;
+  for (int c = lane; c < C; c += 32)                         // (never past C: with a NaN row thr is +inf, and so are the pad entries)
+    if (d32[c] <= thr) { ++ncand; cand = c; }
+  const int total_cand = __reduce_add_sync(FULL, ncand);
+  int bi;
+  if (total_cand == 1) {
+    bi = __reduce_max_sync(FULL, cand);
+  } else if (total_cand == 0) {
+    bi = 0;                                                  // every distance is NaN (non-finite input, reported elsewhere): group 0
+  } else {
+    double best = 0.0;
+    bi = -1;
+    for (int c = lane; c < C; c += 32) {
+      if (d32[c] <= thr) {
+        const float* m = mu_s + (size_t)c * LDM;
+        double dsum = 0.0;
+#pragma unroll 8
+        for (int k = 0; k < R; ++k) {
+          const double diff = __dsub_rn((double)xs[k], (double)m[k]);
+          dsum = __dadd_rn(dsum, __dmul_rn(diff, diff));
+        }
+        if (bi < 0 || dsum < best) { best = dsum; bi = c; }    // a lane meets its centroids in increasing order
+      }
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+      const double ob = __shfl_xor_sync(FULL, best, o);
+      const int oi = __shfl_xor_sync(FULL, bi, o);
+      if (oi >= 0 && (bi < 0 || ob < best || (ob == best && oi < bi))) { best = ob; bi = oi; }
+    }
+  }
+  return min(max(bi, 0), C - 1);
 }
 
 // Exact decision for the rows the fast path could not prove (a few thousand per pass at N = 32760 and 24 heads).
@@ -451,72 +553,7 @@ __global__ void __launch_bounds__(256) k_assign_recheck_staged(const int* __rest
     __syncwarp();
     for (int k = lane; k < R; k += 32) xs[k] = x[k];
     __syncwarp();
-    float best32 = INFINITY;
-    for (int c0 = 0; c0 < C; c0 += 256) {
-      // packed float32 arithmetic, two columns per instruction: (m - x)^2 summed in two partial sums per centroid
-      float2 acc[8];
-      const float* mrow[8];
-#pragma unroll
-      for (int j = 0; j < 8; ++j) { acc[j] = make_float2(0.f, 0.f); mrow[j] = mu_s + (size_t)min(c0 + 32 * j + lane, C - 1) * LDM; }
-#pragma unroll 2
-      for (int k = 0; k < R; k += 4) {
-        const float4 xv = *reinterpret_cast<const float4*>(xs + k);
-        const float2 nx0 = make_float2(-xv.x, -xv.y), nx1 = make_float2(-xv.z, -xv.w);
-#pragma unroll
-        for (int j = 0; j < 8; ++j) {
-          const float4 mv = *reinterpret_cast<const float4*>(mrow[j] + k);
-          const float2 d0 = __fadd2_rn(make_float2(mv.x, mv.y), nx0), d1 = __fadd2_rn(make_float2(mv.z, mv.w), nx1);
-          acc[j] = __ffma2_rn(d0, d0, acc[j]);
-          acc[j] = __ffma2_rn(d1, d1, acc[j]);
-        }
-      }
-#pragma unroll
-      for (int j = 0; j < 8; ++j) {
-        const int c = c0 + 32 * j + lane;
-        if (c < Cp) {
-          const float d = c < C ? acc[j].x + acc[j].y : INFINITY;
-          d32[c] = d;
-          best32 = fminf(best32, d);
-        }
-      }
-    }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) best32 = fminf(best32, __shfl_xor_sync(FULL, best32, o));
-    const float thr = best32 * (1.f + 4.f * (float)(R + 4) * 5.9604645e-8f) + 1e-30f;
-    // candidates: normally one, and then the decision is made (the definition is a chain of float64 additions, about 9 cycles per term,
-    // behind conversions)
-    int ncand = 0, cand = -1;
-    for (int c = lane; c < C; c += 32)                         // (never past C: with a NaN row thr is +inf, and so are the pad entries)
-      if (d32[c] <= thr) { ++ncand; cand = c; }
-    const int total_cand = __reduce_add_sync(FULL, ncand);
-    int bi;
-    if (total_cand == 1) {
-      bi = __reduce_max_sync(FULL, cand);
-    } else if (total_cand == 0) {
-      bi = 0;                                                  // every distance is NaN (non-finite input, reported elsewhere): group 0
-    } else {
-      double best = 0.0;
-      bi = -1;
-      for (int c = lane; c < C; c += 32) {
-        if (d32[c] <= thr) {
-          const float* m = mu_s + (size_t)c * LDM;
-          double dsum = 0.0;
-#pragma unroll 8
-          for (int k = 0; k < R; ++k) {
-            const double diff = __dsub_rn((double)xs[k], (double)m[k]);
-            dsum = __dadd_rn(dsum, __dmul_rn(diff, diff));
-          }
-          if (bi < 0 || dsum < best) { best = dsum; bi = c; }    // a lane meets its centroids in increasing order
-        }
-      }
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) {
-        const double ob = __shfl_xor_sync(FULL, best, o);
-        const int oi = __shfl_xor_sync(FULL, bi, o);
-        if (oi >= 0 && (bi < 0 || ob < best || (ob == best && oi < bi))) { best = ob; bi = oi; }
-      }
-    }
-    bi = min(max(bi, 0), C - 1);
+    const int bi = recheck_row(xs, mu_s, LDM, C, R, d32, lane);
     const int old_a = old != nullptr ? old[gr] : -1;
     __syncwarp();                                              // everyone has read it (`old` may be `assign`)
     if (lane == 0) {
@@ -531,6 +568,390 @@ __global__ void __launch_bounds__(256) k_assign_recheck_staged(const int* __rest
 }
 // shared memory of the kernel above
 static size_t recheck_staged_smem(int C, int R) { return ((size_t)C * (R + 4) + 8 * (size_t)((C + 31) & ~31) + 8 * (size_t)R) * sizeof(float); }
+
+// All passes of a k-means run in one kernel, for at most 256 centroids: a cluster of CTAs per head, each with a contiguous run of the head's row tiles.
+// A pass of the kernels above is three dependent launches, 16 us at two heads of 4770 rows; here it is
+//   centroids from the sums, by every CTA for itself, straight into the operands in shared memory
+//   -> products, scan, decisions as above -> exact recheck of the CTA's own undecided rows -> sums -> barrier of the cluster.
+// The sums stay in global memory (atomics, read past the first-level cache); a second barrier of the cluster keeps them from changing before everyone
+// has read them.  (Centroids dealt out to the CTAs and handed round through the cluster's shared memory: stores to other CTAs move 8 bytes per cycle
+// and SM, 2 to 5 k cycles a pass more than forming all of them.)  Up to four row tiles of at most 128 centroids stay in shared memory for all passes.
+// What an SM sends to the sums is bound by its atomics (a row is 16 sectors of 32 bytes per sum), so the rows that move are listed, and where they are
+// many they are sorted by group, so that a warp adds up rows of one group; in a first pass, all rows in windows of the list's length.
+// Every thread of the cluster meets the same barriers whatever happens: an abort only skips the work in between, and the end of the iteration is read
+// from a counter that all of them see behind a barrier.
+// A pass at two heads of 4770 rows is 15 k cycles: centroids 3, products and decisions of three tiles 5.5, recheck of a row or two 3, barriers 3; its
+// first pass 25.  Runs of eight passes, us, in separate launches and here: 2 heads of 4770 rows and 38 centroids 132, 70; 2 of 4096 float32 rows and 64
+// centroids 143, 76; 8 of 7161 rows and 112 centroids 228, 178.
+constexpr int kKmRunList = 2048;                     // moved rows of a pass that are listed (the others go to the sums at once)
+constexpr int kKmRunSort = 48;                       // listed rows from which they are sorted
+constexpr int kKmRunTiles = 64;                      // row tiles per CTA (a row has 14 bits in the list)
+struct KmRunParams {
+  int N, C, r, R, T, n_chunks, per_cta;
+  const float* phi; int ldphi;
+  const float* xnorm;
+  const float* mu;
+  int from_sums;
+  const int* old;
+  int* assign;
+  i64* sums; int* counts; const int* fx_shift;
+  int* flagged; int* recheck_total; int* err;
+  int* changed; int ld_changed;
+};
+__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
+__device__ __forceinline__ void cluster_arrive_relaxed() { asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory"); }
+__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
+
+// A moved row in the list: row (from the CTA's first), group before (511: none) and group now
+constexpr int kKmNone = 511;
+__device__ __forceinline__ unsigned km_entry(int row, int was, int is) { return (unsigned)row | (unsigned)was << 14 | (unsigned)is << 23; }
+// The moves of a sorted list by one warp: elements lo .. hi - 1, the place of an entry and, in the top bit, whether its row leaves its old group or joins its new one
+__device__ __forceinline__ void km_move_sorted(const unsigned* entries, const unsigned short* list, int lo, int hi, const float* phi, int ldphi,
+                                               i64* sums, int* counts, int R, int r, float scl, int lane) {
+  constexpr int kRows = 8;                                     // rows in flight
+  const int c0 = 2 * lane;
+  const float* at = phi + (c0 < r ? c0 : 0);                   // (without a condition on the loads, so that they go out together)
+  i64 s0 = 0, s1 = 0;
+  int group = -1, count = 0;
+  const auto flush = [&] {
+    if (group >= 0) {
+      if (s0 != 0 && c0 < r) atomicAdd(reinterpret_cast<u64*>(sums + (i64)group * R + c0), (u64)s0);
+      if (s1 != 0 && c0 + 1 < r) atomicAdd(reinterpret_cast<u64*>(sums + (i64)group * R + c0 + 1), (u64)s1);
+      if (lane == 0 && count != 0) atomicAdd(counts + group, count);
+    }
+    s0 = s1 = 0; count = 0;
+  };
+  for (int i0 = lo; i0 < hi; i0 += kRows) {
+    int g[kRows];                                              // group, leaving: - 1 - group
+    float2 x[kRows];
+#pragma unroll
+    for (int u = 0; u < kRows; ++u) {
+      const int l = list[min(i0 + u, hi - 1)];
+      const unsigned e = entries[l & 0x7FFF];
+      g[u] = l & 0x8000 ? -1 - (int)((e >> 14) & 511u) : (int)(e >> 23);
+      x[u] = *reinterpret_cast<const float2*>(at + (i64)(e & 0x3FFFu) * ldphi);
+    }
+#pragma unroll
+    for (int u = 0; u < kRows; ++u) {
+      if (i0 + u >= hi) break;                                 // (uniform)
+      const int sign = g[u] >> 31, gu = g[u] ^ sign;           // 0 or -1
+      if (gu != group) { flush(); group = gu; }
+      const float signed_scale = sign ? -scl : scl;            // (rounded as in km_move)
+      s0 += __float2ll_rn(x[u].x * signed_scale);
+      s1 += __float2ll_rn(x[u].y * signed_scale);
+      count += 1 + 2 * sign;
+    }
+  }
+  flush();
+}
+
+__global__ void __launch_bounds__(kKmThreads, 1)
+k_kmeans_run(const __grid_constant__ CUtensorMap mapXh, const __grid_constant__ CUtensorMap mapXl, KmRunParams prm) {
+  extern __shared__ unsigned char smem_raw[];
+  const uint32_t raw = smem_u32(smem_raw);
+  const uint32_t base = (raw + 1023u) & ~1023u;
+  unsigned char* sm = smem_raw + (base - raw);
+  volatile int* misc = reinterpret_cast<volatile int*>(sm + KmSmem::misc);   // [0] tmem base, [1] abort
+  const uint32_t bars = base + KmSmem::bars;
+  auto bar = [&](int i) { return bars + 8u * i; };
+  constexpr unsigned FULL = 0xffffffffu;
+  constexpr int kWarps = kKmThreads / 32;
+  const int tid = threadIdx.x, warp = __shfl_sync(FULL, tid >> 5, 0), lane = tid & 31;
+  const int bh = blockIdx.y, cta = blockIdx.x, C = prm.C, R = prm.R, LDM = R + 4, n_chunks = prm.n_chunks;
+  // four row stages and one chunk of centroids, or two and two: operands, then float32 values
+  const int xst = n_chunks == 1 ? 4 : 2, xlog = n_chunks == 1 ? 2 : 1;
+  const uint32_t mu_area = (uint32_t)xst * 2 * kXBytes, val_area = mu_area + (uint32_t)n_chunks * kMuStage;
+  static_assert(2 * 2 * kXBytes + 4 * kMuStage <= KmSmem::tiles && 4 * 2 * kXBytes + 2 * kMuStage <= KmSmem::tiles && kKmChunk * (64 + 4) * 4 <= kMuStage, "layouts");
+  static_assert(kKmRunList * 4 <= KmSmem::bars - KmSmem::xchg && kKmEpiWarps * (kKmChunk + 64) * 4 <= KmSmem::bars - KmSmem::xchg, "sorted list, recheck scratch");
+  __shared__ unsigned s_list[kKmRunList];
+  __shared__ float s_max[kWarps];
+  __shared__ int s_start[2 * kKmChunk + 1];
+  __shared__ int s_flagged, s_moved, s_left, s_skip;
+  if (tid == 0) {
+    for (int i = 0; i < KM_BARS; ++i) mbar_init(bar(i), i >= ACC_EMPTY ? 8 : 1);
+    misc[1] = 0;
+    s_flagged = 0; s_moved = 0;
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
+  if (warp == kKmEpiWarps + 1) tmem_alloc(base + KmSmem::misc, 512);
+  if (tid < 256) {                                             // the constant rows (see k_kmeans_assign_tc)
+    const uint32_t one2 = 0x3F803F80u;
+    *reinterpret_cast<uint4*>(sm + KmSmem::ones + tid * 16) = (tid & 8) == 0 ? make_uint4(one2, 0x3F80u, 0u, 0u) : make_uint4(0u, 0u, 0u, 0u);
+  }
+  // operands of the places beyond C: zeros, and a norm larger than any score
+  for (uint32_t e = tid * 16; e < n_chunks * kMuStage; e += kKmThreads * 16)
+    *reinterpret_cast<uint4*>(sm + mu_area + e) = e % kMuStage < 2 * kMuBytes ? make_uint4(0u, 0u, 0u, 0u) : norm_words(kKmFar);
+  pdl_wait();                                                  // features, first centroids and sums come from the kernels before
+  if (tid == 0) s_skip = prm.err != nullptr && *reinterpret_cast<volatile int*>(prm.err) == SPARSEPR_ERR_TIMEOUT;
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  const uint32_t tmem = (uint32_t)misc[0];
+  volatile int* abort_flag = &misc[1];
+  const int row_tiles = (prm.N + 127) / 128, tile0 = cta * prm.per_cta;
+  const int my_tiles = __any_sync(FULL, s_skip) ? 0 : max(0, min(prm.per_cta, row_tiles - tile0));
+  const bool keep = my_tiles <= xst && n_chunks == 1;          // the row tiles stay in shared memory
+  const int row0 = tile0 * 128, my_rows = max(0, min(my_tiles * 128, prm.N - row0));
+  const i64 hrow0 = (i64)bh * prm.N + row0;                    // (rows count from the CTA's first below)
+  const float* phi = prm.phi + hrow0 * prm.ldphi;
+  int* assign = prm.assign + hrow0;
+  int* flagged = prm.flagged + hrow0;
+  const float scl = __int_as_float((127 + prm.fx_shift[bh]) << 23);
+  const double inv_sc = ldexp(1.0, -prm.fx_shift[bh]);
+  i64* sums = prm.sums + (i64)bh * C * R;
+  int* counts = prm.counts + (i64)bh * C;
+  float* values = reinterpret_cast<float*>(sm + val_area);
+  int tiles = my_tiles;                                        // 0 once a wait has run out
+  int kc = 0;                                                  // chunks of this warp's group so far (issuers and epilogue)
+  for (int t = 1;; ++t) {
+    // ---- centroids: words of -2 mu, words of the norm, float32 values
+    const bool from_sums = t > 1 || prm.from_sums;
+    float mx = 0.f;
+    constexpr int kB = 4;                                      // centroids of a warp in flight
+    for (int c0 = warp; c0 < C; c0 += kB * kWarps) {
+      const int k = 2 * lane;
+      int cnt[kB];
+      longlong2 sv[kB];
+      float2 v[kB];
+#pragma unroll
+      for (int b = 0; b < kB; ++b) {
+        const int c = c0 + b * kWarps;
+        cnt[b] = 0;
+        v[b] = make_float2(0.f, 0.f);
+        sv[b] = make_longlong2(0, 0);
+        if (c < C && k < R) {                                  // (columns r to R - 1 hold zeros)
+          if (from_sums) { cnt[b] = __ldcg(counts + c); sv[b] = __ldcg(reinterpret_cast<const longlong2*>(sums + (i64)c * R + k)); }
+          v[b] = t > 1 ? *reinterpret_cast<const float2*>(values + c * LDM + k) : *reinterpret_cast<const float2*>(prm.mu + ((i64)bh * C + c) * R + k);
+        }
+      }
+      float n2[kB];
+#pragma unroll
+      for (int b = 0; b < kB; ++b) {                           // (no branches: the chains of the four run side by side)
+        const GroupMean mean(max(cnt[b], 1), inv_sc);
+        const float mx0 = mean(sv[b].x), mx1 = mean(sv[b].y);
+        v[b].x = cnt[b] > 0 ? mx0 : v[b].x; v[b].y = cnt[b] > 0 ? mx1 : v[b].y;
+        n2[b] = warp_sum(fmaf(v[b].x, v[b].x, v[b].y * v[b].y));             // (7 roundings: 4.2e-7 of it, inside what km_score_error allows for accumulation)
+        mx = fmaxf(mx, n2[b]);
+      }
+#pragma unroll
+      for (int b = 0; b < kB; ++b) {
+        const int c = c0 + b * kWarps;
+        if (c >= C) break;                                     // (uniform)
+        if (k < R) *reinterpret_cast<float2*>(values + c * LDM + k) = v[b];
+        const uint32_t hi = pack_bf16x2(-2.f * v[b].x, -2.f * v[b].y), lo = pack_bf16x2_rest(-2.f * v[b].x, -2.f * v[b].y, hi);
+        unsigned char* st = sm + mu_area + (c / kKmChunk) * kMuStage;
+        const int cc = c % kKmChunk, off = cc * 128 + (((k >> 3) ^ (cc & 7)) << 4) + (k & 7) * 2;      // rows of 128 bytes, 128-byte swizzle
+        *reinterpret_cast<uint32_t*>(st + off) = hi;
+        *reinterpret_cast<uint32_t*>(st + kMuBytes + off) = lo;
+        if (lane == 0) *reinterpret_cast<uint4*>(st + 2 * kMuBytes + cc * 16) = norm_words(n2[b]);
+      }
+    }
+    __syncwarp();
+    cluster_arrive_relaxed();                                  // this warp has read the sums (they are in registers: nothing to be released)
+    if (lane == 0) s_max[warp] = mx;
+    fence_async_smem();                                        // the tensor cores read the operands
+    __syncthreads();
+    float mm = s_max[0];                                       // largest centroid norm of the head, rounded up
+#pragma unroll
+    for (int w = 1; w < kWarps; ++w) mm = fmaxf(mm, s_max[w]);
+    mm = sqrtf(mm) * 1.000001f;
+    cluster_wait();                                            // all CTAs have read the sums: they may change
+    const bool upd = t < prm.T;                                // the last pass needs no sums
+    const int* old = t > 1 ? assign : prm.old != nullptr ? prm.old + hrow0 : nullptr;
+    const bool first = old == nullptr;                         // no row is in a group yet: the sums are formed from all rows behind the pass
+    const int loads = keep ? 0 : (t - 1) * my_tiles;           // row tiles loaded in the passes before
+    if (warp == kKmEpiWarps) {
+      // =========================== TMA producer ============================================
+      if (lane == 0 && (!keep || t == 1)) {
+        for (int tl = 0; tl < tiles; ++tl) {
+          const int n = loads + tl, xs = n & (xst - 1);
+          if (!mbar_wait(bar(X_EMPTY + xs), ((n >> xlog) & 1) ^ 1, abort_flag)) break;
+          mbar_expect_tx(bar(X_FULL + xs), 2 * kXBytes);
+          tma_load_4d(base + KmSmem::x + xs * 2 * kXBytes, &mapXh, bar(X_FULL + xs), 0, row0 + tl * 128, bh, 0);
+          tma_load_4d(base + KmSmem::x + xs * 2 * kXBytes + kXBytes, &mapXl, bar(X_FULL + xs), 0, row0 + tl * 128, bh, 0);
+        }
+      }
+    } else if (warp > kKmEpiWarps) {
+      // =========================== MMA issuers (one per group) ================================
+      const int g = warp - (kKmEpiWarps + 1), ksteps = R / 16;
+      const int n_last = min(kKmChunk, (C - (n_chunks - 1) * kKmChunk + 15) & ~15);
+      const uint32_t idesc_full = idesc_bf16(0, kKmChunk), idesc_last = idesc_bf16(0, n_last);
+      const uint64_t x_desc0 = smem_desc(base + KmSmem::x, 16), m_desc0 = smem_desc(base + mu_area, 16);
+      const uint64_t one_desc = smem_desc_plain(base + KmSmem::ones, 128, 256), w_desc0 = smem_desc_plain(base + mu_area + 2 * kMuBytes, 0, 128);
+      const uint32_t tm = __shfl_sync(FULL, tmem, 0);
+      bool go = true;
+      for (int tl = g; tl < tiles && go; tl += 2) {
+        const int n = loads + tl, xs = n & (xst - 1);
+        if (!keep || t == 1) go = __all_sync(FULL, mbar_wait(bar(X_FULL + xs), (n >> xlog) & 1, abort_flag));
+        for (int ch = 0; ch < n_chunks; ++ch, ++kc) {
+          const int ab = 2 * g + (kc & 1);
+          go = __all_sync(FULL, go && mbar_wait(bar(ACC_EMPTY + ab), ((kc >> 1) & 1) ^ 1, abort_flag));
+          if (!go) break;
+          tc_fence_after();
+          const bool last = ch == n_chunks - 1;
+          const uint64_t moff = (uint64_t)((ch * kMuStage) >> 4);
+          if (elect_one()) {
+            km_product(tm + (uint32_t)ab * kKmChunk, one_desc, w_desc0 + moff, x_desc0 + (uint64_t)((xs * 2 * kXBytes) >> 4), m_desc0 + moff, ksteps,
+                       last ? idesc_last : idesc_full);
+            umma_commit(bar(ACC_FULL + ab));
+            if (last && !keep) umma_commit(bar(X_EMPTY + xs));
+          }
+          __syncwarp();
+        }
+      }
+    } else {
+      // =========================== epilogue: argmin ===========================================
+      const int grp = warp >> 3, hh = (warp >> 2) & 1, wq = warp & 3;
+      const uint32_t acc_addr0 = tmem + ((uint32_t)(wq * 32) << 16) + (uint32_t)grp * (2 * kKmChunk);
+      float* xb = reinterpret_cast<float*>(sm + KmSmem::xchg);
+      int n_changed = 0;
+      bool ok = true;
+      // a row's norm and group are fetched a tile ahead; the two warps of a quadrant finish 16 of its rows each
+      const auto is_mine = [&](int tl) { return tl < tiles && tl * 128 + wq * 32 + lane < my_rows && (lane >> 4) == hh; };
+      const auto norm_of = [&](int tl) { return is_mine(tl) ? prm.xnorm[hrow0 + tl * 128 + wq * 32 + lane] : 0.f; };
+      const auto group_of = [&](int tl) { return !first && is_mine(tl) ? old[tl * 128 + wq * 32 + lane] : -1; };
+      float xn_next = norm_of(grp);
+      int old_next = group_of(grp);
+      for (int tl = grp; tl < tiles; tl += 2) {
+        const int rowbase = tl * 128 + wq * 32, row = rowbase + lane;
+        const bool mine = is_mine(tl);
+        const float xn = xn_next;
+        const int was = old_next >= 0 && old_next < C ? old_next : kKmNone;
+        xn_next = norm_of(tl + 2);
+        old_next = group_of(tl + 2);
+        KmScan scan;
+        for (int ch = 0; ch < n_chunks; ++ch, ++kc) {
+          const int ab = 2 * grp + (kc & 1);
+          ok = __all_sync(FULL, ok && mbar_wait(bar(ACC_FULL + ab), (kc >> 1) & 1, abort_flag));
+          if (ok) {
+            tc_fence_after();
+            scan.chunk(acc_addr0 + (uint32_t)(kc & 1) * kKmChunk, ch * kKmChunk, C, hh);
+            tc_fence_before();
+          }
+          __syncwarp();
+          if (lane == 0) mbar_arrive(bar(ACC_EMPTY + ab));
+        }
+        float best, second;
+        int bi;
+        scan.result(best, second, bi);
+        km_exchange(xb + ((grp * 2 + ((tl >> 1) & 1)) * 2) * 128 + wq * 32 + lane, hh, 1 + grp * 4 + wq, best, second, bi);
+        bi = min(bi, C - 1);                                   // (only rows of non-finite scores could point past C)
+        const bool decided = ok && mine && second - best > 2.f * km_score_error(xn, mm), moved = decided && was != bi;
+        if (decided) {
+          if (moved || t == 1) assign[row] = bi;
+        } else if (ok && mine) {                               // the recheck decides this row
+          flagged[atomicAdd(&s_flagged, 1)] = row;
+          asm volatile("prefetch.global.L1 [%0];" ::"l"(phi + (i64)row * prm.ldphi));
+          asm volatile("prefetch.global.L1 [%0];" ::"l"(phi + (i64)row * prm.ldphi + prm.ldphi - 16));
+        }
+        n_changed += __popc(__ballot_sync(FULL, t == 1 ? decided : moved));
+        const unsigned mask = __ballot_sync(FULL, moved);
+        if (mask && upd && !first) {
+          int at = 0;
+          if (lane == 0) at = atomicAdd(&s_moved, __popc(mask));
+          at = __shfl_sync(FULL, at, 0) + __popc(mask & ((1u << lane) - 1));
+          if (moved && at < kKmRunList) s_list[at] = km_entry(row, was, bi);
+          const unsigned over = __ballot_sync(FULL, moved && at >= kKmRunList);
+          if (over) km_moves(over, phi + (i64)rowbase * prm.ldphi, prm.ldphi, sums, counts, C, R, prm.r, scl, was, bi, lane);
+        }
+      }
+      if (lane == 0 && n_changed) atomicAdd(prm.changed + (i64)t * prm.ld_changed + bh, n_changed);
+    }
+    __syncthreads();
+    if (*abort_flag) tiles = 0;                                // (the same for all threads: nobody waits now)
+    const int n_flagged = tiles ? s_flagged : 0, n_moved = tiles ? min(s_moved, kKmRunList) : 0;
+    const bool sorted = n_moved > kKmRunSort;
+    // ---- exact decisions for the rows that are left, by the epilogue warps; moves row by row, the last warps first
+    if (warp < kKmEpiWarps && n_flagged > 0) {
+      // scratch of a warp: behind the row stages' use (more than 128 centroids, whose tiles are not kept), else where the halves of the columns meet
+      const int Cp = (C + 31) & ~31;
+      float *d32 = reinterpret_cast<float*>(sm + (n_chunks == 1 ? KmSmem::xchg : KmSmem::x)) + warp * (Cp + R), *xs = d32 + Cp;
+      for (int i = warp; i < n_flagged; i += kKmEpiWarps) {
+        const int row = flagged[i], o = first ? -1 : old[row], was = o >= 0 && o < C ? o : kKmNone;
+        __syncwarp();
+        for (int k = lane; k < R; k += 32) xs[k] = phi[(i64)row * prm.ldphi + k];
+        __syncwarp();                                          // (everyone has read the old group, which may lie in `assign`)
+        const int bi = recheck_row(xs, values, LDM, C, R, d32, lane);
+        if (lane == 0) {
+          assign[row] = bi;
+          if (t == 1 || was != bi) atomicAdd(prm.changed + (i64)t * prm.ld_changed + bh, 1);
+        }
+        if (upd && !first && was != bi)
+          km_move(sums, counts, C, R, prm.r, scl, 2 * lane < R ? *reinterpret_cast<const float2*>(xs + 2 * lane) : make_float2(0.f, 0.f), was == kKmNone ? -1 : was, bi, lane);
+      }
+    }
+    if (t == prm.T) {
+      if (tid == 0 && prm.recheck_total != nullptr && n_flagged) atomicAdd(prm.recheck_total, n_flagged);
+      break;
+    }
+    if (!first && !sorted) {
+      for (int i = kWarps - 1 - warp; i < n_moved; i += kWarps) {
+        const unsigned e = s_list[i];
+        const int row = e & 0x3FFFu, was = (e >> 14) & 511u;
+        const float2 x = 2 * lane < prm.r ? *reinterpret_cast<const float2*>(phi + (i64)row * prm.ldphi + 2 * lane) : make_float2(0.f, 0.f);
+        km_move(sums, counts, C, R, prm.r, scl, x, was == kKmNone ? -1 : was, e >> 23, lane);
+      }
+    } else {
+      __syncthreads();                                         // the recheck's groups and scratch
+      unsigned short* list = reinterpret_cast<unsigned short*>(sm + KmSmem::xchg);           // sorted: up to two elements per entry
+      const int in_pass = first ? (tiles ? my_rows : 0) : n_moved;
+      for (int w0 = 0; w0 < in_pass; w0 += kKmRunList) {       // (one round where rows have moved)
+        const int n = min(kKmRunList, in_pass - w0);
+        for (int g = tid; g <= C; g += kKmThreads) s_start[g] = 0;
+        if (first) for (int i = tid; i < n; i += kKmThreads) s_list[i] = km_entry(w0 + i, kKmNone, assign[w0 + i]);
+        __syncthreads();
+        for (int i = tid; i < n; i += kKmThreads) {
+          const unsigned e = s_list[i];
+          atomicAdd(s_start + (e >> 23), 1);
+          if (((e >> 14) & 511u) != kKmNone) atomicAdd(s_start + ((e >> 14) & 511u), 1);
+        }
+        __syncthreads();
+        if (warp == 0) {                                       // exclusive prefix sums over up to 256 groups, total behind them
+          int c[8], sum = 0;
+#pragma unroll
+          for (int u = 0; u < 8; ++u) { c[u] = 8 * lane + u < C ? s_start[8 * lane + u] : 0; sum += c[u]; }
+          int inc = sum;
+#pragma unroll
+          for (int o = 1; o < 32; o <<= 1) { const int up = __shfl_up_sync(FULL, inc, o); if (lane >= o) inc += up; }
+          int at = inc - sum;
+#pragma unroll
+          for (int u = 0; u < 8; ++u) { if (8 * lane + u < C) s_start[8 * lane + u] = at; at += c[u]; }
+          if (lane == 31) s_start[C] = inc;
+        }
+        __syncthreads();
+        for (int i = tid; i < n; i += kKmThreads) {
+          const unsigned e = s_list[i];
+          list[atomicAdd(s_start + (e >> 23), 1)] = (unsigned short)i;
+          if (((e >> 14) & 511u) != kKmNone) list[atomicAdd(s_start + ((e >> 14) & 511u), 1)] = (unsigned short)(i | 0x8000);
+        }
+        __syncthreads();
+        const int total = s_start[C];
+        km_move_sorted(s_list, list, total * warp / kWarps, total * (warp + 1) / kWarps, phi, prm.ldphi, sums, counts, R, prm.r, scl, lane);
+        if (w0 + kKmRunList < in_pass) __syncthreads();        // the list is filled again
+      }
+    }
+    // a pass that changes nothing has reached the fixed point of the iteration
+    __syncwarp();
+    cluster_arrive();
+    cluster_wait();                                            // the sums and the counter of this pass are complete
+    if (tid == 0) { s_left = __ldcg(prm.changed + (i64)t * prm.ld_changed + bh); s_flagged = 0; s_moved = 0; }
+    fence_async_smem();                                        // (scratch in the row stages, which are filled again)
+    __syncthreads();
+    if (s_left == 0) break;                                    // (the same for the whole cluster)
+  }
+  pdl_launch_dependents();
+  tc_fence_before();
+  __syncthreads();
+  if (*abort_flag) {
+    for (int k = 0; k < 64; ++k) __nanosleep(1000);
+    if (tid == 0) set_error(prm.err, SPARSEPR_ERR_TIMEOUT);
+    __syncthreads();
+  }
+  if (warp == kKmEpiWarps + 1) {
+    tc_fence_after();
+    tmem_dealloc(tmem, 512);
+  }
+}
 
 // The same decision without staging, for centroid tables that do not fit into shared memory: grid (X, BH), one CTA per
 // row, one thread per centroid, float64 throughout.
@@ -640,15 +1061,78 @@ __global__ void __launch_bounds__(256) k_split_bf16(const float* __restrict__ x,
 
 constexpr size_t kRecheckSmemMax = 200 * 1024;
 cudaError_t init_kmeans_tc() {
-  const cudaError_t e = cudaFuncSetAttribute(tc::k_assign_recheck_staged, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kRecheckSmemMax);
+  cudaError_t e = cudaFuncSetAttribute(tc::k_assign_recheck_staged, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kRecheckSmemMax);
   if (e != cudaSuccess) return e;
-  return cudaFuncSetAttribute(tc::k_kmeans_assign_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)tc::kKmSmemBytes);
+  e = cudaFuncSetAttribute(tc::k_kmeans_assign_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)tc::kKmSmemBytes);
+  if (e != cudaSuccess) return e;
+  e = cudaFuncSetAttribute(tc::k_kmeans_run, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)tc::kKmSmemBytes);
+  if (e != cudaSuccess) return e;
+  return cudaFuncSetAttribute(tc::k_kmeans_run, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
 }
 bool kmeans_tc_supported() { return tc::tma_available(); }
 
 void launch_split_bf16(const float* x, int ld, i64 rows, int r, __nv_bfloat16* hi, __nv_bfloat16* lo, float* norm,
                        cudaStream_t st) {
   launch_pdl(tc::k_split_bf16, dim3((unsigned)((rows * 8 + 255) / 256)), dim3(256), 0, st, x, ld, rows, r, hi, lo, norm);
+}
+
+// Clusters of s CTAs that run side by side on the current device (0: none), s = 1 .. 16
+static const int* run_clusters() {
+  static int table[64][17];
+  static std::once_flag once[64];
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) { static const int none[17] = {}; return none; }
+  std::call_once(once[dev], [dev] {
+    for (int s = 1; s <= 16; ++s) {
+      cudaLaunchConfig_t cfg{};
+      cfg.gridDim = dim3(s, 1); cfg.blockDim = dim3(tc::kKmThreads); cfg.dynamicSmemBytes = tc::kKmSmemBytes;
+      cudaLaunchAttribute at[1];
+      at[0].id = cudaLaunchAttributeClusterDimension;
+      at[0].val.clusterDim.x = s; at[0].val.clusterDim.y = 1; at[0].val.clusterDim.z = 1;
+      cfg.attrs = at; cfg.numAttrs = 1;
+      int n = 0;
+      if (cudaOccupancyMaxActiveClusters(&n, tc::k_kmeans_run, &cfg) != cudaSuccess) { cudaGetLastError(); n = 0; }
+      table[dev][s] = n;
+    }
+  });
+  return table[dev];
+}
+// CTAs per head for a run in one kernel, 0 where separate passes are faster.  One head's CTAs form a cluster, and all clusters have to be on the GPU at
+// once: the largest that BH heads leave room for.  Of clusters of an odd number of CTAs the last ones that should fit often do not (they share pairs of
+// SMs with others: 25 and 26 clusters of 5 where 26 are promised, 42 to 45 of 3 where 45 are), hence the margin there.
+// A pass in one kernel saves 8 us and 0.45 us per head, measured; clusters leave SMs idle, and a row tile more per CTA than the separate launches
+// have costs 0.9 us for its rows and as much for 256 centroids; the line below is drawn a little to the safe side of that.  Plans in one kernel / separately, us: 2 heads of 4096 rows
+// (32 centroids) 582 / 707, 16 of 17408 (136) 1523 / 1622, 33 of 16384 (128) 1956 / 2372; on the other side 1 of 32768 (256) 1308 / 1025, 16 of 32768
+// 2655 / 2514, 24 of 32768 3242 / 3263.
+int kmeans_run_ctas(int BH, int N, int C, int r) {
+  if (C > 2 * tc::kKmChunk || r > kMaxRank || !kmeans_tc_supported()) return 0;
+  const int row_tiles = (N + 127) / 128, *fit = run_clusters();
+  int s = 0;
+  for (int k = 1; k <= 16 && k <= row_tiles; ++k) if (fit[k] - (k & 1 ? fit[k] / 11 : 0) >= BH) s = k;
+  if (s == 0) return 0;
+  const int per = (row_tiles + s - 1) / s, alone = (int)(((i64)row_tiles * BH + sm_count() - 1) / sm_count());
+  if (per > tc::kKmRunTiles || (per - alone) * (256 + C) > 2000 + 110 * BH) return 0;
+  return (row_tiles + per - 1) / per;
+}
+bool launch_kmeans_run(const KmeansRunArgs& a, cudaStream_t st) {
+  using namespace tc;
+  CUtensorMap mxh, mxl;
+  if (!make_map(&mxh, a.xh, 64, a.N, a.BH, 1, 0, (i64)a.N * 64, 64, 128) || !make_map(&mxl, a.xl, 64, a.N, a.BH, 1, 0, (i64)a.N * 64, 64, 128)) return false;
+  const int s = kmeans_run_ctas(a.BH, a.N, a.C, a.r), row_tiles = (a.N + 127) / 128;
+  KmRunParams p{};
+  p.N = a.N; p.C = a.C; p.r = a.r; p.R = a.R; p.T = a.T; p.n_chunks = (a.C + kKmChunk - 1) / kKmChunk; p.per_cta = (row_tiles + s - 1) / s;
+  p.phi = a.phi; p.ldphi = a.ldphi; p.xnorm = a.xnorm; p.mu = a.mu; p.from_sums = a.from_sums; p.old = a.old; p.assign = a.assign;
+  p.sums = a.sums; p.counts = a.counts; p.fx_shift = a.fx_shift; p.flagged = a.flagged; p.recheck_total = a.recheck_total; p.err = a.err;
+  p.changed = a.changed; p.ld_changed = a.ld_changed;
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3(s, a.BH); cfg.blockDim = dim3(kKmThreads); cfg.dynamicSmemBytes = kKmSmemBytes; cfg.stream = st;
+  cudaLaunchAttribute at[2];
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  at[1].id = cudaLaunchAttributeClusterDimension;
+  at[1].val.clusterDim.x = s; at[1].val.clusterDim.y = 1; at[1].val.clusterDim.z = 1;
+  cfg.attrs = at; cfg.numAttrs = 2;
+  return cudaLaunchKernelEx(&cfg, k_kmeans_run, mxh, mxl, p) == cudaSuccess;
 }
 
 // One assignment pass.  xh/xl: bf16 [BH][N][64]; mh/ml: bf16 [BH][C][64]; sums may be null (no update wanted), else they

@@ -2,7 +2,7 @@
 // Gram matrix, batched Jacobi eigen-decomposition -> feature maps, response
 // projections, k-means assignment/update, stable counting sort, group means.
 #include <algorithm>
-#include "kernels.cuh"
+#include "kmeans_sums.cuh"
 
 namespace spr {
 
@@ -368,10 +368,11 @@ void launch_kmeans_assign(const float* phi, int ldphi, int BH, int N, int r, con
 // and derives the fixed-point shift of the head from max |phi|.
 __global__ void k_kmeans_init(const float* __restrict__ phi, int ldphi, int N, int r, int R, int C, u64 seed, int tag, int head0,
                               float* __restrict__ mu, i64* __restrict__ sums, int* __restrict__ counts,
-                              const unsigned* __restrict__ maxabs_bits, int* __restrict__ fx_shift) {
+                              const unsigned* __restrict__ maxabs_bits, int* __restrict__ fx_shift, int* __restrict__ recheck_total) {
   pdl_wait();                                                   // the features come from the kernel before
   pdl_launch_dependents();
   const int bh = blockIdx.y;
+  if (blockIdx.x == 0 && bh == 0 && threadIdx.x == 0) *recheck_total = 0;
   const u64 U = sample_offset(seed, tag, head0 + bh);
   for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < C * R; e += gridDim.x * blockDim.x) {
     const int c = e / R, k = e % R;
@@ -410,13 +411,7 @@ __global__ void __launch_bounds__(1024) k_kmeans_finalize(float* __restrict__ mu
   pdl_launch_dependents();
   const double inv_sc = update ? ldexp(1.0, -fx_shift[bh]) : 0.0;
   float mx = 0.f;
-  auto store_words = [&](float v, int c) {                       // the three bf16 words of ||mu_c||^2, then zeros
-    const __nv_bfloat16 w0 = __float2bfloat16_rn(v);
-    const float v1 = v - __bfloat162float(w0);
-    const __nv_bfloat16 w1 = __float2bfloat16_rn(v1), w2 = __float2bfloat16_rn(v1 - __bfloat162float(w1));
-    const uint32_t lo = (uint32_t)__bfloat16_as_ushort(w0) | ((uint32_t)__bfloat16_as_ushort(w1) << 16);
-    *reinterpret_cast<uint4*>(mw + ((i64)bh * Cpad + c) * 8) = make_uint4(lo, __bfloat16_as_ushort(w2), 0u, 0u);
-  };
+  auto store_words = [&](float v, int c) { *reinterpret_cast<uint4*>(mw + ((i64)bh * Cpad + c) * 8) = norm_words(v); };
   if (mw != nullptr && blockIdx.y == 0)
     for (int c = C + threadIdx.x; c < Cpad; c += blockDim.x) store_words(kKmFar, c);
   for (int c = blockIdx.y * nw + w; c < C; c += nw * gridDim.y) {
@@ -429,7 +424,7 @@ __global__ void __launch_bounds__(1024) k_kmeans_finalize(float* __restrict__ mu
       if (k < R) {
         v = m[k];
         if (update) {
-          if (cnt > 0 && k < r) { v = (float)((double)s[k] * inv_sc / (double)cnt); m[k] = v; }
+          if (cnt > 0 && k < r) { v = group_mean(s[k], inv_sc, cnt); m[k] = v; }
           if (update == 1) s[k] = 0;
         }
         n2 += (double)v * (double)v;
@@ -460,58 +455,17 @@ __global__ void __launch_bounds__(1024) k_kmeans_finalize(float* __restrict__ mu
 // Fixed-point sums and counts of the features over the groups of a partition [BH][N] (ids outside [0, C) are ignored): the
 // first centroids of a warm start (Appendix C.1; a group that the previous partition left empty keeps the strided row
 // k_kmeans_init gave it), and the sums after the first tensor-core assignment, which later passes only update.
-// Every row is rounded once, as in a later move of that row, so the sums stay exact: x 2^shift = h 2^26 + l with
-// h = rint(x 2^(shift - 26)) and l = rint of what is left, both below 2^26 and added over up to 32 rows in int32.
-// One warp per 32 consecutive rows, lane = columns lane and lane + 32, two rows in flight, one atomic per (group present in
-// the warp, column).  Bound by those atomics (a warp's 32 rows fall into about 20 groups after a cold start): 67 us at
+// One warp per 32 consecutive rows (add_rows_to_sums).  Bound by the atomics (a warp's 32 rows fall into about 20 groups after a cold start): 67 us at
 // 24 heads of 32760 rows and 64 columns, 48 us on the partition of a call before (few groups per warp).
 __global__ void __launch_bounds__(256) k_kmeans_group_sums(const float* __restrict__ phi, int ldphi, int N, int r, int R, int C,
                                                            const int* __restrict__ assign, i64* __restrict__ sums,
                                                            int* __restrict__ counts, const int* __restrict__ fx_shift) {
-  const unsigned FULL = 0xffffffffu;
   pdl_wait();                                                   // the assignment comes from the kernels before
   pdl_launch_dependents();
-  const int bh = blockIdx.y, lane = threadIdx.x & 31;
-  const int rowbase = (blockIdx.x * 8 + (threadIdx.x >> 5)) * 32;
+  const int bh = blockIdx.y, rowbase = (blockIdx.x * 8 + (threadIdx.x >> 5)) * 32;
   if (rowbase >= N) return;
-  const int row = rowbase + lane;
-  int cl_mine = -1;
-  if (row < N) { const int c = assign[(i64)bh * N + row]; if (c >= 0 && c < C) cl_mine = c; }
-  const float s_hi = __int_as_float((127 + fx_shift[bh] - 26) << 23);
-  for (int cb = 0; cb < R; cb += 64) {                         // 64 columns at a time (two passes for raw activations)
-    const int col = cb + lane;
-    const bool ok0 = col < r, ok1 = col + 32 < r;
-    const float* p = phi + ((i64)bh * N + rowbase) * ldphi + col;
-    unsigned todo = __ballot_sync(FULL, cl_mine >= 0);
-    while (todo) {
-      const int leader = __ffs(todo) - 1;
-      const int cl = __shfl_sync(FULL, cl_mine, leader);
-      unsigned m = __ballot_sync(FULL, cl_mine == cl);
-      todo &= ~m;
-      const int n = __popc(m);
-      int h0 = 0, h1 = 0, l0 = 0, l1 = 0;
-      auto add = [&](float xa, float xc) {
-        const float y0 = xa * s_hi, y1 = xc * s_hi;
-        const int a0 = __float2int_rn(y0), a1 = __float2int_rn(y1);
-        h0 += a0; h1 += a1;
-        l0 += __float2int_rn((y0 - (float)a0) * 67108864.f); l1 += __float2int_rn((y1 - (float)a1) * 67108864.f);
-      };
-      while (m) {
-        const float* pa = p + (i64)(__ffs(m) - 1) * ldphi;
-        m &= m - 1;
-        const float* pb = m ? p + (i64)(__ffs(m) - 1) * ldphi : nullptr;
-        m &= m - 1;
-        const float a0 = ok0 ? pa[0] : 0.f, a1 = ok1 ? pa[32] : 0.f;
-        const float b0 = ok0 && pb ? pb[0] : 0.f, b1 = ok1 && pb ? pb[32] : 0.f;
-        add(a0, a1);
-        add(b0, b1);
-      }
-      i64* sp = sums + ((i64)bh * C + cl) * R + col;
-      if (ok0) atomicAdd(reinterpret_cast<u64*>(sp), (u64)((i64)h0 * 67108864ll + l0));
-      if (ok1) atomicAdd(reinterpret_cast<u64*>(sp + 32), (u64)((i64)h1 * 67108864ll + l1));
-      if (lane == 0 && cb == 0) atomicAdd(counts + (i64)bh * C + cl, n);
-    }
-  }
+  const i64 row = (i64)bh * N + rowbase;
+  add_rows_to_sums(phi + row * ldphi, ldphi, N - rowbase, r, R, C, assign + row, sums + (i64)bh * C * R, counts + (i64)bh * C, fx_shift[bh]);
 }
 void launch_kmeans_group_sums(const float* phi, int ldphi, int BH, int N, int r, int C, const int* assign, i64* sums,
                               int* counts, const int* fx_shift, cudaStream_t st) {
@@ -520,10 +474,10 @@ void launch_kmeans_group_sums(const float* phi, int ldphi, int BH, int N, int r,
 }
 
 void launch_kmeans_init(const float* phi, int ldphi, int BH, int N, int r, int C, u64 seed, int tag, int head0, float* mu,
-                        i64* sums, int* counts, const unsigned* maxabs_bits, int* fx_shift, cudaStream_t st) {
+                        i64* sums, int* counts, const unsigned* maxabs_bits, int* fx_shift, int* recheck_total, cudaStream_t st) {
   const int R = feature_ld(r);
   dim3 grid((C * R + 255) / 256, BH);
-  launch_pdl(k_kmeans_init, grid, dim3(256), 0, st, phi, ldphi, N, r, R, C, seed, tag, head0, mu, sums, counts, maxabs_bits, fx_shift);
+  launch_pdl(k_kmeans_init, grid, dim3(256), 0, st, phi, ldphi, N, r, R, C, seed, tag, head0, mu, sums, counts, maxabs_bits, fx_shift, recheck_total);
 }
 void launch_kmeans_finalize(float* mu, float* mu2, float* mumax, i64* sums, int* counts, const int* fx_shift, int BH,
                             int C, int r, int update, cudaStream_t st, __nv_bfloat16* mh, __nv_bfloat16* ml, __nv_bfloat16* mw) {
