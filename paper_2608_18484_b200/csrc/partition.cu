@@ -8,115 +8,155 @@ namespace spr {
 
 // =============================================================================
 // Gram matrices: M_K = Q_s^T Q_s / M_s (Appendix B.1) and
-// M_Q = Ktilde^T Ktilde / (C_k^+ d) (Appendix B.2), float64 accumulation.
-// Grid (D/16, heads): a CTA owns 16 rows of the D x D result; thread t owns column
-// t % D and 8 consecutive rows.  Input rows are staged in shared memory as doubles.
+// M_Q = Ktilde^T Ktilde / (C_k^+ d) (Appendix B.2), float64 accumulation in order of the rows.
+// Bound by the float64 pipe, which takes a warp's instruction every 14 cycles or so on each of an SM's four schedulers (8 to 9 multiply-adds per clock
+// and SM): only the tiles on and above the diagonal are formed (the products of two mirrored entries are the same, a tile is also written mirrored), and
+// they are small, 16 x 16, so that a few heads spread over the SMs.  128 threads, two neighbouring entries each; rows come a chunk ahead.
+// (What the call takes for the sample / the centroids, us: 2 heads of d = 128, 256 and 38 rows, 15 / 6, 24 heads of 256 rows each 30 / 41; with 16 whole
+// rows of the result per CTA 26 / 9 and 48 / 98, with tiles of 32 x 32 by two warps 34 / 17 and 48 / 184.)
 // =============================================================================
-constexpr int kGramChunk = 32;
-constexpr int kGramSlab = 16;
+constexpr int kGramChunk = 64, kGramTile = 16, kGramThreads = 128;
+constexpr int gram_tiles(int d) { return (d / kGramTile) * (d / kGramTile + 1) / 2; }
 
-template <int D>
-__device__ __forceinline__ void gram_accumulate(const double* rows, int nrows, int i0, int j, double (&acc)[8]) {
+template <int D> __device__ __forceinline__ void gram_tile(int t, int& i0, int& j0) {      // t-th tile by rows
+  int i = 0;
+  for (int left = t, n = D / kGramTile;; ++i, --n) {
+    if (left < n) { i0 = i * kGramTile; j0 = (i + left) * kGramTile; return; }
+    left -= n;
+  }
+}
+// rows [kGramChunk][2][kGramTile]: the columns from i0 on, then those from j0 on
+__device__ __forceinline__ void gram_accumulate(const double (*rows)[2][kGramTile], int nrows, double (&acc)[2]) {
+  const int i = threadIdx.x / 8, j = threadIdx.x % 8 * 2;
+#pragma unroll 8
   for (int s = 0; s < nrows; ++s) {
-    const double xj = rows[s * D + j];
-    const double* xi = rows + s * D + i0;                 // the same 8 values for the whole half-block: broadcast
+    const double xi = rows[s][0][i];
+    const double2 xj = *reinterpret_cast<const double2*>(&rows[s][1][j]);
+    acc[0] = fma(xi, xj.x, acc[0]);
+    acc[1] = fma(xi, xj.y, acc[1]);
+  }
+}
+template <int D> __device__ __forceinline__ void gram_store(double* M, int i0, int j0, const double (&acc)[2], double denom) {
+  const int i = i0 + threadIdx.x / 8, j = j0 + threadIdx.x % 8 * 2;
 #pragma unroll
-    for (int k = 0; k < 8; ++k) acc[k] = fma(xi[k], xj, acc[k]);
+  for (int v = 0; v < 2; ++v) {
+    const double m = acc[v] / denom;
+    M[i * D + j + v] = m;
+    if (i0 != j0) M[(j + v) * D + i] = m;
   }
 }
 
 template <typename T, int D>
-__global__ void __launch_bounds__(256) k_sample_gram(const T* __restrict__ Q, i64 sb, i64 sh, i64 sn, int H, int N,
-                                                     int Ms, u64 seed, int head0, double* __restrict__ Mout) {
+__global__ void __launch_bounds__(kGramThreads) k_sample_gram(const T* __restrict__ Q, i64 sb, i64 sh, i64 sn, int H, int N,
+                                                              int Ms, u64 seed, int head0, double* __restrict__ Mout) {
   pdl_launch_dependents();                                     // (inputs of this kernel are the caller's)
-  __shared__ __align__(16) double rows[kGramChunk * D];
-  const int bh = blockIdx.y, b = bh / H, h = bh % H;
+  __shared__ __align__(16) double rows[kGramChunk][2][kGramTile];
+  __shared__ int s_row[2][kGramChunk];                         // sampled rows of this chunk and the next
+  const int bh = blockIdx.y, b = bh / H, h = bh % H, tid = threadIdx.x;
   const T* base = Q + b * sb + h * sh;
   const u64 U = sample_offset(seed, kTagQuerySample, head0 + bh);
-  const int j = threadIdx.x % D, i0 = blockIdx.x * kGramSlab + (threadIdx.x / D) * 8;
-  const bool active = threadIdx.x < 2 * D;
-  double acc[8] = {0, 0, 0, 0, 0, 0, 0, 0};
+  int i0, j0;
+  gram_tile<D>(blockIdx.x, i0, j0);
+  // eight columns of kOwn rows per thread and chunk
+  constexpr int kOwn = kGramChunk * 2 * kGramTile / 8 / kGramThreads, kStep = kGramThreads / 4;
+  const int s = tid / 4, c = tid % 4, col = c < 2 ? i0 + 8 * c : j0 + 8 * (c - 2);
+  float v[kOwn][8] = {};
+  const auto sample = [&](int s0) { if (tid < kGramChunk && s0 + tid < Ms) s_row[(s0 / kGramChunk) & 1][tid] = strided_row(s0 + tid, Ms, N, U); };
+  const auto fetch = [&](int s0) {
+#pragma unroll
+    for (int u = 0; u < kOwn; ++u)
+      if (s0 + s + u * kStep < Ms) load8(base + (i64)s_row[(s0 / kGramChunk) & 1][s + u * kStep] * sn + col, v[u]);
+  };
+  double acc[2] = {0.0, 0.0};
+  sample(0);
+  __syncthreads();
+  fetch(0);
   for (int s0 = 0; s0 < Ms; s0 += kGramChunk) {
-    const int nr = min(kGramChunk, Ms - s0);
-    __syncthreads();
-    for (int t = threadIdx.x; t < nr * (D / 8); t += 256) {
-      const int s = t / (D / 8), c = t % (D / 8);
-      float v[8];
-      load8(base + (i64)strided_row(s0 + s, Ms, N, U) * sn + c * 8, v);
+    sample(s0 + kGramChunk);
+    __syncthreads();                                           // (the chunk before has been read)
 #pragma unroll
-      for (int k = 0; k < 8; ++k) rows[s * D + c * 8 + k] = (double)v[k];
-    }
-    __syncthreads();
-    if (active) gram_accumulate<D>(rows, nr, i0, j, acc);
-  }
-  if (active) {
+    for (int u = 0; u < kOwn; ++u)
 #pragma unroll
-    for (int k = 0; k < 8; ++k) Mout[(i64)bh * D * D + (i64)(i0 + k) * D + j] = acc[k] / (double)Ms;
+      for (int k = 0; k < 8; ++k) rows[s + u * kStep][c / 2][c % 2 * 8 + k] = (double)v[u][k];
+    __syncthreads();
+    if (s0 + kGramChunk < Ms) fetch(s0 + kGramChunk);
+    gram_accumulate(rows, min(kGramChunk, Ms - s0), acc);
   }
+  gram_store<D>(Mout + (i64)bh * D * D, i0, j0, acc, (double)Ms);
 }
 
 // kappa [BH][C][D] float32, n [BH][C] group sizes.  Empty groups are skipped and the
-// remaining centroids are centred by their uniform mean.
+// remaining centroids are centred by their uniform mean (summed in order of the groups).
 template <int D>
-__global__ void __launch_bounds__(256) k_centroid_gram(const float* __restrict__ kappa, const int* __restrict__ n, int C,
-                                                       double* __restrict__ Mout) {
+__global__ void __launch_bounds__(kGramThreads) k_centroid_gram(const float* __restrict__ kappa, const int* __restrict__ n, int C,
+                                                                double* __restrict__ Mout) {
   pdl_wait();                                                   // the group means come from the kernel before
   pdl_launch_dependents();
-  __shared__ __align__(16) double rows[kGramChunk * D];
-  __shared__ double mean[D];
+  __shared__ __align__(16) double rows[kGramChunk][2][kGramTile];
+  __shared__ int s_n[kMaxGroups];
+  __shared__ double s_mean[2 * kGramTile];
   __shared__ int s_cnt;
-  const int bh = blockIdx.y;
-  const float* kp = kappa + (i64)bh * C * D;
-  const int* nn = n + (i64)bh * C;
-  if (threadIdx.x == 0) s_cnt = 0;
+  const int bh = blockIdx.y, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  int i0, j0;
+  gram_tile<D>(blockIdx.x, i0, j0);
+  // lane = one of the 32 columns of the tile's rows, a warp has eight rows of a chunk
+  constexpr int kOwn = kGramChunk / (kGramThreads / 32);
+  const int side = lane / kGramTile, jj = lane % kGramTile;
+  const float* kp = kappa + (i64)bh * C * D + (side ? j0 : i0) + jj;
+  if (tid == 0) s_cnt = 0;
   __syncthreads();
-  {
-    int c = 0;
-    for (int g = threadIdx.x; g < C; g += 256) c += nn[g] > 0;
-    c = warp_sum(c);
-    if ((threadIdx.x & 31) == 0 && c) atomicAdd(&s_cnt, c);
-  }
+  int c = 0;
+  for (int g = tid; g < C; g += kGramThreads) { const int ng = n[(i64)bh * C + g]; s_n[g] = ng; c += ng > 0; }
+  c = warp_sum(c);
+  if (lane == 0 && c) atomicAdd(&s_cnt, c);
   __syncthreads();
   const int cplus = s_cnt;
-  if (threadIdx.x < D) {
-    double m = 0.0;
-    for (int g = 0; g < C; ++g)
-      if (nn[g] > 0) m += (double)kp[(i64)g * D + threadIdx.x];
-    mean[threadIdx.x] = cplus > 0 ? m / cplus : 0.0;
-  }
-  const int j = threadIdx.x % D, i0 = blockIdx.x * kGramSlab + (threadIdx.x / D) * 8;
-  const bool active = threadIdx.x < 2 * D;
-  double acc[8] = {0, 0, 0, 0, 0, 0, 0, 0};
-  for (int g0 = 0; g0 < C; g0 += kGramChunk) {
-    const int nr = min(kGramChunk, C - g0);
-    __syncthreads();
-    for (int t = threadIdx.x; t < nr * D; t += 256) {
-      const int s = t / D, jj = t % D;
-      rows[t] = nn[g0 + s] > 0 ? (double)kp[(i64)(g0 + s) * D + jj] - mean[jj] : 0.0;
-    }
-    __syncthreads();
-    if (active) gram_accumulate<D>(rows, nr, i0, j, acc);
-  }
-  const double denom = cplus > 0 ? (double)cplus * (double)D : 1.0;
-  if (active) {
+  float x[kOwn];
+  const auto fetch = [&](int g0) {
 #pragma unroll
-    for (int k = 0; k < 8; ++k) Mout[(i64)bh * D * D + (i64)(i0 + k) * D + j] = acc[k] / denom;
+    for (int u = 0; u < kOwn; ++u) { const int g = g0 + warp * kOwn + u; x[u] = g < C && s_n[g] > 0 ? kp[(i64)g * D] : 0.f; }
+  };
+  // first the mean, then the products: the rows come twice
+  double acc[2] = {0.0, 0.0}, m = 0.0;
+  for (int pass = 0; pass < 2; ++pass) {
+    const double mean = pass ? s_mean[lane] : 0.0;
+    fetch(0);
+    for (int g0 = 0; g0 < C; g0 += kGramChunk) {
+      const int nr = min(kGramChunk, C - g0);
+      __syncthreads();
+#pragma unroll
+      for (int u = 0; u < kOwn; ++u) {
+        const int g = g0 + warp * kOwn + u;
+        rows[warp * kOwn + u][side][jj] = pass && !(g < C && s_n[g] > 0) ? 0.0 : (double)x[u] - mean;
+      }
+      __syncthreads();
+      if (g0 + kGramChunk < C) fetch(g0 + kGramChunk);
+      if (pass) {
+        gram_accumulate(rows, nr, acc);
+      } else if (warp == 0) {
+#pragma unroll 8
+        for (int u = 0; u < nr; ++u) m += rows[u][side][jj];   // (an empty group adds nothing)
+      }
+    }
+    if (pass == 0 && warp == 0) s_mean[lane] = cplus > 0 ? m / cplus : 0.0;
+    __syncthreads();
   }
+  gram_store<D>(Mout + (i64)bh * D * D, i0, j0, acc, cplus > 0 ? (double)cplus * (double)D : 1.0);
 }
 
 void launch_sample_gram(int dtype, const void* Q, const i64* qs, int BH, int H, int N, int d, int Ms, u64 seed, int head0,
                         double* Mout, cudaStream_t st) {
   if (dtype == SPARSEPR_BF16) {
-    if (d == 128) k_sample_gram<__nv_bfloat16, 128><<<dim3(d / kGramSlab, BH), 256, 0, st>>>((const __nv_bfloat16*)Q, qs[0], qs[1], qs[2], H, N, Ms, seed, head0, Mout);
-    else k_sample_gram<__nv_bfloat16, 64><<<dim3(d / kGramSlab, BH), 256, 0, st>>>((const __nv_bfloat16*)Q, qs[0], qs[1], qs[2], H, N, Ms, seed, head0, Mout);
+    if (d == 128) k_sample_gram<__nv_bfloat16, 128><<<dim3(gram_tiles(d), BH), kGramThreads, 0, st>>>((const __nv_bfloat16*)Q, qs[0], qs[1], qs[2], H, N, Ms, seed, head0, Mout);
+    else k_sample_gram<__nv_bfloat16, 64><<<dim3(gram_tiles(d), BH), kGramThreads, 0, st>>>((const __nv_bfloat16*)Q, qs[0], qs[1], qs[2], H, N, Ms, seed, head0, Mout);
   } else {
-    if (d == 128) k_sample_gram<float, 128><<<dim3(d / kGramSlab, BH), 256, 0, st>>>((const float*)Q, qs[0], qs[1], qs[2], H, N, Ms, seed, head0, Mout);
-    else k_sample_gram<float, 64><<<dim3(d / kGramSlab, BH), 256, 0, st>>>((const float*)Q, qs[0], qs[1], qs[2], H, N, Ms, seed, head0, Mout);
+    if (d == 128) k_sample_gram<float, 128><<<dim3(gram_tiles(d), BH), kGramThreads, 0, st>>>((const float*)Q, qs[0], qs[1], qs[2], H, N, Ms, seed, head0, Mout);
+    else k_sample_gram<float, 64><<<dim3(gram_tiles(d), BH), kGramThreads, 0, st>>>((const float*)Q, qs[0], qs[1], qs[2], H, N, Ms, seed, head0, Mout);
   }
 }
 void launch_centroid_gram(const float* kappa, const int* n, int BH, int C, int d, double* Mout, cudaStream_t st) {
-  if (d == 128) launch_pdl(k_centroid_gram<128>, dim3(128 / kGramSlab, BH), dim3(256), 0, st, kappa, n, C, Mout);
-  else launch_pdl(k_centroid_gram<64>, dim3(64 / kGramSlab, BH), dim3(256), 0, st, kappa, n, C, Mout);
+  if (d == 128) launch_pdl(k_centroid_gram<128>, dim3(gram_tiles(128), BH), dim3(kGramThreads), 0, st, kappa, n, C, Mout);
+  else launch_pdl(k_centroid_gram<64>, dim3(gram_tiles(64), BH), dim3(kGramThreads), 0, st, kappa, n, C, Mout);
 }
 
 // =============================================================================
