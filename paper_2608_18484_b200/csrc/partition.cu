@@ -9,8 +9,8 @@ namespace spr {
 // =============================================================================
 // Gram matrices: M_K = Q_s^T Q_s / M_s (Appendix B.1) and
 // M_Q = Ktilde^T Ktilde / (C_k^+ d) (Appendix B.2), float64 accumulation in order of the rows.
-// Bound by the float64 pipe, which takes a warp's instruction every 14 cycles or so on each of an SM's four schedulers (8 to 9 multiply-adds per clock
-// and SM): only the tiles on and above the diagonal are formed (the products of two mirrored entries are the same, a tile is also written mirrored), and
+// Bound by latency and by conversions to float64 (16 per clock and SM; a warp alone takes 13 cycles for one): the rows of an entry are a chain of multiply-adds.
+// So only the tiles on and above the diagonal are formed (the products of two mirrored entries are the same, a tile is also written mirrored), and
 // they are small, 16 x 16, so that a few heads spread over the SMs.  128 threads, two neighbouring entries each; rows come a chunk ahead.
 // (What the call takes for the sample / the centroids, us: 2 heads of d = 128, 256 and 38 rows, 15 / 6, 24 heads of 256 rows each 30 / 41; with 16 whole
 // rows of the result per CTA 26 / 9 and 48 / 98, with tiles of 32 x 32 by two warps 34 / 17 and 48 / 184.)

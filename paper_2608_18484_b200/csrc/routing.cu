@@ -34,12 +34,15 @@ __global__ void __launch_bounds__(256) k_cell_scores(const float* __restrict__ t
     float acc[kCsRows];
 #pragma unroll
     for (int r = 0; r < kCsRows; ++r) acc[r] = 0.f;
+    const int rows = min(256, Ck - b0);
     for (int k0 = 0; k0 < d; k0 += 32) {
       __syncthreads();
-#pragma unroll 8
-      for (int r = 0; r < 32; ++r) {
-        const int b = b0 + warp * 32 + r;
-        kt[lane][warp * 32 + r] = (b < Ck && k0 + lane < d) ? kappa[((i64)kvh * Ck + b) * d + k0 + lane] : 0.f;
+      for (int r0 = warp; r0 < rows; r0 += 64) {                // rows over the warps, eight of a warp in flight: few groups are one round of loads
+        float v[8];
+#pragma unroll
+        for (int u = 0; u < 8; ++u) { const int b = b0 + r0 + 8 * u; v[u] = b < Ck ? kappa[((i64)kvh * Ck + b) * d + k0 + lane] : 0.f; }
+#pragma unroll
+        for (int u = 0; u < 8; ++u) kt[lane][r0 + 8 * u] = v[u];
       }
       __syncthreads();
 #pragma unroll
@@ -437,7 +440,8 @@ void launch_route_select(const float* score, const int* nq, const int* nk, int B
 // a time, and the largest group set the duration: 343 us beside the cell scores at 480p-like size with 24 heads, now 192 us;
 // whole calls: 2 heads of 4096 float32 tokens 1075 -> 1008 us, 2 heads of 4770 bf16 tokens 1171 -> 1140 us.)  Eight warps fetch 64
 // rows at once; the sums keep the order of the rows (a column is summed by one thread), and a distance is formed by one warp as
-// before, so that the result is the same bit for bit.
+// before, so that the result is the same bit for bit.  Eight butterflies per warp that share their first levels, and roots by full warps
+// (selection alone, us, before and now: 24 heads of 32760 tokens 214, 196, 32 of 18000 158, 145, 40 of 75600 673, 595).
 constexpr int kPdRows = 64, kPdCols = 128;
 __global__ void __launch_bounds__(256) k_probe_dist(const float* __restrict__ phi, int ldphi, int r,
                                                     const int* __restrict__ perm, const int* __restrict__ off, int N,
@@ -496,16 +500,20 @@ __global__ void __launch_bounds__(256) k_probe_dist(const float* __restrict__ ph
       for (int j = 0; j < kCols; ++j)
         if (has[j]) { const double t = (double)x[q][j] - cen[j]; s[q] += t * t; }
     }
-    // eight independent butterflies
+    // the sums over the lanes, as a butterfly gives them; at the first three levels a lane keeps half of the rows that it has, in the end row lane / 4
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
+    for (int half = 4; half > 0; half >>= 1) {
+      const bool upper = lane & (4 * half);
 #pragma unroll
-      for (int q = 0; q < 8; ++q) s[q] += __shfl_xor_sync(0xffffffffu, s[q], o);
+      for (int q = 0; q < half; ++q) s[q] = (upper ? s[q + half] : s[q]) + __shfl_xor_sync(0xffffffffu, upper ? s[q] : s[q + half], 4 * half);
     }
-#pragma unroll
-    for (int q = 0; q < 8; ++q)
-      if (lane == q && p + q < p1) dist[(i64)bh * N + p + q] = sqrt(s[q]);
+    s[0] += __shfl_xor_sync(0xffffffffu, s[0], 2);
+    s[0] += __shfl_xor_sync(0xffffffffu, s[0], 1);
+    if ((lane & 3) == 0 && p + lane / 4 < p1) dist[(i64)bh * N + p + lane / 4] = s[0];
   }
+  // the roots by a thread per row: a warp's float64 root takes 225 cycles whatever its number of lanes
+  __syncthreads();
+  for (int p = p0 + tid; p < p1; p += 256) dist[(i64)bh * N + p] = sqrt(dist[(i64)bh * N + p]);
 }
 
 __global__ void __launch_bounds__(1024) k_probe_pick(const double* __restrict__ dist, const int* __restrict__ perm,
