@@ -186,7 +186,7 @@ struct SideSet {
   cudaEvent_t ev_fork = nullptr, ev_join = nullptr;
   // third stream: the routing beside the gathers; the remainder kernel and the paired tiles beside the single ones
   cudaStream_t side2 = nullptr;
-  cudaEvent_t ev_join2 = nullptr, ev_route = nullptr;
+  cudaEvent_t ev_join2 = nullptr, ev_route = nullptr, ev_select = nullptr;
 };
 namespace {
 std::mutex g_side_mu;
@@ -213,12 +213,14 @@ SideSet* acquire_side_set() {
       cudaStreamCreateWithPriority(&s->side2, cudaStreamNonBlocking, prio_hi) != cudaSuccess ||
       cudaEventCreateWithFlags(&s->ev_join2, cudaEventDisableTiming) != cudaSuccess ||
       cudaEventCreateWithFlags(&s->ev_route, cudaEventDisableTiming) != cudaSuccess ||
+      cudaEventCreateWithFlags(&s->ev_select, cudaEventDisableTiming) != cudaSuccess ||
       cudaEventCreateWithFlags(&s->ev_fork, cudaEventDisableTiming) != cudaSuccess ||
       cudaEventCreateWithFlags(&s->ev_join, cudaEventDisableTiming) != cudaSuccess) {
     if (s->ev_fork) cudaEventDestroy(s->ev_fork);
     if (s->ev_join) cudaEventDestroy(s->ev_join);
     if (s->ev_join2) cudaEventDestroy(s->ev_join2);
     if (s->ev_route) cudaEventDestroy(s->ev_route);
+    if (s->ev_select) cudaEventDestroy(s->ev_select);
     if (s->side) cudaStreamDestroy(s->side);
     if (s->side2) cudaStreamDestroy(s->side2);
     delete s;
@@ -238,7 +240,7 @@ struct sparsepr_plan_s {
   cudaStream_t stream;
   SideSet* set = nullptr;
   cudaStream_t side = nullptr, side2 = nullptr;          // aliases of the set's members
-  cudaEvent_t ev_fork = nullptr, ev_join = nullptr, ev_join2 = nullptr, ev_route = nullptr;
+  cudaEvent_t ev_fork = nullptr, ev_join = nullptr, ev_join2 = nullptr, ev_route = nullptr, ev_select = nullptr;
   // the probe selection of the plan call may still run on `side` when the call returns, and the routing on `side2`: the first
   // attend call orders the former (its probe work follows on the same stream and is joined there), every attend call
   // waits for ev_route; statistics, export and the destructor wait for both themselves
@@ -517,7 +519,7 @@ static sparsepr_status_t make_plan(const sparsepr_shape_t* shape, const sparsepr
   p->set = acquire_side_set();
   if (!p->set) { delete p; return SPARSEPR_ERR_CUDA; }
   p->side = p->set->side; p->side2 = p->set->side2;
-  p->ev_fork = p->set->ev_fork; p->ev_join = p->set->ev_join; p->ev_join2 = p->set->ev_join2; p->ev_route = p->set->ev_route;
+  p->ev_fork = p->set->ev_fork; p->ev_join = p->set->ev_join; p->ev_join2 = p->set->ev_join2; p->ev_route = p->set->ev_route; p->ev_select = p->set->ev_select;
   Carver c(workspace);
   carve_plan(c, r, p);
   *out = p;
@@ -536,13 +538,13 @@ unsigned long long capture_of(cudaStream_t st) {
   if (cudaStreamGetCaptureInfo(st, &status, &id) != cudaSuccess) { cudaGetLastError(); return 0; }
   return status == cudaStreamCaptureStatusActive ? id : 0;
 }
-// Work of an attend call on `st` comes after the routes.  A captured wait can only name work of its own capture: an attend call
-// that is captured on a plan made before the capture waits for the plan here, on the host (the replays find it complete), and
-// one outside the capture of its plan is ordered by whoever launches the graph.
-bool wait_for_routes(const sparsepr_plan_s* p, cudaStream_t st) {
+// Work of an attend call comes after the routes.  A captured wait can only name work of its own capture: for an attend call that is captured on a
+// plan made before the capture this waits for the plan, on the host (the replays find it complete), and one outside the capture of its plan is
+// ordered by whoever launches the graph.  named: neither, the streams have to wait for the plan's events.
+bool find_routes(const sparsepr_plan_s* p, cudaStream_t st, bool* named) {
   const unsigned long long cap = capture_of(st);
-  if (cap == p->capture) return cudaStreamWaitEvent(st, p->ev_route, 0) == cudaSuccess;
-  if (p->capture != 0) return true;
+  *named = cap == p->capture;
+  if (*named || p->capture != 0) return true;
   cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;      // the waits below concern no captured stream
   cudaThreadExchangeStreamCaptureMode(&mode);
   const bool ok = cudaEventSynchronize(p->ev_route) == cudaSuccess && (!p->side_pending || cudaStreamSynchronize(p->side) == cudaSuccess);
@@ -642,6 +644,7 @@ static sparsepr_status_t plan_impl(const sparsepr_shape_t* shape, const sparsepr
   if (!beside) cell_scores();
   launch_route_select(p->score, p->nq, p->nk, r.BH, r.Cq, r.Ck, pair_budget(r), r.density >= 1.0f, p->route_ptr,
                       p->route_idx, p->rstate, nullptr, r.G, rs);
+  cudaEventRecord(p->ev_select, rs);
   launch_tiles(p, rs);
   cudaEventRecord(p->ev_route, rs);
   p->side_pending = beside;                     // not joined here: neither is needed before the attend call
@@ -711,6 +714,7 @@ sparsepr_status_t sparsepr_plan_import(const sparsepr_shape_t* shape, const spar
   k_sizes_from_off<<<dim3((r.Cq + 255) / 256, r.BH), 256, 0, st>>>(p->q_off, r.Cq, p->nq);
   launch_count_pairs(p->q_off, p->kv_off, p->route_ptr, p->route_idx, r.BH, r.Cq, r.Ck, p->rstate, r.G, st);
   launch_tiles(p, st);
+  cudaEventRecord(p->ev_select, st);
   cudaEventRecord(p->ev_route, st);
   if (!launch_ok() || cudaStreamSynchronize(st) != cudaSuccess) { delete p; return SPARSEPR_ERR_CUDA; }
   *out = p;
@@ -738,9 +742,21 @@ static sparsepr_status_t attend_impl(const sparsepr_plan_t* p, const void* Q, co
   launch_gather_rows(r.dtype, Q, r.qs, r.BH, r.H, p->q_perm, r.N, r.d, w.Qg, st);
   launch_gather_rows(r.dtype, K, r.ks, r.BHkv, r.Hkv, p->kv_perm, r.N, r.d, w.Kg, st);
   launch_gather_rows(r.dtype, V, r.vs, r.BHkv, r.Hkv, p->kv_perm, r.N, r.d, w.Vg, st);
-  if (!wait_for_routes(p, st)) return SPARSEPR_ERR_CUDA;
+  // The probe rows and the fit depend only on the gathered K, V and the plan.  The correction is a separate pass, so
+  // they run on the plan's second stream beside the block-sparse kernel, from the end of the selection on (the lists of tiles are made
+  // meanwhile); a profiled call keeps everything on one stream so that stage times add up.
+  const bool fitted = r.mode == 0 && r.M > 0, overlap = fitted && prof == nullptr;
+  bool named = false;
+  if (!find_routes(p, st, &named)) return SPARSEPR_ERR_CUDA;
+  if (overlap) {
+    fork_side(p, st);
+    cudaStreamWaitEvent(p->side2, p->ev_fork, 0);
+  }
+  if (named) {
+    cudaStreamWaitEvent(st, p->ev_route, 0);
+    if (overlap) { cudaStreamWaitEvent(p->side, p->ev_select, 0); cudaStreamWaitEvent(p->side2, p->ev_route, 0); }
+  }
   tm.mark(SPARSEPR_STAGE_GATHER);
-  const bool fitted = r.mode == 0 && r.M > 0;
   AttnArgs aa{};
   aa.dtype = r.dtype; aa.BH = r.BH; aa.H = r.H; aa.N = r.N; aa.d = r.d; aa.scale = r.scale;
   aa.Q = w.Qg; aa.K = w.Kg; aa.V = w.Vg;
@@ -751,14 +767,10 @@ static sparsepr_status_t attend_impl(const sparsepr_plan_t* p, const void* Q, co
   aa.err = p->err;
   const bool tensor = attention_tc_supported(aa);
   if (r.dtype == SPARSEPR_BF16 && !tensor) return SPARSEPR_ERR_CUDA;          // no tensor maps: nothing else serves bf16
-  // The probe rows and the fit depend only on the gathered K, V and the plan.  The correction is a separate pass, so
-  // they run on the plan's second stream beside the block-sparse kernel; a profiled call keeps everything on one
-  // stream so that stage times add up.
-  const bool overlap = fitted && prof == nullptr;
   if (p->side_pending && !overlap) { join_side(p, st); p->side_pending = false; }   // the plan call's probe selection, still on the second stream
   if (fitted) {
     cudaStream_t fs = st;
-    if (overlap) { fork_side(p, st); fs = p->side; }
+    if (overlap) fs = p->side;
     ProbeArgs pa{};
     pa.dtype = r.dtype; pa.BH = r.BH; pa.H = r.H; pa.N = r.N; pa.d = r.d; pa.M = r.M; pa.Ck = r.Ck; pa.Cq = r.Cq;
     pa.n_split = w.n_split; pa.scale = r.scale; pa.Qg = w.Qg; pa.q_inv = p->q_inv; pa.kv_div = r.G;
@@ -783,8 +795,10 @@ static sparsepr_status_t attend_impl(const sparsepr_plan_t* p, const void* Q, co
     if (fitted) aa.O_lo = w.Olo;
     // the packed remainder tiles are few and long, then come the pairs of tiles and the tiles alone, many and short: they share the GPU
     // instead of running one after the other (also in a profiled call: all belong to the ATTENTION stage)
-    if (!overlap) cudaEventRecord(p->ev_fork, st);                // (with the probes' overlap the event is recorded already)
-    cudaStreamWaitEvent(p->side2, p->ev_fork, 0);
+    if (!overlap) {                                               // (with the probes' overlap the streams are forked already)
+      cudaEventRecord(p->ev_fork, st);
+      cudaStreamWaitEvent(p->side2, p->ev_fork, 0);
+    }
     if (!launch_attention_packed(aa, p->rem_pos, p->rem_grp, p->rem_cnt, p->side2)) return SPARSEPR_ERR_CUDA;
     if (attention_tc_pairs(r.BH, r.N, r.d) && !launch_attention_tc(aa, p->side2, true)) return SPARSEPR_ERR_CUDA;
     if (!launch_attention_tc(aa, st)) return SPARSEPR_ERR_CUDA;
