@@ -1,5 +1,6 @@
 // Shared routing (Section 4.3) and query-group-stratified probe selection
 // (Algorithm A.1, Appendix A.2).
+#include <algorithm>
 #include "kernels.cuh"
 
 namespace spr {
@@ -395,6 +396,254 @@ __global__ void __launch_bounds__(kRouteThreads) k_route_select(const float* __r
   }
 }
 
+// The same selection for at most 32 kR query and K/V groups, with the whole score matrix of the head in registers: warp w has the rows w + 16 i, a lane
+// their cells lane + 32 j.  What the kernel above spends on such a head is mostly set-up of its histograms; here the threshold is found by bisection of
+// the bit pattern, a step of which is two additions per cell and one barrier, until a warp can order what is left (two sums of 48 cycles each over a
+// warp make the step, not the cells).  A cell that can be taken has the key bits + 1, any other 0.
+// The kernel above / this one, us, alone: 2 heads of 38 groups 25 / 14, 2 of 64 28 / 16, 8 of 112 51 / 26, 16 of 138 69 / 46.  Beyond 160 groups the
+// matrix no longer fits the registers.
+constexpr int kRouteSmallWarps = 16, kRouteSmallThreads = 32 * kRouteSmallWarps;
+__device__ __forceinline__ i64 warp_sum_cost(i64 v) {           // v >= 0, by 32-bit reductions of 22 bits each
+  const u64 x = (u64)v;
+  const unsigned a = __reduce_add_sync(0xffffffffu, (unsigned)x & 0x3FFFFFu), b = __reduce_add_sync(0xffffffffu, (unsigned)(x >> 22) & 0x3FFFFFu);
+  const unsigned c = __reduce_add_sync(0xffffffffu, (unsigned)(x >> 44));
+  return (i64)((u64)a + ((u64)b << 22) + ((u64)c << 44));
+}
+template <int kR>
+__global__ void __launch_bounds__(kRouteSmallThreads) k_route_select_small(const float* __restrict__ score, const int* __restrict__ nq,
+                                                                      const int* __restrict__ nk, int Cq, int Ck, i64 budget, int select_all,
+                                                                      int* __restrict__ route_ptr, int* __restrict__ route_idx, RouteState* __restrict__ state,
+                                                                      i64* __restrict__ pairs_out, int kv_div) {
+  pdl_wait();                                                   // the scores come from the kernel before
+  pdl_launch_dependents();
+  constexpr unsigned FULL = 0xffffffffu;
+  constexpr int kI = 32 * kR / kRouteSmallWarps, kW = kRouteSmallWarps;     // rows of a warp
+  __shared__ i64 s_cost[2][kW], s_taken;
+  __shared__ uint2 s_pair[2][kW], s_near[32];
+  __shared__ unsigned s_t;
+  __shared__ int s_cnt[32 * kR], scratch[34], s_tie_cnt, s_last_tie, s_near_cnt;
+  __shared__ int s_tie[32];
+  const int bh = blockIdx.x, lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  const unsigned* u = reinterpret_cast<const unsigned*>(score) + (i64)bh * Cq * Ck;
+  const int* nqh = nq + (i64)bh * Cq;
+  const int* nkh = nk + (i64)(bh / kv_div) * Ck;
+  unsigned key[kI][kR];
+  int n_k[kR], n_q[kI], forced[kI];                             // forced: the cell that a row must take, -1: none
+#pragma unroll
+  for (int j = 0; j < kR; ++j) n_k[j] = lane + 32 * j < Ck ? nkh[lane + 32 * j] : 0;
+#pragma unroll
+  for (int i = 0; i < kI; ++i) {
+    const int a = w + kW * i;
+    n_q[i] = a < Cq ? nqh[a] : 0;
+#pragma unroll
+    for (int j = 0; j < kR; ++j) key[i][j] = n_q[i] > 0 && n_k[j] > 0 ? min(u[(i64)a * Ck + lane + 32 * j], 0xFFFFFFFEu) + 1u : 0u;
+  }
+  int turn = 0;
+  const auto block_cost = [&](i64 v) {                          // sum over the CTA, one barrier
+    v = warp_sum_cost(v);
+    i64* buf = s_cost[turn++ & 1];
+    if (lane == 0) buf[w] = v;
+    __syncthreads();
+    return warp_sum_cost(lane < kW ? buf[lane] : 0);
+  };
+  // 1. forced cells: best score, then lowest b
+  i64 cost = 0;
+#pragma unroll
+  for (int i = 0; i < kI; ++i) {
+    unsigned best = 0u;
+#pragma unroll
+    for (int j = 0; j < kR; ++j) best = max(best, key[i][j]);
+    best = __reduce_max_sync(FULL, best);
+    forced[i] = -1;
+    if (best == 0u) continue;                                   // (uniform) no cell in this row
+#pragma unroll
+    for (int j = kR - 1; j >= 0; --j) {
+      const unsigned m = __ballot_sync(FULL, key[i][j] == best);
+      if (m) forced[i] = 32 * j + __ffs(m) - 1;
+    }
+#pragma unroll
+    for (int j = 0; j < kR; ++j)
+      if (lane + 32 * j == forced[i]) { key[i][j] = 0u; cost += (i64)n_q[i] * n_k[j]; }
+  }
+  const i64 rem = budget - block_cost(cost);
+  // 2. the smallest threshold t (keys from t + 1 on) whose cost fits; in 32-bit arithmetic where all cells together cost less than 2^32
+  i64 rows = 0, cols = 0;
+#pragma unroll
+  for (int i = 0; i < kI; ++i) rows += lane == 0 ? n_q[i] : 0;
+#pragma unroll
+  for (int j = 0; j < kR; ++j) cols += n_k[j];
+  cols = warp_sum_cost(cols);
+  const bool narrow = block_cost(rows) * cols < (1ll << 32);
+  // cost and number of the cells with key > t
+  const auto narrow_above = [&](unsigned t, unsigned& n) {
+    unsigned c = 0u, k = 0u;
+#pragma unroll
+    for (int i = 0; i < kI; ++i) {
+      if (n_q[i] == 0) continue;                                // (uniform)
+      unsigned keys = 0u;
+#pragma unroll
+      for (int j = 0; j < kR; ++j) {
+        const bool in = key[i][j] > t;
+        keys += in ? (unsigned)n_k[j] : 0u;
+        k += in;
+      }
+      c += keys * (unsigned)n_q[i];
+    }
+    c = __reduce_add_sync(FULL, c);
+    k = __reduce_add_sync(FULL, k);
+    uint2* buf = s_pair[turn++ & 1];
+    if (lane == 0) buf[w] = make_uint2(c, k);
+    __syncthreads();
+    const uint2 all = lane < kW ? buf[lane] : make_uint2(0u, 0u);
+    n = __reduce_add_sync(FULL, all.y);
+    return (i64)__reduce_add_sync(FULL, all.x);
+  };
+  const auto cost_from = [&](unsigned t) {                      // of the cells with key > t
+    i64 c = 0;
+#pragma unroll
+    for (int i = 0; i < kI; ++i) {
+      if (n_q[i] == 0) continue;                                // (uniform)
+      int keys = 0;
+#pragma unroll
+      for (int j = 0; j < kR; ++j) keys += key[i][j] > t ? n_k[j] : 0;
+      c += (i64)keys * n_q[i];
+    }
+    return block_cost(c);
+  };
+  u64 tstar = select_all ? 0ull : 1ull << 32;
+  i64 taken = 0;
+  if (!select_all && rem >= 0) {
+    unsigned lo = 0u, hi = 0xFFFFFFFFu;                         // the answer lies in [lo, hi]; no key exceeds hi
+    if (narrow) {
+      // bisection until at most 32 keys are left between, which one warp orders
+      unsigned n_lo, n_hi = 0u, n;                              // keys >= lo, > hi
+      const i64 all = narrow_above(0u, n_lo);
+      if (all <= rem) { hi = 0u; taken = all; } else lo = 1u;
+      while (lo < hi && n_lo - n_hi > 32u) {
+        const unsigned mid = lo + ((hi - lo) >> 1);
+        const i64 c = narrow_above(mid, n);
+        if (c <= rem) { hi = mid; taken = c; n_hi = n; } else { lo = mid + 1u; n_lo = n; }
+      }
+      if (lo < hi) {                                            // (uniform)
+        if (threadIdx.x == 0) s_near_cnt = 0;
+        __syncthreads();
+#pragma unroll
+        for (int i = 0; i < kI; ++i)
+#pragma unroll
+          for (int j = 0; j < kR; ++j)
+            if (key[i][j] >= lo && key[i][j] <= hi) s_near[atomicAdd(&s_near_cnt, 1)] = make_uint2(key[i][j], (unsigned)n_q[i] * (unsigned)n_k[j]);
+        __syncthreads();
+        if (w == 0) {
+          // cost above a threshold t: lane 0 also tries t = lo, the others their keys
+          const int m = s_near_cnt;
+          const uint2 e = lane < m ? s_near[lane] : make_uint2(0u, 0u);
+          i64 above = taken, above_lo = taken;
+          for (int l = 0; l < m; ++l) {
+            const unsigned ok = __shfl_sync(FULL, e.x, l), oc = __shfl_sync(FULL, e.y, l);
+            if (ok > e.x) above += oc;
+            if (ok > lo) above_lo += oc;
+          }
+          const unsigned best = above_lo <= rem ? lo : __reduce_min_sync(FULL, lane < m && above <= rem ? e.x : 0xFFFFFFFFu);
+          if (above_lo <= rem) { if (lane == 0) { s_t = lo; s_taken = above_lo; } }
+          else if (lane < m && e.x == best) { s_t = best; s_taken = above; }
+        }
+        __syncthreads();
+        lo = s_t; taken = s_taken;
+      }
+    } else {
+      while (lo < hi) {
+        const unsigned mid = lo + ((hi - lo) >> 1);
+        const i64 c = cost_from(mid);
+        if (c <= rem) { hi = mid; taken = c; } else lo = mid + 1u;
+      }
+    }
+    tstar = lo;
+  }
+  // the cells with bits = tstar - 1, in (a, b) order, as far as they fit
+  if (threadIdx.x == 0) { s_tie_cnt = 0; s_last_tie = -1; }
+  __syncthreads();
+  const bool tie_tier = !select_all && rem >= 0 && tstar > 0;
+  const unsigned tie_key = tie_tier ? (unsigned)tstar : 0u;     // (key of bits tstar - 1; no cell has it where there is no tier: 0 is tested apart)
+  if (tie_tier) {
+#pragma unroll
+    for (int i = 0; i < kI; ++i)
+#pragma unroll
+      for (int j = 0; j < kR; ++j)
+        if (key[i][j] == tie_key) { const int at = atomicAdd(&s_tie_cnt, 1); if (at < 32) s_tie[at] = (w + kW * i) * Ck + lane + 32 * j; }
+    __syncthreads();
+    if (s_tie_cnt <= 32) {
+      if (w == 0) {
+        const int n = s_tie_cnt, idx = lane < n ? s_tie[lane] : 0x7fffffff;
+        const i64 mine = lane < n ? (i64)nqh[idx / Ck] * nkh[idx % Ck] : 0;
+        i64 cum = taken;                                        // cost of the tier's cells up to and including this one
+        for (int l = 0; l < n; ++l) {
+          const int ol = __shfl_sync(FULL, idx, l);
+          const i64 cl = __shfl_sync(FULL, mine, l);
+          if (ol <= idx) cum += cl;
+        }
+        const int last = __reduce_max_sync(FULL, lane < n && cum <= rem ? idx : -1);       // monotone along the order: costs are positive
+        if (lane == 0) s_last_tie = last;
+      }
+    } else {
+      // many equal scores: the largest place up to which they fit, by bisection
+      int lo = -1, hi = Cq * Ck - 1;
+      while (lo < hi) {
+        const int mid = lo + ((hi - lo + 1) >> 1);
+        i64 c = 0;
+#pragma unroll
+        for (int i = 0; i < kI; ++i)
+#pragma unroll
+          for (int j = 0; j < kR; ++j) c += key[i][j] == tie_key && (w + kW * i) * Ck + lane + 32 * j <= mid ? (i64)n_q[i] * n_k[j] : 0;
+        if (taken + block_cost(c) <= rem) lo = mid; else hi = mid - 1;
+      }
+      if (threadIdx.x == 0) s_last_tie = lo;
+    }
+    __syncthreads();
+  }
+  const int last_tie = s_last_tie;
+  const auto selected = [&](int i, int j) {
+    const unsigned k = key[i][j];
+    return lane + 32 * j == forced[i] || (k != 0u && ((u64)k > tstar || (tie_tier && k == tie_key && (w + kW * i) * Ck + lane + 32 * j <= last_tie)));
+  };
+  // 3. counts, offsets, lists
+  cost = 0;
+#pragma unroll
+  for (int i = 0; i < kI; ++i) {
+    const int a = w + kW * i;
+    int n = 0, keys = 0;
+#pragma unroll
+    for (int j = 0; j < kR; ++j) {
+      const bool s = selected(i, j);
+      n += __popc(__ballot_sync(FULL, s));
+      keys += s ? n_k[j] : 0;
+    }
+    cost += (i64)keys * n_q[i];
+    if (lane == 0 && a < Cq) s_cnt[a] = n;
+  }
+  const i64 pairs = block_cost(cost);
+  const int total = block_exclusive_scan(s_cnt, Cq, scratch);
+  int* rp = route_ptr + (i64)bh * (Cq + 1);
+  int* ri = route_idx + (i64)bh * Cq * Ck;
+  for (int a = threadIdx.x; a < Cq; a += kRouteSmallThreads) rp[a] = s_cnt[a];
+  if (threadIdx.x == 0) {
+    rp[Cq] = total;
+    if (state) { state[bh].pairs = pairs; state[bh].cells = total; }
+    if (pairs_out) pairs_out[bh] = pairs;
+  }
+#pragma unroll
+  for (int i = 0; i < kI; ++i) {
+    if (w + kW * i >= Cq) break;                                // (uniform)
+    int pos = s_cnt[w + kW * i];
+#pragma unroll
+    for (int j = 0; j < kR; ++j) {
+      const bool s = selected(i, j);
+      const unsigned m = __ballot_sync(FULL, s);
+      if (s) ri[pos + __popc(m & ((1u << lane) - 1u))] = lane + 32 * j;
+      pos += __popc(m);
+    }
+  }
+}
+
 static size_t route_smem(int Cq, int Ck) {      // forced, cnt, nqs [Cq], nks [Ck] ints, then a warp's 256 int64 cost and int32 key counts
   return (size_t)(3 * Cq + Ck + ((Cq + Ck) & 1)) * sizeof(int) + (size_t)kRouteWarps * 256 * (sizeof(long long) + sizeof(int));
 }
@@ -424,8 +673,17 @@ void launch_count_pairs(const int* q_off, const int* kv_off, const int* route_pt
 void launch_route_select(const float* score, const int* nq, const int* nk, int BH, int Cq, int Ck, i64 budget,
                          int select_all, int* route_ptr, int* route_idx, RouteState* state, i64* pairs_out,
                          int kv_div, cudaStream_t st) {
+  const int groups = std::max(Cq, Ck), div = kv_div < 1 ? 1 : kv_div;
+  if (groups <= 128) {
+    launch_pdl(k_route_select_small<4>, dim3(BH), dim3(kRouteSmallThreads), 0, st, score, nq, nk, Cq, Ck, budget, select_all, route_ptr, route_idx, state, pairs_out, div);
+    return;
+  }
+  if (groups <= 160) {
+    launch_pdl(k_route_select_small<5>, dim3(BH), dim3(kRouteSmallThreads), 0, st, score, nq, nk, Cq, Ck, budget, select_all, route_ptr, route_idx, state, pairs_out, div);
+    return;
+  }
   launch_pdl(k_route_select, dim3(BH), dim3(kRouteThreads), route_smem(Cq, Ck), st, score, nq, nk, Cq, Ck, budget, select_all, route_ptr, route_idx,
-             state, pairs_out, kv_div < 1 ? 1 : kv_div);
+             state, pairs_out, div);
 }
 
 // =============================================================================
