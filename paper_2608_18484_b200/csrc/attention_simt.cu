@@ -12,86 +12,6 @@ constexpr int BM = 64;     // query rows per CTA
 constexpr int BN = 64;     // keys per tile
 constexpr float kLog2e = 1.4426950408889634f;
 
-template <int D> struct SimtSmem {
-  static constexpr int q = D * BM, k = D * BN, v = BN * D, p = BN * BM;
-};
-
-// Transposed tile load: dst[(c)*64 + r] = src_row_r[c]; rows given by a row-pointer functor.
-template <typename T, int D, typename RowPtr>
-__device__ __forceinline__ void load_tile_transposed(float* dst, RowPtr rowptr) {
-  const int r = threadIdx.x & 63;
-  const T* p = rowptr(r);
-#pragma unroll
-  for (int pass = 0; pass < D / 32; ++pass) {
-    const int c = ((threadIdx.x >> 6) + 4 * pass) * 8;
-    float v[8];
-    if (p) load8(p + c, v);
-    else {
-#pragma unroll
-      for (int k = 0; k < 8; ++k) v[k] = 0.f;
-    }
-#pragma unroll
-    for (int k = 0; k < 8; ++k) dst[(c + k) * 64 + r] = v[k];
-  }
-}
-template <typename T, int D, typename RowPtr>
-__device__ __forceinline__ void load_tile_natural(float* dst, RowPtr rowptr) {
-  // 64 rows x D: thread handles 8 consecutive elements; consecutive threads -> consecutive chunks of a row
-  constexpr int CPR = D / 8;
-#pragma unroll
-  for (int e = threadIdx.x; e < 64 * CPR; e += 256) {
-    const int r = e / CPR, c = (e % CPR) * 8;
-    const T* p = rowptr(r);
-    float v[8];
-    if (p) load8(p + c, v);
-    else {
-#pragma unroll
-      for (int k = 0; k < 8; ++k) v[k] = 0.f;
-    }
-    *reinterpret_cast<float4*>(dst + r * D + c) = make_float4(v[0], v[1], v[2], v[3]);
-    *reinterpret_cast<float4*>(dst + r * D + c + 4) = make_float4(v[4], v[5], v[6], v[7]);
-  }
-}
-
-// S[4][4] = Q_tile (rows ty*4..) . K_tile^T (cols tx*4..)
-template <int D>
-__device__ __forceinline__ void qk_tile(const float* Qs, const float* Ks, int ty, int tx, float (&s)[4][4]) {
-#pragma unroll
-  for (int i = 0; i < 4; ++i)
-#pragma unroll
-    for (int j = 0; j < 4; ++j) s[i][j] = 0.f;
-#pragma unroll 8
-  for (int k = 0; k < D; ++k) {
-    const float4 a = *reinterpret_cast<const float4*>(Qs + k * BM + ty * 4);
-    const float4 b = *reinterpret_cast<const float4*>(Ks + k * BN + tx * 4);
-    const float av[4] = {a.x, a.y, a.z, a.w}, bv[4] = {b.x, b.y, b.z, b.w};
-#pragma unroll
-    for (int i = 0; i < 4; ++i)
-#pragma unroll
-      for (int j = 0; j < 4; ++j) s[i][j] = fmaf(av[i], bv[j], s[i][j]);
-  }
-}
-
-// O[4][D/16] += P^T-tile (Ps[j][rows]) . V_tile
-template <int D>
-__device__ __forceinline__ void pv_tile(const float* Ps, const float* Vs, int ty, int tx, int ncols, float (&o)[4][D / 16]) {
-  constexpr int OC = D / 16;
-  for (int j = 0; j < ncols; ++j) {
-    const float4 p = *reinterpret_cast<const float4*>(Ps + j * BM + ty * 4);
-    const float pv[4] = {p.x, p.y, p.z, p.w};
-    float vv[OC];
-#pragma unroll
-    for (int c = 0; c < OC; c += 4) {
-      const float4 v = *reinterpret_cast<const float4*>(Vs + j * D + tx * OC + c);
-      vv[c] = v.x; vv[c + 1] = v.y; vv[c + 2] = v.z; vv[c + 3] = v.w;
-    }
-#pragma unroll
-    for (int i = 0; i < 4; ++i)
-#pragma unroll
-      for (int c = 0; c < OC; ++c) o[i][c] = fmaf(pv[i], vv[c], o[i][c]);
-  }
-}
-
 __device__ __forceinline__ float row16_max(float v) {
 #pragma unroll
   for (int o = 8; o > 0; o >>= 1) v = fmaxf(v, __shfl_xor_sync(0xffffffffu, v, o));
@@ -592,123 +512,238 @@ void launch_attention_f32(const AttnArgs& a, float* part, int* counter, cudaStre
 // omitted ones (Z_U, N_U).  Then O_sp = N_S/Z_S and O_dense = (N_S+N_U)/(Z_S+Z_U).
 // The key range is split across CTAs; partial states are merged afterwards.
 // partial layout: [BH][n_split][M][2][D+2] = (m, l, N[D]) for the S and the U state.
+//
+// Bound by the FMA pipe on large calls, by the chain of a CTA's few key tiles on small ones.  A key belongs to one of a row's
+// two states, and keys are group-major, so both states change hands only where a K/V group ends: a thread multiplies into the
+// row's current state and swaps it with the other one there, which is one product with V per key instead of two.  32 rows per
+// CTA (both states of four rows and the scores fit a thread's registers), packed 4 x 4 score blocks; K of the next tile
+// arrives under the product with V, V under the scores.  With one block of 4 x 4 single multiply-adds per state, 64 rows per CTA
+// and loads that were waited for: 2 heads of 4096 tokens, d = 64, 32 probes 60 us, now 15 us; 8 heads of 7161 tokens, d = 128,
+// 64 probes (beside the attention) 200 us, now 81 us.
 // =============================================================================
-template <typename T, int D>
-__global__ void __launch_bounds__(256) k_probe_rows(ProbeArgs a) {
+constexpr int kProbeRows = 32;
+template <int D> struct ProbeSmem {
+  static constexpr int ld = D + 4, ldp = kProbeRows + 4;
+  static constexpr int q = kProbeRows * ld, k = BN * ld, v = BN * D, p = BN * ldp;
+  static size_t bytes(int Ck) {
+    return (size_t)(q + k + v + p) * sizeof(float) + (size_t)(kProbeRows * ((Ck + 31) / 32) + 2 * BN + Ck) * sizeof(int);
+  }
+};
+template <int D>
+__global__ void __launch_bounds__(kFThreads, 2) k_probe_rows(ProbeArgs a) {
   extern __shared__ __align__(16) float smem[];
-  float* Qs = smem;
-  float* Ks = Qs + SimtSmem<D>::q;
-  float* Vs = Ks + SimtSmem<D>::k;
-  float* Ps = Vs + SimtSmem<D>::v;                           // retained weights
-  float* Pu = Ps + SimtSmem<D>::p;                           // omitted weights
-  unsigned* bitmap = reinterpret_cast<unsigned*>(Pu + SimtSmem<D>::p);   // [64][words]
+  using S = ProbeSmem<D>;
+  float* Qs = smem;                                          // [32][D + 4]
+  float* Ks = Qs + S::q;                                     // [64][D + 4]
+  float* Vs = Ks + S::k;                                     // [64][D]
+  float* Ps = Vs + S::v;                                     // [64 keys][32 rows + 4]
   const int words = (a.Ck + 31) / 32;
-  int* kgrp = reinterpret_cast<int*>(bitmap + 64 * words);   // [64] K/V group of every tile key
-  constexpr int OC = D / 16;
+  unsigned* bitmap = reinterpret_cast<unsigned*>(Ps + S::p); // [32][words] routes of every row's group
+  int* kgrp = reinterpret_cast<int*>(bitmap + kProbeRows * words);   // [2][64] K/V group of every key of this / the next tile
+  int* koff = kgrp + 2 * BN;                                 // [Ck]
+  constexpr int OP = D / 32, CPR = D / 4, R = 4;             // output column pairs, 16-byte chunks of a row, rows per thread
   const int bh = blockIdx.z;
-  const int m0 = blockIdx.y * BM, nrows = min(BM, a.M - m0);
+  const int m0 = blockIdx.y * kProbeRows, nrows = min(kProbeRows, a.M - m0);
   const int tid = threadIdx.x, ty = tid >> 4, tx = tid & 15;
   const int* pidx = a.probe_idx + (i64)bh * a.M + m0;
-  const T* Qb = (const T*)a.Qg + (i64)bh * a.N * D;
+  const float* Qb = (const float*)a.Qg + (i64)bh * a.N * D;
   const int* inv = a.q_inv + (i64)bh * a.N;
-  const T* Kb = (const T*)a.Kg + (i64)bh * a.N * D;
-  const T* Vb = (const T*)a.Vg + (i64)bh * a.N * D;
+  const float* Kb = (const float*)a.Kg + (i64)bh * a.N * D;
+  const float* Vb = (const float*)a.Vg + (i64)bh * a.N * D;
   const int* kvoff = a.kv_off + (i64)bh * (a.Ck + 1);
-
-  for (int e = tid; e < 64 * words; e += 256) bitmap[e] = 0u;
-  __syncthreads();
-  for (int r = tid >> 2; r < nrows; r += 64) {               // 4 threads per probe row
-    const int pi = pidx[r];
-    if (pi < 0) continue;
-    const int g = a.q_assign[(i64)bh * a.N + pi];
-    const int* rp = a.route_ptr + (i64)bh * (a.Cq + 1);
-    const int* ri = a.route_idx + (i64)bh * a.Cq * a.Ck;
-    for (int t = rp[g] + (tid & 3); t < rp[g + 1]; t += 4) atomicOr(&bitmap[r * words + (ri[t] >> 5)], 1u << (ri[t] & 31));
-  }
-  load_tile_transposed<T, D>(Qs, [&](int r) { return (r < nrows && pidx[r] >= 0) ? Qb + (i64)inv[pidx[r]] * D : (const T*)nullptr; });
 
   // key positions of this split, in whole tiles
   const int tiles = (a.N + BN - 1) / BN;
   const int per = (tiles + a.n_split - 1) / a.n_split;
   const int k_begin = min(a.N, (int)blockIdx.x * per * BN), k_end = min(a.N, ((int)blockIdx.x + 1) * per * BN);
 
-  float oS[4][OC], oU[4][OC], mS[4], lS[4], mU[4], lU[4];
+  auto load_keys = [&](const float* base, float* dst, int ld, int t0) {   // one commit group, empty past the last tile
+    if (t0 < k_end) {
+#pragma unroll 8
+      for (int e = tid; e < BN * CPR; e += kFThreads) {
+        const int r = e / CPR, c = (e % CPR) * 4;
+        const bool on = t0 + r < k_end;
+        cp16(dst + r * ld + c, base + (i64)(on ? t0 + r : 0) * D + c, on);
+      }
+    }
+    asm volatile("cp.async.commit_group;" ::: "memory");
+  };
+  auto find_groups = [&](int t0, int* dst) {
+    if (tid < BN) {
+      int lo = 0, hi = t0 + tid < k_end ? a.Ck - 1 : 0;      // last group with koff[g] <= position
+      while (lo < hi) { const int mid = (lo + hi + 1) >> 1; if (koff[mid] <= t0 + tid) lo = mid; else hi = mid - 1; }
+      dst[tid] = lo;
+    }
+  };
+#pragma unroll 4
+  for (int e = tid; e < kProbeRows * CPR; e += kFThreads) {
+    const int r = e / CPR, c = (e % CPR) * 4;
+    const int pi = r < nrows ? pidx[r] : -1;
+    cp16(Qs + r * S::ld + c, Qb + (i64)(pi >= 0 ? inv[pi] : 0) * D + c, pi >= 0);
+  }
+  load_keys(Kb, Ks, S::ld, k_begin);                         // with Q
+  load_keys(Vb, Vs, D, k_begin);
+  for (int e = tid; e < kProbeRows * words; e += kFThreads) bitmap[e] = 0u;
+  for (int e = tid; e < a.Ck; e += kFThreads) koff[e] = kvoff[e];
+  __syncthreads();
+  if ((tid >> 2) < nrows) {                                  // 4 threads per probe row
+    const int r = tid >> 2, pi = pidx[r];
+    if (pi >= 0) {
+      const int g = a.q_assign[(i64)bh * a.N + pi];
+      const int* rp = a.route_ptr + (i64)bh * (a.Cq + 1);
+      const int* ri = a.route_idx + (i64)bh * a.Cq * a.Ck;
+      for (int t = rp[g] + (tid & 3); t < rp[g + 1]; t += 4) atomicOr(&bitmap[r * words + (ri[t] >> 5)], 1u << (ri[t] & 31));
+    }
+  }
+  find_groups(k_begin, kgrp);
+
+  float2 oc[R][OP], oo[R][OP];                               // current state of every row, the other one
+  float mS[R], lS[R], mU[R], lU[R];
+  unsigned cur = 0;                                          // bit i: the retained state of row i is the current one
 #pragma unroll
-  for (int i = 0; i < 4; ++i) {
+  for (int i = 0; i < R; ++i) {
     mS[i] = mU[i] = -INFINITY; lS[i] = lU[i] = 0.f;
 #pragma unroll
-    for (int c = 0; c < OC; ++c) oS[i][c] = oU[i][c] = 0.f;
+    for (int c = 0; c < OP; ++c) oc[i][c] = oo[i][c] = make_float2(0.f, 0.f);
   }
-  const float sc = a.scale * kLog2e;
-  for (int t0 = k_begin; t0 < k_end; t0 += BN) {
-    const int ncols = min(BN, k_end - t0);
-    __syncthreads();
-    if (tid < BN) {
-      int g = 0;
-      if (tid < ncols) {
-        const int pos = t0 + tid;
-        int lo = 0, hi = a.Ck - 1;                     // last group with kvoff[g] <= pos
-        while (lo < hi) { const int mid = (lo + hi + 1) >> 1; if (kvoff[mid] <= pos) lo = mid; else hi = mid - 1; }
-        g = lo;
+  auto turn = [&](unsigned want) {                           // make the states `want` the current ones
+    const unsigned sw = want ^ cur;
+    cur = want;
+    if (sw == 0) return;
+#pragma unroll
+    for (int i = 0; i < R; ++i)
+#pragma unroll
+      for (int c = 0; c < OP; ++c) {
+        const float2 x = oc[i][c], y = oo[i][c];
+        const bool b = (sw >> i) & 1u;
+        oc[i][c] = b ? y : x; oo[i][c] = b ? x : y;
       }
-      kgrp[tid] = g;
-    }
-    load_tile_transposed<T, D>(Ks, [&](int r) { return r < ncols ? Kb + (i64)(t0 + r) * D : (const T*)nullptr; });
-    load_tile_natural<T, D>(Vs, [&](int r) { return r < ncols ? Vb + (i64)(t0 + r) * D : (const T*)nullptr; });
+  };
+  const unsigned* bm = bitmap + ty * R * words;
+  const float sc = a.scale * kLog2e;
+  int phase = 0;
+  for (int t0 = k_begin; t0 < k_end; t0 += BN, phase ^= 1) {
+    const int ncols = min(BN, k_end - t0);
+    const int* kg = kgrp + phase * BN;
+    asm volatile("cp.async.wait_group 1;" ::: "memory");     // Q and K
     __syncthreads();
-    float s[4][4];
-    qk_tile<D>(Qs, Ks, ty, tx, s);
+    float s[R][4];
+    {
+      float2 acc[R][4];
+#pragma unroll
+      for (int i = 0; i < R; ++i)
+#pragma unroll
+        for (int j = 0; j < 4; ++j) acc[i][j] = make_float2(0.f, 0.f);
+      const float* qp = Qs + ty * R * S::ld;
+      const float* kp = Ks + tx * S::ld;
+#pragma unroll 2
+      for (int k = 0; k < D; k += 4) {
+        float4 kk[4], q[R];
+#pragma unroll
+        for (int j = 0; j < 4; ++j) kk[j] = *reinterpret_cast<const float4*>(kp + 16 * j * S::ld + k);
+#pragma unroll
+        for (int i = 0; i < R; ++i) q[i] = *reinterpret_cast<const float4*>(qp + i * S::ld + k);
+#pragma unroll
+        for (int i = 0; i < R; ++i)
+#pragma unroll
+          for (int j = 0; j < 4; ++j) acc[i][j] = __ffma2_rn(make_float2(q[i].x, q[i].y), make_float2(kk[j].x, kk[j].y), acc[i][j]);
+#pragma unroll
+        for (int i = 0; i < R; ++i)
+#pragma unroll
+          for (int j = 0; j < 4; ++j) acc[i][j] = __ffma2_rn(make_float2(q[i].z, q[i].w), make_float2(kk[j].z, kk[j].w), acc[i][j]);
+      }
+#pragma unroll
+      for (int i = 0; i < R; ++i)
+#pragma unroll
+        for (int j = 0; j < 4; ++j) s[i][j] = tx + 16 * j < ncols ? (acc[i][j].x + acc[i][j].y) * sc : -INFINITY;
+    }
+    __syncthreads();                                         // K is consumed
+    load_keys(Kb, Ks, S::ld, t0 + BN);
+    if (t0 + BN < k_end) find_groups(t0 + BN, kgrp + (phase ^ 1) * BN);
     int grp[4];
 #pragma unroll
-    for (int j = 0; j < 4; ++j) grp[j] = kgrp[tx * 4 + j];
+    for (int j = 0; j < 4; ++j) grp[j] = kg[tx + 16 * j];
 #pragma unroll
-    for (int i = 0; i < 4; ++i) {
-      const unsigned* bm = bitmap + (ty * 4 + i) * words;
+    for (int i = 0; i < R; ++i) {
       bool ret[4];
       float mxS = -INFINITY, mxU = -INFINITY;
 #pragma unroll
       for (int j = 0; j < 4; ++j) {
-        const bool valid = tx * 4 + j < ncols;
-        ret[j] = (bm[grp[j] >> 5] >> (grp[j] & 31)) & 1u;
-        s[i][j] = valid ? s[i][j] * sc : -INFINITY;
+        ret[j] = (bm[i * words + (grp[j] >> 5)] >> (grp[j] & 31)) & 1u;
         if (ret[j]) mxS = fmaxf(mxS, s[i][j]); else mxU = fmaxf(mxU, s[i][j]);
       }
       mxS = row16_max(mxS); mxU = row16_max(mxU);
       const float nS = fmaxf(mS[i], mxS), nU = fmaxf(mU[i], mxU);
       const float cS = nS == -INFINITY ? 1.f : exp2f(mS[i] - nS), cU = nU == -INFINITY ? 1.f : exp2f(mU[i] - nU);
       mS[i] = nS; mU[i] = nU;
-      float pS[4], pU[4], sS = 0.f, sU = 0.f;
+      float sS = 0.f, sU = 0.f;
 #pragma unroll
       for (int j = 0; j < 4; ++j) {
-        const float e = exp2f(s[i][j] - (ret[j] ? nS : nU));       // -inf logit -> 0
-        const bool live = s[i][j] > -INFINITY;
-        pS[j] = (live && ret[j]) ? e : 0.f;
-        pU[j] = (live && !ret[j]) ? e : 0.f;
-        sS += pS[j]; sU += pU[j];
+        const float e = s[i][j] > -INFINITY ? exp2f(s[i][j] - (ret[j] ? nS : nU)) : 0.f;   // no weight past the last key
+        s[i][j] = e;
+        sS += ret[j] ? e : 0.f; sU += ret[j] ? 0.f : e;
       }
       lS[i] = lS[i] * cS + sS; lU[i] = lU[i] * cU + sU;
+      const bool is_s = (cur >> i) & 1u;
+      const float cc = is_s ? cS : cU, co = is_s ? cU : cS;
+      if (cc != 1.f || co != 1.f) {
 #pragma unroll
-      for (int c = 0; c < OC; ++c) { oS[i][c] *= cS; oU[i][c] *= cU; }
-#pragma unroll
-      for (int j = 0; j < 4; ++j) { Ps[(tx * 4 + j) * BM + ty * 4 + i] = pS[j]; Pu[(tx * 4 + j) * BM + ty * 4 + i] = pU[j]; }
+        for (int c = 0; c < OP; ++c) { oc[i][c].x *= cc; oc[i][c].y *= cc; oo[i][c].x *= co; oo[i][c].y *= co; }
+      }
     }
-    __syncthreads();
-    pv_tile<D>(Ps, Vs, ty, tx, ncols, oS);
-    pv_tile<D>(Pu, Vs, ty, tx, ncols, oU);
-  }
 #pragma unroll
-  for (int i = 0; i < 4; ++i) {
-    const int r = ty * 4 + i;
+    for (int j = 0; j < 4; ++j)
+      *reinterpret_cast<float4*>(Ps + (tx + 16 * j) * S::ldp + ty * R) = make_float4(s[0][j], s[1][j], s[2][j], s[3][j]);
+    asm volatile("cp.async.wait_group 1;" ::: "memory");     // V
+    __syncthreads();
+    for (int j0 = 0; j0 < ncols;) {                          // the keys of one K/V group after the other
+      const int g = kg[j0];
+      const int j1 = g + 1 < a.Ck ? min(ncols, koff[g + 1] - t0) : ncols;
+      unsigned want = 0;
+#pragma unroll
+      for (int i = 0; i < R; ++i) want |= ((bm[i * words + (g >> 5)] >> (g & 31)) & 1u) << i;
+      turn(want);
+#pragma unroll 4
+      for (int j = j0; j < j1; ++j) {
+        const float4 p = *reinterpret_cast<const float4*>(Ps + j * S::ldp + ty * R);
+        const float pv[R] = {p.x, p.y, p.z, p.w};
+#pragma unroll
+        for (int c = 0; c < OP / 2; ++c) {
+          const float4 v = *reinterpret_cast<const float4*>(Vs + j * D + 64 * c + 4 * tx);
+#pragma unroll
+          for (int i = 0; i < R; ++i) {
+            const float2 pp = make_float2(pv[i], pv[i]);
+            oc[i][2 * c] = __ffma2_rn(pp, make_float2(v.x, v.y), oc[i][2 * c]);
+            oc[i][2 * c + 1] = __ffma2_rn(pp, make_float2(v.z, v.w), oc[i][2 * c + 1]);
+          }
+        }
+      }
+      j0 = j1;
+    }
+    __syncthreads();                                         // V and the probabilities are consumed
+    load_keys(Vb, Vs, D, t0 + BN);
+  }
+  asm volatile("cp.async.wait_all;" ::: "memory");         // (a slice without keys has only fetched Q)
+  turn((1u << R) - 1);
+#pragma unroll
+  for (int i = 0; i < R; ++i) {
+    const int r = ty * R + i;
     const float tS = row16_sum(lS[i]), tU = row16_sum(lU[i]);
     if (r >= nrows) continue;
     float* out = a.partial + ((((i64)bh * a.n_split + blockIdx.x) * a.M + m0 + r) * 2) * (D + 2);
     if (tx == 0) { out[0] = mS[i]; out[1] = tS; out[D + 2] = mU[i]; out[D + 3] = tU; }
 #pragma unroll
-    for (int c = 0; c < OC; ++c) { out[2 + tx * OC + c] = oS[i][c]; out[D + 4 + tx * OC + c] = oU[i][c]; }
+    for (int c = 0; c < OP; ++c) {                           // (rows of the partial states are 8-byte aligned)
+      const int col = 64 * (c >> 1) + 4 * tx + 2 * (c & 1);
+      *reinterpret_cast<float2*>(out + 2 + col) = oc[i][c];
+      *reinterpret_cast<float2*>(out + D + 4 + col) = oo[i][c];
+    }
   }
 }
 
-// merge the split states; one warp per probe row
+// merge the split states; one warp per probe row.  Bound by latency: the maxima are found by the lanes side by side, and the
+// numerators of four slices are on their way at a time (on the two calls above 13 -> 9 us with 16 -> 32 slices, and 56 -> 31 us;
+// eight at a time cost the calls of few slices more than they gained: 20 -> 26 us at 4 slices of 32 heads).
 template <int D>
 __global__ void __launch_bounds__(256) k_probe_merge(const float* __restrict__ partial, int n_split, int M,
                                                      float* __restrict__ X, float* __restrict__ Dn) {
@@ -717,28 +752,46 @@ __global__ void __launch_bounds__(256) k_probe_merge(const float* __restrict__ p
   if (r >= M) return;
   const int lane = threadIdx.x & 31;
   constexpr int PL = D / 32;
+  const float* p0 = partial + ((i64)bh * n_split * M + r) * 2 * (D + 2);   // of split 0
+  const i64 step = (i64)M * 2 * (D + 2);
   float mS = -INFINITY, mU = -INFINITY;
-  for (int s = 0; s < n_split; ++s) {
-    const float* p = partial + ((((i64)bh * n_split + s) * M + r) * 2) * (D + 2);
-    mS = fmaxf(mS, p[0]); mU = fmaxf(mU, p[D + 2]);
-  }
+  for (int s = lane; s < n_split; s += 32) { mS = fmaxf(mS, p0[s * step]); mU = fmaxf(mU, p0[s * step + D + 2]); }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) { mS = fmaxf(mS, __shfl_xor_sync(0xffffffffu, mS, o)); mU = fmaxf(mU, __shfl_xor_sync(0xffffffffu, mU, o)); }
   float lS = 0.f, lU = 0.f, nS[PL], nU[PL];
 #pragma unroll
   for (int c = 0; c < PL; ++c) nS[c] = nU[c] = 0.f;
-  for (int s = 0; s < n_split; ++s) {
-    const float* p = partial + ((((i64)bh * n_split + s) * M + r) * 2) * (D + 2);
-    const float wS = p[0] == -INFINITY ? 0.f : exp2f(p[0] - mS), wU = p[D + 2] == -INFINITY ? 0.f : exp2f(p[D + 2] - mU);
-    // a state without any key (empty key slice, or no retained / omitted key inside it) has weight 0 and its
-    // numerator may never have been written: it is skipped, not multiplied by 0
-    if (wS != 0.f) {
-      lS += p[1] * wS;
+  // a state without any key (empty key slice, or no retained / omitted key inside it) has weight 0 and its numerator may never
+  // have been written: it is fetched with the others (kAhead splits at a time) but left out, not multiplied by 0
+  constexpr int kAhead = 4;
+  for (int s0 = 0; s0 < n_split; s0 += kAhead) {
+    float xS[kAhead][PL], xU[kAhead][PL];
 #pragma unroll
-      for (int c = 0; c < PL; ++c) nS[c] += p[2 + lane + 32 * c] * wS;
+    for (int k = 0; k < kAhead; ++k) {
+      const float* p = p0 + min(s0 + k, n_split - 1) * step;
+#pragma unroll
+      for (int c = 0; c < PL; ++c) { xS[k][c] = p[2 + lane + 32 * c]; xU[k][c] = p[D + 4 + lane + 32 * c]; }
     }
-    if (wU != 0.f) {
-      lU += p[D + 3] * wU;
+    float w = 0.f, z = 0.f;                                  // lane k, 16 + k: weight and sum of state S, U of split s0 + k
+    if ((lane & 15) < kAhead && s0 + (lane & 15) < n_split) {
+      const float* p = p0 + (s0 + (lane & 15)) * step + (lane < 16 ? 0 : D + 2);
+      w = p[0] == -INFINITY ? 0.f : exp2f(p[0] - (lane < 16 ? mS : mU));
+      z = p[1];
+    }
 #pragma unroll
-      for (int c = 0; c < PL; ++c) nU[c] += p[D + 4 + lane + 32 * c] * wU;
+    for (int k = 0; k < kAhead; ++k) {
+      const float wS = __shfl_sync(0xffffffffu, w, k), wU = __shfl_sync(0xffffffffu, w, 16 + k);
+      const float zS = __shfl_sync(0xffffffffu, z, k), zU = __shfl_sync(0xffffffffu, z, 16 + k);
+      if (wS != 0.f) {
+        lS = fmaf(zS, wS, lS);
+#pragma unroll
+        for (int c = 0; c < PL; ++c) nS[c] = fmaf(xS[k][c], wS, nS[c]);
+      }
+      if (wU != 0.f) {
+        lU = fmaf(zU, wU, lU);
+#pragma unroll
+        for (int c = 0; c < PL; ++c) nU[c] = fmaf(xU[k][c], wU, nU[c]);
+      }
     }
   }
   const float mD = fmaxf(mS, mU);
@@ -751,16 +804,12 @@ __global__ void __launch_bounds__(256) k_probe_merge(const float* __restrict__ p
   }
 }
 
-template <int D> static size_t probe_smem_bytes(int Ck) {
-  return (size_t)(SimtSmem<D>::q + SimtSmem<D>::k + SimtSmem<D>::v + 2 * SimtSmem<D>::p) * sizeof(float) +
-         (size_t)64 * ((Ck + 31) / 32) * sizeof(unsigned) + 64 * sizeof(int);
-}
 size_t probe_partial_floats(int BH, int n_split, int M, int d) { return (size_t)BH * n_split * M * 2 * (d + 2); }
 
-template <typename T, int D>
+template <int D>
 static void probe_dispatch(const ProbeArgs& a, cudaStream_t st) {
-  dim3 grid(a.n_split, (a.M + BM - 1) / BM, a.BH);
-  k_probe_rows<T, D><<<grid, 256, probe_smem_bytes<D>(a.Ck), st>>>(a);
+  dim3 grid(a.n_split, (a.M + kProbeRows - 1) / kProbeRows, a.BH);
+  k_probe_rows<D><<<grid, kFThreads, ProbeSmem<D>::bytes(a.Ck), st>>>(a);
   dim3 g2((a.M + 7) / 8, a.BH);
   k_probe_merge<D><<<g2, 256, 0, st>>>(a.partial, a.n_split, a.M, a.X, a.Dn);
 }
@@ -770,7 +819,7 @@ void launch_probe_merge(const ProbeArgs& a, cudaStream_t st) {
   else k_probe_merge<64><<<g2, 256, 0, st>>>(a.partial, a.n_split, a.M, a.X, a.Dn);
 }
 void launch_probe_rows(const ProbeArgs& a, cudaStream_t st) {
-  if (a.d == 128) probe_dispatch<float, 128>(a, st); else probe_dispatch<float, 64>(a, st);
+  if (a.d == 128) probe_dispatch<128>(a, st); else probe_dispatch<64>(a, st);
 }
 
 // O[b,h,probe_idx[m],:] = O_dense of the probe (Eq. 10, first case)
@@ -798,8 +847,8 @@ cudaError_t init_attention_simt() {
   SPR_ATTR(k_attention_f32_dense<128>, F32Smem<128>::bytes);
   SPR_ATTR(k_attention_f32_sparse<64>, F32Smem<64>::bytes);
   SPR_ATTR(k_attention_f32_dense<64>, F32Smem<64>::bytes);
-  SPR_ATTR((k_probe_rows<float, 128>), probe_smem_bytes<128>(kMaxGroups));
-  SPR_ATTR((k_probe_rows<float, 64>), probe_smem_bytes<64>(kMaxGroups));
+  SPR_ATTR(k_probe_rows<128>, ProbeSmem<128>::bytes(kMaxGroups));
+  SPR_ATTR(k_probe_rows<64>, ProbeSmem<64>::bytes(kMaxGroups));
 #undef SPR_ATTR
   return cudaSuccess;
 }
