@@ -161,51 +161,75 @@ void launch_centroid_gram(const float* kappa, const int* n, int BH, int C, int d
 
 // =============================================================================
 // Response projections: phi_K = K F_K (Eq. 6) and phi_Q = RMS-normalised Q F_Q
-// (Eq. 7).  Each thread produces two rows of R outputs; F is staged in shared
+// (Eq. 7).  Each thread produces kRows rows of R outputs; F is staged in shared
 // memory and read by broadcast.  Also tracks max |phi| per head (for the
 // fixed-point centroid sums) and flags non-finite values.
+// Bound by the latency of its loads on small calls and by the FMA pipe on large ones: multiply-adds of two columns to an
+// instruction, and the next eight values of a row are fetched under those of the last eight (24 heads of 16000 rows, d = 128, 64
+// outputs: 261 -> 210 us).
 // =============================================================================
-template <typename T, int D, int R, bool RMS>
+template <typename T, int D, int R, bool RMS, int kRows>
 __global__ void __launch_bounds__(128) k_project(const T* __restrict__ X, i64 sb, i64 sh, i64 sn, int H, int N, int r,
                                                  const float* __restrict__ F, float eps, float* __restrict__ phi,
                                                  int ldphi, unsigned* __restrict__ maxabs_bits, int* err) {
   __shared__ __align__(16) float Fs[D * R];
   const int bh = blockIdx.y, b = bh / H, h = bh % H;
   const float* Fh = F + (i64)bh * D * r;
-  for (int e = threadIdx.x; e < D * R; e += 128) {
+  const T* base = X + b * sb + h * sh;
+  const int row0 = blockIdx.x * (blockDim.x * kRows) + threadIdx.x;
+  const T* p[kRows];
+  float x[kRows][8];
+#pragma unroll
+  for (int u = 0; u < kRows; ++u) {
+    const int row = row0 + u * blockDim.x;
+    p[u] = base + (i64)(row < N ? row : 0) * sn;
+    load8(p[u], x[u]);
+  }
+#pragma unroll 8
+  for (int e = threadIdx.x; e < D * R; e += blockDim.x) {
     const int k = e / R, c = e % R;
     Fs[e] = c < r ? Fh[k * r + c] : 0.f;
   }
   __syncthreads();
-  const T* base = X + b * sb + h * sh;
-  const int row0 = blockIdx.x * 256 + threadIdx.x, row1 = row0 + 128;
-  const bool v0 = row0 < N, v1 = row1 < N;
-  const T* p0 = base + (i64)(v0 ? row0 : 0) * sn;
-  const T* p1 = base + (i64)(v1 ? row1 : 0) * sn;
-  float acc0[R], acc1[R];
+  float2 acc2[kRows][R / 2];
 #pragma unroll
-  for (int c = 0; c < R; ++c) { acc0[c] = 0.f; acc1[c] = 0.f; }
+  for (int u = 0; u < kRows; ++u)
+#pragma unroll
+    for (int c = 0; c < R / 2; ++c) acc2[u][c] = make_float2(0.f, 0.f);
+#pragma unroll 1
   for (int k0 = 0; k0 < D; k0 += 8) {
-    float x0[8], x1[8];
-    load8(p0 + k0, x0);
-    load8(p1 + k0, x1);
+    float nx[kRows][8];
+    const int kn = min(k0 + 8, D - 8);
+#pragma unroll
+    for (int u = 0; u < kRows; ++u) load8(p[u] + kn, nx[u]);
 #pragma unroll
     for (int kk = 0; kk < 8; ++kk) {
       const float4* f4 = reinterpret_cast<const float4*>(Fs + (k0 + kk) * R);
 #pragma unroll
       for (int c = 0; c < R / 4; ++c) {
         const float4 f = f4[c];
-        acc0[4 * c] = fmaf(x0[kk], f.x, acc0[4 * c]); acc0[4 * c + 1] = fmaf(x0[kk], f.y, acc0[4 * c + 1]);
-        acc0[4 * c + 2] = fmaf(x0[kk], f.z, acc0[4 * c + 2]); acc0[4 * c + 3] = fmaf(x0[kk], f.w, acc0[4 * c + 3]);
-        acc1[4 * c] = fmaf(x1[kk], f.x, acc1[4 * c]); acc1[4 * c + 1] = fmaf(x1[kk], f.y, acc1[4 * c + 1]);
-        acc1[4 * c + 2] = fmaf(x1[kk], f.z, acc1[4 * c + 2]); acc1[4 * c + 3] = fmaf(x1[kk], f.w, acc1[4 * c + 3]);
+#pragma unroll
+        for (int u = 0; u < kRows; ++u) {
+          const float2 xx = make_float2(x[u][kk], x[u][kk]);
+          acc2[u][2 * c] = __ffma2_rn(xx, make_float2(f.x, f.y), acc2[u][2 * c]);
+          acc2[u][2 * c + 1] = __ffma2_rn(xx, make_float2(f.z, f.w), acc2[u][2 * c + 1]);
+        }
       }
     }
+#pragma unroll
+    for (int u = 0; u < kRows; ++u)
+#pragma unroll
+      for (int k = 0; k < 8; ++k) x[u][k] = nx[u][k];
   }
   float m = 0.f;
   bool bad = false;
-  auto finish = [&](float (&acc)[R], int row, bool valid) {
-    if (!valid) return;
+#pragma unroll
+  for (int u = 0; u < kRows; ++u) {
+    const int row = row0 + u * blockDim.x;
+    if (row >= N) continue;
+    float acc[R];
+#pragma unroll
+    for (int c = 0; c < R; c += 2) { acc[c] = acc2[u][c / 2].x; acc[c + 1] = acc2[u][c / 2].y; }
     if (RMS) {
       float ss = 0.f;
 #pragma unroll
@@ -223,22 +247,30 @@ __global__ void __launch_bounds__(128) k_project(const T* __restrict__ X, i64 sb
       m = fmaxf(m, fabsf(acc[c]));
       bad |= !(fabsf(acc[c]) <= 3.0e38f);
     }
-  };
-  finish(acc0, row0, v0);
-  finish(acc1, row1, v1);
+  }
   m = warp_max(m);
   if ((threadIdx.x & 31) == 0) atomicMax(maxabs_bits + bh, __float_as_uint(m));
   if (bad) set_error(err, SPARSEPR_ERR_NUMERIC);
 }
 
+template <typename T, int D, int R, bool RMS>
+static void project_rows(const T* X, const i64* xs, int BH, int H, int N, int r, const float* F, float eps,
+                         float* phi, int ldphi, unsigned* maxabs, int* err, cudaStream_t st) {
+  // up to 4 CTAs of 64 rows per SM one row per thread, above two, which halve the reads of F per multiply-add (48 and 64 outputs in
+  // turn, us): 2 x 4096 rows, d = 64: 9.4 and 12.1 against 14.6 and 17.5 with two; 2 x 20000 rows, d = 128: 31.5 and 38.6 against
+  // 32.3 and 41.0; 8 x 7161 rows, d = 128: 42.0 and 62.5 against 33.3 and 42.0
+  if ((i64)BH * N <= 4 * 148 * 64)
+    k_project<T, D, R, RMS, 1><<<dim3((N + 63) / 64, BH), 64, 0, st>>>(X, xs[0], xs[1], xs[2], H, N, r, F, eps, phi, ldphi, maxabs, err);
+  else
+    k_project<T, D, R, RMS, 2><<<dim3((N + 255) / 256, BH), 128, 0, st>>>(X, xs[0], xs[1], xs[2], H, N, r, F, eps, phi, ldphi, maxabs, err);
+}
 template <typename T, int D, bool RMS>
 static void project_dispatch_r(const T* X, const i64* xs, int BH, int H, int N, int r, const float* F, float eps,
                                float* phi, int ldphi, unsigned* maxabs, int* err, cudaStream_t st) {
-  dim3 grid((N + 255) / 256, BH);
-  if (r <= 16) k_project<T, D, 16, RMS><<<grid, 128, 0, st>>>(X, xs[0], xs[1], xs[2], H, N, r, F, eps, phi, ldphi, maxabs, err);
-  else if (r <= 32) k_project<T, D, 32, RMS><<<grid, 128, 0, st>>>(X, xs[0], xs[1], xs[2], H, N, r, F, eps, phi, ldphi, maxabs, err);
-  else if (r <= 48) k_project<T, D, 48, RMS><<<grid, 128, 0, st>>>(X, xs[0], xs[1], xs[2], H, N, r, F, eps, phi, ldphi, maxabs, err);
-  else k_project<T, D, 64, RMS><<<grid, 128, 0, st>>>(X, xs[0], xs[1], xs[2], H, N, r, F, eps, phi, ldphi, maxabs, err);
+  if (r <= 16) project_rows<T, D, 16, RMS>(X, xs, BH, H, N, r, F, eps, phi, ldphi, maxabs, err, st);
+  else if (r <= 32) project_rows<T, D, 32, RMS>(X, xs, BH, H, N, r, F, eps, phi, ldphi, maxabs, err, st);
+  else if (r <= 48) project_rows<T, D, 48, RMS>(X, xs, BH, H, N, r, F, eps, phi, ldphi, maxabs, err, st);
+  else project_rows<T, D, 64, RMS>(X, xs, BH, H, N, r, F, eps, phi, ldphi, maxabs, err, st);
 }
 void launch_project(int dtype, const void* X, const i64* xs, int BH, int H, int N, int d, int r, const float* F,
                     bool rms, float eps, float* phi, int ldphi, unsigned* maxabs, int* err, cudaStream_t st) {
