@@ -350,10 +350,10 @@ struct AttendWs {
   int n_split;
 };
 
-// float32: at most two CTAs per SM in one wave, and two key tiles of 64 per slice where that leaves the GPU idle (with four, 32 of
-// the 148 SMs worked at 2 heads of 4096 tokens)
+// Key slices of the float32 probe rows (16-bit tensors: n_split_tc): one wave of at most two CTAs per SM, and no less than two key
+// tiles of 64 per slice (with four, 32 of the 148 SMs worked at 2 heads of 4096 tokens).
 int probe_splits(const Resolved& r) {
-  if (r.M == 0) return 1;
+  if (r.M == 0 || r.dtype != SPARSEPR_F32) return 1;
   const int row_tiles = (r.M + 31) / 32, key_tiles = (r.N + 63) / 64;
   return std::max(1, std::min(2 * sm_count() / (r.BH * row_tiles), key_tiles / 2));
 }
