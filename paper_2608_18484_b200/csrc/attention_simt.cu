@@ -378,51 +378,74 @@ __global__ void __launch_bounds__(kItemBuckets) k_f32_items(const int* __restric
   if (threadIdx.x == 0) *n_items = total;
 }
 
-// Residual correction of Eq. 9 in place: O <- X + X A + c for the rows X = O (float32).  A CTA takes 32 rows of a head; A is
-// read through L2, thread (ty, tx) = 4 rows x D / 16 columns.
+// Residual correction of Eq. 9 in place: O <- X + X A + c for the rows X = O (float32).  A CTA takes 32 rows of a head, thread
+// (ty, tx) 4 of them x D / 16 columns, two columns to a multiply-add.  Bound by the FMA pipe: A comes through shared memory, 16 of
+// its rows under the arithmetic of the 16 before.  With A read through L2 and single multiply-adds 8 heads of 7161 rows, d = 128,
+// took 103 us, now 45 (64 rows per CTA: 46); 2 of 4096 rows, d = 64, 11.6, now 4.6 (4.8).
+constexpr int kCorrK = 16;
 template <int D>
 __global__ void __launch_bounds__(128) k_correction_f32(const float* __restrict__ A, const float* __restrict__ cvec, int H, int N,
                                                         float* __restrict__ O, i64 ob, i64 oh, i64 on) {
-  __shared__ __align__(16) float xs[32][D + 4];
-  const int bh = blockIdx.y, row0 = blockIdx.x * 32, nr = min(32, N - row0);
+  constexpr int R = 4, ld = D + 4, OP = D / 32;
+  __shared__ __align__(16) float xs[8 * R * ld], as[2 * kCorrK * D];
+  const int bh = blockIdx.y, row0 = blockIdx.x * 8 * R, nr = min(8 * R, N - row0);
   const int tid = threadIdx.x, ty = tid >> 4, tx = tid & 15;
   float* Ob = O + (bh / H) * ob + (bh % H) * oh;
-  for (int e = tid; e < 32 * (D / 4); e += 128) {
+  const float* Ah = A + (i64)bh * D * D;
+  auto fetch = [&](int k0) {
+    float* dst = as + (k0 / kCorrK & 1) * kCorrK * D;
+#pragma unroll
+    for (int e = tid * 4; e < kCorrK * D; e += 512) cp16(dst + e, Ah + k0 * D + e, true);
+    asm volatile("cp.async.commit_group;" ::: "memory");
+  };
+#pragma unroll 8
+  for (int e = tid; e < 8 * R * (D / 4); e += 128) {
     const int r = e / (D / 4), c = (e % (D / 4)) * 4;
-    *reinterpret_cast<float4*>(&xs[r][c]) = r < nr ? *reinterpret_cast<const float4*>(Ob + (i64)(row0 + r) * on + c) : make_float4(0.f, 0.f, 0.f, 0.f);
+    cp16(xs + r * ld + c, Ob + (i64)(row0 + min(r, nr - 1)) * on + c, r < nr);
   }
-  __syncthreads();
-  const float* Ah = A + (i64)bh * D * D + 4 * tx;
-  float acc[4][D / 16];
+  fetch(0);
+  float2 acc[R][OP];
 #pragma unroll
-  for (int i = 0; i < 4; ++i)
+  for (int i = 0; i < R; ++i)
 #pragma unroll
-    for (int c = 0; c < D / 16; ++c) acc[i][c] = 0.f;
-#pragma unroll 4
-  for (int k = 0; k < D; ++k) {
-    float x[4];
+    for (int c = 0; c < OP; ++c) acc[i][c] = make_float2(0.f, 0.f);
+  for (int k0 = 0; k0 < D; k0 += kCorrK) {
+    asm volatile("cp.async.wait_group 0;" ::: "memory");
+    __syncthreads();                                     // this chunk is there, the one before is consumed
+    if (k0 + kCorrK < D) fetch(k0 + kCorrK);
+    const float* ac = as + (k0 / kCorrK & 1) * kCorrK * D + 4 * tx;
+#pragma unroll 2
+    for (int k = 0; k < kCorrK; k += 4) {
+      float x[R][4];
 #pragma unroll
-    for (int i = 0; i < 4; ++i) x[i] = xs[ty * 4 + i][k];
-#pragma unroll
-    for (int c = 0; c < D / 64; ++c) {
-      const float4 v = __ldg(reinterpret_cast<const float4*>(Ah + (i64)k * D + 64 * c));
-#pragma unroll
-      for (int i = 0; i < 4; ++i) {
-        acc[i][4 * c] = fmaf(x[i], v.x, acc[i][4 * c]); acc[i][4 * c + 1] = fmaf(x[i], v.y, acc[i][4 * c + 1]);
-        acc[i][4 * c + 2] = fmaf(x[i], v.z, acc[i][4 * c + 2]); acc[i][4 * c + 3] = fmaf(x[i], v.w, acc[i][4 * c + 3]);
+      for (int i = 0; i < R; ++i) {
+        const float4 v = *reinterpret_cast<const float4*>(xs + (ty * R + i) * ld + k0 + k);
+        x[i][0] = v.x; x[i][1] = v.y; x[i][2] = v.z; x[i][3] = v.w;
       }
+#pragma unroll
+      for (int u = 0; u < 4; ++u)
+#pragma unroll
+        for (int c = 0; c < OP / 2; ++c) {
+          const float4 v = *reinterpret_cast<const float4*>(ac + (k + u) * D + 64 * c);
+#pragma unroll
+          for (int i = 0; i < R; ++i) {
+            const float2 xx = make_float2(x[i][u], x[i][u]);
+            acc[i][2 * c] = __ffma2_rn(xx, make_float2(v.x, v.y), acc[i][2 * c]);
+            acc[i][2 * c + 1] = __ffma2_rn(xx, make_float2(v.z, v.w), acc[i][2 * c + 1]);
+          }
+        }
     }
   }
 #pragma unroll
-  for (int c = 0; c < D / 64; ++c) {
+  for (int c = 0; c < OP / 2; ++c) {
     const float4 cv = *reinterpret_cast<const float4*>(cvec + (i64)bh * D + 64 * c + 4 * tx);
 #pragma unroll
-    for (int i = 0; i < 4; ++i) {
-      const int r = ty * 4 + i;
+    for (int i = 0; i < R; ++i) {
+      const int r = ty * R + i;
       if (r >= nr) continue;
-      const float4 x = *reinterpret_cast<const float4*>(&xs[r][64 * c + 4 * tx]);
+      const float4 x = *reinterpret_cast<const float4*>(xs + r * ld + 64 * c + 4 * tx);
       *reinterpret_cast<float4*>(Ob + (i64)(row0 + r) * on + 64 * c + 4 * tx) =
-          make_float4(x.x + (cv.x + acc[i][4 * c]), x.y + (cv.y + acc[i][4 * c + 1]), x.z + (cv.z + acc[i][4 * c + 2]), x.w + (cv.w + acc[i][4 * c + 3]));
+          make_float4(x.x + (cv.x + acc[i][2 * c].x), x.y + (cv.y + acc[i][2 * c].y), x.z + (cv.z + acc[i][2 * c + 1].x), x.w + (cv.w + acc[i][2 * c + 1].y));
     }
   }
 }
@@ -742,8 +765,8 @@ __global__ void __launch_bounds__(kFThreads, 2) k_probe_rows(ProbeArgs a) {
 }
 
 // merge the split states; one warp per probe row.  Bound by latency: the maxima are found by the lanes side by side, and the
-// numerators of four slices are on their way at a time (on the two calls above 13 -> 9 us with 16 -> 32 slices, and 56 -> 31 us;
-// eight at a time cost the calls of few slices more than they gained: 20 -> 26 us at 4 slices of 32 heads).
+// numerators of four slices are on their way at a time (on the two calls above 13 us with 16 slices -> 12 with 32, and 56 -> 32 us;
+// eight at a time: 9 and 31 us, but 20 -> 26 us at 4 slices of 32 heads).
 template <int D>
 __global__ void __launch_bounds__(256) k_probe_merge(const float* __restrict__ partial, int n_split, int M,
                                                      float* __restrict__ X, float* __restrict__ Dn) {
