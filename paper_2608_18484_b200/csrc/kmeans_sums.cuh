@@ -21,6 +21,22 @@ struct GroupMean {
     return (float)fma(fma(-q, n, a), y, q);
   }
 };
+// Squared norms of four rows by a warp, of each of which a lane has two columns (zeros beyond the row): in float64, rounded once.  A lane gets the
+// norm of row lane / 8: at the first two levels of the butterfly it keeps half of the rows that it has.
+__device__ __forceinline__ float norms_of_four(const float2 (&v)[4], int lane) {
+  double s[4];
+#pragma unroll
+  for (int b = 0; b < 4; ++b) s[b] = (double)v[b].x * (double)v[b].x + (double)v[b].y * (double)v[b].y;
+#pragma unroll
+  for (int half = 2; half > 0; half >>= 1) {
+    const bool upper = lane & (8 * half);
+#pragma unroll
+    for (int b = 0; b < half; ++b) s[b] = (upper ? s[b + half] : s[b]) + __shfl_xor_sync(0xffffffffu, upper ? s[b] : s[b + half], 8 * half);
+  }
+#pragma unroll
+  for (int o = 4; o > 0; o >>= 1) s[0] += __shfl_xor_sync(0xffffffffu, s[0], o);
+  return (float)s[0];
+}
 // the three bf16 words of ||mu_c||^2 (all bits of a float32), then zeros: a row of the operand of the norm step
 __device__ __forceinline__ uint4 norm_words(float v) {
   const __nv_bfloat16 w0 = __float2bfloat16_rn(v);

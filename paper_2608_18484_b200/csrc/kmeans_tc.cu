@@ -724,14 +724,17 @@ k_kmeans_run(const __grid_constant__ CUtensorMap mapXh, const __grid_constant__ 
           v[b] = t > 1 ? *reinterpret_cast<const float2*>(values + c * LDM + k) : *reinterpret_cast<const float2*>(prm.mu + ((i64)bh * C + c) * R + k);
         }
       }
-      float n2[kB];
 #pragma unroll
       for (int b = 0; b < kB; ++b) {                           // (no branches: the chains of the four run side by side)
         const GroupMean mean(max(cnt[b], 1), inv_sc);
         const float mx0 = mean(sv[b].x), mx1 = mean(sv[b].y);
         v[b].x = cnt[b] > 0 ? mx0 : v[b].x; v[b].y = cnt[b] > 0 ? mx1 : v[b].y;
-        n2[b] = warp_sum(fmaf(v[b].x, v[b].x, v[b].y * v[b].y));             // (7 roundings: 4.2e-7 of it, inside what km_score_error allows for accumulation)
-        mx = fmaxf(mx, n2[b]);
+      }
+      const float n2 = norms_of_four(v, lane);                 // of centroid lane / 8 of the four
+      mx = fmaxf(mx, n2);
+      if ((lane & 7) == 0 && c0 + lane / 8 * kWarps < C) {
+        const int c = c0 + lane / 8 * kWarps;
+        *reinterpret_cast<uint4*>(sm + mu_area + (c / kKmChunk) * kMuStage + 2 * kMuBytes + c % kKmChunk * 16) = norm_words(n2);
       }
 #pragma unroll
       for (int b = 0; b < kB; ++b) {
@@ -743,11 +746,11 @@ k_kmeans_run(const __grid_constant__ CUtensorMap mapXh, const __grid_constant__ 
         const int cc = c % kKmChunk, off = cc * 128 + (((k >> 3) ^ (cc & 7)) << 4) + (k & 7) * 2;      // rows of 128 bytes, 128-byte swizzle
         *reinterpret_cast<uint32_t*>(st + off) = hi;
         *reinterpret_cast<uint32_t*>(st + kMuBytes + off) = lo;
-        if (lane == 0) *reinterpret_cast<uint4*>(st + 2 * kMuBytes + cc * 16) = norm_words(n2[b]);
       }
     }
     __syncwarp();
     cluster_arrive_relaxed();                                  // this warp has read the sums (they are in registers: nothing to be released)
+    mx = warp_max(mx);
     if (lane == 0) s_max[warp] = mx;
     fence_async_smem();                                        // the tensor cores read the operands
     __syncthreads();
