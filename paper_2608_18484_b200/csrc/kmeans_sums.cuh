@@ -7,7 +7,8 @@ namespace spr {
 // Mean of a group from its fixed-point sum (inv_scale = 2^-shift): the definition of an updated centroid
 __device__ __forceinline__ float group_mean(i64 sum, double inv_scale, int count) { return (float)((double)sum * inv_scale / (double)count); }
 
-// The same, to the bit, for several sums of one group: quotients by a reciprocal y of the count and one correction.  a / n lies at least 2^-54 / n away
+// The same, to the bit, for several sums of one group: a reciprocal y of the count by Newton-Raphson steps, and quotients with one correction by
+// their remainder (Markstein, "Computation of elementary functions on the IBM RISC System/6000 processor", 1990).  a / n lies at least 2^-54 / n away
 // (relatively) from any midpoint between two float64 that is not itself, n < 2^31, and q + (a - q n) y, the remainder being exact, misses it by 2^-104.
 struct GroupMean {
   double scale, n, y;
