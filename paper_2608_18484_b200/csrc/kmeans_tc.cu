@@ -581,8 +581,8 @@ static size_t recheck_staged_smem(int C, int R) { return ((size_t)C * (R + 4) + 
 // Every thread of the cluster meets the same barriers whatever happens: an abort only skips the work in between, and the end of the iteration is read
 // from a counter that all of them see behind a barrier.
 // A pass at two heads of 4770 rows is 15 k cycles: centroids 3, products and decisions of three tiles 5.5, recheck of a row or two 3, barriers 3; its
-// first pass 25.  Runs of eight passes, us, in separate launches and here: 2 heads of 4770 rows and 38 centroids 132, 70; 2 of 4096 float32 rows and 64
-// centroids 143, 76; 8 of 7161 rows and 112 centroids 228, 178.
+// first pass 25.  Runs of eight passes, us, in separate launches and here: 2 heads of 4770 rows and 38 centroids 132, 72; 2 of 4096 float32 rows and 64
+// centroids 143, 76; 8 of 7161 rows and 112 centroids 228, 176.
 constexpr int kKmRunList = 2048;                     // moved rows of a pass that are listed (the others go to the sums at once)
 constexpr int kKmRunSort = 48;                       // listed rows from which they are sorted
 constexpr int kKmRunTiles = 64;                      // row tiles per CTA (a row has 14 bits in the list)
@@ -748,17 +748,26 @@ k_kmeans_run(const __grid_constant__ CUtensorMap mapXh, const __grid_constant__ 
         *reinterpret_cast<uint32_t*>(st + kMuBytes + off) = lo;
       }
     }
-    __syncwarp();
-    cluster_arrive_relaxed();                                  // this warp has read the sums (they are in registers: nothing to be released)
     mx = warp_max(mx);
     if (lane == 0) s_max[warp] = mx;
     fence_async_smem();                                        // the tensor cores read the operands
     __syncthreads();
+    // Every warp has read the sums; they may change once all CTAs have.  One warp's release carries the reads of all, which lie before the barrier
+    // above: that of the producer, which has nothing to load in most passes.  The others wait for the cluster when their first product is under way
+    // or read: in front of the moves, and of the prefetches for the recheck (waiting empties the first-level cache).  Runs of keys and queries, us, so,
+    // with the wait behind all products, and with a release and the wait in front of them: 2 heads of 4770 rows 72 and 78, 73 and 80, 73 and 80; 8 of
+    // 7161 float32 rows 168 and 184, 171 and 186, 173 and 190; 16 of 17550 rows, d = 64, 344 and 363, 344 and 364, 352 and 375.
+    if (warp == kKmEpiWarps) cluster_arrive(); else cluster_arrive_relaxed();
+    bool may_move = false;                                     // this warp has waited for the cluster
+    const auto wait_for_cluster = [&] {
+      __syncwarp();
+      if (!may_move) cluster_wait();                           // (uniform)
+      may_move = true;
+    };
     float mm = s_max[0];                                       // largest centroid norm of the head, rounded up
 #pragma unroll
     for (int w = 1; w < kWarps; ++w) mm = fmaxf(mm, s_max[w]);
     mm = sqrtf(mm) * 1.000001f;
-    cluster_wait();                                            // all CTAs have read the sums: they may change
     const bool upd = t < prm.T;                                // the last pass needs no sums
     const int* old = t > 1 ? assign : prm.old != nullptr ? prm.old + hrow0 : nullptr;
     const bool first = old == nullptr;                         // no row is in a group yet: the sums are formed from all rows behind the pass
@@ -774,6 +783,7 @@ k_kmeans_run(const __grid_constant__ CUtensorMap mapXh, const __grid_constant__ 
           tma_load_4d(base + KmSmem::x + xs * 2 * kXBytes + kXBytes, &mapXl, bar(X_FULL + xs), 0, row0 + tl * 128, bh, 0);
         }
       }
+      wait_for_cluster();
     } else if (warp > kKmEpiWarps) {
       // =========================== MMA issuers (one per group) ================================
       const int g = warp - (kKmEpiWarps + 1), ksteps = R / 16;
@@ -801,6 +811,7 @@ k_kmeans_run(const __grid_constant__ CUtensorMap mapXh, const __grid_constant__ 
           }
           __syncwarp();
         }
+        wait_for_cluster();
       }
     } else {
       // =========================== epilogue: argmin ===========================================
@@ -836,6 +847,7 @@ k_kmeans_run(const __grid_constant__ CUtensorMap mapXh, const __grid_constant__ 
         }
         float best, second;
         int bi;
+        wait_for_cluster();
         scan.result(best, second, bi);
         km_exchange(xb + ((grp * 2 + ((tl >> 1) & 1)) * 2) * 128 + wq * 32 + lane, hh, 1 + grp * 4 + wq, best, second, bi);
         bi = min(bi, C - 1);                                   // (only rows of non-finite scores could point past C)
@@ -862,6 +874,7 @@ k_kmeans_run(const __grid_constant__ CUtensorMap mapXh, const __grid_constant__ 
     }
     __syncthreads();
     if (*abort_flag) tiles = 0;                                // (the same for all threads: nobody waits now)
+    wait_for_cluster();
     const int n_flagged = tiles ? s_flagged : 0, n_moved = tiles ? min(s_moved, kKmRunList) : 0;
     const bool sorted = n_moved > kKmRunSort;
     // ---- exact decisions for the rows that are left, by the epilogue warps; moves row by row, the last warps first
