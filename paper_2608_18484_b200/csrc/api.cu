@@ -745,15 +745,15 @@ static sparsepr_status_t attend_impl(const sparsepr_plan_t* p, const void* Q, co
   // they run on the plan's second stream beside the block-sparse kernel, from the end of the selection on (the lists of tiles are made
   // meanwhile); a profiled call keeps everything on one stream so that stage times add up.
   const bool fitted = r.mode == 0 && r.M > 0, overlap = fitted && prof == nullptr;
+  const bool third = overlap && r.dtype == SPARSEPR_BF16;       // float32 calls have nothing for the third stream, and would not join it
   bool named = false;
   if (!find_routes(p, st, &named)) return SPARSEPR_ERR_CUDA;
-  if (overlap) {
-    fork_side(p, st);
-    cudaStreamWaitEvent(p->side2, p->ev_fork, 0);
-  }
+  if (overlap) fork_side(p, st);
+  if (third) cudaStreamWaitEvent(p->side2, p->ev_fork, 0);
   if (named) {
     cudaStreamWaitEvent(st, p->ev_route, 0);
-    if (overlap) { cudaStreamWaitEvent(p->side, p->ev_select, 0); cudaStreamWaitEvent(p->side2, p->ev_route, 0); }
+    if (overlap) cudaStreamWaitEvent(p->side, p->ev_select, 0);
+    if (third) cudaStreamWaitEvent(p->side2, p->ev_route, 0);
   }
   tm.mark(SPARSEPR_STAGE_GATHER);
   AttnArgs aa{};
