@@ -256,10 +256,13 @@ __global__ void __launch_bounds__(128) k_project(const T* __restrict__ X, i64 sb
 template <typename T, int D, int R, bool RMS>
 static void project_rows(const T* X, const i64* xs, int BH, int H, int N, int r, const float* F, float eps,
                          float* phi, int ldphi, unsigned* maxabs, int* err, cudaStream_t st) {
-  // up to 4 CTAs of 64 rows per SM one row per thread, above two, which halve the reads of F per multiply-add (48 and 64 outputs in
-  // turn, us): 2 x 4096 rows, d = 64: 9.4 and 12.1 against 14.6 and 17.5 with two; 2 x 20000 rows, d = 128: 31.5 and 38.6 against
-  // 32.3 and 41.0; 8 x 7161 rows, d = 128: 42.0 and 62.5 against 33.3 and 42.0
-  if ((i64)BH * N <= 4 * 148 * 64)
+  // One row per thread or two, which halve the reads of F per multiply-add: a call takes as long as the CTAs that one SM gets, and one more of 64 rows
+  // costs 2 / 5 of one more of 256.  Measured, us, one row against two, float32, d = 128 with 64 outputs: 2 x 9251 rows (2 CTAs of 64 on an SM, 1 of 256)
+  // 25.5, 29.2; 2 x 10001 (3, 1) 29.6, 28.9; 2 x 18001 (4, 1) 35.7, 29.5; 32 x 1126 (4, 2) 35.3, 43.9; 2 x 20001 (5, 2) 41.8, 43.7; 2 x 25001 (6, 2) 48.0,
+  // 43.9; 8 x 10001 (9, 3) 80.8, 62.6.  d = 64 with 48: 2 x 4001 (1, 1) 12.6, 14.6; 2 x 18001 (4, 1) 19.4, 15.5; 2 x 20001 (5, 2) 21.5, 23.5; 2 x 25001 (6, 2)
+  // 23.6, 23.5; with 16 outputs the two differ by a microsecond or two.
+  const i64 sms = sm_count(), one = ((i64)BH * ((N + 63) / 64) + sms - 1) / sms, two = ((i64)BH * ((N + 255) / 256) + sms - 1) / sms;
+  if (2 * one <= 5 * two)
     k_project<T, D, R, RMS, 1><<<dim3((N + 63) / 64, BH), 64, 0, st>>>(X, xs[0], xs[1], xs[2], H, N, r, F, eps, phi, ldphi, maxabs, err);
   else
     k_project<T, D, R, RMS, 2><<<dim3((N + 255) / 256, BH), 128, 0, st>>>(X, xs[0], xs[1], xs[2], H, N, r, F, eps, phi, ldphi, maxabs, err);
