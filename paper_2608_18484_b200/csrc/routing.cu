@@ -400,8 +400,8 @@ __global__ void __launch_bounds__(kRouteThreads) k_route_select(const float* __r
 // their cells lane + 32 j.  What the kernel above spends on such a head is mostly set-up of its histograms; here the threshold is found by bisection of
 // the bit pattern, a step of which is two additions per cell and one barrier, until a warp can order what is left (two sums of 48 cycles each over a
 // warp make the step, not the cells).  A cell that can be taken has the key bits + 1, any other 0.
-// The kernel above / this one, us, alone: 2 heads of 38 groups 25 / 14, 2 of 64 28 / 16, 8 of 112 51 / 26, 16 of 138 69 / 46.  Beyond 160 groups the
-// matrix no longer fits the registers.
+// The kernel above / this one, us, alone: 2 heads of 38 groups 25 / 14, 2 of 64 28 / 16, 8 of 112 51 / 26, 16 of 138 69 / 46.  For more than
+// 128 groups the matrix takes 50 of a thread's 128 registers and 136 bytes of the rest are spilled; beyond 160 the kernel above.
 constexpr int kRouteSmallWarps = 16, kRouteSmallThreads = 32 * kRouteSmallWarps;
 __device__ __forceinline__ i64 warp_sum_cost(i64 v) {           // v >= 0, by 32-bit reductions of 22 bits each
   const u64 x = (u64)v;
