@@ -379,9 +379,9 @@ __global__ void __launch_bounds__(kItemBuckets) k_f32_items(const int* __restric
 }
 
 // Residual correction of Eq. 9 in place: O <- X + X A + c for the rows X = O (float32).  A CTA takes 32 rows of a head, thread
-// (ty, tx) 4 of them x D / 16 columns, two columns to a multiply-add.  Bound by the FMA pipe: A comes through shared memory, 16 of
-// its rows under the arithmetic of the 16 before.  With A read through L2 and single multiply-adds 8 heads of 7161 rows, d = 128,
-// took 103 us, now 45 (64 rows per CTA: 46); 2 of 4096 rows, d = 64, 11.6, now 4.6 (4.8).
+// (ty, tx) 4 of them x D / 16 columns, two columns to a multiply-add.  Bound by reads of shared memory (85 % of their rate, FMA pipe 64 %, at
+// 8 heads of 7161 rows, d = 128): A comes through it, 16 of its rows under the arithmetic of the 16 before.  With A read through L2 and
+// single multiply-adds that call took 103 us, now 45 (64 rows per CTA: 46); 2 heads of 4096 rows, d = 64, 11.6, now 4.6 (4.8).
 constexpr int kCorrK = 16;
 template <int D>
 __global__ void __launch_bounds__(128) k_correction_f32(const float* __restrict__ A, const float* __restrict__ cvec, int H, int N,
@@ -536,7 +536,8 @@ void launch_attention_f32(const AttnArgs& a, float* part, int* counter, cudaStre
 // The key range is split across CTAs; partial states are merged afterwards.
 // partial layout: [BH][n_split][M][2][D+2] = (m, l, N[D]) for the S and the U state.
 //
-// Bound by the FMA pipe on large calls, by the chain of a CTA's few key tiles on small ones.  A key belongs to one of a row's
+// Bound by the latency of a few warps' dependent steps: two CTAs to an SM leave two warps to a scheduler, which issue in 39 % of the
+// cycles (FMA pipe 43 %, shared memory 57 %, at 8 heads of 7161 tokens, d = 128).  A key belongs to one of a row's
 // two states, and keys are group-major, so both states change hands only where a K/V group ends: a thread multiplies into the
 // row's current state and swaps it with the other one there, which is one product with V per key instead of two.  32 rows per
 // CTA (both states of four rows and the scores fit a thread's registers), packed 4 x 4 score blocks; K of the next tile

@@ -164,9 +164,9 @@ void launch_centroid_gram(const float* kappa, const int* n, int BH, int C, int d
 // (Eq. 7).  Each thread produces kRows rows of R outputs; F is staged in shared
 // memory and read by broadcast.  Also tracks max |phi| per head (for the
 // fixed-point centroid sums) and flags non-finite values.
-// Bound by the latency of its loads on small calls and by the FMA pipe on large ones: multiply-adds of two columns to an
-// instruction, and the next eight values of a row are fetched under those of the last eight (24 heads of 16000 rows, d = 128, 64
-// outputs: 261 -> 210 us).
+// Bound by latency on small calls and by reads of F from shared memory on large ones (8 heads of 7161 rows, d = 128, 64 outputs: 224 CTAs, shared memory
+// 68 % of its rate while one is on an SM, FMA pipe 38 %): multiply-adds of two columns to an instruction, and the next eight values of a row are
+// fetched under those of the last eight (24 heads of 16000 rows, d = 128, 64 outputs: 261 -> 210 us).
 // =============================================================================
 template <typename T, int D, int R, bool RMS, int kRows>
 __global__ void __launch_bounds__(128) k_project(const T* __restrict__ X, i64 sb, i64 sh, i64 sn, int H, int N, int r,
